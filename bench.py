@@ -547,10 +547,13 @@ def gemv_copies(mats) -> int:
 
 
 def gemv_kernel_names(mats, B: int) -> str:
-    """The kernels wq4_gemv's size rule picks for the set (batch 1-2, K % 256 == 0)."""
+    """The kernels wq4_gemv's size rules pick for the set (K % 256 == 0)."""
     names = []
     for _, N, K in mats:
-        k = "gemv_mma_kernel" if B <= 2 and K % 256 == 0 and N * K >= 12 << 20 else "gemv_tma_kernel"
+        if B > 2 or (B == 2 and N * K >= 8 << 20):
+            k = "bgemv_tma_kernel"
+        else:
+            k = "gemv_mma_kernel" if B == 1 and N * K >= 12 << 20 else "gemv_tma_kernel"
         if k not in names:
             names.append(k)
     return "+".join(names)
@@ -562,7 +565,7 @@ def gemv_io_bytes(mats, B: int) -> int:
 
 def gemv_source_sha() -> str:
     h = hashlib.sha256()
-    for f in ("wq4_gemv.cu", "wq4_items.cuh", "wq4_device.cuh"):
+    for f in ("wq4_gemv.cu", "wq4_bgemv.cu", "wq4_items.cuh", "wq4_device.cuh"):
         h.update(open(os.path.join(ROOT, "paper_2412_15803_gb300", "csrc", f), "rb").read())
     return h.hexdigest()[:16]
 

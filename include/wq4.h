@@ -68,9 +68,11 @@ enum wq4_status {
  * memory).
  *   W_packed : uint32 [N][K/8], 16-byte aligned.
  *   scales   : fp16 bits [N][K/32], 2-byte aligned (16-byte aligned and
- *              K % 256 == 0 select the TMA-staged fast paths: at batch 1-2
- *              from 12 Mi weights the legacy-tensor-path kernel, exact in
- *              fp16 products with fp32 sums, else the CUDA-core one).
+ *              K % 256 == 0 select the TMA-staged fast paths: batch 1 from
+ *              12 Mi weights, batch 2 from 8 Mi and every larger batch run on
+ *              the legacy tensor path, exact in fp16 products with fp32 sums,
+ *              else the CUDA cores; other rows at batch 3 and up run on the
+ *              legacy tensor path too).
  *   x        : fp16 bits [batch][K], 16-byte aligned.
  *   y        : fp16 bits [batch][N], 2-byte aligned; must not overlap x, W or
  *              scales.
@@ -128,8 +130,8 @@ int wq4_pack_host(const uint8_t* q_host, uint32_t* W_host, int N, int K);
 /*
  * Test hook: which kernel wq4_gemv takes at batch 1-2 with K % 256 == 0 and
  * 16-byte aligned scales, for every later call in this process.  0 (the
- * default) picks by size (the legacy-tensor-path kernel from 12 Mi weights
- * up, the CUDA-core kernel below), 1 always the legacy-tensor-path kernel,
+ * default) picks by size (the legacy-tensor-path kernels from 12 Mi weights
+ * up, 8 Mi at batch 2, the CUDA-core kernel below), 1 always a legacy-tensor-path kernel,
  * 2 always the CUDA-core kernel.  Results agree within the tolerance; no
  * counterpart in the paper.  WQ4_ERR_INVALID for another value.
  */

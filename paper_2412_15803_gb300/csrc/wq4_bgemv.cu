@@ -1,0 +1,859 @@
+// wq4_bgemv.cu -- the fused dequantize x GEMV for several activation rows
+// (batch 3-32, and batch 1-2 where the TMA-staged kernels do not apply): one
+// decode step of a serving batch through one projection (Section 3, Table 1).
+//
+// y[b][n] = fp16( sum_k (q(n,k) - 7) * s[n][k/32] * x[b][k] )
+//
+// The contraction runs on mma.sync m16n8k16 with the activations as the 16
+// rows and eight weight rows as the columns: per 32-code group and tile of
+// eight rows two MMAs add the group's exact fp16 products (q - 7) x in fp32,
+// and the group's scales multiply the fp32 result into the running sums, so
+// no weight is ever rounded and every fp16 scale is valid.  (tcgen05 would
+// need the scale inside the fp16 operand, or one accumulator per group.)
+//
+// A CTA owns tiles of 8 R RG weight rows; its 16 warps are RG row groups of R
+// tiles times KS slices of every K chunk, and the slices' sums are added in
+// slice order in shared memory at the tile's end: the same inputs give the
+// same bits.  Chunks of KG groups (codes, scales, activations) move through a
+// four-stage cp.async ring; rows are padded so that ldmatrix of the codes and
+// the 16-byte loads of the activations are free of bank conflicts.  The next
+// tile's chunks are in flight while a tile is finished.
+//
+// Two forms: rows that tensor copies can take (K % 256 == 0, 16-byte aligned
+// scales) run in bgemv_tma_kernel below, others in bgemv_kernel.  Measured
+// (us a launch in a graph over rotated copies, before: CUDA-core kernels that
+// read the activations through L1): 3072 x 8192 batch 8 76.5 -> 6.8,
+// 16384 x 3072 batch 8 100 -> 9.0 and batch 32 387 -> 17.8, 128256 x 4096
+// batch 8 927 -> 56 (5.3 TB/s) and batch 32 3739 -> 136; 1003 x 2080 (copy
+// ring) batch 5 7.3 -> 4.1.  Up to batch 8 the wide shapes are bound by
+// instruction issue and HBM together, at batch 32 by the MMAs (two per tile,
+// group and eight activation rows) and their issue; the narrow ones by the
+// launch and a chunk's latency.
+#include "wq4.h"
+#include "wq4_device.cuh"
+#include "wq4_host.h"
+#include "wq4_items.cuh"
+#include "wq4_tc.cuh"
+
+#include <cuda_runtime.h>
+
+#include <algorithm>
+#include <atomic>
+
+namespace wq4 {
+namespace {
+
+constexpr int kBWarps = 16;
+constexpr int kBThreads = kBWarps * 32;
+constexpr int kBStages = 4;
+constexpr int kScaleRegs = 4;      // scales a thread carries per chunk (S2)
+
+struct BGemvParams {
+    const uint32_t* W;
+    const uint16_t* s;
+    const uint16_t* x;
+    uint16_t* y;
+    int N, K, batch;
+    int lkg;               // log2 of the groups per chunk
+    int ks, gpw;           // K slices, groups of a chunk per slice (even)
+    int tiles, nch;        // row tiles, chunks along K
+    uint32_t stage_bytes, scale_off, x_off, red_off;
+    int y4;                // two outputs may be stored at once
+};
+
+__device__ __forceinline__ void cp_async16(uint32_t dst, const void* src)
+{
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst), "l"(src) : "memory");
+}
+
+// Copies `bytes` (0 or 16) bytes and fills the rest of the 16 with zeros.
+__device__ __forceinline__ void cp_async16z(uint32_t dst, const void* src, uint32_t bytes)
+{
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(dst), "l"(src), "r"(bytes) : "memory");
+}
+
+__device__ __forceinline__ void cp_async4(uint32_t dst, const void* src)
+{
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(dst), "l"(src) : "memory");
+}
+
+__device__ __forceinline__ void cp_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
+
+template <int N>
+__device__ __forceinline__ void cp_wait()
+{
+    asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory");
+}
+
+__device__ __forceinline__ void ldsm_x4_b(uint32_t addr, uint32_t r[4])
+{
+    asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0, %1, %2, %3}, [%4];"
+                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3])
+                 : "r"(addr)
+                 : "memory");
+}
+
+// d += A B (m16n8k16, fp16 in, fp32 out); see mma_16816 for the fragments.
+__device__ __forceinline__ void mma_acc(float d[4], uint32_t a0, uint32_t a1, uint32_t a2, uint32_t a3, uint32_t b0,
+                                        uint32_t b1)
+{
+    const float c[4] = {d[0], d[1], d[2], d[3]};
+    mma_16816(d, a0, a1, a2, a3, b0, b1, c);
+}
+
+// XT: tiles of eight activation rows (batch <= 8 XT); R: tiles of eight
+// weight rows per warp; S2: scales at any 2-byte address (else copied in
+// 4-byte aligned pairs).
+template <int XT, int R, bool S2>
+__global__ void __launch_bounds__(kBThreads, 1) bgemv_kernel(const BGemvParams p)
+{
+    extern __shared__ __align__(1024) uint8_t smem[];
+    constexpr int MT = (XT + 1) / 2;                  // MMA row blocks of 16 activation rows
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int g = lane >> 2, c = lane & 3;
+    const int KG = 1 << p.lkg, G = p.K >> 5;
+    const int ks = p.ks, rgs = kBWarps / ks, TR = 8 * R * rgs;
+    const int rg = warp / ks, sl = warp - rg * ks;    // row group and K slice of this warp
+    const uint32_t cpitch = 16u * KG + 16u, spitch = 2u * KG + 16u, xpitch = 64u * KG + 64u;
+    const uint32_t smem0 = smem_addr(smem);
+    const int mytiles = (p.tiles - static_cast<int>(blockIdx.x) + static_cast<int>(gridDim.x) - 1) / static_cast<int>(gridDim.x);
+    const int total = mytiles * p.nch;
+
+    // ---- chunk loads: this thread's place in each copy is fixed; the row
+    // advances by a constant step
+    int lc = 0, ln0 = static_cast<int>(blockIdx.x) * TR, lstage = 0;
+    [[maybe_unused]] uint16_t sreg[S2 ? kScaleRegs : 1];
+    [[maybe_unused]] uint32_t sdst = 0;                                // stage the carried scales belong to
+    [[maybe_unused]] int sng = 0;
+    const size_t wrow = static_cast<size_t>(G) * 16, srow = static_cast<size_t>(G) * 2;
+    const int crow = tid >> p.lkg, ccol = tid & (KG - 1), cstep = kBThreads >> p.lkg;
+    constexpr int kLsg = S2 ? 0 : 1;                  // log2 of the scales per copy
+    const int lsu = p.lkg - kLsg;                     // log2 of the scale copies per row
+    const int qrow = tid >> lsu, qcol = (tid & ((1 << lsu) - 1)) << kLsg, qstep = kBThreads >> lsu;
+    const int xrow = tid >> (p.lkg + 2), xcol = tid & (4 * KG - 1), xstep = kBThreads >> (p.lkg + 2);
+    auto issue_w = [&](int stage, int n0, int ch) {
+        const uint32_t base = smem0 + stage * p.stage_bytes;
+        const int g0 = ch << p.lkg, ng = min(KG, G - g0), last = p.N - 1 - n0;   // rows past N repeat the last
+        if (ccol < ng) {
+            const uint8_t* src = reinterpret_cast<const uint8_t*>(p.W) + static_cast<size_t>(n0) * wrow + 16 * (g0 + ccol);
+            uint32_t dst = base + crow * cpitch + 16 * ccol;
+            for (int row = crow; row < TR; row += cstep, dst += cstep * cpitch)
+                cp_async16(dst, src + static_cast<size_t>(min(row, last)) * wrow);
+        }
+        const uint8_t* src = reinterpret_cast<const uint8_t*>(p.s) + static_cast<size_t>(n0) * srow + 2 * (g0 + qcol);
+        if constexpr (!S2) {
+            if (qcol < ng) {
+                uint32_t dst = base + p.scale_off + qrow * spitch + 2 * qcol;
+                for (int row = qrow; row < TR; row += qstep, dst += qstep * spitch)
+                    cp_async4(dst, src + static_cast<size_t>(min(row, last)) * srow);
+            }
+        } else {
+            // scales at any 2-byte address: through registers, stored one chunk later
+#pragma unroll
+            for (int q = 0; q < kScaleRegs; ++q) {
+                const int row = qrow + q * qstep;
+                if (row < TR && qcol < ng)
+                    sreg[q] = __ldg(reinterpret_cast<const uint16_t*>(src + static_cast<size_t>(min(row, last)) * srow));
+            }
+            sdst = base + p.scale_off + qrow * spitch + 2 * qcol;
+            sng = ng;
+        }
+    };
+    auto flush_scales = [&]() {
+        if constexpr (S2) {
+#pragma unroll
+            for (int q = 0; q < kScaleRegs; ++q) {
+                // an odd last group is paired with one of scale 0
+                if (qrow + q * qstep < TR && qcol < ((sng + 1) & ~1))
+                    asm volatile("st.shared.b16 [%0], %1;" ::"r"(sdst + q * qstep * spitch),
+                                 "h"(qcol < sng ? sreg[q] : static_cast<uint16_t>(0))
+                                 : "memory");
+            }
+            sng = 0;
+        }
+    };
+    auto issue_x = [&](int stage, int ch) {
+        const int g0 = ch << p.lkg, ng = min(KG, G - g0), xg = xcol >> 2;
+        if (xg >= ((ng + 1) & ~1)) return;
+        const uint32_t bytes = xg < ng ? 16u : 0u;     // an odd last group is paired with one of zeros
+        const uint8_t* src = reinterpret_cast<const uint8_t*>(p.x) + 64 * static_cast<size_t>(g0) + (xg < ng ? 16 * xcol : 0);
+        uint32_t dst = smem0 + stage * p.stage_bytes + p.x_off + xrow * xpitch + 16 * xcol;
+        for (int row = xrow; row < 8 * XT; row += xstep, dst += xstep * xpitch)   // rows past the batch repeat the last
+            cp_async16z(dst, src + static_cast<size_t>(min(row, p.batch - 1)) * (2 * static_cast<size_t>(p.K)), bytes);
+    };
+    auto advance = [&]() {
+        if (++lc == p.nch) {
+            lc = 0;
+            ln0 += static_cast<int>(gridDim.x) * TR;
+        }
+        lstage = (lstage + 1) & (kBStages - 1);
+    };
+
+    grid_dependents_launch();
+    // weights of the first chunks may be fetched while the previous kernel of
+    // the stream finishes; activations only after it (programmatic dependent launch)
+    {
+        int c1 = 0, n1 = ln0;
+        for (int i = 0; i < kBStages - 1 && i < total; ++i) {
+            issue_w(i, n1, c1);
+            flush_scales();
+            if (++c1 == p.nch) {
+                c1 = 0;
+                n1 += static_cast<int>(gridDim.x) * TR;
+            }
+        }
+    }
+    grid_dependency_wait();
+    for (int i = 0; i < kBStages - 1; ++i) {
+        if (i < total) {
+            issue_x(lstage, lc);
+            advance();
+        }
+        cp_commit();
+    }
+
+    // ---- this lane's shared-memory offsets within a stage
+    const int m = lane >> 3, lr = lane & 7;           // ldmatrix: matrix and row of this lane's address
+    uint32_t coff;
+    if (R == 1) coff = (8 * rg + lr) * cpitch + 16 * (m & 1);                          // groups j, j + 1
+    else if (R == 2) coff = (16 * rg + 8 * (m & 1) + lr) * cpitch + 16 * (m >> 1);     // 2 tiles x 2 groups
+    else coff = (8 * R * rg + 8 * min(m, R - 1) + lr) * cpitch;                        // R tiles of one group
+    const uint32_t soff = p.scale_off + (8 * R * rg + 2 * c) * spitch;
+    const uint32_t xoff = p.x_off + g * xpitch + 16 * c;
+    const int j0 = sl * p.gpw;
+
+    float acc[R][XT][2];
+#pragma unroll
+    for (int r = 0; r < R; ++r)
+#pragma unroll
+        for (int t = 0; t < XT; ++t) acc[r][t][0] = acc[r][t][1] = 0.f;
+
+    int ch = 0, stage = 0, n0 = static_cast<int>(blockIdx.x) * TR;
+    for (int f = 0; f < total; ++f) {
+        cp_wait<kBStages - 2>();
+        __syncthreads();
+        flush_scales();                                // of chunk f + 2: read three barriers after its load
+        if (f + kBStages - 1 < total) {
+            issue_w(lstage, ln0, lc);
+            issue_x(lstage, lc);
+            advance();
+        }
+        cp_commit();
+
+        const uint32_t base = smem0 + stage * p.stage_bytes;
+        const int ng = min(KG, G - (ch << p.lkg));
+        const int jend = min(j0 + p.gpw, ng);           // whole pairs: an odd last group has a zero partner
+        for (int j = j0; j < jend; j += 2) {
+            uint32_t sc0[R], sc1[R];                   // scales of groups j, j + 1: rows 2c and 2c + 1
+#pragma unroll
+            for (int r = 0; r < R; ++r) {
+                sc0[r] = lds_u32(base + soff + (8 * r) * spitch + 2 * j);
+                sc1[r] = lds_u32(base + soff + (8 * r + 1) * spitch + 2 * j);
+            }
+            uint32_t w[2][R > 2 ? 4 : 2];
+            if (R == 1) {
+                ldsm_x2(base + coff + 16 * j, w[0][0], w[1][0]);
+            } else if (R == 2) {
+                uint32_t t[4];
+                ldsm_x4_b(base + coff + 16 * j, t);
+                w[0][0] = t[0];
+                w[0][1] = t[1];
+                w[1][0] = t[2];
+                w[1][1] = t[3];
+            } else {
+                ldsm_x4_b(base + coff + 16 * j, w[0]);
+                ldsm_x4_b(base + coff + 16 * j + 16, w[1]);
+            }
+#pragma unroll
+            for (int h = 0; h < 2; ++h) {
+                uint4 v[2 * MT];
+#pragma unroll
+                for (int t = 0; t < XT; ++t) v[t] = pair_permute(lds_v4(base + xoff + (8 * t) * xpitch + 64 * (j + h)));
+                if (XT & 1) v[XT] = make_uint4(0u, 0u, 0u, 0u);
+#pragma unroll
+                for (int r = 0; r < R; ++r) {
+                    uint32_t q[4];
+                    unpack_word(w[h][r], q);
+                    const float s0 = h ? hi_f(sc0[r]) : lo_f(sc0[r]), s1 = h ? hi_f(sc1[r]) : lo_f(sc1[r]);
+#pragma unroll
+                    for (int mt = 0; mt < MT; ++mt) {
+                        float d[4] = {0.f, 0.f, 0.f, 0.f};
+                        mma_acc(d, v[2 * mt].x, v[2 * mt + 1].x, v[2 * mt].y, v[2 * mt + 1].y, q[0], q[1]);
+                        mma_acc(d, v[2 * mt].z, v[2 * mt + 1].z, v[2 * mt].w, v[2 * mt + 1].w, q[2], q[3]);
+                        acc[r][2 * mt][0] = fmaf(s0, d[0], acc[r][2 * mt][0]);
+                        acc[r][2 * mt][1] = fmaf(s1, d[1], acc[r][2 * mt][1]);
+                        if (2 * mt + 1 < XT) {
+                            acc[r][2 * mt + 1 < XT ? 2 * mt + 1 : 0][0] = fmaf(s0, d[2], acc[r][2 * mt + 1 < XT ? 2 * mt + 1 : 0][0]);
+                            acc[r][2 * mt + 1 < XT ? 2 * mt + 1 : 0][1] = fmaf(s1, d[3], acc[r][2 * mt + 1 < XT ? 2 * mt + 1 : 0][1]);
+                        }
+                    }
+                }
+            }
+        }
+        stage = (stage + 1) & (kBStages - 1);
+        if (++ch < p.nch) continue;
+
+        // ---- the tile is complete: lane (g, c) holds rows 8 r + 2c, + 1 of
+        // its row group for batch rows 8 t + g
+        auto store = [&](int row, int b, float v0, float v1) {
+            const int n = n0 + row;
+            if (b >= p.batch || n >= p.N) return;
+            uint16_t* out = p.y + static_cast<size_t>(b) * p.N + n;
+            const uint16_t h0 = float_to_half_bits(v0), h1 = float_to_half_bits(v1);
+            if (p.y4) {
+                *reinterpret_cast<uint32_t*>(out) = pack2(h0, h1);   // N even, n even
+            } else {
+                out[0] = h0;
+                if (n + 1 < p.N) out[1] = h1;
+            }
+        };
+        if (ks == 1) {
+#pragma unroll
+            for (int r = 0; r < R; ++r)
+#pragma unroll
+                for (int t = 0; t < XT; ++t) store(8 * (R * rg + r) + 2 * c, 8 * t + g, acc[r][t][0], acc[r][t][1]);
+        } else {
+            float2* red = reinterpret_cast<float2*>(smem + p.red_off);   // [warp][r][t][lane]
+#pragma unroll
+            for (int r = 0; r < R; ++r)
+#pragma unroll
+                for (int t = 0; t < XT; ++t)
+                    red[((warp * R + r) * XT + t) * 32 + lane] = make_float2(acc[r][t][0], acc[r][t][1]);
+            __syncthreads();
+            // slices added in order; the next tile's sums are stored only
+            // after a later barrier
+            for (int e = tid; e < rgs * R * XT * 32; e += kBThreads) {
+                const int ln = e & 31, q = e >> 5;                       // q = (row group, r, t)
+                const int t = q % XT, qr = q / XT;
+                const int r = qr % R, grp = qr / R;
+                const float2* src = red + ((grp * ks * R + r) * XT + t) * 32 + ln;
+                float2 sum = src[0];
+                for (int k = 1; k < ks; ++k) {
+                    const float2 o = src[k * R * XT * 32];
+                    sum.x += o.x;
+                    sum.y += o.y;
+                }
+                store(8 * (R * grp + r) + 2 * (ln & 3), 8 * t + (ln >> 2), sum.x, sum.y);
+            }
+        }
+#pragma unroll
+        for (int r = 0; r < R; ++r)
+#pragma unroll
+            for (int t = 0; t < XT; ++t) acc[r][t][0] = acc[r][t][1] = 0.f;
+        ch = 0;
+        n0 += static_cast<int>(gridDim.x) * TR;
+    }
+    cp_wait<0>();
+}
+
+// ------------------------------------------------- tensor-copy kernel --
+//
+// K % 256 == 0 and 16-byte aligned scales.  Weights are the 16 rows of the
+// MMA here (row tiles of 16, two MMAs per 32-code group, tile and eight
+// activation rows), which takes ~20 % fewer instructions a weight than
+// activations as the rows while the batch leaves half of those empty.  A
+// producer lane brings each K chunk with three tensor copies: TR rows of
+// codes (boxes of 128 bytes = 8 groups, 128-byte swizzle), TR rows of scales
+// (16 bytes a box) and the batch's activations (boxes of 64 = 2 groups,
+// 128-byte swizzle; rows past the batch read as zeros), each matrix seen as
+// (position in the box, row, box).  One copy a matrix and chunk matters: with
+// one copy per box the producer's issue rate (~85 cycles a copy) bound the
+// narrow shapes.  The consumer warps wait only for the chunk they are at and
+// drift apart by up to the ring's depth.
+// Consumer warps: 16 (96 registers a thread beside the producer) up to batch
+// 16, else 8 (168) with up to 48 weight rows each: at 96 registers the sums of
+// 24-32 activation rows spilled (128256 x 4096, batch 32: 396 us, with 8 warps
+// 130; 12 warps 137, and narrow matrices lose their 8 K slices).
+template <int XT>
+constexpr int kTWarps = XT <= 2 ? 16 : 8;
+constexpr int kTMaxSlots = 8;
+constexpr int kTHeader = 1024;                    // full[8], empty[8]
+
+struct TGemvParams {
+    uint16_t* y;
+    int N, K, batch;
+    int lkg;               // log2 of the groups per chunk (8, 16 or 32)
+    int wrows;             // weight rows per warp: a multiple of 8 up to 32 (48 with 8 warps)
+    int ks, gpw;           // K slices, groups of a chunk per slice (2, 4 or 8)
+    int tiles, nch, nslots;
+    uint32_t slot_bytes, scale_off, x_off, red_off;
+    int y4;                // two outputs may be stored at once
+    uint32_t* err;
+};
+
+// Activation row (of a tile of eight) that lane group g holds: neighbouring
+// groups take rows four apart, so that the eight lanes of a 16-byte load phase
+// (two rows, four chunks) hit different halves of the swizzled 128-byte lines.
+__device__ __forceinline__ int x_row(int g) { return ((g & 1) << 2) | (g >> 1); }
+
+__device__ __forceinline__ float lo_scale(uint32_t v) { return __low2float(*reinterpret_cast<const __half2*>(&v)); }
+__device__ __forceinline__ float hi_scale(uint32_t v) { return __high2float(*reinterpret_cast<const __half2*>(&v)); }
+
+// XT: tiles of eight activation rows; R: row tiles of 16 per warp (the last
+// one may hold eight rows; its other eight read what follows and are dropped).
+template <int XT, int R>
+__global__ void __launch_bounds__(32 * (kTWarps<XT> + 1), 1)
+    bgemv_tma_kernel(const __grid_constant__ CUtensorMap tm_w, const __grid_constant__ CUtensorMap tm_s,
+                     const __grid_constant__ CUtensorMap tm_x, const TGemvParams p)
+{
+    extern __shared__ __align__(1024) uint8_t smem[];
+    constexpr int NW = kTWarps<XT>, kConsumers = 32 * NW;
+    uint64_t* full = reinterpret_cast<uint64_t*>(smem);
+    uint64_t* empty = full + kTMaxSlots;
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int ks = p.ks, rgs = NW / ks, TR = p.wrows * rgs;
+    const int grid = static_cast<int>(gridDim.x), nch = p.nch, nslots = p.nslots;
+    const int mytiles = (p.tiles - static_cast<int>(blockIdx.x) + grid - 1) / grid;
+
+    if (tid == kConsumers) {
+        for (int i = 0; i < nslots; ++i) {
+            mbar_init(&full[i], 1);
+            mbar_init(&empty[i], NW);
+        }
+        mbar_fence_init();
+    }
+    __syncthreads();
+    grid_dependents_launch();
+
+    if (warp == NW) {
+        // ---------------------------------------------------- producer
+        if (lane == 0) {
+            const int boxes = 1 << (p.lkg - 3), total = mytiles * nch;
+            const uint32_t bytes = boxes * (TR * 144 + XT * 4096);
+            auto load_w = [&](int slot, int n0, int ch) {
+                uint8_t* base = smem + kTHeader + static_cast<size_t>(slot) * p.slot_bytes;
+                mbar_arrive_expect_tx(&full[slot], bytes);
+                tc::tma_load_3d(base, &tm_w, 0, n0, ch * boxes, &full[slot]);
+                tc::tma_load_3d(base + p.scale_off, &tm_s, 0, n0, ch * boxes, &full[slot]);
+            };
+            auto load_x = [&](int slot, int ch) {
+                uint8_t* base = smem + kTHeader + static_cast<size_t>(slot) * p.slot_bytes;
+                tc::tma_load_3d(base + p.x_off, &tm_x, 0, 0, 4 * ch * boxes, &full[slot]);
+            };
+            // weights may be fetched while the previous kernel of the stream
+            // finishes, activations only after it (programmatic dependent launch)
+            int n0 = static_cast<int>(blockIdx.x) * TR, ch = 0;
+            const int early = min(nslots, total);
+            for (int f = 0; f < early; ++f) {
+                load_w(f, n0, ch);
+                if (++ch == nch) {
+                    ch = 0;
+                    n0 += grid * TR;
+                }
+            }
+            grid_dependency_wait();
+            for (int f = 0, c = 0; f < early; ++f) {
+                load_x(f, c);
+                if (++c == nch) c = 0;
+            }
+            int slot = 0, par = 0, f = early;
+            for (; f < total; ++f) {
+                if (!mbar_wait(&empty[slot], par, p.err)) break;
+                load_w(slot, n0, ch);
+                load_x(slot, ch);
+                if (++ch == nch) {
+                    ch = 0;
+                    n0 += grid * TR;
+                }
+                if (++slot == nslots) {
+                    slot = 0;
+                    par ^= 1;
+                }
+            }
+            // every copy issued has landed before the CTA's memory goes away
+            for (int i = max(0, f - nslots); i < f; ++i) mbar_wait(&full[i % nslots], (i / nslots) & 1, p.err);
+        }
+        return;
+    }
+
+    // -------------------------------------------------------- consumers
+    grid_dependency_wait();               // y is written after the previous kernel
+    const int g = lane >> 2, c = lane & 3;
+    const int rg = warp / ks, sl = warp - rg * ks;    // row group and K slice of this warp
+    const int m = lane >> 3, lr = lane & 7;           // ldmatrix: matrix and row of this lane's address
+    const int j0 = sl * p.gpw;                        // first group of the slice (a slice lies in one box of 8)
+    const uint32_t smem0 = smem_addr(smem) + kTHeader;
+    // matrices of a tile: rows 0-7 and 8-15 of group j, then of group j + 1
+    const uint32_t coff = ((j0 >> 3) * TR + rg * p.wrows + 8 * (m & 1) + lr) * 128;
+    const uint32_t soff = p.scale_off + ((j0 >> 3) * TR + rg * p.wrows + g) * 16;
+    const uint32_t xoff = p.x_off + (j0 >> 1) * (XT * 1024) + x_row(g) * 128 + ((c ^ x_row(g)) << 4);
+
+    float acc[R][XT][4];       // rows 16 r + g (0, 1) and + 8 (2, 3), activation rows 8 t + x_row(2c), x_row(2c + 1)
+#pragma unroll
+    for (int r = 0; r < R; ++r)
+#pragma unroll
+        for (int t = 0; t < XT; ++t) acc[r][t][0] = acc[r][t][1] = acc[r][t][2] = acc[r][t][3] = 0.f;
+
+    int slot = 0, par = 0, n0 = static_cast<int>(blockIdx.x) * TR;
+    const int G = p.K >> 5;
+    bool ok = true;
+    for (int it = 0; it < mytiles; ++it, n0 += grid * TR) {
+        for (int ch = 0; ch < nch; ++ch) {
+            if (ok) ok = mbar_wait(&full[slot], par, p.err);   // after a wait gave up, none is waited for
+            const uint32_t base = smem0 + slot * p.slot_bytes;
+            const int npair = min(p.gpw, G - (ch << p.lkg) - j0) >> 1;   // G is a multiple of 8
+            const uint32_t cb = base + coff;
+            uint32_t sa = base + soff + 2 * (j0 & 7), xa = base + xoff;
+            int j = (j0 & 7) + (m >> 1);
+#pragma unroll 1
+            for (int k = 0; k < npair; ++k, sa += 4, xa += XT * 1024, j += 2) {
+                uint32_t w[R][4], sa0[R], sb0[R];
+                const uint32_t ca = cb + ((j ^ lr) << 4);
+#pragma unroll
+                for (int r = 0; r < R; ++r) {
+                    ldsm_x4_b(ca + 2048 * r, w[r]);
+                    sa0[r] = lds_u32(sa + 256 * r);        // scales of groups j, j + 1: row g
+                    sb0[r] = lds_u32(sa + 256 * r + 128);  // ... and row g + 8
+                }
+#pragma unroll
+                for (int h = 0; h < 2; ++h) {
+                    uint32_t qa[R][4], qb[R][4];
+#pragma unroll
+                    for (int r = 0; r < R; ++r) {
+                        unpack_word(w[r][2 * h], qa[r]);
+                        unpack_word(w[r][2 * h + 1], qb[r]);
+                    }
+#pragma unroll
+                    for (int t = 0; t < XT; ++t) {
+                        const uint4 v = pair_permute(lds_v4((xa ^ (64 * h)) + 1024 * t));
+#pragma unroll
+                        for (int r = 0; r < R; ++r) {
+                            const float s0 = h ? hi_scale(sa0[r]) : lo_scale(sa0[r]);
+                            const float s1 = h ? hi_scale(sb0[r]) : lo_scale(sb0[r]);
+                            float d[4] = {0.f, 0.f, 0.f, 0.f};
+                            mma_acc(d, qa[r][0], qb[r][0], qa[r][1], qb[r][1], v.x, v.y);
+                            mma_acc(d, qa[r][2], qb[r][2], qa[r][3], qb[r][3], v.z, v.w);
+                            acc[r][t][0] = fmaf(s0, d[0], acc[r][t][0]);
+                            acc[r][t][1] = fmaf(s0, d[1], acc[r][t][1]);
+                            acc[r][t][2] = fmaf(s1, d[2], acc[r][t][2]);
+                            acc[r][t][3] = fmaf(s1, d[3], acc[r][t][3]);
+                        }
+                    }
+                }
+            }
+            __syncwarp();
+            if (lane == 0) mbar_arrive(&empty[slot]);
+            if (++slot == nslots) {
+                slot = 0;
+                par ^= 1;
+            }
+        }
+
+        // ---- the tile is complete
+        if (ks == 1) {
+#pragma unroll
+            for (int r = 0; r < R; ++r)
+#pragma unroll
+                for (int t = 0; t < XT; ++t)
+#pragma unroll
+                    for (int i = 0; i < 4; ++i) {
+                        const int row = 16 * r + g + 8 * (i >> 1), n = n0 + rg * p.wrows + row;
+                        const int b = 8 * t + x_row(2 * c + (i & 1));
+                        if (row < p.wrows && n < p.N && b < p.batch)
+                            p.y[static_cast<size_t>(b) * p.N + n] = float_to_half_bits(acc[r][t][i]);
+                    }
+        } else {
+            // [warp][activation row][weight row]; the pitch spreads a store over the banks
+            constexpr int P = 16 * R + 4;
+            float* red = reinterpret_cast<float*>(smem + p.red_off);
+            float* mine = red + warp * (8 * XT * P) + 2 * c * P + g;
+#pragma unroll
+            for (int r = 0; r < R; ++r)
+#pragma unroll
+                for (int t = 0; t < XT; ++t) {
+                    float* q = mine + 8 * t * P + 16 * r;
+                    q[0] = acc[r][t][0];
+                    q[P] = acc[r][t][1];
+                    q[8] = acc[r][t][2];
+                    q[P + 8] = acc[r][t][3];
+                }
+            named_barrier_sync(1, kConsumers);
+            const int hrows = p.wrows >> 1;                              // pairs of rows per row group
+            for (int e = tid; e < rgs * hrows * 8 * XT; e += kConsumers) {
+                const int pr = e % hrows, q = e / hrows;                 // row pair; column and row group
+                const int col = q % (8 * XT), grp = q / (8 * XT);
+                const float2* src = reinterpret_cast<const float2*>(red + (grp * ks * 8 * XT + col) * P + 2 * pr);
+                float2 sum = src[0];
+                for (int k = 1; k < ks; ++k) {                           // slices added in order
+                    const float2 o = src[k * (8 * XT * P / 2)];
+                    sum.x += o.x;
+                    sum.y += o.y;
+                }
+                const int n = n0 + grp * p.wrows + 2 * pr, b = (col & ~7) + x_row(col & 7);
+                if (b < p.batch && n < p.N) {
+                    uint16_t* out = p.y + static_cast<size_t>(b) * p.N + n;
+                    const uint16_t h0 = float_to_half_bits(sum.x), h1 = float_to_half_bits(sum.y);
+                    if (p.y4) {
+                        *reinterpret_cast<uint32_t*>(out) = pack2(h0, h1);   // N even, n even
+                    } else {
+                        out[0] = h0;
+                        if (n + 1 < p.N) out[1] = h1;
+                    }
+                }
+            }
+            named_barrier_sync(1, kConsumers);                            // the sums' buffer is free again
+        }
+#pragma unroll
+        for (int r = 0; r < R; ++r)
+#pragma unroll
+            for (int t = 0; t < XT; ++t) acc[r][t][0] = acc[r][t][1] = acc[r][t][2] = acc[r][t][3] = 0.f;
+    }
+}
+
+// ----------------------------------------------------------------- host --
+
+struct BPlan {
+    int R = 0, ks = 0, lkg = 0, tiles = 0, nch = 0;
+    uint32_t stage_bytes = 0, scale_off = 0, x_off = 0, red_off = 0;
+    size_t smem = 0;
+};
+
+// Tiles per warp, K slices and chunk length: the least estimated SM cycles.
+// Per chunk the larger of the instructions of a scheduler's four warps, the
+// MMA time (one m16n8k16 per two cycles and SM) and the copies at 50 bytes
+// per cycle, plus a barrier; per tile the slices' sum.
+bool plan_bgemv(int sms, size_t smem_max, int N, int K, int XT, bool s2, BPlan* best)
+{
+    const int G = K / 32, MT = (XT + 1) / 2;
+    double best_c = 0.0;
+    for (int R = 1; R <= 4; ++R)
+        for (int ks = 1; ks <= kBWarps; ks *= 2)
+            for (int lkg = 3; lkg <= 5; ++lkg) {
+                const int KG = 1 << lkg, gpw = KG / ks;
+                if (gpw < 2) continue;
+                const int rgs = kBWarps / ks, TR = 8 * R * rgs;
+                if (s2 && (R > 2 || TR * KG > kScaleRegs * kBThreads)) continue;
+                BPlan q;
+                q.R = R;
+                q.ks = ks;
+                q.lkg = lkg;
+                q.scale_off = static_cast<uint32_t>(TR * (16 * KG + 16));
+                q.x_off = static_cast<uint32_t>(align_up(q.scale_off + TR * (2 * KG + 16), 16));
+                q.stage_bytes = static_cast<uint32_t>(align_up(q.x_off + 8 * XT * (64 * KG + 64), 128));
+                q.red_off = q.stage_bytes * kBStages;
+                q.smem = q.red_off + (ks > 1 ? static_cast<size_t>(kBWarps) * R * XT * 256 : 0);
+                if (q.smem > smem_max) continue;
+                q.tiles = (N + TR - 1) / TR;
+                q.nch = (G + KG - 1) / KG;
+                const int rounds = (q.tiles + sms - 1) / sms;
+                const double instr = gpw * (5.0 * XT + 4 + R * (13.0 + 2 * MT + 2 * XT)) + 20.0 +
+                                     (TR * KG * 1.5 + 32.0 * XT * KG) / kBThreads * 8.0;
+                const double mma = static_cast<double>(kBWarps) * gpw * R * 2 * MT * 2.0;
+                const double copy = (TR * 18.0 * KG + 512.0 * XT * KG) / 50.0;
+                const double chunk = std::max(std::max(4.6 * instr, mma), copy) + 150.0;
+                const double cost = rounds * (q.nch * chunk + (ks > 1 ? 150.0 + 20.0 * R * XT : 30.0 * R)) + 1500.0;
+                if (best->R == 0 || cost < best_c) {
+                    best_c = cost;
+                    *best = q;
+                }
+            }
+    return best->R != 0;
+}
+
+template <int XT, int R, bool S2>
+cudaError_t launch_one(const cudaLaunchConfig_t& cfg, const BGemvParams& p, int smem_max)
+{
+    static std::atomic<bool> ready[64];                // per device; setting the attribute twice is harmless
+    int dev = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e != cudaSuccess) return e;
+    if (dev >= 64 || !ready[dev].load()) {
+        e = cudaFuncSetAttribute(bgemv_kernel<XT, R, S2>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_max);
+        if (e != cudaSuccess) return e;
+        if (dev < 64) ready[dev].store(true);
+    }
+    return cudaLaunchKernelEx(&cfg, bgemv_kernel<XT, R, S2>, p);
+}
+
+template <int XT>
+cudaError_t launch_xt(int R, bool s2, const cudaLaunchConfig_t& cfg, const BGemvParams& p, int smem_max)
+{
+    if (s2) return R == 1 ? launch_one<XT, 1, true>(cfg, p, smem_max) : launch_one<XT, 2, true>(cfg, p, smem_max);
+    switch (R) {
+        case 1: return launch_one<XT, 1, false>(cfg, p, smem_max);
+        case 2: return launch_one<XT, 2, false>(cfg, p, smem_max);
+        case 3: return launch_one<XT, 3, false>(cfg, p, smem_max);
+        default: return launch_one<XT, 4, false>(cfg, p, smem_max);
+    }
+}
+
+// The tensor-copy kernel's split: as plan_bgemv, without copy instructions
+// in the warps (a chunk costs them a wait and an arrival).
+struct TPlan {
+    int wrows = 0, ks = 0, lkg = 0, tiles = 0, nch = 0, nslots = 0;
+    uint32_t slot_bytes = 0, scale_off = 0, x_off = 0, red_off = 0;
+    size_t smem = 0;
+};
+
+bool plan_tma(int sms, size_t smem_max, int N, int K, int XT, TPlan* best)
+{
+    const int G = K / 32, NW = XT <= 2 ? kTWarps<1> : kTWarps<4>;
+    double best_c = 0.0;
+    for (int wrows = 8; wrows <= (NW == 16 ? 32 : 48); wrows += 8)
+        for (int ks = 1; ks <= NW; ks *= 2)
+            for (int lkg = 3; lkg <= 5; ++lkg) {
+                const int KG = 1 << lkg, gpw = KG / ks, boxes = KG / 8, R = (wrows + 15) / 16;
+                if (gpw < 2 || gpw > 8) continue;
+                const int rgs = NW / ks, TR = wrows * rgs;
+                if (TR > 256) continue;
+                TPlan q;
+                q.wrows = wrows;
+                q.ks = ks;
+                q.lkg = lkg;
+                q.scale_off = static_cast<uint32_t>(boxes * TR * 128);
+                q.x_off = static_cast<uint32_t>(align_up(q.scale_off + boxes * TR * 16, 1024));
+                q.slot_bytes = q.x_off + boxes * XT * 4096;
+                const size_t red = ks > 1 ? static_cast<size_t>(NW) * 8 * XT * (16 * R + 4) * 4 : 0;
+                if (smem_max < kTHeader + red) continue;
+                const int nslots = static_cast<int>((smem_max - kTHeader - red) / q.slot_bytes);
+                if (nslots < 3) continue;
+                q.nslots = std::min(nslots, kTMaxSlots);
+                q.red_off = kTHeader + q.nslots * q.slot_bytes;
+                q.smem = q.red_off + red;
+                q.tiles = (N + TR - 1) / TR;
+                q.nch = (G + KG - 1) / KG;
+                const int rounds = (q.tiles + sms - 1) / sms;
+                const double instr = gpw * (5.0 * XT + 4 + R * (22.0 + 6 * XT)) + 30.0;
+                const double mma = static_cast<double>(NW) * gpw * R * 2 * XT * 2.0;
+                const double copy = (TR * 18.0 * KG + 512.0 * XT * KG) / 45.0;
+                const double chunk = std::max(std::max((NW == 16 ? 5.0 : 3.0) * instr, mma * 1.1), copy);
+                double cost = rounds * (q.nch * chunk + (ks > 1 ? 200.0 + 40.0 * R * XT : 80.0 * R)) + 1500.0;
+                if (wrows % 16 != 0) cost *= 1.03;                 // half a tile's MMAs are dropped
+                if (XT == 4 && R == 3) cost *= 1.08;               // a few registers spill
+                if (best->wrows == 0 || cost < best_c) {
+                    best_c = cost;
+                    *best = q;
+                }
+            }
+    return best->wrows != 0;
+}
+
+template <int XT, int R>
+cudaError_t launch_tma(const cudaLaunchConfig_t& cfg, const CUtensorMap* tm, const TGemvParams& p, int smem_max)
+{
+    static std::atomic<bool> ready[64];                // per device; setting the attribute twice is harmless
+    int dev = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e != cudaSuccess) return e;
+    if (dev >= 64 || !ready[dev].load()) {
+        e = cudaFuncSetAttribute(bgemv_tma_kernel<XT, R>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_max);
+        if (e != cudaSuccess) return e;
+        if (dev < 64) ready[dev].store(true);
+    }
+    return cudaLaunchKernelEx(&cfg, bgemv_tma_kernel<XT, R>, tm[0], tm[1], tm[2], p);
+}
+
+template <int XT>
+cudaError_t launch_tma_xt(int R, const cudaLaunchConfig_t& cfg, const CUtensorMap* tm, const TGemvParams& p, int smem_max)
+{
+    if (R == 1) return launch_tma<XT, 1>(cfg, tm, p, smem_max);
+    if constexpr (kTWarps<XT> == 8)
+        if (R == 3) return launch_tma<XT, 3>(cfg, tm, p, smem_max);
+    return launch_tma<XT, 2>(cfg, tm, p, smem_max);
+}
+
+int launch_bgemv_tma(const DeviceInfo* di, const uint32_t* W, const uint16_t* s, const uint16_t* x, uint16_t* y, int N,
+                     int K, int batch, cudaStream_t stream)
+{
+    const int XT = (batch + 7) / 8;
+    TPlan b;
+    if (!plan_tma(di->sm_count, static_cast<size_t>(di->smem_optin), N, K, XT, &b)) return WQ4_ERR_CUDA;
+    const int NW = XT <= 2 ? kTWarps<1> : kTWarps<4>;
+    const int TR = b.wrows * (NW / b.ks), R = (b.wrows + 15) / 16;
+    const uint32_t boxes = 1u << (b.lkg - 3);
+    const uint64_t Ku = static_cast<uint64_t>(K), Nu = static_cast<uint64_t>(N);
+    CUtensorMap tm[3];
+    if (!encode_tensor_map_3d(&tm[0], CU_TENSOR_MAP_DATA_TYPE_UINT8, W, {128, Nu, Ku / 256}, {Ku / 2, 128},
+                              {128, static_cast<uint32_t>(TR), boxes}, CU_TENSOR_MAP_SWIZZLE_128B) ||
+        !encode_tensor_map_3d(&tm[1], CU_TENSOR_MAP_DATA_TYPE_UINT16, s, {8, Nu, Ku / 256}, {Ku / 16, 16},
+                              {8, static_cast<uint32_t>(TR), boxes}, CU_TENSOR_MAP_SWIZZLE_NONE) ||
+        !encode_tensor_map_3d(&tm[2], CU_TENSOR_MAP_DATA_TYPE_FLOAT16, x, {64, static_cast<uint64_t>(batch), Ku / 64},
+                              {Ku * 2, 128}, {64, static_cast<uint32_t>(8 * XT), 4 * boxes}, CU_TENSOR_MAP_SWIZZLE_128B))
+        return WQ4_ERR_CUDA;
+    TGemvParams p;
+    p.y = y;
+    p.N = N;
+    p.K = K;
+    p.batch = batch;
+    p.lkg = b.lkg;
+    p.wrows = b.wrows;
+    p.ks = b.ks;
+    p.gpw = (1 << b.lkg) / b.ks;
+    p.tiles = b.tiles;
+    p.nch = b.nch;
+    p.nslots = b.nslots;
+    p.slot_bytes = b.slot_bytes;
+    p.scale_off = b.scale_off;
+    p.x_off = b.x_off;
+    p.red_off = b.red_off;
+    p.y4 = (N % 2) == 0 && aligned(y, 4);
+    p.err = status_word();
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(std::min(b.tiles, di->sm_count));
+    cfg.blockDim = dim3(32 * (NW + 1));
+    cfg.dynamicSmemBytes = b.smem;
+    cfg.stream = stream;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    cudaError_t e;
+    switch (XT) {
+        case 1: e = launch_tma_xt<1>(R, cfg, tm, p, di->smem_optin); break;
+        case 2: e = launch_tma_xt<2>(R, cfg, tm, p, di->smem_optin); break;
+        case 3: e = launch_tma_xt<3>(R, cfg, tm, p, di->smem_optin); break;
+        default: e = launch_tma_xt<4>(R, cfg, tm, p, di->smem_optin); break;
+    }
+    return e == cudaSuccess ? WQ4_OK : WQ4_ERR_CUDA;
+}
+
+}  // namespace
+
+int launch_bgemv(const DeviceInfo* di, const uint32_t* W, const uint16_t* s, const uint16_t* x, uint16_t* y, int N,
+                 int K, int batch, cudaStream_t stream)
+{
+    if ((K % 256) == 0 && aligned(s, 16)) return launch_bgemv_tma(di, W, s, x, y, N, K, batch, stream);
+    const int XT = (batch + 7) / 8;
+    BGemvParams p;
+    const bool s2 = (K % 64) != 0 || !aligned(s, 4);
+    BPlan b;
+    if (!plan_bgemv(di->sm_count, static_cast<size_t>(di->smem_optin), N, K, XT, s2, &b)) return WQ4_ERR_CUDA;
+    p.W = W;
+    p.s = s;
+    p.x = x;
+    p.y = y;
+    p.N = N;
+    p.K = K;
+    p.batch = batch;
+    p.lkg = b.lkg;
+    p.ks = b.ks;
+    p.gpw = (1 << b.lkg) / b.ks;
+    p.tiles = b.tiles;
+    p.nch = b.nch;
+    p.stage_bytes = b.stage_bytes;
+    p.scale_off = b.scale_off;
+    p.x_off = b.x_off;
+    p.red_off = b.red_off;
+    p.y4 = (N % 2) == 0 && aligned(y, 4);
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(std::min(b.tiles, di->sm_count));
+    cfg.blockDim = dim3(kBThreads);
+    cfg.dynamicSmemBytes = b.smem;
+    cfg.stream = stream;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    cudaError_t e;
+    switch (XT) {
+        case 1: e = launch_xt<1>(b.R, s2, cfg, p, di->smem_optin); break;
+        case 2: e = launch_xt<2>(b.R, s2, cfg, p, di->smem_optin); break;
+        case 3: e = launch_xt<3>(b.R, s2, cfg, p, di->smem_optin); break;
+        default: e = launch_xt<4>(b.R, s2, cfg, p, di->smem_optin); break;
+    }
+    return e == cudaSuccess ? WQ4_OK : WQ4_ERR_CUDA;
+}
+
+}  // namespace wq4

@@ -3,23 +3,24 @@
 //
 // y[b][n] = fp16( sum_k (q(n,k) - 7) * s[n][k/32] * x[b][k] ), the projection
 // every decoded token applies to every 4-bit weight matrix (Section 3,
-// Table 1).  Two kernels:
+// Table 1).  The kernels of batch 1-2 (batch 2 from 8 Mi weights and every
+// larger batch run in wq4_bgemv.cu):
 //
-//  * gemv_mma_kernel<B> (batch B <= 2, K % 256 == 0, 16-byte aligned scales):
-//    the persistent decode chain's weight stream for one projection.  A
+//  * gemv_mma_kernel (batch 1, K % 256 == 0, 16-byte aligned scales): the
+//    persistent decode chain's weight stream for one projection.  A
 //    producer warp streams the CTA's word rows (pairs of rows) through a
 //    ring of shared-memory slots with 1-D bulk copies; 15 consumer warps take
 //    work items (superpair of row pairs, K part) round-robin in ring order
 //    and run them on the legacy tensor path (wq4_items.cuh: exact fp16
 //    q - 7, eight groups of x as the MMA's columns, scales in fp32 on the
 //    diagonal); K parts are added in part order in shared memory.
-//  * gemv_tma_kernel<B> (batch B <= 4, K % 256 == 0): one persistent CTA per
+//  * gemv_tma_kernel<B> (batch B <= 2, K % 256 == 0): one persistent CTA per
 //    SM.  A producer warp streams the CTA's contiguous block of rows through a
 //    ring of shared-memory slots with 1-D bulk copies (TMA) and mbarriers;
 //    consumer warps take rows round-robin, unpack in registers and accumulate
 //    in fp32 against the activations staged once in shared memory ("GEMM
 //    tiling" and "kernel fusion" of Section 2.3, by hand).
-//  * gemv_generic_kernel<BT> (any K % 32 == 0, batch up to 32, scales of any
+//  * gemv_generic_kernel<B> (batch B <= 2, any K % 32 == 0, scales of any
 //    2-byte alignment): warp per row, weights loaded straight into registers,
 //    activations read through L1.
 #include "wq4_device.cuh"
@@ -35,12 +36,6 @@
 namespace wq4 {
 
 __device__ uint32_t g_status_word;
-
-// Programmatic dependent launch: wait for the previous grid of the stream
-// (complete, memory visible) / let the next one launch.  No effect when the
-// launch did not ask for it.
-__device__ __forceinline__ void grid_dependency_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
-__device__ __forceinline__ void grid_dependents_launch() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 
 constexpr int kGemvConsumerWarps = 8;
 constexpr int kGemvThreads = (kGemvConsumerWarps + 1) * 32;
@@ -155,7 +150,6 @@ __global__ void __launch_bounds__(kGemvThreads, 1) gemv_tma_kernel(const GemvTma
     }
 }
 
-// Generic path: warp per row, batch processed in tiles of BT rows of x.
 // ------------------------------------------------------ gemv_mma_kernel --
 
 constexpr int kMmaWarps = 15;                         // consumer warps
@@ -187,9 +181,9 @@ struct GemvMmaParams {
 // first item.  A warp waits only on the chunks holding its items; the plan
 // keeps nslots + ceil(15 / items per chunk) <= nbars so that no parity wait
 // can alias, as in the chain kernel.
-template <int B>
 __global__ void __launch_bounds__(kMmaThreads, 1) gemv_mma_kernel(const GemvMmaParams p)
 {
+    constexpr int B = 1;                          // activation rows
     extern __shared__ __align__(1024) uint8_t smem[];
     uint64_t* full = reinterpret_cast<uint64_t*>(smem);
     uint64_t* empty = full + kMmaFullBars;
@@ -379,12 +373,11 @@ __global__ void __launch_bounds__(kMmaThreads, 1) gemv_mma_kernel(const GemvMmaP
     }
 }
 
-template <int BT>
+template <int B>
 __global__ void __launch_bounds__(256) gemv_generic_kernel(const uint32_t* __restrict__ W,
                                                            const uint16_t* __restrict__ s,
                                                            const uint16_t* __restrict__ x,
-                                                           uint16_t* __restrict__ y, int N, int K,
-                                                           int batch)
+                                                           uint16_t* __restrict__ y, int N, int K)
 {
     const int lane = threadIdx.x & 31;
     const int gw = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
@@ -393,36 +386,31 @@ __global__ void __launch_bounds__(256) gemv_generic_kernel(const uint32_t* __res
     for (int n = gw; n < N; n += nw) {
         const uint4* crow = reinterpret_cast<const uint4*>(W + static_cast<size_t>(n) * (K >> 3));
         const uint16_t* srow = s + static_cast<size_t>(n) * gpr;
-        for (int b0 = 0; b0 < batch; b0 += BT) {
-            float acc[BT];
+        float acc[B];
 #pragma unroll
-            for (int b = 0; b < BT; ++b) acc[b] = 0.f;
-            for (int g = lane; g < gpr; g += 32) {
-                const uint4 cw = __ldg(crow + g);
-                const float sc = half_bits_to_float(__ldg(srow + g));
-                uint32_t pq[16];
-                unpack_word(cw.x, pq + 0);
-                unpack_word(cw.y, pq + 4);
-                unpack_word(cw.z, pq + 8);
-                unpack_word(cw.w, pq + 12);
+        for (int b = 0; b < B; ++b) acc[b] = 0.f;
+        for (int g = lane; g < gpr; g += 32) {
+            const uint4 cw = __ldg(crow + g);
+            const float sc = half_bits_to_float(__ldg(srow + g));
+            uint32_t pq[16];
+            unpack_word(cw.x, pq + 0);
+            unpack_word(cw.y, pq + 4);
+            unpack_word(cw.z, pq + 8);
+            unpack_word(cw.w, pq + 12);
 #pragma unroll
-                for (int b = 0; b < BT; ++b) {
-                    if (b0 + b < batch) {
-                        const uint4* xb =
-                            reinterpret_cast<const uint4*>(x + static_cast<size_t>(b0 + b) * K) + g * 4;
-                        const float a0 = fma8(pq + 0, __ldg(xb + 0), 0.f);
-                        const float a1 = fma8(pq + 4, __ldg(xb + 1), 0.f);
-                        const float a2 = fma8(pq + 8, __ldg(xb + 2), 0.f);
-                        const float a3 = fma8(pq + 12, __ldg(xb + 3), 0.f);
-                        acc[b] = fmaf(sc, (a0 + a1) + (a2 + a3), acc[b]);
-                    }
-                }
+            for (int b = 0; b < B; ++b) {
+                const uint4* xb = reinterpret_cast<const uint4*>(x + static_cast<size_t>(b) * K) + g * 4;
+                const float a0 = fma8(pq + 0, __ldg(xb + 0), 0.f);
+                const float a1 = fma8(pq + 4, __ldg(xb + 1), 0.f);
+                const float a2 = fma8(pq + 8, __ldg(xb + 2), 0.f);
+                const float a3 = fma8(pq + 12, __ldg(xb + 3), 0.f);
+                acc[b] = fmaf(sc, (a0 + a1) + (a2 + a3), acc[b]);
             }
+        }
 #pragma unroll
-            for (int b = 0; b < BT; ++b) {
-                const float v = warp_sum(acc[b]);
-                if (lane == b && b0 + b < batch) y[static_cast<size_t>(b0 + b) * N + n] = float_to_half_bits(v);
-            }
+        for (int b = 0; b < B; ++b) {
+            const float v = warp_sum(acc[b]);
+            if (lane == b) y[static_cast<size_t>(b) * N + n] = float_to_half_bits(v);
         }
     }
 }
@@ -474,10 +462,9 @@ bool set_tma_attr(int smem)
            cudaSuccess;
 }
 
-template <int B>
 bool set_mma_attr(int smem)
 {
-    return cudaFuncSetAttribute(gemv_mma_kernel<B>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) ==
+    return cudaFuncSetAttribute(gemv_mma_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) ==
            cudaSuccess;
 }
 
@@ -495,9 +482,7 @@ const DeviceInfo* current_device_info(int* device_out)
         if (cudaDeviceGetAttribute(&d.smem_optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev) != cudaSuccess)
             return nullptr;
         if (cudaDeviceGetAttribute(&d.coop_launch, cudaDevAttrCooperativeLaunch, dev) != cudaSuccess) return nullptr;
-        if (!set_tma_attr<1>(d.smem_optin) || !set_tma_attr<2>(d.smem_optin) || !set_tma_attr<3>(d.smem_optin) ||
-            !set_tma_attr<4>(d.smem_optin) || !set_mma_attr<1>(d.smem_optin) || !set_mma_attr<2>(d.smem_optin))
-            return nullptr;
+        if (!set_tma_attr<1>(d.smem_optin) || !set_tma_attr<2>(d.smem_optin) || !set_mma_attr(d.smem_optin)) return nullptr;
         void* ptr = nullptr;
         if (cudaGetSymbolAddress(&ptr, g_status_word) != cudaSuccess) return nullptr;
         g_status_ptr[dev] = static_cast<uint32_t*>(ptr);
@@ -580,8 +565,8 @@ bool plan_mma(const DeviceInfo* di, int N, int K, int B, MmaPlan* pl)
     return true;
 }
 
-// Which batch 1-2 kernel a call takes (wq4_test_gemv_path): 0 the size rule,
-// 1 the legacy-tensor-path kernel wherever it applies, 2 the CUDA-core one.
+// Which batch 1-2 kernel a call takes (wq4_test_gemv_path): 0 the size rules,
+// 1 the legacy-tensor-path kernels wherever they apply, 2 the CUDA-core one.
 std::atomic<int> g_gemv_path{0};
 
 // Below ~12 M weights a launch is bound by its fixed costs (x staging, the
@@ -593,17 +578,34 @@ std::atomic<int> g_gemv_path{0};
 // 16384 x 3072 8.69 / 12.20, 128256 x 3072 45.1 / 75.1.
 constexpr int64_t kMmaMinWeights = int64_t(12) << 20;
 
+// From here on batch 2 takes the batched kernel (wq4_bgemv.cu): batch 2, us
+// (batched / the CUDA-core kernel here, or above 12 Mi weights the two-row
+// form that gemv_mma_kernel had): 2048 x 2048 2.99 / 3.00, 512 x 14336 6.86 /
+// 4.36, 3072 x 3072 3.68 / 4.70, 16384 x 3072 9.15 / 10.61, 128256 x 3072
+// 43.8 / 57.4.  At batch 1 the kernels here stay ahead (128256 x 3072 42.4 /
+// 43.8).
+constexpr int64_t kBatch2MinWeights = int64_t(8) << 20;
+
+// Rows that the bulk copies cannot take (K % 256 != 0 or unaligned scales):
+// the batched kernel's copy ring from here on at batch 1 and 2, the warp-per-row
+// kernel below.  us (ring / warp per row): batch 1 1003 x 2080 4.83 / 2.99,
+// 20000 x 3104 27.5 / 21.6, 100000 x 3104 78.6 / 95.4; batch 2 1003 x 2080
+// 4.62 / 4.27, 4000 x 2080 6.53 / 7.33, 100000 x 3104 78.5 / 155.8.
+constexpr int64_t kRingMinWeights[3] = {0, int64_t(128) << 20, int64_t(6) << 20};
+
 int launch_gemv(const uint32_t* W, const uint16_t* s, const uint16_t* x, uint16_t* y, int N, int K, int batch,
                 cudaStream_t stream)
 {
     int dev = 0;
     const DeviceInfo* di = current_device_info(&dev);
     if (!di) return WQ4_ERR_CUDA;
-    MmaPlan mp;
     const int path = g_gemv_path.load();
-    const bool big = static_cast<int64_t>(N) * K >= kMmaMinWeights;
-    if (path != 2 && (big || path == 1) && batch <= 2 && (K % 256) == 0 && aligned(s, 16) &&
-        plan_mma(di, N, K, batch, &mp)) {
+    const int64_t weights = static_cast<int64_t>(N) * K;
+    const bool bulk = (K % 256) == 0 && aligned(s, 16);
+    if (batch > 2 || (batch == 2 && bulk && path != 2 && (weights >= kBatch2MinWeights || path == 1)))
+        return launch_bgemv(di, W, s, x, y, N, K, batch, stream);
+    MmaPlan mp;
+    if (path != 2 && (weights >= kMmaMinWeights || path == 1) && batch == 1 && bulk && plan_mma(di, N, K, batch, &mp)) {
         GemvMmaParams p;
         p.W = W;
         p.s = s;
@@ -628,14 +630,12 @@ int launch_gemv(const uint32_t* W, const uint16_t* s, const uint16_t* x, uint16_
         cfg.stream = stream;
         cfg.attrs = attr;
         cfg.numAttrs = 1;
-        const cudaError_t e = batch == 1 ? cudaLaunchKernelEx(&cfg, gemv_mma_kernel<1>, p)
-                                         : cudaLaunchKernelEx(&cfg, gemv_mma_kernel<2>, p);
+        const cudaError_t e = cudaLaunchKernelEx(&cfg, gemv_mma_kernel, p);
         return e == cudaSuccess ? WQ4_OK : WQ4_ERR_CUDA;
     }
     const size_t row_bytes = static_cast<size_t>(K) / 2 + static_cast<size_t>(K) / 16;
     const size_t x_bytes = align_up(static_cast<size_t>(batch) * K * 2, 128);
-    const bool fast = batch <= 4 && (K % 256) == 0 && aligned(s, 16) &&
-                      kHeaderBytes + x_bytes + 2 * align_up(row_bytes, 128) <= static_cast<size_t>(di->smem_optin);
+    const bool fast = bulk && kHeaderBytes + x_bytes + 2 * align_up(row_bytes, 128) <= static_cast<size_t>(di->smem_optin);
     if (fast) {
         const int grid = N < di->sm_count ? N : di->sm_count;
         const int rows_per_cta = (N + grid - 1) / grid;
@@ -675,27 +675,20 @@ int launch_gemv(const uint32_t* W, const uint16_t* s, const uint16_t* x, uint16_
         cfg.stream = stream;
         cfg.attrs = attr;
         cfg.numAttrs = 1;
-        cudaError_t e;
-        switch (batch) {
-            case 1: e = cudaLaunchKernelEx(&cfg, gemv_tma_kernel<1>, p); break;
-            case 2: e = cudaLaunchKernelEx(&cfg, gemv_tma_kernel<2>, p); break;
-            case 3: e = cudaLaunchKernelEx(&cfg, gemv_tma_kernel<3>, p); break;
-            default: e = cudaLaunchKernelEx(&cfg, gemv_tma_kernel<4>, p); break;
-        }
+        const cudaError_t e = batch == 1 ? cudaLaunchKernelEx(&cfg, gemv_tma_kernel<1>, p)
+                                         : cudaLaunchKernelEx(&cfg, gemv_tma_kernel<2>, p);
         if (e != cudaSuccess) return WQ4_ERR_CUDA;
+    } else if (weights >= kRingMinWeights[batch]) {
+        return launch_bgemv(di, W, s, x, y, N, K, batch, stream);
     } else {
         const int warps_per_block = 8;
         int grid = (N + warps_per_block - 1) / warps_per_block;
         const int cap = di->sm_count * 8;
         if (grid > cap) grid = cap;
         if (batch == 1)
-            gemv_generic_kernel<1><<<grid, 256, 0, stream>>>(W, s, x, y, N, K, batch);
-        else if (batch == 2)
-            gemv_generic_kernel<2><<<grid, 256, 0, stream>>>(W, s, x, y, N, K, batch);
-        else if (batch <= 4)
-            gemv_generic_kernel<4><<<grid, 256, 0, stream>>>(W, s, x, y, N, K, batch);
+            gemv_generic_kernel<1><<<grid, 256, 0, stream>>>(W, s, x, y, N, K);
         else
-            gemv_generic_kernel<8><<<grid, 256, 0, stream>>>(W, s, x, y, N, K, batch);
+            gemv_generic_kernel<2><<<grid, 256, 0, stream>>>(W, s, x, y, N, K);
     }
     return cudaGetLastError() == cudaSuccess ? WQ4_OK : WQ4_ERR_CUDA;
 }

@@ -4,6 +4,7 @@
 #include <cuda.h>
 #include <cuda_runtime.h>
 
+#include <array>
 #include <cstddef>
 #include <cstdint>
 
@@ -26,6 +27,17 @@ uint32_t* status_word();
 bool encode_tensor_map_2d(CUtensorMap* m, CUtensorMapDataType dt, const void* base, uint64_t inner,
                           uint64_t outer, uint64_t row_bytes, uint32_t box_inner, uint32_t box_outer,
                           CUtensorMapSwizzle swz);
+
+// 3-D tiled tensor map: extents innermost first, byte strides of the outer two
+// dimensions, box extents.
+bool encode_tensor_map_3d(CUtensorMap* m, CUtensorMapDataType dt, const void* base, const std::array<uint64_t, 3>& dims,
+                          const std::array<uint64_t, 2>& strides, const std::array<uint32_t, 3>& box,
+                          CUtensorMapSwizzle swz);
+
+// wq4_gemv for the batches and sizes that the TMA-staged kernels do not take
+// (wq4_bgemv.cu): any N, K % 32 == 0, batch 1-32, scales at any 2-byte address.
+int launch_bgemv(const DeviceInfo* di, const uint32_t* W, const uint16_t* s, const uint16_t* x, uint16_t* y, int N,
+                 int K, int batch, cudaStream_t stream);
 
 inline bool aligned(const void* p, size_t a)
 {

@@ -660,6 +660,18 @@ bool encode_tensor_map_2d(CUtensorMap* m, CUtensorMapDataType dt, const void* ba
                CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
+bool encode_tensor_map_3d(CUtensorMap* m, CUtensorMapDataType dt, const void* base, const std::array<uint64_t, 3>& dims,
+                          const std::array<uint64_t, 2>& strides, const std::array<uint32_t, 3>& box,
+                          CUtensorMapSwizzle swz)
+{
+    PFN_cuTensorMapEncodeTiled_v12000 enc = encode_fn();
+    if (!enc) return false;
+    cuuint64_t d[3] = {dims[0], dims[1], dims[2]}, st[2] = {strides[0], strides[1]};
+    cuuint32_t bx[3] = {box[0], box[1], box[2]}, es[3] = {1, 1, 1};
+    return enc(m, dt, 3, const_cast<void*>(base), d, st, bx, es, CU_TENSOR_MAP_INTERLEAVE_NONE, swz,
+               CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+}
+
 struct TcPlan {
     std::vector<TcMatMaps> mats;   // [4L + 1]
     CUtensorMap xH[2], xF;
