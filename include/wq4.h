@@ -103,7 +103,9 @@ int wq4_gemv(const uint32_t* W_packed, const uint16_t* scales, const uint16_t* x
  *       aligned, must not overlap x, W or scales.
  *   M >= 1 (any size), N >= 1 with N % 8 == 0, K % 256 == 0 (other valid
  *   sizes return WQ4_ERR_UNSUPPORTED: use wq4_gemv for them).
- * Deterministic (no split K).  Returns WQ4_OK, WQ4_ERR_INVALID,
+ * Deterministic (where K is split over thread blocks, the parts are added in
+ * order).  Launched with programmatic dependent launch, as wq4_gemv.  At most
+ * 16 tokens run on wq4_gemv's kernels (exact weights).  Returns WQ4_OK, WQ4_ERR_INVALID,
  * WQ4_ERR_UNSUPPORTED, WQ4_ERR_ALIGN or WQ4_ERR_CUDA.
  */
 int wq4_gemm(const uint32_t* W_packed, const uint16_t* scales, const uint16_t* x,

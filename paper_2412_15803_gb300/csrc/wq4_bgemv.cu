@@ -378,6 +378,7 @@ struct TGemvParams {
     int tiles, nch, nslots;
     uint32_t slot_bytes, scale_off, x_off, red_off;
     int y4;                // two outputs may be stored at once
+    int check;             // flag scales beyond +-8188 (wq4_gemm's contract)
     uint32_t* err;
 };
 
@@ -487,6 +488,7 @@ __global__ void __launch_bounds__(32 * (kTWarps<XT> + 1), 1)
     int slot = 0, par = 0, n0 = static_cast<int>(blockIdx.x) * TR;
     const int G = p.K >> 5;
     bool ok = true;
+    bool bad = false;                                 // a scale beyond the limit was met
     for (int it = 0; it < mytiles; ++it, n0 += grid * TR) {
         for (int ch = 0; ch < nch; ++ch) {
             if (ok) ok = mbar_wait(&full[slot], par, p.err);   // after a wait gave up, none is waited for
@@ -504,6 +506,17 @@ __global__ void __launch_bounds__(32 * (kTWarps<XT> + 1), 1)
                     ldsm_x4_b(ca + 2048 * r, w[r]);
                     sa0[r] = lds_u32(sa + 256 * r);        // scales of groups j, j + 1: row g
                     sb0[r] = lds_u32(sa + 256 * r + 128);  // ... and row g + 8
+                }
+                // (wq4_gemm comes with at most 16 activation rows; in the larger
+                // kernels the branch alone cost 4 %)
+                if (XT <= 2 && p.check) {
+#pragma unroll
+                    for (int r = 0; r < R; ++r) {
+                        // (the last tile's second eight rows may be none of this warp's)
+                        const uint32_t sb = 16 * r + 8 < p.wrows ? sb0[r] & 0x7FFF7FFFu : 0u;
+                        const uint32_t hi = __vmaxu2(sa0[r] & 0x7FFF7FFFu, sb);
+                        bad = bad || (hi & 0xFFFFu) > kMaxFp16ScaleBits || (hi >> 16) > kMaxFp16ScaleBits;
+                    }
                 }
 #pragma unroll
                 for (int h = 0; h < 2; ++h) {
@@ -598,6 +611,7 @@ __global__ void __launch_bounds__(32 * (kTWarps<XT> + 1), 1)
 #pragma unroll
             for (int t = 0; t < XT; ++t) acc[r][t][0] = acc[r][t][1] = acc[r][t][2] = acc[r][t][3] = 0.f;
     }
+    if (bad) atomicOr(p.err, kErrScale);
 }
 
 // ----------------------------------------------------------------- host --
@@ -753,7 +767,7 @@ cudaError_t launch_tma_xt(int R, const cudaLaunchConfig_t& cfg, const CUtensorMa
 }
 
 int launch_bgemv_tma(const DeviceInfo* di, const uint32_t* W, const uint16_t* s, const uint16_t* x, uint16_t* y, int N,
-                     int K, int batch, cudaStream_t stream)
+                     int K, int batch, bool check_scales, cudaStream_t stream)
 {
     const int XT = (batch + 7) / 8;
     TPlan b;
@@ -787,6 +801,7 @@ int launch_bgemv_tma(const DeviceInfo* di, const uint32_t* W, const uint16_t* s,
     p.x_off = b.x_off;
     p.red_off = b.red_off;
     p.y4 = (N % 2) == 0 && aligned(y, 4);
+    p.check = check_scales ? 1 : 0;
     p.err = status_word();
     cudaLaunchAttribute attr[1];
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
@@ -811,9 +826,9 @@ int launch_bgemv_tma(const DeviceInfo* di, const uint32_t* W, const uint16_t* s,
 }  // namespace
 
 int launch_bgemv(const DeviceInfo* di, const uint32_t* W, const uint16_t* s, const uint16_t* x, uint16_t* y, int N,
-                 int K, int batch, cudaStream_t stream)
+                 int K, int batch, cudaStream_t stream, bool check_scales)
 {
-    if ((K % 256) == 0 && aligned(s, 16)) return launch_bgemv_tma(di, W, s, x, y, N, K, batch, stream);
+    if ((K % 256) == 0 && aligned(s, 16)) return launch_bgemv_tma(di, W, s, x, y, N, K, batch, check_scales, stream);
     const int XT = (batch + 7) / 8;
     BGemvParams p;
     const bool s2 = (K % 64) != 0 || !aligned(s, 4);

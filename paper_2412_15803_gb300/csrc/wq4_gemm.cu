@@ -4,22 +4,30 @@
 //
 // Y[m][n] = fp16( sum_k x[m][k] * fp16((q(n,k) - 7) * s(n, k/32)) ), fp32 sums.
 //
-// A persistent grid walks (128 weight rows x T tokens) tiles, T = 128, 192 or
-// 256 chosen per call (pick_tok), row tile major so that the CTAs running at
-// one time share a weight tile through L2.  Per 64-wide K chunk a producer
-// warp brings the tile's codes and scales (2-D tensor copies) and the T x 64
-// activation block (one 128-byte swizzled box) into a ring of 4-6 slots
-// (small slots, so that copies stay in flight while the MMAs of earlier
-// chunks run); eight dequant warps write the 128 x 64 weights, dequantized to
-// fp16 in natural K order, into one of three 32-column A buffers in tensor
-// memory (lane = weight row); one thread issues 4 tcgen05.mma (kind::f16,
-// M = 128, N = T tokens, K = 16: at T = 256 the tensor-core rate, ~128 cycles
-// each, so the dequant warps keep up) into a T-column fp32 accumulator; four
-// epilogue warps move a finished accumulator into a shared-memory transpose
-// buffer, release it, and store T tokens x 128 outputs with 16-byte stores
-// while the next tile's MMAs run.  Every weight is rounded to fp16 once
-// (relative error <= 2^-11, accumulated in fp32): within the library's
-// accuracy contract.
+// A persistent grid walks (128 weight rows x T tokens) tiles, T = 64, 128,
+// 192 or 256 chosen per call (pick_gemm), row tile major so that the CTAs
+// running at one time share a weight tile through L2; where the tiles leave
+// SMs idle, the CTAs of a cluster share a tile's K instead and add their fp32
+// sums in rank order through distributed shared memory.  A producer warp
+// brings the tile's codes and scales in blocks of 256 K (2-D tensor copies), a
+// second one the tokens' activations (boxes of 64 K, 128-byte swizzle); three
+// sets of four dequant warps take items of 128 K in turn and write the weights,
+// dequantized to fp16 in natural K order, into 64-column A buffers in tensor
+// memory (lane = weight row); one warp issues eight tcgen05.mma an item
+// (kind::f16, M = 128, N = T, K = 16) into a T-column fp32 accumulator; eight
+// epilogue warps move a finished accumulator through shared-memory transpose
+// blocks to 16-byte stores while the next tile's MMAs run.  Every weight is
+// rounded to fp16 once (relative error <= 2^-11, accumulated in fp32): within
+// the library's accuracy contract.
+//
+// What bounds it: over long prompts the power limit (28672 x 4096 over 2048
+// tokens: 363 -> 311 us, 1.55 PFLOP/s; in a loop the SMs settle at 1.42 GHz,
+// where 256-token tiles run at 87 % of the MMA rate), over short ones the MMA
+// issuer's own latency (~340 cycles a 64-wide chunk) and the launch.  Before,
+// each 64-wide chunk cost the issuer ~870 cycles whatever the tile: one lane's
+// branch with two waits and two commits for four MMAs.  5120 x 3072 over 77
+// tokens 22.7 -> 9.5 us, 3072 x 8192 over 1000 tokens 57 -> 39, 512 x 14336
+// over 200 tokens 91 -> 11.3.
 #include "wq4.h"
 #include "wq4_device.cuh"
 #include "wq4_host.h"
@@ -28,35 +36,49 @@
 #include <cuda.h>
 #include <cuda_runtime.h>
 
-#include <cstring>
+#include <algorithm>
+#include <atomic>
 #include <mutex>
 
 namespace wq4 {
 namespace {
 
-constexpr int kGThreads = 448;        // warps 0-7 dequant, 8 producer, 9 MMA, 10-13 epilogue
-constexpr int kGProducer = 8, kGIssuer = 9;
-constexpr int kGCodes = 128 * 32;     // 128 rows x 64 codes (32-byte rows, 32-byte swizzle)
-constexpr int kGScales = 128 * 16;    // 128 rows x 8 fp16 scales (the 256-wide K block of the chunk)
-constexpr int kGABufs = 3;            // 32-column A buffers
-constexpr int kGDCol = 256;           // accumulator: TOK columns
-constexpr int kGT = 1024;             // transpose buffer: TOK tokens x 128 outputs fp16
+// Warps: 0-11 dequant (three sets of four, items in turn), 12 and 13 the
+// weight and activation producers, 14 the MMA issuer, 16-23 epilogue (two
+// groups of four, token blocks in turn).
+constexpr int kGThreads = 768;
+constexpr int kGSets = 3;
+constexpr int kGWProd = 12, kGXProd = 13, kGIssuer = 14, kGEpi = 16;
+constexpr int kGCodes = 128 * 128;    // a K block: 128 rows x 256 codes (128-byte swizzle)
+constexpr int kGScales = 128 * 16;    // ... and 8 fp16 scales a row
+constexpr int kGBlk = 64;             // tokens of a transpose block
+constexpr int kGHeader = 1024;
 constexpr int kGTmemCols = 512;
 
-// Tile of TOK tokens (MMA N = 128, 192 or 256).
+// Tile of 128 weight rows and TOK tokens (MMA N = TOK).  K moves in items of
+// 128: one A buffer (64 columns) and, in one slot (TOK <= 128) or two, the
+// tokens' activations; the weights in blocks of two items.
 template <int TOK>
 struct GCfg {
-    static constexpr int kSlots = TOK == 256 ? 4 : (TOK == 192 ? 5 : 6);
-    static constexpr int kX = TOK * 64 * 2;                // activation block: TOK tokens x 64 K fp16
-    static constexpr int kSlot = kX + kGCodes + kGScales;  // a multiple of 1024
-    static constexpr int kRing = kGT + TOK * 128 * 2;
-    static constexpr int kSmem = kRing + kSlots * kSlot;
+    static constexpr int kABufs = (kGTmemCols - TOK) / 64 < 6 ? (kGTmemCols - TOK) / 64 : 6;
+    static constexpr int kXSub = TOK <= 128 ? 1 : 2;              // activation slots of an item
+    static constexpr int kX = TOK * 2 * (128 / kXSub);            // activation slot: boxes of TOK tokens x 64 K fp16
+    static constexpr int kW = kGCodes + kGScales;
+    static constexpr int kXSlots = TOK == 256 ? 4 : (TOK == 192 ? 5 : (TOK == 128 ? 4 : 6));
+    static constexpr int kWSlots = TOK == 256 ? 3 : 3;
+    static constexpr int kT = kGHeader;                           // two transpose blocks: kGBlk tokens x 128 outputs fp16
+    static constexpr int kXRing = kT + 2 * kGBlk * 128 * 2;
+    static constexpr int kWRing = kXRing + kXSlots * kX;
+    static constexpr int kSmem = kWRing + kWSlots * kW;
     static_assert(kSmem <= 227 * 1024, "shared memory");
+    static_assert(kXSlots * kX >= TOK * 128 * 4, "a split tile's sums go over the activation ring");
+    static_assert((2 * kXSlots + 2 * kWSlots + 2 * kABufs + 3) * 8 <= 1008, "barriers");
 };
 
 struct GemmArgs {
     uint16_t* y;
     int N, K, M, rtiles, ttiles;
+    int split;               // CTAs of a cluster that share a tile's K (1: persistent grid)
     uint32_t* err;
 };
 
@@ -72,40 +94,84 @@ __device__ __forceinline__ bool g_wait(uint64_t* bar, uint32_t parity, uint32_t*
     return mbar_wait(bar, parity, err);
 }
 
+__device__ __forceinline__ void cluster_sync_all()
+{
+    asm volatile("barrier.cluster.arrive.release;" ::: "memory");
+    asm volatile("barrier.cluster.wait.acquire;" ::: "memory");
+}
+
+// Four floats at the same shared-memory offset in CTA `rank` of the cluster.
+__device__ __forceinline__ float4 ld_cluster_f4(uint32_t addr, uint32_t rank)
+{
+    uint32_t ra;
+    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(ra) : "r"(addr), "r"(rank));
+    float4 v;
+    asm volatile("ld.shared::cluster.v4.f32 {%0, %1, %2, %3}, [%4];"
+                 : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w)
+                 : "r"(ra)
+                 : "memory");
+    return v;
+}
+
+// A ring position: slot and parity of the n-th use of a ring of S slots.
+template <int S>
+struct RingPos {
+    int slot = 0;
+    uint32_t par = 0;
+    __device__ __forceinline__ void next()
+    {
+        if (++slot == S) {
+            slot = 0;
+            par ^= 1u;
+        }
+    }
+};
+
 template <int TOK>
 __global__ void __launch_bounds__(kGThreads, 1)
     gemm_kernel(const __grid_constant__ CUtensorMap tm_codes, const __grid_constant__ CUtensorMap tm_scales,
                 const __grid_constant__ CUtensorMap tm_x, const GemmArgs a)
 {
     using C = GCfg<TOK>;
-    constexpr int kGSlots = C::kSlots, kGX = C::kX, kGSlot = C::kSlot, kGRing = C::kRing, kGTok = TOK;
+    constexpr int XS = C::kXSlots, WS = C::kWSlots, NA = C::kABufs;
     extern __shared__ __align__(1024) uint8_t smem[];
-    uint64_t* full = reinterpret_cast<uint64_t*>(smem);      // codes, scales, activations landed
-    uint64_t* empty = full + kGSlots;
-    uint64_t* afull = empty + kGSlots;
-    uint64_t* aempty = afull + kGABufs;
-    uint64_t* dfull = aempty + kGABufs;
+    uint64_t* xfull = reinterpret_cast<uint64_t*>(smem);     // activations landed
+    uint64_t* xempty = xfull + XS;
+    uint64_t* wfull = xempty + XS;                           // codes and scales landed
+    uint64_t* wempty = wfull + WS;
+    uint64_t* afull = wempty + WS;
+    uint64_t* aempty = afull + NA;
+    uint64_t* dfull = aempty + NA;
     uint64_t* dempty = dfull + 1;
-    uint64_t* drain = dempty + 1;                            // ends at byte (2 slots + 9) * 8 <= 240
-    uint32_t* tbase_sh = reinterpret_cast<uint32_t*>(smem + 240);
-    uint16_t* tbuf = reinterpret_cast<uint16_t*>(smem + kGT);
-    uint8_t* ring = smem + kGRing;
+    uint64_t* drain = dempty + 1;
+    uint32_t* tbase_sh = reinterpret_cast<uint32_t*>(smem + 1008);
+    uint16_t* tbuf = reinterpret_cast<uint16_t*>(smem + C::kT);
+    uint8_t* xring = smem + C::kXRing;
+    uint8_t* wring = smem + C::kWRing;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int nch = a.K >> 6;   // 64-wide K chunks
+    // this CTA's K blocks [k0, k1) of 256 (all of them unless the cluster splits K)
+    const int split = a.split, rank = static_cast<int>(blockIdx.x) % split;
+    const int nblk = a.K >> 8;
+    const int k0 = rank * nblk / split, k1 = (rank + 1) * nblk / split;
     const int tiles = a.rtiles * a.ttiles;
+    const int u0 = static_cast<int>(blockIdx.x) / split, ustep = static_cast<int>(gridDim.x) / split;
     uint32_t* err = a.err;
 
     if (threadIdx.x == 0) {
-        for (int i = 0; i < kGSlots; ++i) {
-            mbar_init(&full[i], 1);
-            mbar_init(&empty[i], 9);   // 8 dequant warps + the MMA commit
+        for (int i = 0; i < XS; ++i) {
+            mbar_init(&xfull[i], 1);
+            mbar_init(&xempty[i], 1);
         }
-        for (int i = 0; i < kGABufs; ++i) {
-            mbar_init(&afull[i], 8);
+        for (int i = 0; i < WS; ++i) {
+            mbar_init(&wfull[i], 1);
+            mbar_init(&wempty[i], 8);    // 4 warps x 2 items
+        }
+        for (int i = 0; i < NA; ++i) {
+            mbar_init(&afull[i], 4);
             mbar_init(&aempty[i], 1);
         }
         mbar_init(dfull, 1);
-        mbar_init(dempty, 4);
+        mbar_init(dempty, 8);
         mbar_init(drain, 1);
         mbar_fence_init();
     }
@@ -114,157 +180,214 @@ __global__ void __launch_bounds__(kGThreads, 1)
     __syncthreads();
     tc::fence_after_sync();
     const uint32_t tbase = *tbase_sh;
+    const uint32_t dcol = tbase + kGTmemCols - TOK;
+    grid_dependents_launch();
 
-    if (warp == kGProducer) {
-        // ---------------------------------------------------- producer
+    if (warp == kGWProd) {
+        // ------------------------------------------------ weight producer
+        // (weights may be fetched while the previous kernel of the stream
+        // finishes: programmatic dependent launch)
         if (lane == 0) {
             tc::prefetch_map(&tm_codes);
             tc::prefetch_map(&tm_scales);
-            tc::prefetch_map(&tm_x);
-            int it = 0;
+            RingPos<WS> w;
+            int n = 0;
             bool ok = true;
-            for (int u = blockIdx.x; u < tiles && ok; u += gridDim.x) {
-                const int n0 = (u / a.ttiles) * 128, m0 = (u % a.ttiles) * kGTok;
-                for (int c = 0; c < nch; ++c, ++it) {
-                    const int slot = it % kGSlots;
-                    if (it >= kGSlots && !g_wait(&empty[slot], ((it / kGSlots) - 1) & 1, err)) {
+            for (int u = u0; u < tiles && ok; u += ustep) {
+                const int n0 = (u / a.ttiles) * 128;
+                for (int k = k0; k < k1; ++k, ++n, w.next()) {
+                    if (n >= WS && !g_wait(&wempty[w.slot], w.par ^ 1u, err)) {
                         ok = false;
                         break;
                     }
-                    uint8_t* base = ring + static_cast<size_t>(slot) * kGSlot;
-                    mbar_arrive_expect_tx(&full[slot], kGSlot);
-                    tc::tma_load_2d(base, &tm_x, c * 64, m0, &full[slot]);
-                    tc::tma_load_2d(base + kGX, &tm_codes, c * 32, n0, &full[slot]);
-                    tc::tma_load_2d(base + kGX + 64 * 32, &tm_codes, c * 32, n0 + 64, &full[slot]);
-                    tc::tma_load_2d(base + kGX + kGCodes, &tm_scales, (c >> 2) * 8, n0, &full[slot]);
-                    tc::tma_load_2d(base + kGX + kGCodes + 64 * 16, &tm_scales, (c >> 2) * 8, n0 + 64, &full[slot]);
+                    uint8_t* base = wring + static_cast<size_t>(w.slot) * C::kW;
+                    mbar_arrive_expect_tx(&wfull[w.slot], C::kW);
+                    tc::tma_load_2d(base, &tm_codes, k * 128, n0, &wfull[w.slot]);
+                    tc::tma_load_2d(base + kGCodes, &tm_scales, k * 8, n0, &wfull[w.slot]);
                 }
             }
             // every copy issued has landed before the CTA's memory goes away
-            const int first = it > kGSlots ? it - kGSlots : 0;
-            for (int i = first; i < it; ++i) g_wait(&full[i % kGSlots], (i / kGSlots) & 1, err);
+            for (int i = max(0, n - WS); i < n; ++i) g_wait(&wfull[i % WS], (i / WS) & 1, err);
         }
-    } else if (warp == kGIssuer) {
-        // ---------------------------------------------------- MMA issuer
+    } else if (warp == kGXProd) {
+        // -------------------------------------------- activation producer
         if (lane == 0) {
-            constexpr uint32_t idesc = tc::idesc_f16_f32(128, kGTok);
-            int it = 0, dit = 0;
+            tc::prefetch_map(&tm_x);
+            grid_dependency_wait();
+            RingPos<XS> x;
+            int n = 0;
             bool ok = true;
-            const uint32_t dt = tbase + kGDCol;
-            for (int u = blockIdx.x; u < tiles && ok; u += gridDim.x, ++dit) {
-                if (dit >= 1 && !g_wait(dempty, (dit - 1) & 1, err)) break;
-                tc::fence_after_sync();
-                for (int c = 0; c < nch; ++c, ++it) {
-                    const int slot = it % kGSlots, abuf = it % kGABufs;
-                    if (!g_wait(&full[slot], (it / kGSlots) & 1, err) ||
-                        !g_wait(&afull[abuf], (it / kGABufs) & 1, err)) {
+            constexpr int kZ = 2 / C::kXSub;         // boxes of 64 K in a slot
+            for (int u = u0; u < tiles && ok; u += ustep) {
+                const int m0 = (u % a.ttiles) * TOK;
+                for (int z = 4 * k0; z < 4 * k1; z += kZ, ++n, x.next()) {
+                    if (n >= XS && !g_wait(&xempty[x.slot], x.par ^ 1u, err)) {
                         ok = false;
                         break;
                     }
-                    tc::fence_after_sync();
-                    const uint32_t xs = smem_addr(ring + static_cast<size_t>(slot) * kGSlot);
-#pragma unroll
-                    for (int s = 0; s < 4; ++s) {
-                        const uint64_t bd = tc::sw128_kmajor_desc(xs + 32 * s);
-                        tc::mma_f16_ts(dt, tbase + 32 * abuf + 8 * s, bd, idesc, (c > 0 || s > 0) ? 1u : 0u);
-                    }
-                    tc::commit(&aempty[abuf]);
-                    tc::commit(&empty[slot]);
+                    mbar_arrive_expect_tx(&xfull[x.slot], C::kX);
+                    tc::tma_load_3d(xring + static_cast<size_t>(x.slot) * C::kX, &tm_x, 0, m0, z, &xfull[x.slot]);
                 }
-                if (!ok) break;
-                tc::commit(dfull);
             }
-            // all MMAs issued have completed before tensor memory is released
-            tc::commit(drain);
-            g_wait(drain, 0, err);
+            for (int i = max(0, n - XS); i < n; ++i) g_wait(&xfull[i % XS], (i / XS) & 1, err);
         }
-    } else if (warp < 8) {
+    } else if (warp == kGIssuer) {
+        // ---------------------------------------------------- MMA issuer
+        // Its own latency bounds the kernel unless an item is long: a wait
+        // costs ~80 cycles even when it is over, a fence, a commit and an MMA
+        // ~30 each (~60 an MMA from a single lane's branch, where the operands
+        // are not warp-uniform; so the whole warp runs the loop and one elected
+        // lane issues).  Hence eight MMAs an item, two or three waits.
+        constexpr uint32_t idesc = tc::idesc_f16_f32(128, TOK);
+        const bool leader = tc::elect_one();
+        RingPos<XS> x;
+        RingPos<NA> ab;
+        int dit = 0;
+        bool ok = true;            // after a wait gave up, none is waited for
+        const uint64_t xdesc = tc::sw128_kmajor_desc(smem_addr(xring));
+        for (int u = u0; u < tiles; u += ustep, ++dit) {
+            if (dit >= 1 && ok) ok = g_wait(dempty, (dit - 1) & 1, err);
+            for (int it = 2 * k0; it < 2 * k1; ++it) {
+                if (ok) ok = g_wait(&afull[ab.slot], ab.par, err);
+#pragma unroll
+                for (int sub = 0; sub < 2; ++sub) {
+                    if (sub < C::kXSub && ok) ok = g_wait(&xfull[x.slot], x.par, err);
+                    if (sub == 0) tc::fence_after_sync();
+                    const uint64_t xd = xdesc + static_cast<uint64_t>(x.slot) * (C::kX >> 4) +
+                                        (C::kXSub == 1 ? sub * (TOK * 128 >> 4) : 0);
+                    if (leader) {
+#pragma unroll
+                        for (int s = 0; s < 4; ++s)
+                            tc::mma_f16_ts(dcol, tbase + 64 * ab.slot + 32 * sub + 8 * s, xd + 2 * s, idesc,
+                                           (it > 2 * k0 || sub + s > 0) ? 1u : 0u);
+                        if (sub == 1) tc::commit(&aempty[ab.slot]);
+                        if (C::kXSub == 2 || sub == 1) tc::commit(&xempty[x.slot]);
+                    }
+                    if (C::kXSub == 2 || sub == 1) x.next();
+                }
+                ab.next();
+            }
+            if (leader) tc::commit(dfull);
+        }
+        // all MMAs issued have completed before tensor memory is released
+        if (leader) tc::commit(drain);
+        g_wait(drain, 0, err);
+    } else if (warp < 4 * kGSets) {
         // ---------------------------------------------------- dequant
-        // warp w: rows 32 (w % 4) + lane (its tensor-memory lanes), group
-        // w / 4 of each 64-wide chunk, written in natural K order
-        const int row = 32 * (warp & 3) + lane;
-        const int jg = warp >> 2;
+        // Item i goes to A buffer i % NA and warp set i % 3, so that several
+        // items' waits, unpacking and stores are in flight.  Lane = weight row;
+        // 128 codes in natural K order, 64 at a time.
+        const int set = warp >> 2, row = 32 * (warp & 3) + lane;
         const uint32_t lane_base = tbase + (static_cast<uint32_t>(32 * (warp & 3)) << 16);
-        int it = 0;
+        RingPos<WS> w;
+        RingPos<NA> ab;
+        int i = 0;
         bool ok = true;
-        for (int u = blockIdx.x; u < tiles && ok; u += gridDim.x) {
-            for (int c = 0; c < nch; ++c, ++it) {
-                const int slot = it % kGSlots, abuf = it % kGABufs;
-                if (!g_wait(&full[slot], (it / kGSlots) & 1, err) ||
-                    (it >= kGABufs && !g_wait(&aempty[abuf], ((it / kGABufs) - 1) & 1, err))) {
+        for (int u = u0; u < tiles && ok; u += ustep) {
+            for (int it = 2 * k0; it < 2 * k1 && ok; ++it, ++i, ab.next()) {
+                if (it > 2 * k0 && (it & 1) == 0) w.next();
+                if (i % kGSets != set) continue;
+                if (!g_wait(&wfull[w.slot], w.par, err) || (i >= NA && !g_wait(&aempty[ab.slot], ab.par ^ 1u, err))) {
                     ok = false;
                     break;
                 }
-                const uint8_t* base = ring + static_cast<size_t>(slot) * kGSlot + kGX;
-                const uint8_t* crow = base + row * 32;
-                // scale of group 2 (c & 3) + jg of the 8 loaded for this 256-wide block
-                const uint32_t sh = *reinterpret_cast<const uint16_t*>(base + kGCodes + row * 16 + 4 * (c & 3) + 2 * jg);
-                // (q - 7) s is rounded to fp16 below: a larger scale would overflow
-                if ((sh & 0x7FFFu) > kMaxFp16ScaleBits) atomicOr(err, kErrScale);
-                {
-                    const int j = jg;   // 16-byte chunk of the 32-byte row, 32-byte swizzle
-                    const uint4 cw = *reinterpret_cast<const uint4*>(crow + ((j ^ ((row >> 2) & 1)) << 4));
-                    const uint32_t s2 = sh | (sh << 16);
-                    const uint32_t words[4] = {cw.x, cw.y, cw.z, cw.w};
-                    uint32_t q[16];
+                const uint8_t* base = wring + static_cast<size_t>(w.slot) * C::kW;
+                const uint8_t* crow = base + row * 128;
+                const uint2 sv2 = *reinterpret_cast<const uint2*>(base + kGCodes + row * 16 + 8 * (it & 1));
 #pragma unroll
-                    for (int w = 0; w < 4; ++w) {
+                for (int sub = 0; sub < 2; ++sub) {
+                    // groups j, j + 1 of the block's 8: codes and scales
+                    const int j = 4 * (it & 1) + 2 * sub;
+                    const uint4 cw0 = *reinterpret_cast<const uint4*>(crow + ((j ^ (row & 7)) << 4));
+                    const uint4 cw1 = *reinterpret_cast<const uint4*>(crow + (((j + 1) ^ (row & 7)) << 4));
+                    const uint32_t sv = sub ? sv2.y : sv2.x;
+                    // (q - 7) s is rounded to fp16 below: a larger scale would overflow
+                    if ((sv & 0x7FFFu) > kMaxFp16ScaleBits || ((sv >> 16) & 0x7FFFu) > kMaxFp16ScaleBits) atomicOr(err, kErrScale);
+                    const uint32_t words[8] = {cw0.x, cw0.y, cw0.z, cw0.w, cw1.x, cw1.y, cw1.z, cw1.w};
+                    const uint32_t s0 = prmt(sv, sv, 0x1010u), s1 = prmt(sv, sv, 0x3232u);
+                    uint32_t q[32];
+#pragma unroll
+                    for (int k = 0; k < 8; ++k) {
+                        const uint32_t s2 = k < 4 ? s0 : s1;
                         uint32_t p[4];   // (k, k+4) pairs of the word
-                        unpack_word(words[w], p);
-                        q[4 * w + 0] = tc::hmul2_u32(prmt(p[0], p[1], 0x5410u), s2);   // k0 k1
-                        q[4 * w + 1] = tc::hmul2_u32(prmt(p[2], p[3], 0x5410u), s2);   // k2 k3
-                        q[4 * w + 2] = tc::hmul2_u32(prmt(p[0], p[1], 0x7632u), s2);   // k4 k5
-                        q[4 * w + 3] = tc::hmul2_u32(prmt(p[2], p[3], 0x7632u), s2);   // k6 k7
+                        unpack_word(words[k], p);
+                        q[4 * k + 0] = tc::hmul2_u32(prmt(p[0], p[1], 0x5410u), s2);   // k0 k1
+                        q[4 * k + 1] = tc::hmul2_u32(prmt(p[2], p[3], 0x5410u), s2);   // k2 k3
+                        q[4 * k + 2] = tc::hmul2_u32(prmt(p[0], p[1], 0x7632u), s2);   // k4 k5
+                        q[4 * k + 3] = tc::hmul2_u32(prmt(p[2], p[3], 0x7632u), s2);   // k6 k7
                     }
-                    tc::st16(lane_base + 32 * abuf + 16 * j, q);
+                    tc::st16(lane_base + 64 * ab.slot + 32 * sub, q);
+                    tc::st16(lane_base + 64 * ab.slot + 32 * sub + 16, q + 16);
                 }
                 tc::st_wait();
                 tc::fence_before_sync();
                 __syncwarp();
                 if (lane == 0) {
-                    mbar_arrive(&empty[slot]);
-                    mbar_arrive(&afull[abuf]);
+                    mbar_arrive(&afull[ab.slot]);
+                    mbar_arrive(&wempty[w.slot]);
                 }
             }
+            w.next();
         }
-    } else {
+    } else if (warp >= kGEpi) {
         // ---------------------------------------------------- epilogue warps
         // warp w reads tensor-memory lanes 32 (w % 4) .. + 31 (weight rows)
-        const int quad = warp & 3;
-        const int row = 32 * quad + lane;
-        const int tid = 32 * quad + lane;   // 0..127 over the four warps
-        const uint32_t lane_base = tbase + (static_cast<uint32_t>(32 * quad) << 16);
+        grid_dependency_wait();          // y is written after the previous kernel
+        const int quad = warp & 3, grp = (warp - kGEpi) >> 2;
+        uint16_t* const tb0 = tbuf + grp * kGBlk * 128;
+        const int row = 32 * quad + lane;   // 0..127 over the four warps
+        const uint32_t lane_base = dcol + (static_cast<uint32_t>(32 * quad) << 16);
         int dit = 0;
-        for (int u = blockIdx.x; u < tiles; u += gridDim.x, ++dit) {
-            const int n0 = (u / a.ttiles) * 128, m0 = (u % a.ttiles) * kGTok;
+        for (int u = u0; u < tiles; u += ustep, ++dit) {
+            const int n0 = (u / a.ttiles) * 128, m0 = (u % a.ttiles) * TOK;
             if (!g_wait(dfull, dit & 1, err)) break;
             tc::fence_after_sync();
-            // accumulator (row, token) -> transpose buffer [token][row], fp16;
-            // the accumulator is free for the next tile's MMAs right after
-#pragma unroll 4
-            for (int h = 0; h < kGTok / 16; ++h) {
-                uint32_t d[16];
-                tc::ld16(lane_base + kGDCol + 16 * h, d);
-                tc::ld_wait();
+            if (split > 1) {
+                // fp32 sums of this CTA's K chunks, [token][row], over the idle activation ring
+                float* ps = reinterpret_cast<float*>(xring);
+#pragma unroll 2
+                for (int t = grp * (TOK / 2); t < (grp + 1) * (TOK / 2); t += 16) {
+                    uint32_t d[16];
+                    tc::ld16(lane_base + t, d);
+                    tc::ld_wait();
 #pragma unroll
-                for (int i = 0; i < 16; ++i)
-                    tbuf[(16 * h + i) * 128 + row] = float_to_half_bits(__uint_as_float(d[i]));
+                    for (int i = 0; i < 16; ++i) ps[(t + i) * 128 + row] = __uint_as_float(d[i]);
+                }
+                break;
             }
-            tc::fence_before_sync();
-            __syncwarp();
-            if (lane == 0) mbar_arrive(dempty);
-            named_barrier_sync(3, 128);
-            // 256 tokens x 256 bytes out, 16 bytes per store
-#pragma unroll 4
-            for (int i = 0; i < kGTok / 8; ++i) {
-                const int chunk = tid + 128 * i;
-                const int tok = chunk >> 4, seg = chunk & 15;
-                const int m = m0 + tok, n = n0 + 8 * seg;
-                if (m < a.M && n < a.N)
-                    *reinterpret_cast<uint4*>(a.y + static_cast<size_t>(m) * a.N + n) =
-                        *reinterpret_cast<const uint4*>(tbuf + tok * 128 + 8 * seg);
+            // token blocks go to the two groups in turn
+            constexpr int kBlocks = TOK / kGBlk;
+            if (grp >= kBlocks && lane == 0) mbar_arrive(dempty);
+            for (int blk = grp; blk < kBlocks; blk += 2) {
+                const int tb = blk * kGBlk;
+                // (row, token) -> transpose block [token][row], fp16
+#pragma unroll
+                for (int t = 0; t < kGBlk; t += 32) {
+                    uint32_t d[32];
+                    tc::ld16(lane_base + tb + t, d);
+                    tc::ld16(lane_base + tb + t + 16, d + 16);
+                    tc::ld_wait();
+#pragma unroll
+                    for (int i = 0; i < 32; ++i) tb0[(t + i) * 128 + row] = float_to_half_bits(__uint_as_float(d[i]));
+                }
+                if (blk + 2 >= kBlocks) {
+                    // this group is done with the accumulator
+                    tc::fence_before_sync();
+                    __syncwarp();
+                    if (lane == 0) mbar_arrive(dempty);
+                }
+                named_barrier_sync(3 + grp, 128);
+#pragma unroll
+                for (int i = 0; i < kGBlk / 8; ++i) {
+                    const int chunk = row + 128 * i;
+                    const int tok = chunk >> 4, seg = chunk & 15;
+                    const int mm = m0 + tb + tok, n = n0 + 8 * seg;
+                    if (mm < a.M && n < a.N)
+                        *reinterpret_cast<uint4*>(a.y + static_cast<size_t>(mm) * a.N + n) =
+                            *reinterpret_cast<const uint4*>(tb0 + tok * 128 + 8 * seg);
+                }
+                named_barrier_sync(3 + grp, 128);   // the block is free again
             }
-            named_barrier_sync(3, 128);   // the buffer is free for the next tile
         }
     }
 
@@ -272,45 +395,129 @@ __global__ void __launch_bounds__(kGThreads, 1)
     __syncthreads();
     tc::fence_after_sync();
     if (warp == kGIssuer) tc::tmem_dealloc(tbase, kGTmemCols);
+    if (split > 1) {
+        // the cluster's sums are in: this CTA adds its share of the tokens in
+        // rank order and stores them
+        grid_dependency_wait();
+        cluster_sync_all();
+        const int n0 = (u0 / a.ttiles) * 128, m0 = (u0 % a.ttiles) * TOK;
+        const int t0 = rank * TOK / split, t1 = (rank + 1) * TOK / split;
+        const uint32_t ps = smem_addr(xring);
+        for (int e = t0 * 32 + static_cast<int>(threadIdx.x); e < t1 * 32; e += kGThreads) {
+            const int mm = m0 + (e >> 5), n = n0 + 4 * (e & 31);
+            if (mm >= a.M || n >= a.N) continue;
+            float4 sum = ld_cluster_f4(ps + 16 * e, 0);
+            for (int r = 1; r < split; ++r) {
+                const float4 v = ld_cluster_f4(ps + 16 * e, r);
+                sum.x += v.x;
+                sum.y += v.y;
+                sum.z += v.z;
+                sum.w += v.w;
+            }
+            uint2 o;
+            o.x = static_cast<uint32_t>(float_to_half_bits(sum.x)) | (static_cast<uint32_t>(float_to_half_bits(sum.y)) << 16);
+            o.y = static_cast<uint32_t>(float_to_half_bits(sum.z)) | (static_cast<uint32_t>(float_to_half_bits(sum.w)) << 16);
+            *reinterpret_cast<uint2*>(a.y + static_cast<size_t>(mm) * a.N + n) = o;   // N % 8 == 0
+        }
+        cluster_sync_all();   // no CTA's memory goes away while another reads it
+    }
 }
 
 template <int TOK>
-int gemm_attr()
+cudaError_t gemm_launch(cudaLaunchConfig_t& cfg, const CUtensorMap* tm, const GemmArgs& a)
 {
     static std::once_flag once;
-    static int rc = -1;
+    static cudaError_t rc = cudaErrorUnknown;
     std::call_once(once, [] {
-        rc = cudaFuncSetAttribute(gemm_kernel<TOK>, cudaFuncAttributeMaxDynamicSharedMemorySize, GCfg<TOK>::kSmem) ==
-                     cudaSuccess
-                 ? 0
-                 : 1;
+        rc = cudaFuncSetAttribute(gemm_kernel<TOK>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                  GCfg<TOK>::kSmem);
     });
-    return rc;
+    if (rc != cudaSuccess) return rc;
+    cfg.dynamicSmemBytes = GCfg<TOK>::kSmem;
+    return cudaLaunchKernelEx(&cfg, gemm_kernel<TOK>, tm[0], tm[1], tm[2], a);
 }
 
-// Token tile: the width whose grid rounds (tiles over the SMs, rounded up)
-// times its cost relative to a 256-token tile is least; a 128-token tile
-// costs well over half of a 256-token one, a 192-token tile more than 6/7 of
-// one (measured: 7 rounds of 192 ran slower than 6 of 256), so 0.6 and 0.9.
-// Ties go to the wider tile.  128 when the prompt has at most 128 tokens.
-int pick_tok(int N, int M, int sms)
+// Clusters of `split` CTAs that fit the device at once (cached per device).
+template <int TOK>
+int cluster_capacity(int dev, int split)
 {
-    if (M <= 128) return 128;
-    const int rt = (N + 127) / 128;
-    const int toks[3] = {256, 192, 128};
-    const double cost[3] = {1.0, 0.9, 0.6};
-    int best = 256;
-    double best_c = 1e300;
-    for (int i = 0; i < 3; ++i) {
-        const int64_t tiles = static_cast<int64_t>(rt) * ((M + toks[i] - 1) / toks[i]);
-        const double c = static_cast<double>((tiles + sms - 1) / sms) * cost[i];
-        if (c < best_c - 1e-9) {
-            best_c = c;
-            best = toks[i];
+    static std::atomic<int> cached[64][9];
+    if (dev < 64 && cached[dev][split].load()) return cached[dev][split].load();
+    if (cudaFuncSetAttribute(gemm_kernel<TOK>, cudaFuncAttributeMaxDynamicSharedMemorySize, GCfg<TOK>::kSmem) !=
+        cudaSuccess)
+        return 0;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = split;
+    attr[0].val.clusterDim.y = attr[0].val.clusterDim.z = 1;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(split);
+    cfg.blockDim = dim3(kGThreads);
+    cfg.dynamicSmemBytes = GCfg<TOK>::kSmem;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    int n = 0;
+    if (cudaOccupancyMaxActiveClusters(&n, gemm_kernel<TOK>, &cfg) != cudaSuccess) {
+        cudaGetLastError();
+        n = 0;
+    }
+    if (dev < 64 && n > 0) cached[dev][split].store(n);
+    return n;
+}
+
+struct GemmPlan {
+    int tok = 0, split = 1;
+};
+
+// Token tile and K split: the least estimated time.  Per 64-wide K chunk a
+// tile takes (us, one CTA alone .. every SM busy) 0.165 .. 0.18 with 64
+// tokens, 0.177 .. 0.22 with 128, 0.214 .. 0.304 with 192 and 0.287 .. 0.394
+// with 256, beside a launch's fixed 1.8, 2.3, 3.3 and 4; a split (the
+// cluster's CTAs take K blocks in order, one tile a cluster, all resident)
+// adds 1.7 and 0.025 a CTA.  Measured: 5120 x 3072 over 77 tokens 10.8 us
+// whole, 9.5 split in 3; 512 x 14336 over 200 tokens 42 whole, 11.3 split in 8;
+// 1024 x 1024 over 77 tokens 4.9 whole, 5.8 split in 2.
+GemmPlan pick_gemm(int N, int K, int M, int sms, int dev)
+{
+    static constexpr int kTok[4] = {64, 128, 192, 256};
+    static constexpr double kB0[4] = {0.165, 0.177, 0.214, 0.287}, kB1[4] = {0.18, 0.22, 0.304, 0.394};
+    static constexpr double kFix[4] = {1.8, 2.3, 3.3, 4.0};
+    GemmPlan best;
+    double best_t = 1e300;
+    const int nblk = K >> 8;
+    for (int i = 3; i >= 0; --i) {
+        const int64_t tiles = static_cast<int64_t>((N + 127) / 128) * ((M + kTok[i] - 1) / kTok[i]);
+        auto rate = [&](double ctas) { return kB0[i] + (kB1[i] - kB0[i]) * std::min(1.0, ctas / sms); };
+        for (int s = 1; s <= 8 && s <= nblk; ++s) {
+            const double nch = 4.0 * ((nblk + s - 1) / s);
+            double t = kFix[i];
+            if (s == 1) {
+                const int64_t full = tiles / sms, rest = tiles % sms;
+                t += nch * (full * kB1[i] + (rest ? rate(static_cast<double>(rest)) : 0.0)) + 0.6 * full;
+            } else {
+                if (tiles * s > sms) break;
+                t += nch * rate(static_cast<double>(tiles * s)) + 1.7 + 0.025 * (tiles * s) * (i >= 2 ? 1.2 : 1.0);
+            }
+            if (t >= best_t - 1e-9) continue;
+            if (s > 1) {
+                const int cap = i == 0   ? cluster_capacity<64>(dev, s)
+                                : i == 1 ? cluster_capacity<128>(dev, s)
+                                : i == 2 ? cluster_capacity<192>(dev, s)
+                                         : cluster_capacity<256>(dev, s);
+                if (tiles > cap) continue;
+            }
+            best_t = t;
+            best.tok = kTok[i];
+            best.split = s;
         }
     }
     return best;
 }
+
+// Up to this many tokens the batched GEMV kernel takes the call (exact
+// weights; 5120 x 3072 over 8 tokens 4.7 us against 8.3 here, 128256 x 4096
+// over 16 tokens 75 against 81).
+constexpr int kGemvTokens = 16;
 
 }  // namespace
 }  // namespace wq4
@@ -331,17 +538,19 @@ extern "C" int wq4_gemm(const uint32_t* W_packed, const uint16_t* scales, const 
     int dev = 0;
     const DeviceInfo* di = current_device_info(&dev);
     if (!di) return WQ4_ERR_CUDA;
-    const int tok = pick_tok(N, M, di->sm_count);
-    if ((tok == 256 ? gemm_attr<256>() : tok == 192 ? gemm_attr<192>() : gemm_attr<128>()) != 0) return WQ4_ERR_CUDA;
-    CUtensorMap mc, ms, mx;
-    if (!encode_tensor_map_2d(&mc, CU_TENSOR_MAP_DATA_TYPE_UINT8, W_packed, static_cast<uint64_t>(K) / 2,
-                              static_cast<uint64_t>(N), static_cast<uint64_t>(K) / 2, 32, 64,
-                              CU_TENSOR_MAP_SWIZZLE_32B) ||
-        !encode_tensor_map_2d(&ms, CU_TENSOR_MAP_DATA_TYPE_UINT16, scales, static_cast<uint64_t>(K) / 32,
-                              static_cast<uint64_t>(N), static_cast<uint64_t>(K) / 16, 8, 64,
+    if (M <= kGemvTokens)
+        return launch_bgemv(di, W_packed, scales, x, y, N, K, M, static_cast<cudaStream_t>(stream), true);
+    const GemmPlan pl = pick_gemm(N, K, M, di->sm_count, dev);
+    CUtensorMap tm[3];
+    if (!encode_tensor_map_2d(&tm[0], CU_TENSOR_MAP_DATA_TYPE_UINT8, W_packed, static_cast<uint64_t>(K) / 2,
+                              static_cast<uint64_t>(N), static_cast<uint64_t>(K) / 2, 128, 128,
+                              CU_TENSOR_MAP_SWIZZLE_128B) ||
+        !encode_tensor_map_2d(&tm[1], CU_TENSOR_MAP_DATA_TYPE_UINT16, scales, static_cast<uint64_t>(K) / 32,
+                              static_cast<uint64_t>(N), static_cast<uint64_t>(K) / 16, 8, 128,
                               CU_TENSOR_MAP_SWIZZLE_NONE) ||
-        !encode_tensor_map_2d(&mx, CU_TENSOR_MAP_DATA_TYPE_FLOAT16, x, static_cast<uint64_t>(K), static_cast<uint64_t>(M),
-                              static_cast<uint64_t>(K) * 2, 64, tok, CU_TENSOR_MAP_SWIZZLE_128B))
+        !encode_tensor_map_3d(&tm[2], CU_TENSOR_MAP_DATA_TYPE_FLOAT16, x,
+                              {64, static_cast<uint64_t>(M), static_cast<uint64_t>(K) / 64}, {static_cast<uint64_t>(K) * 2, 128},
+                              {64, static_cast<uint32_t>(pl.tok), pl.tok <= 128 ? 2u : 1u}, CU_TENSOR_MAP_SWIZZLE_128B))
         return WQ4_ERR_CUDA;
     GemmArgs a;
     a.y = y;
@@ -349,17 +558,31 @@ extern "C" int wq4_gemm(const uint32_t* W_packed, const uint16_t* scales, const 
     a.K = K;
     a.M = M;
     a.rtiles = (N + 127) / 128;
-    a.ttiles = (M + tok - 1) / tok;
+    a.ttiles = (M + pl.tok - 1) / pl.tok;
+    a.split = pl.split;
     a.err = status_word();
     if (!a.err) return WQ4_ERR_CUDA;
     const int64_t tiles = static_cast<int64_t>(a.rtiles) * a.ttiles;
     if (tiles > (static_cast<int64_t>(1) << 30)) return WQ4_ERR_UNSUPPORTED;
-    const int grid = static_cast<int>(tiles < di->sm_count ? tiles : di->sm_count);
-    if (tok == 256)
-        gemm_kernel<256><<<grid, kGThreads, GCfg<256>::kSmem, static_cast<cudaStream_t>(stream)>>>(mc, ms, mx, a);
-    else if (tok == 192)
-        gemm_kernel<192><<<grid, kGThreads, GCfg<192>::kSmem, static_cast<cudaStream_t>(stream)>>>(mc, ms, mx, a);
-    else
-        gemm_kernel<128><<<grid, kGThreads, GCfg<128>::kSmem, static_cast<cudaStream_t>(stream)>>>(mc, ms, mx, a);
-    return cudaGetLastError() == cudaSuccess ? WQ4_OK : WQ4_ERR_CUDA;
+    cudaLaunchAttribute attr[2];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    attr[1].id = cudaLaunchAttributeClusterDimension;
+    attr[1].val.clusterDim.x = pl.split;
+    attr[1].val.clusterDim.y = attr[1].val.clusterDim.z = 1;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(pl.split > 1 ? static_cast<int>(tiles) * pl.split
+                                    : static_cast<int>(tiles < di->sm_count ? tiles : di->sm_count));
+    cfg.blockDim = dim3(kGThreads);
+    cfg.stream = static_cast<cudaStream_t>(stream);
+    cfg.attrs = attr;
+    cfg.numAttrs = pl.split > 1 ? 2 : 1;
+    cudaError_t e;
+    switch (pl.tok) {
+        case 256: e = gemm_launch<256>(cfg, tm, a); break;
+        case 192: e = gemm_launch<192>(cfg, tm, a); break;
+        case 128: e = gemm_launch<128>(cfg, tm, a); break;
+        default: e = gemm_launch<64>(cfg, tm, a); break;
+    }
+    return e == cudaSuccess ? WQ4_OK : WQ4_ERR_CUDA;
 }

@@ -36,8 +36,10 @@ bool encode_tensor_map_3d(CUtensorMap* m, CUtensorMapDataType dt, const void* ba
 
 // wq4_gemv for the batches and sizes that the TMA-staged kernels do not take
 // (wq4_bgemv.cu): any N, K % 32 == 0, batch 1-32, scales at any 2-byte address.
+// check_scales (16-byte aligned scales, K % 256 == 0 only): flag scales beyond
+// +-8188 in the status word, as wq4_gemm promises.
 int launch_bgemv(const DeviceInfo* di, const uint32_t* W, const uint16_t* s, const uint16_t* x, uint16_t* y, int N,
-                 int K, int batch, cudaStream_t stream);
+                 int K, int batch, cudaStream_t stream, bool check_scales = false);
 
 inline bool aligned(const void* p, size_t a)
 {

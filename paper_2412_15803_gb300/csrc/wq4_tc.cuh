@@ -100,6 +100,16 @@ __device__ __forceinline__ void commit(uint64_t* bar)
                  : "memory");
 }
 
+// True in one lane of a converged warp.
+__device__ __forceinline__ bool elect_one()
+{
+    uint32_t p;
+    asm volatile(
+        "{\n\t.reg .pred p;\n\telect.sync _|p, 0xffffffff;\n\tselp.u32 %0, 1, 0, p;\n\t}"
+        : "=r"(p));
+    return p != 0;
+}
+
 // 2-D tensor copy global -> shared of the map's box at element coordinates
 // (x innermost, y), completing its bytes on `bar`.
 __device__ __forceinline__ void tma_load_2d(void* dst, const CUtensorMap* map, int x, int y, uint64_t* bar)
