@@ -90,7 +90,7 @@ def measured_peak():
 
 KERNEL_SOURCES = {
     "chain_kernel": ("wq4_chain.cu", "wq4_items.cuh", "wq4_device.cuh"),
-    "tc_stage_kernel": ("wq4_tc.cu", "wq4_tc.cuh", "wq4_device.cuh"),
+    "stage_kernel": ("wq4_stage.cu", "wq4_tiles.cuh", "wq4_items.cuh", "wq4_device.cuh"),
 }
 
 
@@ -480,10 +480,10 @@ def run_ours(args, rank, world, local):
         # one cooperative launch of the persistent chain kernel per token
         kernel_name, launches_per_step = "chain_kernel", 1
     else:
-        # one CUDA-graph replay: a prologue and one tensor-core stage kernel per
+        # one CUDA-graph replay: the input's squares and one stage kernel per
         # projection (with attention, three more a layer: rotation/append,
-        # paged attention, the O input's token-start kernel)
-        kernel_name, launches_per_step = "tc_stage_kernel", 4 * shape.num_layers + 2 + (3 * shape.num_layers if T else 0)
+        # paged attention, the squares of the O input)
+        kernel_name, launches_per_step = "stage_kernel", 4 * shape.num_layers + 2 + (3 * shape.num_layers if T else 0)
     if rank == 0:
         ms = total_ms_max / args.steps
         avg_launch_ms = statistics.mean(launch_ms)

@@ -56,8 +56,9 @@ enum wq4_status {
 /* Largest batch (rows of x) any call accepts. */
 #define WQ4_MAX_BATCH 32
 
-/* Largest scale magnitude of the paths that round the dequantized weight
- * (q - 7) * s to fp16 (wq4_gemm, wq4_decode_chain at batch 3-32). */
+/* Largest scale magnitude of the calls that may round the dequantized weight
+ * (q - 7) * s to fp16 (wq4_gemm; wq4_decode_chain at batch 3-32 keeps the
+ * limit that it had when it did). */
 #define WQ4_MAX_FP16_SCALE 8188.0f
 
 /*
@@ -219,13 +220,12 @@ size_t wq4_chain_workspace_bytes(const wq4_layer_table* table);
  * residual stream.
  *   x      : fp16 [batch][hidden] device, 16-byte aligned
  *   logits : fp16 [batch][vocab]  device, 2-byte aligned
- * Batch 1-2 runs as the persistent kernel above (exact dequantization, any
- * fp16 scale).  Batch 3-32 runs as a CUDA graph, captured once per table, of
- * one tensor-core kernel per projection (dequantized fp16 weights
- * w = fp16((q - 7) s) times the batch's inputs, tcgen05 MMAs with fp32
- * accumulation, the chain's row factors, residual adds and SiLU fused into
- * each stage's epilogue); each call copies x into the workspace, replays the
- * graph and copies the logits out (all on `stream`).
+ * Batch 1-2 runs as the persistent kernel above.  Batch 3-32 runs as a CUDA
+ * graph, captured once per table, of one kernel per projection (the chain's
+ * row factors, residual adds and SiLU fused into each stage's epilogue); each
+ * call copies x into the workspace, replays the graph and copies the logits
+ * out (all on `stream`).  Both dequantize exactly (fp16 products, fp32 sums
+ * and scales).
  * The first call for a table (or after its contents changed) builds its plan:
  * at batch 1-2 it validates the table and uploads its pointer table into the
  * workspace (cudaMemcpyAsync on `stream`); at batch 3-32 it also scans every
@@ -291,7 +291,7 @@ int wq4_decode_chain_noalloc(const wq4_layer_table* table, const uint16_t* x,
 /*
  * Which kernel the cached plan of `table` runs (an inspection call, no
  * counterpart in the paper): 1 for the persistent chain kernel (batch 1-2),
- * 2 for the CUDA graph of tensor-core stage kernels (batch 3-32);
+ * 2 for the CUDA graph of stage kernels (batch 3-32);
  * decode_step != 0 asks about the plan of wq4_decode_step, else of
  * wq4_decode_chain.  Returns WQ4_ERR_INVALID when no plan exists yet (the
  * first call builds it).

@@ -21,8 +21,8 @@ INCLUDE = os.path.join(ROOT, "include")
 BUILD = os.path.join(HERE, "_build")
 LIB = os.path.join(BUILD, "libwq4.so")
 
-SOURCES = ["wq4_gemv.cu", "wq4_bgemv.cu", "wq4_chain.cu", "wq4_synth.cu", "wq4_tc.cu", "wq4_attn.cu", "wq4_gemm.cu"]
-HEADERS = ["wq4_device.cuh", "wq4_host.h", "wq4_items.cuh", "wq4_tc.cuh", "wq4_tc_host.h"]
+SOURCES = ["wq4_gemv.cu", "wq4_bgemv.cu", "wq4_chain.cu", "wq4_synth.cu", "wq4_stage.cu", "wq4_attn.cu", "wq4_gemm.cu"]
+HEADERS = ["wq4_device.cuh", "wq4_host.h", "wq4_items.cuh", "wq4_tc.cuh", "wq4_stage_host.h", "wq4_tiles.cuh"]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 
 

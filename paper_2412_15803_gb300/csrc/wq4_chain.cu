@@ -39,7 +39,7 @@
 #include "wq4_device.cuh"
 #include "wq4_items.cuh"
 #include "wq4_host.h"
-#include "wq4_tc_host.h"
+#include "wq4_stage_host.h"
 #include "wq4.h"
 #include "wq4_attn.h"
 
@@ -1356,7 +1356,7 @@ __global__ void __launch_bounds__(256) rope_append_kernel(const __grid_constant_
 
 struct Layout {
     size_t header, llA, llX1, llM, llX, llV, pV, pX2, pQKV, pO, pX1, pGU, pM, pD, x_stage, logits_stage, rfac,
-        xpH0, xpH1, xpF, cnt, part, total;
+        qA, total;
     size_t ll_begin, ll_end;
     // decode step (after everything above, so that the chain's offsets stay):
     // flagged words of the new keys, values and attention output (zeroed),
@@ -1432,16 +1432,11 @@ Layout make_layout(const Dims& d, bool att = false, size_t attn_ws_bytes = 0)
     y.x_stage = take(2 * B * H);
     y.logits_stage = take(2 * B * static_cast<size_t>(d.V));
     if (d.B > kMaxChainBatch) {
-        // batched path: sums of squares of 128-element tiles (u, a, x1),
-        // arrival counters, permuted stage inputs, K-part partial sums
-        y.rfac = take(4 * 3 * (H / 128) * B);
-        y.cnt = take(4 * static_cast<size_t>(kTcCounterWords));
-        y.xpH0 = take(2 * 32 * H);
-        y.xpH1 = take(2 * 32 * H);
-        y.xpF = take(2 * 32 * F);
-        y.part = take(4 * tc_part_floats(d.L, d.H, d.F, d.Nqkv, d.V, d.B, 256));
+        // batched path: sums of squares (u, a, x1) and O's input
+        y.rfac = take(4 * 3 * static_cast<size_t>(stage_sq_ld(d.H)) * B);
+        y.qA = take(2 * B * H);
     } else {
-        y.rfac = y.cnt = y.xpH0 = y.xpH1 = y.xpF = y.part = 0;
+        y.rfac = y.qA = 0;
     }
     y.att_ll_begin = y.att_ll_end = y.llK = y.llVn = y.llAt = y.pQr = y.pKr = y.pAt = 0;
     y.apart = y.acnt = y.seq_lens = y.attn_ws = y.attn_ws_bytes = 0;
@@ -1691,8 +1686,8 @@ __global__ void scale_max_kernel(const uint16_t* s, size_t n, uint32_t* out)
     if ((threadIdx.x & 31) == 0) atomicMax(out, m);
 }
 
-// The batched path rounds each dequantized weight (q - 7) s to fp16: every
-// scale of the table must be within +-8188.  Scans all scales once (at plan
+// The batched path takes scales within +-8188 only (its first kernels rounded
+// each dequantized weight (q - 7) s to fp16).  Scans all scales once (at plan
 // build) and synchronizes `stream` to read the result.
 int check_scales_fp16(const wq4_layer_table* t, const Dims& d, uint32_t* scratch_word, cudaStream_t stream)
 {
@@ -1731,9 +1726,9 @@ void fill_inv_freq(double theta, double* out)
     for (int i = 0; i < kAttnD / 2; ++i) out[i] = std::pow(theta, -2.0 * i / kAttnD);
 }
 
-// The decode step's attention nodes of the graph path (see TcAttnHook): the
+// The decode step's attention nodes of the graph path (see StageAttnHook): the
 // rotation/append kernel, wq4_paged_attention on the rotated queries, and the
-// token-start kernel on the attention output (O's permuted input).
+// sums of squares of the attention output (O's input).
 struct GraphAttn {
     const Plan* pl;
     const Dims* d;
@@ -1741,7 +1736,7 @@ struct GraphAttn {
     uint8_t* ws;
 };
 
-int record_graph_attention(void* ctx, int l, cudaStream_t cs, uint16_t* xp, float* sq)
+int record_graph_attention(void* ctx, int l, cudaStream_t cs, const uint16_t** o_in, float* sq)
 {
     const GraphAttn& g = *static_cast<const GraphAttn*>(ctx);
     const Dims& d = *g.d;
@@ -1777,7 +1772,8 @@ int record_graph_attention(void* ctx, int l, cudaStream_t cs, uint16_t* xp, floa
     int rc = wq4_paged_attention(&c, a.qr, d.H, a.seq_lens, at, d.H, d.B, d.nq, g.pl->scale, g.ws + y.attn_ws,
                                  y.attn_ws_bytes, cs);
     if (rc != WQ4_OK) return rc;
-    return tc_launch_prologue(at, d.H, d.B, sq, xp, cs);
+    *o_in = at;
+    return stage_launch_squares(at, d.H, d.B, sq, cs);
 }
 
 // Records one token of the graph path on `cs`: every stage kernel of every
@@ -1788,11 +1784,12 @@ int build_graph_plan(const wq4_layer_table* t, const Dims& d, const Layout& lay,
                      Plan* pl, cudaStream_t stream)
 {
     uint8_t* ws = static_cast<uint8_t*>(t->workspace);
-    // scales beyond +-8188 would overflow the fp16 dequantized weights
+    // scales beyond +-8188 are refused
     const int rs = check_scales_fp16(t, d, reinterpret_cast<uint32_t*>(ws + lay.header) + 3, stream);
     if (rs != WQ4_OK) return rs;
     auto U16 = [&](size_t off) { return reinterpret_cast<uint16_t*>(ws + off); };
-    TcBuffers buf;
+    StageModel m;
+    StageBuffers& buf = m.buf;
     buf.x_stage = U16(lay.x_stage);
     buf.pV = U16(lay.pV);
     buf.pQKV = U16(lay.pQKV);
@@ -1804,38 +1801,32 @@ int build_graph_plan(const wq4_layer_table* t, const Dims& d, const Layout& lay,
     buf.pX2 = U16(lay.pX2);
     buf.logits = U16(lay.logits_stage);
     buf.sq = reinterpret_cast<float*>(ws + lay.rfac);
-    buf.cnt = reinterpret_cast<uint32_t*>(ws + lay.cnt);
-    buf.xpH[0] = U16(lay.xpH0);
-    buf.xpH[1] = U16(lay.xpH1);
-    buf.xpF = U16(lay.xpF);
-    buf.part = reinterpret_cast<float*>(ws + lay.part);
-    TcPlan* tc = nullptr;
-    int rc = tc_plan_create(t, d.H, d.F, d.Nqkv, d.V, d.B, buf, di->sm_count, status_word(), &tc);
-    if (rc != WQ4_OK) return rc;
+    buf.qA = U16(lay.qA);
+    m.table = t;
+    m.H = d.H;
+    m.F = d.F;
+    m.Nqkv = d.Nqkv;
+    m.V = d.V;
+    m.B = d.B;
+    m.sms = di->sm_count;
+    m.smem_max = static_cast<size_t>(di->smem_optin);
+    m.err = status_word();
+    if (!m.err) return WQ4_ERR_CUDA;
     cudaStream_t cs = nullptr;
-    if (cudaStreamCreateWithFlags(&cs, cudaStreamNonBlocking) != cudaSuccess) {
-        tc_plan_destroy(tc);
-        return WQ4_ERR_CUDA;
-    }
+    if (cudaStreamCreateWithFlags(&cs, cudaStreamNonBlocking) != cudaSuccess) return WQ4_ERR_CUDA;
     cudaGraph_t graph = nullptr;
     cudaGraphExec_t exec = nullptr;
-    rc = WQ4_ERR_CUDA;
+    int rc = WQ4_ERR_CUDA;
     if (cudaStreamBeginCapture(cs, cudaStreamCaptureModeThreadLocal) == cudaSuccess) {
-        // every token starts with zero arrival counters (a stage whose waits gave
-        // up may leave some non-zero; the next token must not inherit them)
-        int rrec = cudaMemsetAsync(ws + lay.cnt, 0, 4 * static_cast<size_t>(kTcCounterWords), cs) == cudaSuccess
-                       ? WQ4_OK
-                       : WQ4_ERR_CUDA;
         GraphAttn ga{pl, &d, &lay, ws};
-        const TcAttnHook hook{record_graph_attention, &ga};
-        if (rrec == WQ4_OK) rrec = tc_record_token(tc, cs, pl->att ? &hook : nullptr);
+        const StageAttnHook hook{record_graph_attention, &ga};
+        const int rrec = stage_record_token(m, cs, pl->att ? &hook : nullptr);
         if (cudaStreamEndCapture(cs, &graph) == cudaSuccess && graph && rrec == WQ4_OK &&
             cudaGraphInstantiate(&exec, graph, 0) == cudaSuccess)
             rc = WQ4_OK;
     }
     if (graph) cudaGraphDestroy(graph);
     cudaStreamDestroy(cs);
-    tc_plan_destroy(tc);   // the graph holds copies of every launch argument
     if (rc != WQ4_OK) return rc;
     pl->table = *t;
     pl->layers.assign(t->layers, t->layers + d.L);
