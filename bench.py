@@ -481,9 +481,9 @@ def run_ours(args, rank, world, local):
         kernel_name, launches_per_step = "chain_kernel", 1
     else:
         # one CUDA-graph replay: the input's squares and one stage kernel per
-        # projection (with attention, three more a layer: rotation/append,
-        # paged attention, the squares of the O input)
-        kernel_name, launches_per_step = "stage_kernel", 4 * shape.num_layers + 2 + (3 * shape.num_layers if T else 0)
+        # projection (with attention, the token's rotations and two more a layer:
+        # rotation/append and paged attention)
+        kernel_name, launches_per_step = "stage_kernel", 4 * shape.num_layers + 2 + (2 * shape.num_layers + 1 if T else 0)
     if rank == 0:
         ms = total_ms_max / args.steps
         avg_launch_ms = statistics.mean(launch_ms)

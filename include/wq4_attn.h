@@ -82,7 +82,9 @@ size_t wq4_paged_attention_workspace_bytes(int batch, int n_q_heads, int n_kv_he
  *                16-byte aligned, not shared by concurrent calls.
  * Sequences are split across the GPU's thread blocks by tokens in equal
  * shares and the shares are merged in a fixed order: the same inputs on the
- * same device give the same bits.  Returns WQ4_OK, WQ4_ERR_INVALID,
+ * same device give the same bits.  Launched with programmatic dependent
+ * launch; everything is read after the previous kernel in `stream` has
+ * completed.  Returns WQ4_OK, WQ4_ERR_INVALID,
  * WQ4_ERR_ALIGN, WQ4_ERR_UNSUPPORTED (head_dim != 128, group > 8) or
  * WQ4_ERR_CUDA.
  */

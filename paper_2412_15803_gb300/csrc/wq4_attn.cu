@@ -44,8 +44,11 @@ constexpr int kSlotBytes = 2 * kTile * kD * 2;   // keys + values of one tile: 8
 constexpr int kBoxBytes = kTile * 64 * 2;        // 16 rows x 64 dims: 2 KiB
 constexpr int kPartHdr = 16;                     // floats: M[8], L[8]
 constexpr int kCtasPerSm = 2;
-constexpr int kMaxParts = kConsumers * kD;      // parts of one segment the merge stages: grid <= 512
-constexpr int kMinShare = 16;                   // fewest tiles of a CTA's share (small batches: fewer parts to merge)
+constexpr int kMaxParts = 512;                  // parts of one segment the merge stages: grid <= 512
+// Fewest tiles of a CTA's share (or the whole sequence, if shorter): smaller
+// shares only add parts to merge.
+constexpr int kShareMin = 8;
+constexpr int kShareWhole = 32;   // fair shares up to this many tiles are cut at the segments' ends
 
 // Shared memory map (dynamic, base 1024-aligned).
 constexpr int kOffRing = 0;
@@ -55,10 +58,11 @@ constexpr int kOffMrow = kOffMisc + 64;                           // [W][8] floa
 constexpr int kOffLrow = kOffMrow + kConsumers * kMaxGroup * 4;   // [W][8] floats
 constexpr int kOffScr = kOffLrow + kConsumers * kMaxGroup * 4;    // [W][G][128] floats
 constexpr int kOffPre = kOffScr + kConsumers * kMaxGroup * kD * 4;  // int [batch + 1]
+static_assert(kMaxParts * kMaxGroup * 4 <= kOffPre - kOffScr, "merge scratch");
 
 size_t attn_smem_bytes(int batch)
 {
-    return 1024 + kOffPre + static_cast<size_t>(batch + 1) * 4;
+    return 1024 + kOffPre + 2 * static_cast<size_t>(batch + 1) * 4;   // pre, parts
 }
 
 struct AttnParams {
@@ -73,6 +77,8 @@ struct AttnParams {
     int q_stride, out_stride, pt_stride;
     int batch, Hkv, G, page_size, num_pages;
     float sl2;                   // scale * log2(e)
+    float* sq;                   // per (row, head) sums of squares of the outputs, [batch][sq_ld]; null: none
+    int sq_ld;
 };
 
 // ------------------------------------------------------------ device ---
@@ -168,24 +174,53 @@ __device__ __forceinline__ Piece find_piece(const int* pre, int batch, int Hkv, 
     return p;
 }
 
+// The same when every CTA takes one piece: parts[b] = pieces of one head's
+// segment summed over sequences < b; a sequence's tiles are cut evenly.
+__device__ __forceinline__ Piece whole_piece(const int* pre, const int* parts, int batch, int Hkv, int cta)
+{
+    int lo = 0, hi = batch - 1;
+    while (lo < hi) {
+        const int mid = (lo + hi + 1) >> 1;
+        if (Hkv * parts[mid] <= cta) lo = mid;
+        else hi = mid - 1;
+    }
+    Piece p;
+    p.b = lo;
+    const int tb = pre[lo + 1] - pre[lo], np = parts[lo + 1] - parts[lo];
+    const int i = cta - Hkv * parts[lo];
+    p.h = i / np;
+    const int k = i - p.h * np;
+    p.t0 = k * tb / np;
+    p.t1 = (k + 1) * tb / np;
+    p.seg = p.b * Hkv + p.h;
+    p.first = cta - k;
+    p.npieces = np;
+    p.slot = cta + p.seg;
+    return p;
+}
+
 __global__ void __launch_bounds__(kThreads, kCtasPerSm) paged_attn_kernel(const __grid_constant__ AttnParams P)
 {
     extern __shared__ uint8_t smem_raw[];
     uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
     uint64_t* full = reinterpret_cast<uint64_t*>(smem + kOffBars);
     uint64_t* empty = full + kSlots;
-    volatile int* misc = reinterpret_cast<volatile int*>(smem + kOffMisc);   // [0] abort, [1] last arriver
+    volatile int* misc = reinterpret_cast<volatile int*>(smem + kOffMisc);   // [0] abort, [1] last arriver, [2] one piece per CTA
     float* mrow = reinterpret_cast<float*>(smem + kOffMrow);
     float* lrow = reinterpret_cast<float*>(smem + kOffLrow);
     float* scr = reinterpret_cast<float*>(smem + kOffScr);
     int* pre = reinterpret_cast<int*>(smem + kOffPre);
+    int* parts = pre + P.batch + 1;
 
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const int max_tok = P.pt_stride * P.page_size;
 
-    // tile prefix over the batch (warp 0), barriers (thread 32)
+    // tile prefix over the batch (warp 0), barriers (thread 32); every input may
+    // come from the previous kernel of the stream (programmatic dependent launch)
+    grid_dependents_launch();
+    if (warp != 1) grid_dependency_wait();
     if (warp == 0) {
-        int carry = 0;
+        int carry = 0, longest = 0;
         for (int b0 = 0; b0 < P.batch; b0 += 32) {
             const int b = b0 + lane;
             int tiles = 0;
@@ -197,6 +232,7 @@ __global__ void __launch_bounds__(kThreads, kCtasPerSm) paged_attn_kernel(const 
                 }
                 tiles = T > 0 ? (T + kTile - 1) / kTile : 0;
             }
+            longest = max(longest, tiles);
             int incl = tiles;
 #pragma unroll
             for (int o = 1; o < 32; o <<= 1) {
@@ -207,6 +243,39 @@ __global__ void __launch_bounds__(kThreads, kCtasPerSm) paged_attn_kernel(const 
             carry += __shfl_sync(0xffffffffu, incl, 31);
         }
         if (lane == 0) pre[P.batch] = carry;
+        __syncwarp();
+        // One piece per CTA where that costs little balance: shares of R tiles,
+        // cut at the segments' ends, R the least that leaves a CTA for each.
+        // (A CTA whose share meets a second segment pays a piece's fixed cost,
+        // ~2 us, twice: 2 x 4096 tokens 14.1 us against 12.0; one 64-token
+        // sequence of 8 heads on two CTAs 9.9 us, on eight 3.9.)
+        // Large shares skip it: the search costs more than the second piece.
+        longest = __reduce_max_sync(0xffffffffu, longest);
+        const int grid = static_cast<int>(gridDim.x);
+        const int fair = (P.Hkv * carry + grid - 1) / grid;
+        bool fits = false;
+        int R = max(fair, min(kShareMin, max(longest, 1)));
+        for (int tries = 0; fair <= kShareWhole && tries < 4 && !fits; ++tries, R += 1 + R / 8) {
+            const float inv = 1.f / static_cast<float>(R);
+            int sum = 0;
+            for (int b0 = 0; b0 < P.batch; b0 += 32) {
+                const int b = b0 + lane;
+                // ceil(tiles / R): tiles < 2^21 here, the half keeps the quotient off the whole numbers
+                const int np = b < P.batch ? __float2int_rz((static_cast<float>(pre[b + 1] - pre[b] + R) - 0.5f) * inv) : 0;
+                int incl = np;
+#pragma unroll
+                for (int o = 1; o < 32; o <<= 1) {
+                    const int v = __shfl_up_sync(0xffffffffu, incl, o);
+                    if (lane >= o) incl += v;
+                }
+                if (b < P.batch) parts[b] = sum + incl - np;
+                sum += __shfl_sync(0xffffffffu, incl, 31);
+            }
+            if (lane == 0) parts[P.batch] = sum;
+            fits = P.Hkv * sum <= grid;
+        }
+        __syncwarp();
+        if (lane == 0) misc[2] = fits ? 1 : 0;
     } else if (tid == 32) {
         for (int i = 0; i < kSlots; ++i) {
             mbar_init(&full[i], 1);
@@ -216,13 +285,18 @@ __global__ void __launch_bounds__(kThreads, kCtasPerSm) paged_attn_kernel(const 
         misc[1] = 0;
         mbar_fence_init();
     }
+    if (warp == 1) grid_dependency_wait();
     __syncthreads();
 
     const int total = P.Hkv * pre[P.batch];
-    const int R = max((total + static_cast<int>(gridDim.x) - 1) / static_cast<int>(gridDim.x), kMinShare);
     const int cta = blockIdx.x;
-    const int g_begin = min(total, cta * R);
-    const int g_end = min(total, g_begin + R);
+    const bool whole = misc[2] != 0;
+    const int R = max((total + static_cast<int>(gridDim.x) - 1) / static_cast<int>(gridDim.x), kShareMin);
+    const int g_begin = whole ? 0 : min(total, cta * R);
+    const int g_end = whole ? (cta < P.Hkv * parts[P.batch] ? 1 : 0) : min(total, g_begin + R);
+    auto piece = [&](int g) {
+        return whole ? whole_piece(pre, parts, P.batch, P.Hkv, cta) : find_piece(pre, P.batch, P.Hkv, g, g_end, R, cta);
+    };
     const int G = P.G;
 
     if (warp == kConsumers) {
@@ -235,7 +309,7 @@ __global__ void __launch_bounds__(kThreads, kCtasPerSm) paged_attn_kernel(const 
         int i = 0;   // CTA-wide tile counter
         bool ok = true;
         for (int g = g_begin; g < g_end && ok;) {
-            const Piece pc = find_piece(pre, P.batch, P.Hkv, g, g_end, R, cta);
+            const Piece pc = piece(g);
             const int32_t* pt = P.page_table + static_cast<size_t>(pc.b) * P.pt_stride;
             for (int t = pc.t0; t < pc.t1 && ok; t += 32) {
                 // page ids of up to 32 tiles, one per lane
@@ -276,7 +350,7 @@ __global__ void __launch_bounds__(kThreads, kCtasPerSm) paged_attn_kernel(const 
                     if (!ok) break;
                 }
             }
-            g += pc.t1 - pc.t0;
+            g += whole ? 1 : pc.t1 - pc.t0;
         }
         // drain: the last copy issued into each slot has landed before exit
         if (lane == 0) {
@@ -295,6 +369,8 @@ __global__ void __launch_bounds__(kThreads, kCtasPerSm) paged_attn_kernel(const 
         if (pre[b + 1] == pre[b]) {
             uint16_t* ob = P.out + static_cast<size_t>(b) * P.out_stride;
             for (int e = tid; e < P.Hkv * G * kD; e += kConsumers * 32) ob[e] = 0;
+            if (P.sq)
+                for (int e = tid; e < P.Hkv * G; e += kConsumers * 32) P.sq[static_cast<size_t>(b) * P.sq_ld + e] = 0.f;
         }
     }
 
@@ -303,7 +379,7 @@ __global__ void __launch_bounds__(kThreads, kCtasPerSm) paged_attn_kernel(const 
     const uint32_t ring = smem_addr(smem + kOffRing);
     int ibase = 0;                     // CTA-wide index of the piece's first tile
     for (int g = g_begin; g < g_end;) {
-        const Piece pc = find_piece(pre, P.batch, P.Hkv, g, g_end, R, cta);
+        const Piece pc = piece(g);
         const int ntile = pc.t1 - pc.t0;
         int T = P.seq_lens[pc.b];
         T = T > max_tok ? max_tok : T;
@@ -430,28 +506,42 @@ __global__ void __launch_bounds__(kThreads, kCtasPerSm) paged_attn_kernel(const 
         }
         named_barrier_sync(1, kConsumers * 32);
         float* part = P.part + static_cast<size_t>(pc.slot) * (kPartHdr + G * kD);
-        for (int e = tid; e < G * (kD / 2); e += kConsumers * 32) {
-            const int gg = e / (kD / 2), d = 2 * (e % (kD / 2));
+        // a warp per query head, four dimensions a lane
+        auto store = [&](int gg, float a0, float a1, float a2, float a3, float L) {
+            const float inv = L > 0.f ? 1.f / L : 0.f;
+            const int head = pc.h * G + gg;
+            uint32_t* ob = reinterpret_cast<uint32_t*>(P.out + static_cast<size_t>(pc.b) * P.out_stride + head * kD + 4 * lane);
+            const uint32_t w0 = pack_half2(a0 * inv, a1 * inv), w1 = pack_half2(a2 * inv, a3 * inv);
+            ob[0] = w0;
+            ob[1] = w1;
+            if (P.sq) {
+                const float2 f0 = unpack_half2(w0), f1 = unpack_half2(w1);
+                const float t = warp_sum(fmaf(f0.x, f0.x, f0.y * f0.y) + fmaf(f1.x, f1.x, f1.y * f1.y));
+                if (lane == 0) P.sq[static_cast<size_t>(pc.b) * P.sq_ld + head] = t;
+            }
+        };
+        for (int gg = warp; gg < G; gg += kConsumers) {
+            const int d = 4 * lane;
             float M = -INFINITY;
 #pragma unroll
             for (int w = 0; w < kConsumers; ++w) M = fmaxf(M, mrow[w * kMaxGroup + gg]);
             const float Ms = M == -INFINITY ? 0.f : M;
-            float L = 0.f, O0 = 0.f, O1 = 0.f;
+            float L = 0.f, O0 = 0.f, O1 = 0.f, O2 = 0.f, O3 = 0.f;
 #pragma unroll
             for (int w = 0; w < kConsumers; ++w) {
                 const float f = exp2f(mrow[w * kMaxGroup + gg] - Ms);
                 L += lrow[w * kMaxGroup + gg] * f;
-                const float2 ov = *reinterpret_cast<const float2*>(scr + (w * kMaxGroup + gg) * kD + d);
+                const float4 ov = *reinterpret_cast<const float4*>(scr + (w * kMaxGroup + gg) * kD + d);
                 O0 += ov.x * f;
                 O1 += ov.y * f;
+                O2 += ov.z * f;
+                O3 += ov.w * f;
             }
             if (pc.npieces == 1) {
-                const float inv = L > 0.f ? 1.f / L : 0.f;
-                uint16_t* ob = P.out + static_cast<size_t>(pc.b) * P.out_stride + static_cast<size_t>(pc.h * G + gg) * kD;
-                *reinterpret_cast<uint32_t*>(ob + d) = pack_half2(O0 * inv, O1 * inv);
+                store(gg, O0, O1, O2, O3, L);
             } else {
-                *reinterpret_cast<float2*>(part + kPartHdr + gg * kD + d) = make_float2(O0, O1);
-                if (d == 0) {
+                *reinterpret_cast<float4*>(part + kPartHdr + gg * kD + d) = make_float4(O0, O1, O2, O3);
+                if (lane == 0) {
                     part[gg] = M;
                     part[kMaxGroup + gg] = L;
                 }
@@ -465,79 +555,67 @@ __global__ void __launch_bounds__(kThreads, kCtasPerSm) paged_attn_kernel(const 
                 misc[1] = (old == static_cast<uint32_t>(pc.npieces - 1)) ? 1 : 0;
             }
             named_barrier_sync(1, kConsumers * 32);
-            if (misc[1]) {
-                __threadfence();
-                // Merge parts p = 0..np-1 of this segment.  (1) per head row: 16
-                // threads run the online max/normaliser merge over the parts'
-                // (M_p, L_p), then a fixed shuffle tree joins them; the factors
-                // 2^(M_p - M*) land in shared memory.  (2) every output element
-                // sums f_p * O_p in part order, loads independent of each other.
-                const int np = pc.npieces;
+            if (misc[1]) __threadfence();
+            for (int gg = warp; misc[1] && gg < G; gg += kConsumers) {
+                // Merge parts p = 0..np-1 of this segment, a warp per head.  The
+                // lanes read the parts' (M_p, L_p) and, at the same time, the
+                // first parts' outputs; the running maximum and normaliser are
+                // joined by a fixed shuffle tree and the factors 2^(M_p - M*)
+                // left in shared memory; every output element then sums
+                // f_p * O_p in part order.
+                const int np = pc.npieces, d = 4 * lane;
                 const size_t pstride = kPartHdr + static_cast<size_t>(G) * kD;
                 const float* pbase = P.part + static_cast<size_t>(pc.first + pc.seg) * pstride;
-                float* fsm = scr;     // [np][8] (np <= kMaxParts)
-                float* mls = mrow;    // M*[8], L*[8]
-                {
-                    const int gg = tid >> 4, sub = tid & 15;
-                    float m = -INFINITY, l = 0.f;
-                    if (gg < G) {
-#pragma unroll 4
-                        for (int p = sub; p < np; p += 16) {
-                            const float Mp = __ldcg(pbase + p * pstride + gg);
-                            const float Lp = __ldcg(pbase + p * pstride + kMaxGroup + gg);
-                            fsm[p * kMaxGroup + gg] = Mp;
-                            const float mn = fmaxf(m, Mp);
-                            const float ms = mn == -INFINITY ? 0.f : mn;
-                            l = l * exp2f(m - ms) + Lp * exp2f(Mp - ms);
-                            m = mn;
-                        }
-                    }
+                const float* po = pbase + kPartHdr + gg * kD + d;
+                constexpr int kPre = 8;
+                float4 pre[kPre];
 #pragma unroll
-                    for (int o = 1; o < 16; o <<= 1) {
-                        const float m2 = __shfl_xor_sync(0xffffffffu, m, o);
-                        const float l2 = __shfl_xor_sync(0xffffffffu, l, o);
-                        const float mn = fmaxf(m, m2);
-                        const float ms = mn == -INFINITY ? 0.f : mn;
-                        l = l * exp2f(m - ms) + l2 * exp2f(m2 - ms);
-                        m = mn;
-                    }
-                    if (gg < G && sub == 0) {
-                        mls[gg] = m;
-                        mls[kMaxGroup + gg] = l;
-                    }
-                    named_barrier_sync(1, kConsumers * 32);
-                    if (gg < G) {
-                        const float ms = mls[gg] == -INFINITY ? 0.f : mls[gg];
-                        for (int p = sub; p < np; p += 16) fsm[p * kMaxGroup + gg] = exp2f(fsm[p * kMaxGroup + gg] - ms);
-                    }
-                    named_barrier_sync(1, kConsumers * 32);
+                for (int p = 0; p < kPre; ++p)
+                    pre[p] = p < np ? __ldcg(reinterpret_cast<const float4*>(po + p * pstride)) : make_float4(0.f, 0.f, 0.f, 0.f);
+                float* fsm = scr;     // [np][8] (np <= kMaxParts), column gg is this warp's
+                float m = -INFINITY, l = 0.f;
+#pragma unroll 4
+                for (int p = lane; p < np; p += 32) {
+                    const float Mp = __ldcg(pbase + p * pstride + gg);
+                    const float Lp = __ldcg(pbase + p * pstride + kMaxGroup + gg);
+                    fsm[p * kMaxGroup + gg] = Mp;
+                    const float mn = fmaxf(m, Mp);
+                    const float ms = mn == -INFINITY ? 0.f : mn;
+                    l = l * exp2f(m - ms) + Lp * exp2f(Mp - ms);
+                    m = mn;
                 }
-                for (int e = tid; e < G * (kD / 4); e += kConsumers * 32) {
-                    const int gg = e / (kD / 4), d = 4 * (e % (kD / 4));
-                    const float* po = pbase + kPartHdr + gg * kD + d;
-                    float a0 = 0.f, a1 = 0.f, a2 = 0.f, a3 = 0.f;
+#pragma unroll
+                for (int o = 1; o < 32; o <<= 1) {
+                    const float m2 = __shfl_xor_sync(0xffffffffu, m, o);
+                    const float l2 = __shfl_xor_sync(0xffffffffu, l, o);
+                    const float mn = fmaxf(m, m2);
+                    const float ms = mn == -INFINITY ? 0.f : mn;
+                    l = l * exp2f(m - ms) + l2 * exp2f(m2 - ms);
+                    m = mn;
+                }
+                const float ms = m == -INFINITY ? 0.f : m;
+                for (int p = lane; p < np; p += 32) fsm[p * kMaxGroup + gg] = exp2f(fsm[p * kMaxGroup + gg] - ms);
+                __syncwarp();
+                float a0 = 0.f, a1 = 0.f, a2 = 0.f, a3 = 0.f;
+                auto add = [&](const float4& ov, int p) {
+                    const float f = fsm[p * kMaxGroup + gg];
+                    a0 = fmaf(ov.x, f, a0);
+                    a1 = fmaf(ov.y, f, a1);
+                    a2 = fmaf(ov.z, f, a2);
+                    a3 = fmaf(ov.w, f, a3);
+                };
+#pragma unroll
+                for (int p = 0; p < kPre; ++p)
+                    if (p < np) add(pre[p], p);
 #pragma unroll 8
-                    for (int p = 0; p < np; ++p) {
-                        const float f = fsm[p * kMaxGroup + gg];
-                        const float4 ov = __ldcg(reinterpret_cast<const float4*>(po + p * pstride));
-                        a0 = fmaf(ov.x, f, a0);
-                        a1 = fmaf(ov.y, f, a1);
-                        a2 = fmaf(ov.z, f, a2);
-                        a3 = fmaf(ov.w, f, a3);
-                    }
-                    const float L = mls[kMaxGroup + gg];
-                    const float inv = L > 0.f ? 1.f / L : 0.f;
-                    uint16_t* ob =
-                        P.out + static_cast<size_t>(pc.b) * P.out_stride + static_cast<size_t>(pc.h * G + gg) * kD + d;
-                    reinterpret_cast<uint32_t*>(ob)[0] = pack_half2(a0 * inv, a1 * inv);
-                    reinterpret_cast<uint32_t*>(ob)[1] = pack_half2(a2 * inv, a3 * inv);
-                }
-                if (tid == 0) P.cnt[pc.seg] = 0u;
+                for (int p = kPre; p < np; ++p) add(__ldcg(reinterpret_cast<const float4*>(po + p * pstride)), p);
+                store(gg, a0, a1, a2, a3, l);
             }
+            if (tid == 0 && misc[1]) P.cnt[pc.seg] = 0u;
         }
         named_barrier_sync(1, kConsumers * 32);   // scratch and flags free for the next piece
         ibase += ntile;
-        g += ntile;
+        g += whole ? 1 : ntile;
     }
 }
 
@@ -616,9 +694,11 @@ extern "C" size_t wq4_paged_attention_workspace_bytes(int batch, int n_q_heads, 
     return cnt_bytes + (static_cast<size_t>(grid) + segs) * (kPartHdr + G * kD) * 4;
 }
 
-extern "C" int wq4_paged_attention(const wq4_kv_cache* cache, const uint16_t* q, int q_stride,
-                                   const int32_t* seq_lens, uint16_t* out, int out_stride, int batch, int n_q_heads,
-                                   float scale, void* workspace, size_t workspace_bytes, void* stream)
+namespace wq4 {
+
+int launch_paged_attention(const wq4_kv_cache* cache, const uint16_t* q, int q_stride, const int32_t* seq_lens,
+                           uint16_t* out, int out_stride, int batch, int n_q_heads, float scale, void* workspace,
+                           size_t workspace_bytes, float* sq, int sq_ld, cudaStream_t stream)
 {
     if (!check_cache(cache) || !q || !seq_lens || !out || !workspace) return WQ4_ERR_INVALID;
     if (batch < 1 || batch > WQ4_ATTN_MAX_BATCH) return WQ4_ERR_INVALID;
@@ -678,9 +758,30 @@ extern "C" int wq4_paged_attention(const wq4_kv_cache* cache, const uint16_t* q,
     p.page_size = cache->page_size;
     p.num_pages = cache->num_pages;
     p.sl2 = static_cast<float>(static_cast<double>(scale) * 1.4426950408889634);
+    p.sq = sq;
+    p.sq_ld = sq_ld;
     if (!p.err) return WQ4_ERR_CUDA;
-    paged_attn_kernel<<<grid, kThreads, attn_smem_bytes(batch), static_cast<cudaStream_t>(stream)>>>(p);
-    return cudaGetLastError() == cudaSuccess ? WQ4_OK : WQ4_ERR_CUDA;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(grid);
+    cfg.blockDim = dim3(kThreads);
+    cfg.dynamicSmemBytes = attn_smem_bytes(batch);
+    cfg.stream = stream;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, paged_attn_kernel, p) == cudaSuccess ? WQ4_OK : WQ4_ERR_CUDA;
+}
+
+}  // namespace wq4
+
+extern "C" int wq4_paged_attention(const wq4_kv_cache* cache, const uint16_t* q, int q_stride,
+                                   const int32_t* seq_lens, uint16_t* out, int out_stride, int batch, int n_q_heads,
+                                   float scale, void* workspace, size_t workspace_bytes, void* stream)
+{
+    return launch_paged_attention(cache, q, q_stride, seq_lens, out, out_stride, batch, n_q_heads, scale, workspace,
+                                  workspace_bytes, nullptr, 0, static_cast<cudaStream_t>(stream));
 }
 
 extern "C" int wq4_kv_append(const wq4_kv_cache* cache, const uint16_t* new_k, const uint16_t* new_v, int new_stride,

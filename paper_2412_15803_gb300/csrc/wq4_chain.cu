@@ -1303,35 +1303,49 @@ struct RopeAppendArgs {
     const uint16_t* qkv;        // [B][Nqkv]
     uint16_t* qr;               // [B][H] rotated queries
     uint16_t* kr;               // [B][Hkv 128] rotated keys
-    int32_t* seq_lens;          // [B]
     const int32_t* positions;   // [B]
     KvLayer kv;
     int P, Hkv, H, Nqkv;
     uint32_t* err;
+    const double2* rope;        // [B][64] the token's rotations (rope_start_kernel)
+};
+
+struct RopeStartArgs {
+    double2* rope;              // [B][64]
+    int32_t* seq_lens;          // [B]
+    const int32_t* positions;   // [B]
     double inv_freq[kAttnD / 2];
 };
 
+// Token start of the decode step: the rows' rotations (fp64 sincos, the same in
+// every layer) and sequence lengths.
+__global__ void __launch_bounds__(kAttnD / 2) rope_start_kernel(const __grid_constant__ RopeStartArgs a)
+{
+    grid_dependents_launch();
+    grid_dependency_wait();
+    const int b = blockIdx.x, i = threadIdx.x;
+    const int pos = __ldg(a.positions + b);
+    double sn, cn;
+    sincos(static_cast<double>(pos < 0 ? 0 : pos) * a.inv_freq[i], &sn, &cn);
+    a.rope[b * (kAttnD / 2) + i] = make_double2(cn, sn);
+    if (i == 0) a.seq_lens[b] = pos < 0 ? 0 : pos + 1;
+}
+
+// grid: (word blocks, batch rows)
 __global__ void __launch_bounds__(256) rope_append_kernel(const __grid_constant__ RopeAppendArgs a)
 {
-    __shared__ double2 rope[kAttnD / 2];
-    asm volatile("griddepcontrol.wait;" ::: "memory");
-    const int b = blockIdx.x;
+    grid_dependents_launch();
+    grid_dependency_wait();
+    const int b = blockIdx.y;
     const int pos = __ldg(a.positions + b);
-    if (threadIdx.x < kAttnD / 2) {
-        double sn, cn;
-        sincos(static_cast<double>(pos < 0 ? 0 : pos) * a.inv_freq[threadIdx.x], &sn, &cn);
-        rope[threadIdx.x] = make_double2(cn, sn);
-    }
-    if (threadIdx.x == 0) a.seq_lens[b] = pos < 0 ? 0 : pos + 1;
-    __syncthreads();
-    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     const int H = a.H, KD = a.Hkv * kAttnD;
     const uint32_t* row = reinterpret_cast<const uint32_t*>(a.qkv + static_cast<size_t>(b) * a.Nqkv);
-    for (int w = threadIdx.x; w < (H + 2 * KD) / 2; w += blockDim.x) {
+    const double2* rope = a.rope + b * (kAttnD / 2);
+    for (int w = blockIdx.x * blockDim.x + threadIdx.x; w < (H + 2 * KD) / 2; w += gridDim.x * blockDim.x) {
         const int n = 2 * w;
-        const uint32_t x = row[w];
+        const uint32_t x = __ldcg(row + w);
         if (n < H + KD) {
-            const double2 cs = rope[(n & (kAttnD - 1)) >> 1];
+            const double2 cs = __ldcg(rope + ((n & (kAttnD - 1)) >> 1));
             const double u0 = half_bits_to_float(static_cast<uint16_t>(x & 0xFFFFu));
             const double u1 = half_bits_to_float(static_cast<uint16_t>(x >> 16));
             const uint32_t rw = pack2(double_to_half_bits(u0 * cs.x - u1 * cs.y), double_to_half_bits(u0 * cs.y + u1 * cs.x));
@@ -1362,7 +1376,7 @@ struct Layout {
     // flagged words of the new keys, values and attention output (zeroed),
     // traces, split partials and counters (batch 1-2), or the sequence
     // lengths and wq4_paged_attention's workspace (batch 3-32)
-    size_t att_ll_begin, att_ll_end, llK, llVn, llAt, pQr, pKr, pAt, apart, acnt, seq_lens, attn_ws, attn_ws_bytes;
+    size_t att_ll_begin, att_ll_end, llK, llVn, llAt, pQr, pKr, pAt, apart, acnt, seq_lens, rope, attn_ws, attn_ws_bytes;
 };
 
 struct Dims {
@@ -1439,7 +1453,7 @@ Layout make_layout(const Dims& d, bool att = false, size_t attn_ws_bytes = 0)
         y.rfac = y.qA = 0;
     }
     y.att_ll_begin = y.att_ll_end = y.llK = y.llVn = y.llAt = y.pQr = y.pKr = y.pAt = 0;
-    y.apart = y.acnt = y.seq_lens = y.attn_ws = y.attn_ws_bytes = 0;
+    y.apart = y.acnt = y.seq_lens = y.rope = y.attn_ws = y.attn_ws_bytes = 0;
     if (att) {
         const size_t KD = static_cast<size_t>(d.Hkv) * kAttnD, G = d.Hkv > 0 ? d.nq / d.Hkv : 0;
         y.att_ll_begin = o;
@@ -1455,6 +1469,7 @@ Layout make_layout(const Dims& d, bool att = false, size_t attn_ws_bytes = 0)
             y.acnt = take(4 * L * B * d.Hkv);
         } else {
             y.seq_lens = take(4 * B);
+            y.rope = take(sizeof(double2) * B * (kAttnD / 2));
             y.attn_ws = take(attn_ws_bytes);
             y.attn_ws_bytes = attn_ws_bytes;
         }
@@ -1727,14 +1742,34 @@ void fill_inv_freq(double theta, double* out)
 }
 
 // The decode step's attention nodes of the graph path (see StageAttnHook): the
-// rotation/append kernel, wq4_paged_attention on the rotated queries, and the
-// sums of squares of the attention output (O's input).
+// rotation/append kernel and wq4_paged_attention on the rotated queries, which
+// also leaves the squares of its output (O's input).
 struct GraphAttn {
     const Plan* pl;
     const Dims* d;
     const Layout* lay;
     uint8_t* ws;
 };
+
+// Token start of the decode step: rotations and sequence lengths.
+int record_graph_rope(const Plan& pl, const Dims& d, const Layout& y, uint8_t* ws, cudaStream_t cs)
+{
+    RopeStartArgs a;
+    a.rope = reinterpret_cast<double2*>(ws + y.rope);
+    a.seq_lens = reinterpret_cast<int32_t*>(ws + y.seq_lens);
+    a.positions = pl.positions;
+    fill_inv_freq(pl.theta, a.inv_freq);
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(d.B);
+    cfg.blockDim = dim3(kAttnD / 2);
+    cfg.stream = cs;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, rope_start_kernel, a) == cudaSuccess ? WQ4_OK : WQ4_ERR_CUDA;
+}
 
 int record_graph_attention(void* ctx, int l, cudaStream_t cs, const uint16_t** o_in, float* sq)
 {
@@ -1748,8 +1783,9 @@ int record_graph_attention(void* ctx, int l, cudaStream_t cs, const uint16_t** o
     a.qkv = reinterpret_cast<const uint16_t*>(g.ws + y.pQKV) + static_cast<size_t>(l) * B * d.Nqkv;
     a.qr = reinterpret_cast<uint16_t*>(g.ws + y.pQr) + static_cast<size_t>(l) * B * H;
     a.kr = reinterpret_cast<uint16_t*>(g.ws + y.pKr) + static_cast<size_t>(l) * B * KD;
-    a.seq_lens = reinterpret_cast<int32_t*>(g.ws + y.seq_lens);
+    int32_t* seq_lens = reinterpret_cast<int32_t*>(g.ws + y.seq_lens);
     a.positions = g.pl->positions;
+    a.rope = reinterpret_cast<const double2*>(g.ws + y.rope);
     a.kv = kv_layer(c);
     a.P = c.page_size;
     a.Hkv = d.Hkv;
@@ -1757,23 +1793,21 @@ int record_graph_attention(void* ctx, int l, cudaStream_t cs, const uint16_t** o
     a.Nqkv = d.Nqkv;
     a.err = status_word();
     if (!a.err) return WQ4_ERR_CUDA;
-    fill_inv_freq(g.pl->theta, a.inv_freq);
     cudaLaunchAttribute attr[1];
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr[0].val.programmaticStreamSerializationAllowed = 1;
     cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(d.B);
+    cfg.gridDim = dim3((d.H + 2 * static_cast<int>(KD)) / 2 / 256, d.B);   // one word a thread (H, KD: multiples of 128)
+    if (cfg.gridDim.x < 1) cfg.gridDim.x = 1;
     cfg.blockDim = dim3(256);
     cfg.stream = cs;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
     if (cudaLaunchKernelEx(&cfg, rope_append_kernel, a) != cudaSuccess) return WQ4_ERR_CUDA;
     uint16_t* at = reinterpret_cast<uint16_t*>(g.ws + y.pAt) + static_cast<size_t>(l) * B * H;
-    int rc = wq4_paged_attention(&c, a.qr, d.H, a.seq_lens, at, d.H, d.B, d.nq, g.pl->scale, g.ws + y.attn_ws,
-                                 y.attn_ws_bytes, cs);
-    if (rc != WQ4_OK) return rc;
     *o_in = at;
-    return stage_launch_squares(at, d.H, d.B, sq, cs);
+    return launch_paged_attention(&c, a.qr, d.H, seq_lens, at, d.H, d.B, d.nq, g.pl->scale, g.ws + y.attn_ws,
+                                  y.attn_ws_bytes, sq, stage_sq_ld(d.H), cs);
 }
 
 // Records one token of the graph path on `cs`: every stage kernel of every
@@ -1820,7 +1854,8 @@ int build_graph_plan(const wq4_layer_table* t, const Dims& d, const Layout& lay,
     if (cudaStreamBeginCapture(cs, cudaStreamCaptureModeThreadLocal) == cudaSuccess) {
         GraphAttn ga{pl, &d, &lay, ws};
         const StageAttnHook hook{record_graph_attention, &ga};
-        const int rrec = stage_record_token(m, cs, pl->att ? &hook : nullptr);
+        int rrec = pl->att ? record_graph_rope(*pl, d, lay, ws, cs) : WQ4_OK;
+        if (rrec == WQ4_OK) rrec = stage_record_token(m, cs, pl->att ? &hook : nullptr);
         if (cudaStreamEndCapture(cs, &graph) == cudaSuccess && graph && rrec == WQ4_OK &&
             cudaGraphInstantiate(&exec, graph, 0) == cudaSuccess)
             rc = WQ4_OK;

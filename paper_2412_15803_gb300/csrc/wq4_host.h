@@ -4,6 +4,8 @@
 #include <cuda.h>
 #include <cuda_runtime.h>
 
+#include "wq4_attn.h"
+
 #include <array>
 #include <cstddef>
 #include <cstdint>
@@ -21,6 +23,12 @@ const DeviceInfo* current_device_info(int* device_out);
 
 // Device address of the library's status word on the current device.
 uint32_t* status_word();
+
+// wq4_paged_attention that also leaves the sums of squares of every (row,
+// query head)'s outputs in sq [batch][sq_ld] (null: none).
+int launch_paged_attention(const wq4_kv_cache* cache, const uint16_t* q, int q_stride, const int32_t* seq_lens,
+                           uint16_t* out, int out_stride, int batch, int n_q_heads, float scale, void* workspace,
+                           size_t workspace_bytes, float* sq, int sq_ld, cudaStream_t stream);
 
 // 2-D tiled tensor map (driver entry point, no libcuda link): dims
 // {inner, outer} elements, row pitch row_bytes, box {box_inner, box_outer}.
