@@ -66,7 +66,7 @@ constexpr int kChainMaxSlots = 16;
 // for every stage, which bounds how far ahead of the oldest unconsumed chunk
 // a warp can be (nslots - 1 + ceil(NW / items per slot) chunks).
 constexpr int kFullBars = 48;
-constexpr int kMaxChainBatch = 2;   // larger batches take the tensor-core graph path
+constexpr int kMaxChainBatch = 2;   // larger batches take the stage kernels of the graph path
 // A ring slot is released after kSlotRelease arrivals: one per item consumed
 // from it, plus (kSlotRelease - items) from the warp that consumed its first
 // item.  Only warps that own items of a chunk touch its barriers.
@@ -148,8 +148,8 @@ static_assert(sizeof(ChainParams) <= 32764, "kernel parameter space");
 // new k and v to the layer's paged cache and publishes them as flagged words;
 // at the start of the O stage every CTA computes its splits of the decode
 // attention (a (row, kv head, token range) each, fp32 online softmax over the
-// cached tokens plus the new one), the last split of each (row, kv head) to
-// arrive merges the partials and publishes the attention output, which the O
+// cached tokens plus the new one), the splits of a (row, kv head) exchange
+// their partials and publish the attention output, a share each, which the O
 // stage stages in place of the query block.
 constexpr int kAttnD = 128;          // head dimension
 constexpr int kAttnMaxGroup = 8;     // query heads per kv head
@@ -175,8 +175,7 @@ struct ChainParamsA : ChainParams {
     uint16_t* pQr;                 // [L][B][H] rotated queries
     uint16_t* pKr;                 // [L][B][Hkv 128] rotated keys
     uint16_t* pAt;                 // [L][B][H] attention output
-    float* apart;                  // [L][B][Hkv][S][G][kAttnPart] split partials
-    uint32_t* acnt;                // [L][B][Hkv] splits arrived
+    uint64_t* apart;               // [L][B][Hkv][S][G][kAttnPart] split partials (flagged fp32)
     double inv_freq[kAttnD / 2];   // theta^(-2i / 128)
     KvLayer kv[kChainMaxLayers];
 };
@@ -361,6 +360,26 @@ __device__ __forceinline__ uint32_t ll_load(const uint64_t* addr, uint32_t tag, 
         }
     }
     return static_cast<uint32_t>(a);
+}
+
+// Two consecutive flagged fp32 words at a 16-byte aligned address.
+__device__ __forceinline__ float2 ll_load_f2(const uint64_t* addr, uint32_t epoch, uint32_t* err, uint32_t* abort,
+                                             uint64_t limit_ns)
+{
+    uint64_t a, b;
+    ll_load2_raw(addr, a, b);
+    if (static_cast<uint32_t>(a >> 32) != epoch || static_cast<uint32_t>(b >> 32) != epoch) {
+        const uint64_t t0 = globaltimer_ns();
+        for (uint32_t it = 0;; ++it) {
+            ll_load2_raw(addr, a, b);
+            if (static_cast<uint32_t>(a >> 32) == epoch && static_cast<uint32_t>(b >> 32) == epoch) break;
+            if ((it & 63) == 63 && gave_up(t0, epoch, abort, limit_ns)) {
+                atomicOr(err, kErrFlagTimeout);
+                break;
+            }
+        }
+    }
+    return make_float2(__uint_as_float(static_cast<uint32_t>(a)), __uint_as_float(static_cast<uint32_t>(b)));
 }
 
 // fp16(a + b): the fp32 sum of two fp16 values rounded to fp16 equals the
@@ -550,66 +569,132 @@ __device__ __forceinline__ float warp_allsum(float v)
 // the start of the O stage.  Row b's T = positions[b] + 1 tokens are cut into
 // S_b = min(S, ceil(T / kAttnSplitTokens)) equal ranges; unit u = blockIdx.x
 // + k * gridDim.x is (row b, kv head h, range c), ranges c >= S_b are empty.
-// The unit's warps take U consecutive tokens at a time (lane: dimensions
-// 4 lane .. 4 lane + 3; the range's page ids are staged in shared memory
-// first), keeping a running maximum, sum and weighted value sum per query
-// head of the group; the warps are combined in shared memory in warp order
-// (one head at a time).  With one range the unit publishes a = o / l
-// itself; otherwise it stores its (o, m, l) and the last range of (b, h) to
-// arrive merges all S_b of them in range order and publishes a.
-// Shared memory: xs area = qs[G][128] | wp[NW][kAttnPart]; header area from
-// kHdrRes (res and part are free until the O stage's staging) = acc[G][kAttnPart] |
-// pages[kAttnPageWindow].
+// The range's cached keys and values come through the weight ring: which they
+// are is known from the token's start, so the producer warp streams them like
+// weights, between the layer's QKV and O chunks, and they have landed by the
+// time the queries have.  (Read by the warps themselves once the queries were
+// in, they cost ~5 us of latency a layer: 3B, 4096 tokens, 1212 -> 1082 us a
+// token; the flagged exchange between the ranges 1082 -> 1017, the combine of
+// four heads at a time 1017 -> 981.)  The new token's key and value are polled with the queries.  The
+// warps take blocks of 16 tokens in ring order, keeping a running maximum, sum
+// and weighted value sum per query head of the group; they are combined in
+// shared memory in warp order (one head at a time).  With one range the unit
+// publishes a = o / l itself; otherwise it publishes its (o, m, l), and each of
+// the S_b ranges merges its share of the output over all of them.
+// Shared memory: xs area = qs[G][128] | wp[min(G, kAttnHeads)][NW][kAttnPart];
+// header area from kHdrRes (res and part are free until the O stage's staging)
+// = newkv[2][64], then the merge's ml[kAttnMaxSplits][G] | po (at most G * 64
+// + kAttnMaxSplits pairs).
+constexpr int kAttnHeads = 4;                // heads combined at a time
 constexpr int kAttnSplitTokens = 128;
-constexpr int kAttnPageWindow = 256;
-static_assert(kHdrRes + 4 * (kAttnMaxGroup * kAttnPart + kAttnPageWindow + kAttnD) <= kChainHeader,
+constexpr int kAttnMaxChunk = 64;            // tokens of a ring slot, at most
+static_assert(kHdrRes + 8 * (kAttnMaxSplits * kAttnMaxGroup + kAttnMaxGroup * kAttnD / 2 + kAttnMaxSplits) <= kChainHeader,
               "attention scratch overlaps the staged input");
 
+struct AttnUnit {
+    int b, h, c, Sb, pos;
+    int t0, t1;          // the range's tokens
+    int te;              // ... of which [t0, te) are in the cache (the new one is not)
+};
+
+// Unit u, or false when its range is empty.
+template <int B>
+__device__ __forceinline__ bool attn_unit(const ChainParamsA& p, int l, const int* pos_sh, int u, AttnUnit* a)
+{
+    a->b = u / (p.Hkv * p.S);
+    const int rr = u - a->b * (p.Hkv * p.S);
+    a->h = rr / p.S;
+    a->c = rr - a->h * p.S;
+    a->pos = pos_sh[a->b];
+    const int T = min(a->pos, p.kv[l].pt_stride * p.P - 1) + 1; // 0 for an invalid position
+    const int Sb = (T + kAttnSplitTokens - 1) / kAttnSplitTokens;
+    a->Sb = Sb < 1 ? 1 : (Sb > p.S ? p.S : Sb);
+    if (a->c >= a->Sb) return false;
+    const int each = T / a->Sb, over = T - each * a->Sb;        // the first `over` ranges take one more
+    a->t0 = a->c * each + min(a->c, over);
+    a->t1 = a->t0 + each + (a->c < over ? 1 : 0);
+    a->te = (a->pos >= a->t0 && a->pos < a->t1) ? a->pos : a->t1;
+    return true;
+}
+
+// Tokens of one ring slot (keys, then values, 256 bytes a token each).
+__device__ __forceinline__ int attn_chunk_tokens(uint32_t slot_bytes)
+{
+    return min(kAttnMaxChunk, static_cast<int>(slot_bytes / (4 * kAttnD))) & ~15;
+}
+
+// Producer lane: the bulk copies of tokens [ta, tb) of a unit into one slot.
+// Rows of a page id outside the pool become zeros (and are flagged).
+__device__ __forceinline__ void attn_copy(const ChainParamsA& p, int l, const AttnUnit& a, int ta, int tb, int ct,
+                                          uint8_t* dst, uint64_t* fb, uint64_t pol)
+{
+    const KvLayer& kv = p.kv[l];
+    const int P = p.P, p0 = ta / P;
+    const int32_t* pt = kv.pt + static_cast<size_t>(a.b) * kv.pt_stride + p0;
+    constexpr int kRuns = kAttnMaxChunk / 16 + 1;               // pages of at least 16 tokens
+    int pg[kRuns];
+    uint32_t bytes = 0;
+#pragma unroll
+    for (int i = 0; i < kRuns; ++i) pg[i] = (p0 + i) * P < tb ? __ldg(pt + i) : -1;
+#pragma unroll
+    for (int i = 0; i < kRuns; ++i) {
+        const int x0 = max(ta, (p0 + i) * P), x1 = min(tb, (p0 + i + 1) * P);
+        if (x0 >= x1) continue;
+        if (pg[i] >= 0 && pg[i] < kv.num_pages) {
+            bytes += static_cast<uint32_t>(x1 - x0) * (4 * kAttnD);
+        } else {
+            atomicOr(p.err, kErrPageId);
+            pg[i] = -1;
+            uint4* kz = reinterpret_cast<uint4*>(dst + (x0 - ta) * (2 * kAttnD));
+            uint4* vz = reinterpret_cast<uint4*>(dst + (ct + x0 - ta) * (2 * kAttnD));
+            for (int e = 0; e < (x1 - x0) * (2 * kAttnD / 16); ++e) kz[e] = vz[e] = make_uint4(0u, 0u, 0u, 0u);
+            asm volatile("fence.proxy.async.shared::cta;" ::: "memory");   // before a later copy into the slot
+        }
+    }
+    mbar_arrive_expect_tx(fb, bytes);
+#pragma unroll
+    for (int i = 0; i < kRuns; ++i) {
+        const int x0 = max(ta, (p0 + i) * P), x1 = min(tb, (p0 + i + 1) * P);
+        if (x0 >= x1 || pg[i] < 0) continue;
+        const size_t row = (static_cast<size_t>(pg[i]) * p.Hkv + a.h) * P + (x0 - (p0 + i) * P);
+        const uint32_t n = static_cast<uint32_t>(x1 - x0) * (2 * kAttnD);
+        bulk_g2s(dst + (x0 - ta) * (2 * kAttnD), kv.k + row * kAttnD, n, fb, pol);
+        bulk_g2s(dst + (ct + x0 - ta) * (2 * kAttnD), kv.v + row * kAttnD, n, fb, pol);
+    }
+}
+
+// Returns the ring chunks of the CTA's units; ord0: the first one's ordinal.
 template <int B, int NW, int G>
-__device__ __forceinline__ void attention_phase(const ChainParamsA& p, int l, uint32_t epoch, float* scratch, const int* pos_sh,
-                                             int* flag_sh, uint8_t* smem)
+__device__ __forceinline__ int attention_phase(const ChainParamsA& p, int l, uint32_t epoch, float* scratch, const int* pos_sh,
+                                               uint8_t* smem, uint64_t* full, uint64_t* empty,
+                                             uint8_t* slots, int ord0)
 {
     constexpr int kConsumers = NW * 32;
     constexpr int kBlk = 16;                   // tokens of a warp's block: one per lane pair
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int H = p.H, Hkv = p.Hkv, S = p.S, KD = Hkv * kAttnD, P = p.P;
+    const int H = p.H, Hkv = p.Hkv, S = p.S, KD = Hkv * kAttnD;
     const float scale = p.scale * 1.4426950408889634f;   // base-2 scores
-    // the layer's cache and the outputs in registers (the parameter block is
-    // reached through a generic pointer here)
-    const KvLayer kv = p.kv[l];
+    // the outputs in registers (the parameter block is reached through a
+    // generic pointer here)
     uint16_t* const pAt = p.pAt;
     uint64_t* const llAt = p.llAt;
     const uint32_t repAt = p.repAt;
-    float* const apart = p.apart;
-    uint32_t* const acnt = p.acnt;
-    uint32_t* const err = p.err;
     uint32_t* qh = reinterpret_cast<uint32_t*>(scratch);                        // [G][64] fp16 pairs of q
     float* wp = scratch + G * kAttnD;
-    float* acc = reinterpret_cast<float*>(smem + kHdrRes);                       // [G][kAttnPart]
-    int* pages = reinterpret_cast<int*>(smem + kHdrRes) + G * kAttnPart;          // [kAttnPageWindow]
-    uint32_t* newkv = reinterpret_cast<uint32_t*>(pages + kAttnPageWindow);      // [2][64] the new key, value words
+    uint32_t* newkv = reinterpret_cast<uint32_t*>(smem + kHdrRes);               // [2][64] the new key, value words
     const int nunits = B * Hkv * S;
+    const int ct = attn_chunk_tokens(p.slot_bytes), bpc = ct / kBlk;            // tokens, blocks per chunk
     const uint64_t* qsrc = p.llA + ((blockIdx.x & 1) ? p.rep.A : 0u) + static_cast<size_t>(l) * B * (H / 2);
+    int chunks = 0;
     for (int u = blockIdx.x; u < nunits; u += gridDim.x) {
-        const int b = u / (Hkv * S);
-        const int rr = u - b * (Hkv * S);
-        const int h = rr / S, c = rr - h * S;
-        const int pos = pos_sh[b];
-        int T = pos + 1;                                        // 0 for an invalid position
-        const int cap = kv.pt_stride * P;
-        if (T > cap) {
-            T = cap;
-            if (threadIdx.x == 0 && c == 0) atomicOr(err, kErrSeqLen);
-        }
-        int Sb = (T + kAttnSplitTokens - 1) / kAttnSplitTokens;
-        Sb = Sb < 1 ? 1 : (Sb > S ? S : Sb);
-        if (c >= Sb) continue;                                  // uniform over the CTA
-        const int t0 = static_cast<int>(static_cast<int64_t>(c) * T / Sb);
-        const int t1 = static_cast<int>(static_cast<int64_t>(c + 1) * T / Sb);
+        AttnUnit au;
+        if (!attn_unit<B>(p, l, pos_sh, u, &au)) continue;      // uniform over the CTA
+        const int b = au.b, h = au.h, c = au.c, Sb = au.Sb, pos = au.pos;
+        if (threadIdx.x == 0 && c == 0 && pos >= p.kv[l].pt_stride * p.P) atomicOr(p.err, kErrSeqLen);
         named_barrier_sync(1, kConsumers);                      // scratch free
         // the group's queries and, in the range holding the new token, its key
         // and value words: all polled at once
-        const bool has_new = pos >= t0 && pos < t1;
+        const bool has_new = pos >= au.t0 && pos < au.t1;
         for (int e = threadIdx.x; e < G * (kAttnD / 2) + (has_new ? kAttnD : 0); e += kConsumers) {
             if (e < G * (kAttnD / 2)) {
                 const int j = e / (kAttnD / 2), w = e - j * (kAttnD / 2);
@@ -629,111 +714,79 @@ __device__ __forceinline__ void attention_phase(const ChainParamsA& p, int l, ui
             ls[j] = 0.f;
             o[j][0] = o[j][1] = o[j][2] = o[j][3] = 0.f;
         }
-        const int32_t* ptb = kv.pt + static_cast<size_t>(b) * kv.pt_stride;
         const int half = lane & 1, ti = lane >> 1;
-        // the range in windows of kAttnPageWindow pages
-        for (int wbeg = t0; wbeg < t1; wbeg += kAttnPageWindow * P - (wbeg % P)) {
-            const int wp0 = wbeg / P;
-            const int wend = min(t1, (wp0 + kAttnPageWindow) * P);
-            const int npg = (wend - 1) / P - wp0 + 1;
-            named_barrier_sync(1, kConsumers);                  // previous window's pages consumed; q written
-            for (int i = threadIdx.x; i < npg; i += kConsumers) {
-                const int pid = __ldg(ptb + wp0 + i);
-                pages[i] = (pid >= 0 && pid < kv.num_pages) ? pid : -1;
-                if (pid < 0 || pid >= kv.num_pages) atomicOr(err, kErrPageId);
-            }
-            named_barrier_sync(1, kConsumers);
-            // blocks of 16 tokens per warp: lane pair (2 i, 2 i + 1) scores token
-            // base + i over dimensions 64 half .. 64 half + 63 (fp16 products
-            // exact in fp32, fp32 sums), then every lane accumulates the value
-            // rows' dimensions 4 lane .. 4 lane + 3 with the broadcast weights
-            for (int base = wbeg + warp * kBlk; base < wend; base += NW * kBlk) {
-                const int t = base + ti;
-                const bool valid = t < wend;
-                float sp[G][2];
+        const int nblk = (au.te - au.t0 + kBlk - 1) / kBlk;
+        named_barrier_sync(1, kConsumers);                      // queries written
+        // blocks of 16 tokens per warp, in ring order: lane pair (2 i, 2 i + 1)
+        // scores token i over dimensions 64 half .. 64 half + 63 (fp16 products
+        // exact in fp32, fp32 sums), then every lane accumulates the value
+        // rows' dimensions 4 lane .. 4 lane + 3 with the broadcast weights
+        for (int it = warp; it < nblk; it += NW) {
+            const int k = it / bpc, i0 = k * bpc;               // the block's chunk and that chunk's first block
+            const int ord = ord0 + chunks + k;
+            const int slot = ord % p.nslots, qb = ord / p.nbars;
+            mbar_wait(&full[ord - qb * p.nbars], static_cast<uint32_t>(qb) & 1u, p.err);
+            const uint32_t ka = smem_addr(slots + static_cast<size_t>(slot) * p.slot_bytes) + (it - i0) * (kBlk * 2 * kAttnD);
+            const uint32_t va = ka + ct * (2 * kAttnD);
+            const int nb = min(kBlk, au.te - (au.t0 + it * kBlk));
+            const bool valid = ti < nb;
+            float sp[G][2];
 #pragma unroll
-                for (int j = 0; j < G; ++j) sp[j][0] = sp[j][1] = 0.f;
-                // the key half-row in two passes of four 16-byte chunks
-                const uint4* krow = nullptr;
-                const uint4* knew4 = nullptr;
-                if (valid && t == pos) {
-                    knew4 = reinterpret_cast<const uint4*>(newkv + 32 * half);
-                } else if (valid) {
-                    const int pi = t / P;
-                    const int page = pages[pi - wp0];
-                    if (page >= 0)
-                        krow = reinterpret_cast<const uint4*>(
-                            kv.k + ((static_cast<size_t>(page) * Hkv + h) * P + (t - pi * P)) * kAttnD + 64 * half);
-                }
+            for (int j = 0; j < G; ++j) sp[j][0] = sp[j][1] = 0.f;
+            // the key half-row in 16-byte chunks, each lane starting at its own,
+            // so that eight lanes read eight bank groups
+            const uint32_t krow = ka + ti * (2 * kAttnD) + 128 * half;
+            const uint32_t qrow = smem_addr(qh) + 128 * half;
 #pragma unroll
-                for (int ps = 0; ps < 2; ++ps) {
-                    uint4 kc[4];
-#pragma unroll
-                    for (int cc = 0; cc < 4; ++cc)
-                        kc[cc] = knew4 ? knew4[4 * ps + cc] : (krow ? __ldg(krow + 4 * ps + cc) : make_uint4(0u, 0u, 0u, 0u));
-#pragma unroll
-                    for (int cc = 0; cc < 4; ++cc) {
-#pragma unroll
-                        for (int j = 0; j < G; ++j) {
-                            // a shared-memory load per use: held in registers across the
-                            // blocks, the group's queries would spill
-                            const uint4 qc = lds_v4(smem_addr(qh + j * (kAttnD / 2) + 32 * half + 4 * (4 * ps + cc)));
-                            float& a = sp[j][cc & 1];
-                            a = fma_h2(a, qc.x, kc[cc].x);
-                            a = fma_h2(a, qc.y, kc[cc].y);
-                            a = fma_h2(a, qc.z, kc[cc].z);
-                            a = fma_h2(a, qc.w, kc[cc].w);
-                        }
-                    }
-                }
-                float pw[G];
+            for (int cc = 0; cc < 8; ++cc) {
+                const uint32_t off = 16u * ((cc + lane) & 7);
+                const uint4 kc = lds_v4(krow + off);
 #pragma unroll
                 for (int j = 0; j < G; ++j) {
-                    float sc = sp[j][0] + sp[j][1];
-                    sc = (sc + __shfl_xor_sync(0xffffffffu, sc, 1)) * scale;
-                    if (!valid) sc = -INFINITY;
-                    float bm = sc;                             // the block's maximum (token base is valid)
-#pragma unroll
-                    for (int off = 16; off > 1; off >>= 1) bm = fmaxf(bm, __shfl_xor_sync(0xffffffffu, bm, off));
-                    const float mn = fmaxf(m[j], bm);
-                    const float corr = fast_exp2(m[j] - mn);
-                    pw[j] = valid ? fast_exp2(sc - mn) : 0.f;
-                    float bs = half ? 0.f : pw[j];             // each token once
-#pragma unroll
-                    for (int off = 16; off > 0; off >>= 1) bs += __shfl_xor_sync(0xffffffffu, bs, off);
-                    ls[j] = fmaf(ls[j], corr, bs);
-                    o[j][0] *= corr;
-                    o[j][1] *= corr;
-                    o[j][2] *= corr;
-                    o[j][3] *= corr;
-                    m[j] = mn;
+                    // a shared-memory load per use: held in registers across the
+                    // blocks, the group's queries would spill
+                    const uint4 qc = lds_v4(qrow + j * (2 * kAttnD) + off);
+                    float& a = sp[j][cc & 1];
+                    a = fma_h2(a, qc.x, kc.x);
+                    a = fma_h2(a, qc.y, kc.y);
+                    a = fma_h2(a, qc.z, kc.z);
+                    a = fma_h2(a, qc.w, kc.w);
                 }
-                const int nb = min(kBlk, wend - base);
-                // every value row of the block in flight at once, then the sums
-                uint2 vv[kBlk];
+            }
+            float pw[G];
 #pragma unroll
-                for (int i = 0; i < kBlk; ++i) {
-                    const int tt = base + i;
-                    vv[i] = make_uint2(0u, 0u);
-                    if (i < nb) {
-                        if (tt == pos) {
-                            vv[i] = make_uint2(newkv[64 + 2 * lane], newkv[64 + 2 * lane + 1]);
-                        } else {
-                            const int pi = tt / P;
-                            const int page = pages[pi - wp0];
-                            if (page >= 0)
-                                vv[i] = __ldg(reinterpret_cast<const uint2*>(
-                                                  kv.v + ((static_cast<size_t>(page) * Hkv + h) * P + (tt - pi * P)) * kAttnD) +
-                                              lane);
-                        }
-                    }
-                }
+            for (int j = 0; j < G; ++j) {
+                float sc = sp[j][0] + sp[j][1];
+                sc = (sc + __shfl_xor_sync(0xffffffffu, sc, 1)) * scale;
+                if (!valid) sc = -INFINITY;
+                float bm = sc;                                 // the block's maximum (its first token is valid)
 #pragma unroll
-                for (int i = 0; i < kBlk; ++i) {
-                    const float w0 = lo_f(vv[i].x), w1 = hi_f(vv[i].x), w2 = lo_f(vv[i].y), w3 = hi_f(vv[i].y);
+                for (int off = 16; off > 1; off >>= 1) bm = fmaxf(bm, __shfl_xor_sync(0xffffffffu, bm, off));
+                const float mn = fmaxf(m[j], bm);
+                const float corr = fast_exp2(m[j] - mn);
+                pw[j] = valid ? fast_exp2(sc - mn) : 0.f;
+                float bs = half ? 0.f : pw[j];                 // each token once
+#pragma unroll
+                for (int off = 16; off > 0; off >>= 1) bs += __shfl_xor_sync(0xffffffffu, bs, off);
+                ls[j] = fmaf(ls[j], corr, bs);
+                o[j][0] *= corr;
+                o[j][1] *= corr;
+                o[j][2] *= corr;
+                o[j][3] *= corr;
+                m[j] = mn;
+            }
+#pragma unroll
+            for (int i = 0; i < kBlk; ++i) {
+                if (i < nb) {                                  // rows past the range hold anything
+                    uint2 vv;
+                    asm volatile("ld.shared.v2.b32 {%0, %1}, [%2];"
+                                 : "=r"(vv.x), "=r"(vv.y)
+                                 : "r"(va + i * (2 * kAttnD) + 8 * lane)
+                                 : "memory");
+                    const float w0 = lo_f(vv.x), w1 = hi_f(vv.x), w2 = lo_f(vv.y), w3 = hi_f(vv.y);
 #pragma unroll
                     for (int j = 0; j < G; ++j) {
-                        const float pi_ = __shfl_sync(0xffffffffu, pw[j], 2 * i);   // 0 past the window's end
+                        const float pi_ = __shfl_sync(0xffffffffu, pw[j], 2 * i);
                         o[j][0] = fmaf(pi_, w0, o[j][0]);
                         o[j][1] = fmaf(pi_, w1, o[j][1]);
                         o[j][2] = fmaf(pi_, w2, o[j][2]);
@@ -741,126 +794,142 @@ __device__ __forceinline__ void attention_phase(const ChainParamsA& p, int l, ui
                     }
                 }
             }
+            __syncwarp();
+            // one arrival per block; the chunk's first block brings the rest
+            if (lane == 0)
+                mbar_arrive_count(&empty[slot], it == i0 ? kSlotRelease + 1u - static_cast<uint32_t>(min(bpc, nblk - i0)) : 1u);
         }
-        // combine the warps in warp order, one query head at a time, into acc
+        chunks += (nblk + bpc - 1) / bpc;
+        if (has_new && warp == nblk % NW) {
+            // the new token, its dimensions over the lanes
 #pragma unroll
-        for (int j = 0; j < G; ++j) {
-            float* mine = wp + warp * kAttnPart;
-            reinterpret_cast<float4*>(mine)[lane] = make_float4(o[j][0], o[j][1], o[j][2], o[j][3]);
-            if (lane == 0) {
-                mine[kAttnD] = m[j];
-                mine[kAttnD + 1] = ls[j];
+            for (int j = 0; j < G; ++j) {
+                float sc = fma_h2(0.f, qh[j * (kAttnD / 2) + 2 * lane], newkv[2 * lane]);
+                sc = fma_h2(sc, qh[j * (kAttnD / 2) + 2 * lane + 1], newkv[2 * lane + 1]);
+                sc = warp_allsum(sc) * scale;
+                const float mn = fmaxf(m[j], sc);
+                const float corr = fast_exp2(m[j] - mn), pn = fast_exp2(sc - mn);
+                const uint32_t v0 = newkv[64 + 2 * lane], v1 = newkv[64 + 2 * lane + 1];
+                ls[j] = fmaf(ls[j], corr, pn);
+                o[j][0] = fmaf(o[j][0], corr, pn * lo_f(v0));
+                o[j][1] = fmaf(o[j][1], corr, pn * hi_f(v0));
+                o[j][2] = fmaf(o[j][2], corr, pn * lo_f(v1));
+                o[j][3] = fmaf(o[j][3], corr, pn * hi_f(v1));
+                m[j] = mn;
+            }
+        }
+        // combine the warps in warp order, up to four query heads at a time, a
+        // thread per pair of dimensions.  One range: its result is the attention
+        // output.  Else it publishes its (o, m, l) as flagged words, and every
+        // range merges its share of the output's pairs over all ranges, in range
+        // order: one exchange, where an arrival counter and a last range that
+        // merges alone took a fence, an atomic and two dependent loads (~2 us more)
+        uint64_t* const rp = p.apart + (((static_cast<size_t>(l) * B + b) * Hkv + h) * S) * G * kAttnPart;
+#pragma unroll
+        for (int j0 = 0; j0 < G; j0 += kAttnHeads) {
+            constexpr int HP = G < kAttnHeads ? G : kAttnHeads;      // heads of a pass (the last may hold fewer)
+            if (j0 > 0) named_barrier_sync(1, kConsumers);           // the previous heads' partials were read
+#pragma unroll
+            for (int i = 0; i < HP; ++i) {
+                if (j0 + i >= G) break;
+                const int j = j0 + i < G ? j0 + i : 0;
+                float* mine = wp + (i * NW + warp) * kAttnPart;
+                reinterpret_cast<float4*>(mine)[lane] = make_float4(o[j][0], o[j][1], o[j][2], o[j][3]);
+                if (lane == 0) {
+                    mine[kAttnD] = m[j];
+                    mine[kAttnD + 1] = ls[j];
+                }
             }
             named_barrier_sync(1, kConsumers);
-            if (threadIdx.x < kAttnD) {
-                const int d = threadIdx.x;
+            for (int e = threadIdx.x; e < min(HP, G - j0) * (kAttnD / 2); e += kConsumers) {
+                const int i = e / (kAttnD / 2), w = e - i * (kAttnD / 2), j = j0 + i;
+                const float* hp = wp + i * NW * kAttnPart;
                 float M = -INFINITY;
 #pragma unroll
-                for (int w = 0; w < NW; ++w) M = fmaxf(M, wp[w * kAttnPart + kAttnD]);
-                float Ls = 0.f, Od = 0.f;
-                if (M != -INFINITY) {
-#pragma unroll
-                    for (int w = 0; w < NW; ++w) {
-                        const float f = fast_exp2(wp[w * kAttnPart + kAttnD] - M);   // 0 for a warp without tokens
-                        Ls = fmaf(f, wp[w * kAttnPart + kAttnD + 1], Ls);
-                        Od = fmaf(f, wp[w * kAttnPart + d], Od);
-                    }
-                }
-                acc[j * kAttnPart + d] = Od;
-                if (d == 0) {
-                    acc[j * kAttnPart + kAttnD] = M;
-                    acc[j * kAttnPart + kAttnD + 1] = Ls;
-                }
-            }
-            named_barrier_sync(1, kConsumers);
-        }
-        if (Sb == 1) {
-            // one range: this unit's result is the attention output
-            for (int e = threadIdx.x; e < G * (kAttnD / 2); e += kConsumers) {
-                const int j = e / (kAttnD / 2), w = e - j * (kAttnD / 2);
-                const float Ls = acc[j * kAttnPart + kAttnD + 1];
-                const float a0 = Ls > 0.f ? acc[j * kAttnPart + 2 * w] / Ls : 0.f;
-                const float a1 = Ls > 0.f ? acc[j * kAttnPart + 2 * w + 1] / Ls : 0.f;
-                const uint32_t aw = pack2(float_to_half_bits(a0), float_to_half_bits(a1));
-                const int n = (h * G + j) * kAttnD + 2 * w;
-                *reinterpret_cast<uint32_t*>(pAt + (static_cast<size_t>(l) * B + b) * H + n) = aw;
-                ll_store2(llAt + (static_cast<size_t>(l) * B + b) * (H / 2) + n / 2, repAt, aw, epoch);
-            }
-            continue;                                           // the next unit starts with a barrier
-        }
-        // store the range's partial, then arrive
-        float* dst = apart + ((((static_cast<size_t>(l) * B + b) * Hkv + h) * S + c) * G) * kAttnPart;
-        for (int e = threadIdx.x; e < G * (kAttnD + 2); e += kConsumers) {
-            const int j = e / (kAttnD + 2), d = e - j * (kAttnD + 2);
-            dst[j * kAttnPart + d] = acc[j * kAttnPart + d];
-        }
-        __threadfence();
-        named_barrier_sync(1, kConsumers);
-        if (threadIdx.x == 0) {
-            const uint32_t prev = atomicAdd(acnt + (static_cast<size_t>(l) * B + b) * Hkv + h, 1u);
-            *flag_sh = (prev == static_cast<uint32_t>(Sb - 1)) ? 1 : 0;
-            __threadfence();
-        }
-        named_barrier_sync(1, kConsumers);
-        if (*flag_sh) {
-            // every range of (b, h) is in: merge them in range order; the ranges'
-            // (m, l) first (all loads in flight), then per thread a pair of
-            // dimensions of a head with its Sb loads in flight
-            const float* src = apart + (((static_cast<size_t>(l) * B + b) * Hkv + h) * S) * G * kAttnPart;
-            float2* ml = reinterpret_cast<float2*>(wp);              // [Sb][G]
-            for (int e = threadIdx.x; e < Sb * G; e += kConsumers)
-                ml[e] = __ldcg(reinterpret_cast<const float2*>(src + e * kAttnPart + kAttnD));
-            named_barrier_sync(1, kConsumers);
-            for (int e = threadIdx.x; e < G * (kAttnD / 2); e += kConsumers) {
-                const int j = e / (kAttnD / 2), w = e - j * (kAttnD / 2);
-                float M = -INFINITY;
-                for (int cc = 0; cc < Sb; ++cc) M = fmaxf(M, ml[cc * G + j].x);
+                for (int q = 0; q < NW; ++q) M = fmaxf(M, hp[q * kAttnPart + kAttnD]);
                 float Ls = 0.f, O0 = 0.f, O1 = 0.f;
                 if (M != -INFINITY) {
-                    constexpr int kBatch = 16;                  // loads in flight per thread
-                    for (int c0 = 0; c0 < Sb; c0 += kBatch) {
-                        float2 ov[kBatch];
 #pragma unroll
-                        for (int i = 0; i < kBatch; ++i)
-                            ov[i] = (c0 + i < Sb)
-                                        ? __ldcg(reinterpret_cast<const float2*>(src + ((c0 + i) * G + j) * kAttnPart) + w)
-                                        : make_float2(0.f, 0.f);
-#pragma unroll
-                        for (int i = 0; i < kBatch; ++i) {
-                            if (c0 + i >= Sb) break;
-                            const float2 mlc = ml[(c0 + i) * G + j];
-                            const float f = fast_exp2(mlc.x - M);
-                            Ls = fmaf(f, mlc.y, Ls);
-                            O0 = fmaf(f, ov[i].x, O0);
-                            O1 = fmaf(f, ov[i].y, O1);
-                        }
+                    for (int q = 0; q < NW; ++q) {
+                        const float2 mq = *reinterpret_cast<const float2*>(hp + q * kAttnPart + kAttnD);
+                        const float2 ov = *reinterpret_cast<const float2*>(hp + q * kAttnPart + 2 * w);
+                        const float f = fast_exp2(mq.x - M);   // 0 for a warp without tokens
+                        Ls = fmaf(f, mq.y, Ls);
+                        O0 = fmaf(f, ov.x, O0);
+                        O1 = fmaf(f, ov.y, O1);
                     }
                 }
-                const float a0 = Ls > 0.f ? O0 / Ls : 0.f, a1 = Ls > 0.f ? O1 / Ls : 0.f;
-                const uint32_t aw = pack2(float_to_half_bits(a0), float_to_half_bits(a1));
-                const int n = (h * G + j) * kAttnD + 2 * w;
-                *reinterpret_cast<uint32_t*>(pAt + (static_cast<size_t>(l) * B + b) * H + n) = aw;
-                ll_store2(llAt + (static_cast<size_t>(l) * B + b) * (H / 2) + n / 2, repAt, aw, epoch);
+                if (Sb == 1) {
+                    const float a0 = Ls > 0.f ? O0 / Ls : 0.f, a1 = Ls > 0.f ? O1 / Ls : 0.f;
+                    const uint32_t aw = pack2(float_to_half_bits(a0), float_to_half_bits(a1));
+                    const int n = (h * G + j) * kAttnD + 2 * w;
+                    *reinterpret_cast<uint32_t*>(pAt + (static_cast<size_t>(l) * B + b) * H + n) = aw;
+                    ll_store2(llAt + (static_cast<size_t>(l) * B + b) * (H / 2) + n / 2, repAt, aw, epoch);
+                } else {
+                    uint64_t* dst = rp + (static_cast<size_t>(c) * G + j) * kAttnPart;
+                    ll_store(dst + 2 * w, __float_as_uint(O0), epoch);
+                    ll_store(dst + 2 * w + 1, __float_as_uint(O1), epoch);
+                    if (w == 0) {
+                        ll_store(dst + kAttnD, __float_as_uint(M), epoch);
+                        ll_store(dst + kAttnD + 1, __float_as_uint(Ls), epoch);
+                    }
+                }
             }
-            if (threadIdx.x == 0) acnt[(static_cast<size_t>(l) * B + b) * Hkv + h] = 0u;   // for the next token
+        }
+        if (Sb == 1) continue;                                       // the next unit starts with a barrier
+        constexpr int W = G * (kAttnD / 2);
+        const int w0 = c * W / Sb, nw = (c + 1) * W / Sb - w0;
+        float2* ml = reinterpret_cast<float2*>(smem + kHdrRes);      // [Sb][G]
+        float2* po = ml + kAttnMaxSplits * G;                        // [Sb][nw]
+        for (int e = threadIdx.x; e < Sb * (G + nw); e += kConsumers) {
+            const int r = e / (G + nw), i = e - r * (G + nw);        // range; its i-th word pair
+            const int j = i < G ? i : (w0 + i - G) / (kAttnD / 2);
+            const int d = i < G ? kAttnD : 2 * ((w0 + i - G) % (kAttnD / 2));
+            const float2 v = ll_load_f2(rp + (static_cast<size_t>(r) * G + j) * kAttnPart + d, epoch, p.err, p.abort, p.wait_ns);
+            if (i < G) ml[r * G + i] = v;
+            else po[r * nw + i - G] = v;
+        }
+        named_barrier_sync(1, kConsumers);
+        for (int e = threadIdx.x; e < nw; e += kConsumers) {
+            const int w = w0 + e, j = w / (kAttnD / 2);
+            float M = -INFINITY;
+            for (int r = 0; r < Sb; ++r) M = fmaxf(M, ml[r * G + j].x);
+            float Ls = 0.f, O0 = 0.f, O1 = 0.f;
+            if (M != -INFINITY) {
+#pragma unroll 4
+                for (int r = 0; r < Sb; ++r) {
+                    const float2 mr = ml[r * G + j], ov = po[r * nw + e];
+                    const float f = fast_exp2(mr.x - M);
+                    Ls = fmaf(f, mr.y, Ls);
+                    O0 = fmaf(f, ov.x, O0);
+                    O1 = fmaf(f, ov.y, O1);
+                }
+            }
+            const float a0 = Ls > 0.f ? O0 / Ls : 0.f, a1 = Ls > 0.f ? O1 / Ls : 0.f;
+            const uint32_t aw = pack2(float_to_half_bits(a0), float_to_half_bits(a1));
+            const int n = h * G * kAttnD + 2 * w;
+            *reinterpret_cast<uint32_t*>(pAt + (static_cast<size_t>(l) * B + b) * H + n) = aw;
+            ll_store2(llAt + (static_cast<size_t>(l) * B + b) * (H / 2) + n / 2, repAt, aw, epoch);
         }
     }
     named_barrier_sync(1, kConsumers);                          // scratch free for the staging
+    return chunks;
 }
 
 template <int B, int NW>
-__device__ __forceinline__ void attention_dispatch(const ChainParamsA& p, int l, uint32_t epoch, float* scratch,
-                                                   const int* pos_sh, int* flag_sh, uint8_t* smem)
+__device__ __forceinline__ int attention_dispatch(const ChainParamsA& p, int l, uint32_t epoch, float* scratch,
+                                                  const int* pos_sh, uint8_t* smem, uint64_t* full,
+                                                  uint64_t* empty, uint8_t* slots, int ord0)
 {
     switch (p.G) {
-        case 1: attention_phase<B, NW, 1>(p, l, epoch, scratch, pos_sh, flag_sh, smem); break;
-        case 2: attention_phase<B, NW, 2>(p, l, epoch, scratch, pos_sh, flag_sh, smem); break;
-        case 3: attention_phase<B, NW, 3>(p, l, epoch, scratch, pos_sh, flag_sh, smem); break;
-        case 4: attention_phase<B, NW, 4>(p, l, epoch, scratch, pos_sh, flag_sh, smem); break;
-        case 5: attention_phase<B, NW, 5>(p, l, epoch, scratch, pos_sh, flag_sh, smem); break;
-        case 6: attention_phase<B, NW, 6>(p, l, epoch, scratch, pos_sh, flag_sh, smem); break;
-        case 7: attention_phase<B, NW, 7>(p, l, epoch, scratch, pos_sh, flag_sh, smem); break;
-        default: attention_phase<B, NW, 8>(p, l, epoch, scratch, pos_sh, flag_sh, smem); break;
+        case 1: return attention_phase<B, NW, 1>(p, l, epoch, scratch, pos_sh, smem, full, empty, slots, ord0);
+        case 2: return attention_phase<B, NW, 2>(p, l, epoch, scratch, pos_sh, smem, full, empty, slots, ord0);
+        case 3: return attention_phase<B, NW, 3>(p, l, epoch, scratch, pos_sh, smem, full, empty, slots, ord0);
+        case 4: return attention_phase<B, NW, 4>(p, l, epoch, scratch, pos_sh, smem, full, empty, slots, ord0);
+        case 5: return attention_phase<B, NW, 5>(p, l, epoch, scratch, pos_sh, smem, full, empty, slots, ord0);
+        case 6: return attention_phase<B, NW, 6>(p, l, epoch, scratch, pos_sh, smem, full, empty, slots, ord0);
+        case 7: return attention_phase<B, NW, 7>(p, l, epoch, scratch, pos_sh, smem, full, empty, slots, ord0);
+        default: return attention_phase<B, NW, 8>(p, l, epoch, scratch, pos_sh, smem, full, empty, slots, ord0);
     }
 }
 
@@ -944,6 +1013,31 @@ __global__ void __launch_bounds__((NW + 1) * 32, 1)
                 const StageInfo in = info[g.type];
                 const int w0 = in.w0, w1 = in.w0 + in.nwords, wps = in.wps;
                 const int wpr = g.K >> 3, gpr = g.K >> 5;
+                if constexpr (ATT) {
+                    // the cached keys and values of this CTA's attention ranges
+                    if (g.type == kO) {
+                        const int* pos_sh = reinterpret_cast<const int*>(smem + p.rope_off + kPosOff);
+                        const int ct = attn_chunk_tokens(p.slot_bytes);
+                        for (int u = blockIdx.x; u < B * p.Hkv * p.S; u += gridDim.x) {
+                            AttnUnit au;
+                            if (!attn_unit<B>(p, g.layer, pos_sh, u, &au)) continue;
+                            for (int ta = au.t0; ta < au.te; ta += ct, ++ord) {
+                                if (round > 0) mbar_wait(&empty[slot], (round - 1) & 1, p.err);
+                                attn_copy(p, g.layer, au, ta, min(au.te, ta + ct), ct,
+                                          slots + static_cast<size_t>(slot) * p.slot_bytes, &full[fbi], pol);
+                                if (++slot == p.nslots) {
+                                    slot = 0;
+                                    ++round;
+                                }
+                                if (++fbi == p.nbars) fbi = 0;
+                            }
+                            if (au.te < au.t1) {               // the new token's page, read by nobody, is flagged too
+                                const int page = __ldg(p.kv[g.layer].pt + static_cast<size_t>(au.b) * p.kv[g.layer].pt_stride + au.pos / p.P);
+                                if (page < 0 || page >= p.kv[g.layer].num_pages) atomicOr(p.err, kErrPageId);
+                            }
+                        }
+                    }
+                }
                 for (int wa = w0; wa < w1; wa += wps, ++ord) {
                     const int wb = min(w1, wa + wps);
                     if (round > 0) mbar_wait(&empty[slot], (round - 1) & 1, p.err);
@@ -985,8 +1079,8 @@ __global__ void __launch_bounds__((NW + 1) * 32, 1)
                 // every CTA takes its splits of the layer's attention, words or not
                 if (g.type == kO) {
                     int* pos_sh = reinterpret_cast<int*>(smem + p.rope_off + kPosOff);
-                    attention_dispatch<B, NW>(p, g.layer, epoch, reinterpret_cast<float*>(xs), pos_sh,
-                                              pos_sh + kMaxChainBatch, smem);
+                    cord0 += attention_dispatch<B, NW>(p, g.layer, epoch, reinterpret_cast<float*>(xs), pos_sh,
+                                                       smem, full, empty, slots, cord0);
                 }
             }
             if (in.nwords <= 0) continue;
@@ -1231,19 +1325,31 @@ __global__ void __launch_bounds__((NW + 1) * 32, 1)
             }
 
             // -- every part of every word is in: add the parts in part order and
-            //    publish the words, one thread per (superpair, batch row) on the
-            //    first warps (spreading the entries over all warps, one lane
-            //    each, measured 0.2 ms a token slower)
+            //    publish the words, one thread per (word, batch row) on the first
+            //    warps (spreading the entries over all warps, one lane each,
+            //    measured 0.2 ms a token slower)
             if (g.type != kLM) named_barrier_sync(1, kConsumers);
-            for (int e = threadIdx.x; g.type != kLM && e < nsp * B; e += kConsumers) {
-                const int sl = e / B, b = e - sl * B;
+            for (int e = threadIdx.x; g.type != kLM && e < nwd * B; e += kConsumers) {
+                const int wc = e / B, b = e - wc * B;         // word (stage-relative)
+                const int sl = wc >> sps;
                 const float4* pp = part + sl * q * B + b;
-                float4 sum = pp[0];
-                for (int r = 1; r < q; ++r) {
-                    const float4 t4 = pp[r * B];
-                    sum.x += t4.x; sum.y += t4.y; sum.z += t4.z; sum.w += t4.w;
+                float4 sum;
+                if (g.type == kGU) {
+                    sum = pp[0];
+                    for (int r = 1; r < q; ++r) {
+                        const float4 t4 = pp[r * B];
+                        sum.x += t4.x; sum.y += t4.y; sum.z += t4.z; sum.w += t4.w;
+                    }
+                } else {
+                    // the word's two rows: the superpair's first or second half
+                    const float2* p2 = reinterpret_cast<const float2*>(pp) + (wc & (spw - 1));
+                    float2 s2 = p2[0];
+                    for (int r = 1; r < q; ++r) {
+                        const float2 t2 = p2[2 * r * B];
+                        s2.x += t2.x; s2.y += t2.y;
+                    }
+                    sum = make_float4(s2.x, s2.y, 0.f, 0.f);
                 }
-                const int wc = sl << sps;                     // first word (stage-relative)
 #pragma unroll
                 for (int bb = 0; bb < B; ++bb) {
                     if (bb != b) continue;
@@ -1252,8 +1358,6 @@ __global__ void __launch_bounds__((NW + 1) * 32, 1)
                             const double2* rope = reinterpret_cast<const double2*>(smem + p.rope_off);
                             const int* pos_sh = reinterpret_cast<const int*>(smem + p.rope_off + kPosOff);
                             qkv_epilogue_attn<B>(p, l, w0 + wc, bb, sum.x, sum.y, rf[bb], epoch, rope, pos_sh);
-                            if (spw == 2 && wc + 1 < nwd)
-                                qkv_epilogue_attn<B>(p, l, w0 + wc + 1, bb, sum.z, sum.w, rf[bb], epoch, rope, pos_sh);
                             continue;
                         }
                     }
@@ -1263,9 +1367,6 @@ __global__ void __launch_bounds__((NW + 1) * 32, 1)
                         const bool resid = (g.type == kO || g.type == kDOWN);
                         word_epilogue<B>(p, g, w0 + wc, bb, sum.x, sum.y, 0.f, 0.f, rf[bb],
                                          resid ? res[bb * nwd + wc] : 0u, epoch);
-                        if (spw == 2 && wc + 1 < nwd)
-                            word_epilogue<B>(p, g, w0 + wc + 1, bb, sum.z, sum.w, 0.f, 0.f, rf[bb],
-                                             resid ? res[bb * nwd + wc + 1] : 0u, epoch);
                     }
                 }
             }
@@ -1374,9 +1475,9 @@ struct Layout {
     size_t ll_begin, ll_end;
     // decode step (after everything above, so that the chain's offsets stay):
     // flagged words of the new keys, values and attention output (zeroed),
-    // traces, split partials and counters (batch 1-2), or the sequence
+    // traces, split partials (flagged, zeroed; batch 1-2), or the sequence
     // lengths and wq4_paged_attention's workspace (batch 3-32)
-    size_t att_ll_begin, att_ll_end, llK, llVn, llAt, pQr, pKr, pAt, apart, acnt, seq_lens, rope, attn_ws, attn_ws_bytes;
+    size_t att_ll_begin, att_ll_end, llK, llVn, llAt, pQr, pKr, pAt, apart, seq_lens, rope, attn_ws, attn_ws_bytes;
 };
 
 struct Dims {
@@ -1453,21 +1554,19 @@ Layout make_layout(const Dims& d, bool att = false, size_t attn_ws_bytes = 0)
         y.rfac = y.qA = 0;
     }
     y.att_ll_begin = y.att_ll_end = y.llK = y.llVn = y.llAt = y.pQr = y.pKr = y.pAt = 0;
-    y.apart = y.acnt = y.seq_lens = y.rope = y.attn_ws = y.attn_ws_bytes = 0;
+    y.apart = y.seq_lens = y.rope = y.attn_ws = y.attn_ws_bytes = 0;
     if (att) {
         const size_t KD = static_cast<size_t>(d.Hkv) * kAttnD, G = d.Hkv > 0 ? d.nq / d.Hkv : 0;
         y.att_ll_begin = o;
         y.llK = take(8 * L * B * (KD / 2));
         y.llVn = take(8 * L * B * (KD / 2));
         y.llAt = take(8 * 2 * L * B * (H / 2));          // two replicas
+        if (d.B <= kMaxChainBatch) y.apart = take(8 * L * B * d.Hkv * kAttnMaxSplits * G * kAttnPart);
         y.att_ll_end = o;
         y.pQr = take(2 * L * B * H);
         y.pKr = take(2 * L * B * KD);
         y.pAt = take(2 * L * B * H);
-        if (d.B <= kMaxChainBatch) {
-            y.apart = take(4 * L * B * d.Hkv * kAttnMaxSplits * G * kAttnPart);
-            y.acnt = take(4 * L * B * d.Hkv);
-        } else {
+        if (d.B > kMaxChainBatch) {
             y.seq_lens = take(4 * B);
             y.rope = take(sizeof(double2) * B * (kAttnD / 2));
             y.attn_ws = take(attn_ws_bytes);
@@ -1914,9 +2013,6 @@ int build_plan(const wq4_layer_table* t, const wq4_decode_attn* a, Plan* pl, cud
         // flagged words start at zero (epoch 0 never matches); counters at zero
         if (cudaMemsetAsync(ws + lay.att_ll_begin, 0, lay.att_ll_end - lay.att_ll_begin, stream) != cudaSuccess)
             return WQ4_ERR_CUDA;
-        if (lay.acnt && cudaMemsetAsync(ws + lay.acnt, 0, 4 * static_cast<size_t>(d.L) * d.B * d.Hkv, stream) !=
-                            cudaSuccess)
-            return WQ4_ERR_CUDA;
         if (lay.attn_ws && cudaMemsetAsync(ws + lay.attn_ws, 0, lay.attn_ws_bytes, stream) != cudaSuccess)
             return WQ4_ERR_CUDA;
     }
@@ -1928,7 +2024,10 @@ int build_plan(const wq4_layer_table* t, const wq4_decode_attn* a, Plan* pl, cud
     if (d.L > kChainMaxLayers) return WQ4_ERR_UNSUPPORTED;
     size_t xb = align_up(static_cast<size_t>(d.B) * 2 * (d.H > d.F ? d.H : d.F), 128);
     // the attention's scratch (queries of a group, per-warp partials) lives in the staging area
-    if (a) xb = std::max(xb, align_up(4 * static_cast<size_t>(kAttnMaxGroup * kAttnD + kChainWarps * kAttnPart), 128));
+    if (a) {
+        const int G = d.nq / d.Hkv;
+        xb = std::max(xb, align_up(4 * static_cast<size_t>(G * kAttnD + std::min(G, kAttnHeads) * kChainWarps * kAttnPart), 128));
+    }
     const uint32_t x_bytes = static_cast<uint32_t>(xb);
     // the rotation table (double2 [B][64]), the positions and a flag sit after the ring
     const size_t rope_bytes = a ? align_up(static_cast<size_t>(d.B) * (kAttnD / 2) * 16 + 16, 128) : 0;
@@ -2100,8 +2199,7 @@ int launch_chain(const Plan& pl, const uint16_t* x, uint16_t* logits, cudaStream
         p.pQr = reinterpret_cast<uint16_t*>(ws + y.pQr);
         p.pKr = reinterpret_cast<uint16_t*>(ws + y.pKr);
         p.pAt = reinterpret_cast<uint16_t*>(ws + y.pAt);
-        p.apart = reinterpret_cast<float*>(ws + y.apart);
-        p.acnt = reinterpret_cast<uint32_t*>(ws + y.acnt);
+        p.apart = reinterpret_cast<uint64_t*>(ws + y.apart);
         fill_inv_freq(pl.theta, p.inv_freq);
         for (int l = 0; l < pl.dims.L; ++l) p.kv[l] = kv_layer(pl.kv[l]);
         switch (pl.dims.B) {
