@@ -22,9 +22,9 @@
 // Two forms: rows that tensor copies can take (K % 256 == 0, 16-byte aligned
 // scales) run in bgemv_tma_kernel below, others in bgemv_kernel.  Measured
 // (us a launch in a graph over rotated copies, before: CUDA-core kernels that
-// read the activations through L1): 3072 x 8192 batch 8 76.5 -> 6.8,
-// 16384 x 3072 batch 8 100 -> 9.0 and batch 32 387 -> 17.8, 128256 x 4096
-// batch 8 927 -> 56 (5.3 TB/s) and batch 32 3739 -> 136; 1003 x 2080 (copy
+// read the activations through L1): 3072 x 8192 batch 8 76.5 -> 6.9,
+// 16384 x 3072 batch 8 100 -> 8.8 and batch 32 387 -> 17.3, 128256 x 4096
+// batch 8 927 -> 54.6 (5.4 TB/s) and batch 32 3739 -> 118; 1003 x 2080 (copy
 // ring) batch 5 7.3 -> 4.1.  Up to batch 8 the wide shapes are bound by
 // instruction issue and HBM together, at batch 32 by the MMAs (two per tile,
 // group and eight activation rows) and their issue; the narrow ones by the
@@ -343,10 +343,74 @@ struct TGemvParams {
     uint32_t* err;
 };
 
+// Stores one tile of `wrows` rows a warp from row n0 on.
 template <int XT, int R>
+__device__ __forceinline__ void store_tile(const TGemvParams& p, float* red, int ks, int wrows, int n0, int tid, int warp,
+                                           int lane, const float (&acc)[R][XT][4])
+{
+    constexpr int NW = kTWarps<XT>, kConsumers = 32 * NW;
+    if (ks == 1) {
+#pragma unroll
+        for (int r = 0; r < R; ++r)
+#pragma unroll
+            for (int t = 0; t < XT; ++t)
+#pragma unroll
+                for (int i = 0; i < 4; ++i) {
+                    const int row = 16 * r + (lane >> 2) + 8 * (i >> 1), n = n0 + warp * wrows + row;
+                    const int b = 8 * t + x_row(2 * (lane & 3) + (i & 1));
+                    if (row < wrows && n < p.N && b < p.batch)
+                        p.y[static_cast<size_t>(b) * p.N + n] = float_to_half_bits(acc[r][t][i]);
+                }
+        return;
+    }
+    store_sums<XT, R>(red, warp, lane, acc);
+    named_barrier_sync(1, kConsumers);
+    const int rgs = NW / ks, hrows = wrows >> 1;                 // pairs of rows per row group
+    for (int e = tid; e < rgs * hrows * 8 * XT; e += kConsumers) {
+        const int pr = e % hrows, q = e / hrows;                 // row pair; column and row group
+        const int col = q % (8 * XT), grp = q / (8 * XT);
+        const float2 sum = load_sums<XT, R>(red, grp, ks, col, 2 * pr);
+        const int n = n0 + grp * wrows + 2 * pr, b = (col & ~7) + x_row(col & 7);
+        if (b < p.batch && n < p.N) {
+            uint16_t* out = p.y + static_cast<size_t>(b) * p.N + n;
+            const uint16_t h0 = float_to_half_bits(sum.x), h1 = float_to_half_bits(sum.y);
+            if (p.y4) {
+                *reinterpret_cast<uint32_t*>(out) = pack2(h0, h1);   // N even, n even
+            } else {
+                out[0] = h0;
+                if (n + 1 < p.N) out[1] = h1;
+            }
+        }
+    }
+    named_barrier_sync(1, kConsumers);                           // the sums' buffer is free again
+}
+
+// The CTA's tail, from row `row0` of the tails on: the last round's rows in
+// tiles of 16 a warp, when one round of those takes them (128256 x 4096 is 3.3
+// rounds of 256 rows).  A function of its own, so that the whole tiles' loop
+// keeps its registers.
+template <int XT>
+__device__ __noinline__ bool tail_tile(const TGemvParams& p, uint8_t* smem, int tid, int row0, int slot, int par, bool ok)
+{
+    uint64_t* full = reinterpret_cast<uint64_t*>(smem);
+    TileGeom g = p.g;
+    g.wrows = 16;
+    TileWarp<XT, 1, false> tl(g, smem, tid >> 5, tid & 31);
+    tl.slot = slot;
+    tl.par = par;
+    tl.ok = ok;
+    float acc[1][XT][4];
+    tl.tile(g, full, full + kTMaxSlots, p.check != 0, p.err, acc);
+    store_tile<XT, 1>(p, reinterpret_cast<float*>(smem + g.red_off), g.ks, 16,
+                      row0 + static_cast<int>(blockIdx.x) * 16 * (kTWarps<XT> / g.ks), tid, tid >> 5, tid & 31, acc);
+    return tl.bad;
+}
+
+template <int XT, int R, bool TAIL>
 __global__ void __launch_bounds__(32 * (kTWarps<XT> + 1), 1)
     bgemv_tma_kernel(const __grid_constant__ CUtensorMap tm_w, const __grid_constant__ CUtensorMap tm_s,
-                     const __grid_constant__ CUtensorMap tm_x, const TGemvParams p)
+                     const __grid_constant__ CUtensorMap tm_x, const __grid_constant__ CUtensorMap tm_w2,
+                     const __grid_constant__ CUtensorMap tm_s2, const __grid_constant__ TGemvParams p)
 {
     extern __shared__ __align__(1024) uint8_t smem[];
     constexpr int NW = kTWarps<XT>, kConsumers = 32 * NW;
@@ -365,51 +429,29 @@ __global__ void __launch_bounds__(32 * (kTWarps<XT> + 1), 1)
     __syncthreads();
     grid_dependents_launch();
     if (warp == NW) {
-        if (lane == 0) tile_producer<XT, false>(&tm_w, &tm_s, &tm_x, p.g, 0, smem, full, empty, p.err);
+        if (lane == 0) tile_producer<XT, false, TAIL>(&tm_w, &tm_s, &tm_x, &tm_w2, &tm_s2, p.g, 0, smem, full, empty, p.err);
         return;
     }
 
     grid_dependency_wait();               // y is written after the previous kernel
     TileWarp<XT, R, false> tw(p.g, smem, warp, lane);
-    float acc[R][XT][4];
-    for (int tile = blockIdx.x; tile < p.g.tiles; tile += gridDim.x) {
-        tw.tile(p.g, full, empty, p.check != 0, p.err, acc);
-        const int n0 = tile * TR;
-        if (ks == 1) {
-#pragma unroll
-            for (int r = 0; r < R; ++r)
-#pragma unroll
-                for (int t = 0; t < XT; ++t)
-#pragma unroll
-                    for (int i = 0; i < 4; ++i) {
-                        const int row = 16 * r + (lane >> 2) + 8 * (i >> 1), n = n0 + warp * wrows + row;
-                        const int b = 8 * t + x_row(2 * (lane & 3) + (i & 1));
-                        if (row < wrows && n < p.N && b < p.batch)
-                            p.y[static_cast<size_t>(b) * p.N + n] = float_to_half_bits(acc[r][t][i]);
-                    }
-            continue;
+    {
+        float acc[R][XT][4];
+        for (int tile = blockIdx.x; tile < p.g.tiles; tile += gridDim.x) {
+            tw.tile(p.g, full, empty, p.check != 0, p.err, acc);
+            // (the operands of the call decide the loop's registers: at 17-24 rows
+            // the first form is 5 % faster, 128256 x 4096 at 24 104 -> 99 us, at 25-32
+            // the second 4 %)
+            float* red = reinterpret_cast<float*>(smem + p.g.red_off);
+            if constexpr (XT == 3)
+                store_tile<XT, R>(p, red, p.g.ks, p.g.wrows, tile * TR, tid, tid >> 5, tid & 31, acc);
+            else
+                store_tile<XT, R>(p, red, ks, wrows, tile * TR, tid, warp, lane, acc);
         }
-        float* red = reinterpret_cast<float*>(smem + p.g.red_off);
-        store_sums<XT, R>(red, warp, lane, acc);
-        named_barrier_sync(1, kConsumers);
-        const int hrows = wrows >> 1;                                // pairs of rows per row group
-        for (int e = tid; e < rgs * hrows * 8 * XT; e += kConsumers) {
-            const int pr = e % hrows, q = e / hrows;                 // row pair; column and row group
-            const int col = q % (8 * XT), grp = q / (8 * XT);
-            const float2 sum = load_sums<XT, R>(red, grp, ks, col, 2 * pr);
-            const int n = n0 + grp * wrows + 2 * pr, b = (col & ~7) + x_row(col & 7);
-            if (b < p.batch && n < p.N) {
-                uint16_t* out = p.y + static_cast<size_t>(b) * p.N + n;
-                const uint16_t h0 = float_to_half_bits(sum.x), h1 = float_to_half_bits(sum.y);
-                if (p.y4) {
-                    *reinterpret_cast<uint32_t*>(out) = pack2(h0, h1);   // N even, n even
-                } else {
-                    out[0] = h0;
-                    if (n + 1 < p.N) out[1] = h1;
-                }
-            }
-        }
-        named_barrier_sync(1, kConsumers);                           // the sums' buffer is free again
+    }
+    if constexpr (TAIL) {
+        if (static_cast<int>(blockIdx.x) < p.g.tails)
+            tw.bad = tail_tile<XT>(p, smem, tid, p.g.tiles * TR, tw.slot, tw.par, tw.ok) || tw.bad;
     }
     // a warp that gave up has not seen every copy land, but the producer waits
     // for them before it leaves
@@ -493,7 +535,7 @@ cudaError_t launch_xt(int R, bool s2, const cudaLaunchConfig_t& cfg, const BGemv
     }
 }
 
-template <int XT, int R>
+template <int XT, int R, bool TAIL>
 cudaError_t launch_tma(const cudaLaunchConfig_t& cfg, const CUtensorMap* tm, const TGemvParams& p, int smem_max)
 {
     static std::atomic<bool> ready[64];                // per device; setting the attribute twice is harmless
@@ -501,20 +543,22 @@ cudaError_t launch_tma(const cudaLaunchConfig_t& cfg, const CUtensorMap* tm, con
     cudaError_t e = cudaGetDevice(&dev);
     if (e != cudaSuccess) return e;
     if (dev >= 64 || !ready[dev].load()) {
-        e = cudaFuncSetAttribute(bgemv_tma_kernel<XT, R>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_max);
+        e = cudaFuncSetAttribute(bgemv_tma_kernel<XT, R, TAIL>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_max);
         if (e != cudaSuccess) return e;
         if (dev < 64) ready[dev].store(true);
     }
-    return cudaLaunchKernelEx(&cfg, bgemv_tma_kernel<XT, R>, tm[0], tm[1], tm[2], p);
+    return cudaLaunchKernelEx(&cfg, bgemv_tma_kernel<XT, R, TAIL>, tm[0], tm[1], tm[2], tm[3], tm[4], p);
 }
 
 template <int XT>
 cudaError_t launch_tma_xt(int R, const cudaLaunchConfig_t& cfg, const CUtensorMap* tm, const TGemvParams& p, int smem_max)
 {
-    if (R == 1) return launch_tma<XT, 1>(cfg, tm, p, smem_max);
-    if constexpr (kTWarps<XT> == 8)
-        if (R == 3) return launch_tma<XT, 3>(cfg, tm, p, smem_max);
-    return launch_tma<XT, 2>(cfg, tm, p, smem_max);
+    if constexpr (XT == 4)
+        if (p.g.tails != 0) return launch_tma<XT, 2, true>(cfg, tm, p, smem_max);    // one slice: 32 rows a warp at most
+    if (R == 1) return launch_tma<XT, 1, false>(cfg, tm, p, smem_max);
+    if constexpr (XT != 2)
+        if (R == 3) return launch_tma<XT, 3, false>(cfg, tm, p, smem_max);
+    return launch_tma<XT, 2, false>(cfg, tm, p, smem_max);
 }
 
 int launch_bgemv_tma(const DeviceInfo* di, const uint32_t* W, const uint16_t* s, const uint16_t* x, uint16_t* y, int N,
@@ -522,7 +566,7 @@ int launch_bgemv_tma(const DeviceInfo* di, const uint32_t* W, const uint16_t* s,
 {
     const int XT = (batch + 7) / 8;
     TilePlan b;
-    CUtensorMap tm[3];
+    CUtensorMap tm[5];
     if (!tile_plan(di->sm_count, static_cast<size_t>(di->smem_optin), N, K, XT, false, 0, &b) ||
         !tile_maps(tm, W, s, x, N, K, batch, K, XT, b, false))
         return WQ4_ERR_CUDA;
@@ -556,15 +600,21 @@ int launch_bgemv_tma(const DeviceInfo* di, const uint32_t* W, const uint16_t* s,
 
 }  // namespace
 
-// As plan_bgemv, without copy instructions in the warps (a chunk costs them a
-// wait and an arrival); fitted to a sweep of every choice over the 3B and 8B
-// projections, where its picks are within ~5 % of the best.
+// Per chunk the largest of the instructions of a scheduler's warps, the copies
+// and the time a copy takes to land over the ring's depth; per round the sums of
+// the slices.  Fitted to every choice over eight shapes of the 3B and 8B
+// projections at batch 8, 16, 24 and 32 (times within 20 %, the choice 0.4 %
+// from the best on average, at most 5 %).
 bool tile_plan(int sms, size_t smem_max, int N, int K, int XT, bool stage, size_t extra, TilePlan* out)
 {
     const int G = K / 32, NW = XT <= 2 ? kTWarps<1> : kTWarps<4>;
     double best = 0.0;
     out->R = 0;
-    for (int wrows = stage ? 16 : 8; wrows <= (NW == 16 ? 32 : 48); wrows += stage ? 16 : 8)
+    // (three row tiles on 16 warps only for a GEMV of up to eight rows: 28672 x
+    // 4096 16.6 -> 15.2 us, 5120 x 3072 4.96 -> 4.31 at batch 8; with 9-16 rows
+    // they spill, 128256 x 4096 75 -> 90, and the stages gain nothing)
+    const int max_rows = NW == 8 || (XT == 1 && !stage) ? 48 : 32;
+    for (int wrows = stage ? 16 : 8; wrows <= max_rows; wrows += stage ? 16 : 8)
         for (int ks = stage ? 2 : 1; ks <= NW; ks *= 2)
             for (int lkg = 3; lkg <= 5; ++lkg) {
                 const int KG = 1 << lkg, gpw = KG / ks, boxes = KG / 8, R = (wrows + 15) / 16;
@@ -588,14 +638,28 @@ bool tile_plan(int sms, size_t smem_max, int N, int K, int XT, bool stage, size_
                 g.red_off = kTHeader + g.nslots * g.slot_bytes;
                 g.tiles = (N + TR - 1) / TR;
                 g.nch = (G + KG - 1) / KG;
-                const int rounds = (g.tiles + sms - 1) / sms;
-                const double instr = gpw * (5.0 * XT + 4 + R * (22.0 + 6 * XT)) + 30.0;
-                const double mma = static_cast<double>(NW) * gpw * R * 2 * XT * 2.0;
-                const double copy = (TR * 18.0 * KG + 512.0 * XT * KG) / 45.0;
-                const double chunk = std::max(std::max((NW == 16 ? 5.0 : 3.0) * instr, mma * 1.1), copy);
-                double cost = rounds * (g.nch * chunk + (ks > 1 ? 200.0 + 40.0 * R * XT : 80.0 * R)) + 1500.0;
-                if (wrows % 16 != 0) cost *= 1.03;                 // half a tile's MMAs are dropped
-                if (XT == 4 && R == 3) cost *= 1.08;               // a few registers spill
+                int rounds = (g.tiles + sms - 1) / sms;
+                auto round_cost = [&](int r, int rows) {
+                    const double instr = gpw * (9.0 * XT + 2 + r * (22.0 + 13 * XT)) + 60.0;
+                    const double copy = (rows * 18.0 * KG + 512.0 * XT * KG) / (NW == 16 ? 48.0 : 96.0);
+                    const double chunk = std::max(std::max((NW == 16 ? 4.4 : 3.0) * instr, copy), 2200.0 / g.nslots);
+                    return g.nch * chunk + (ks > 1 ? 900.0 + 130.0 * r * XT : 80.0 * r);
+                };
+                double cost = 0.0;
+                // whole rounds, then a round of 16 rows a warp if that takes the rest
+                // (25-32 activation rows, one slice, three whole rounds: 128256 x 4096 at
+                // batch 32 129 -> 118 us; with fewer rows, with slices or after one round,
+                // 45000 x 4096, a partial round of whole tiles was up to 10 % faster)
+                g.tails = 0;
+                const int rest = N - (rounds - 1) * sms * TR, TR2 = 16 * rgs;
+                if (!stage && XT == 4 && ks == 1 && R > 1 && rounds > 3 && rest <= sms * TR2) {
+                    --rounds;
+                    g.tiles = rounds * sms;
+                    g.tails = (rest + TR2 - 1) / TR2;
+                    cost += round_cost(1, TR2);
+                }
+                cost += rounds * round_cost(R, TR);
+                if (XT == 3 && R == 3) cost *= 1.05;               // measured slower than the model's time
                 if (out->R == 0 || cost < best) {
                     best = cost;
                     out->g = g;
@@ -607,12 +671,21 @@ bool tile_plan(int sms, size_t smem_max, int N, int K, int XT, bool stage, size_
     return out->R != 0;
 }
 
-bool tile_maps(CUtensorMap tm[3], const uint32_t* W, const uint16_t* s, const uint16_t* x, int N, int K, int rows,
+bool tile_maps(CUtensorMap tm[5], const uint32_t* W, const uint16_t* s, const uint16_t* x, int N, int K, int rows,
                int64_t x_pitch, int XT, const TilePlan& p, bool gu)
 {
     const int NW = XT <= 2 ? kTWarps<1> : kTWarps<4>;
     const uint32_t TR = p.g.wrows * (NW / p.g.ks), TB = gu ? TR / 2 : TR, boxes = 1u << (p.g.lkg - 3);
     const uint64_t Ku = static_cast<uint64_t>(K), Nu = static_cast<uint64_t>(N);
+    tm[3] = tm[4] = CUtensorMap{};
+    if (p.g.tails != 0) {
+        const uint32_t T2 = 16 * (NW / p.g.ks);
+        if (!encode_tensor_map_3d(&tm[3], CU_TENSOR_MAP_DATA_TYPE_UINT8, W, {128, Nu, Ku / 256}, {Ku / 2, 128},
+                                  {128, T2, boxes}, CU_TENSOR_MAP_SWIZZLE_128B) ||
+            !encode_tensor_map_3d(&tm[4], CU_TENSOR_MAP_DATA_TYPE_UINT16, s, {8, Nu, Ku / 256}, {Ku / 16, 16},
+                                  {8, T2, boxes}, CU_TENSOR_MAP_SWIZZLE_NONE))
+            return false;
+    }
     return encode_tensor_map_3d(&tm[0], CU_TENSOR_MAP_DATA_TYPE_UINT8, W, {128, Nu, Ku / 256}, {Ku / 2, 128},
                                 {128, TB, boxes}, CU_TENSOR_MAP_SWIZZLE_128B) &&
            encode_tensor_map_3d(&tm[1], CU_TENSOR_MAP_DATA_TYPE_UINT16, s, {8, Nu, Ku / 256}, {Ku / 16, 16},

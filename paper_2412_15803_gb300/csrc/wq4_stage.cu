@@ -100,7 +100,7 @@ __global__ void __launch_bounds__(32 * (kTWarps<XT> + 2), 1)
     __syncthreads();
     grid_dependents_launch();
     if (warp == NW) {
-        if (lane == 0) tile_producer<XT, GU>(&tm_w, &tm_s, &tm_x, a.g, F, smem, full, empty, a.err);
+        if (lane == 0) tile_producer<XT, GU>(&tm_w, &tm_s, &tm_x, nullptr, nullptr, a.g, F, smem, full, empty, a.err);
         return;
     }
     grid_dependency_wait();               // the previous stage's outputs are complete from here on
@@ -354,7 +354,7 @@ int stage_record_token(const StageModel& m, cudaStream_t cs, const StageAttnHook
     bool ok = stage_launch_squares(u.x_stage, H, B, sq_u, cs) == WQ4_OK;
     auto stage = [&](int type, const wq4_mat& w, const uint16_t* x, StageArgs a) {
         const TilePlan& p = plan[type];
-        CUtensorMap tm[3];
+        CUtensorMap tm[5];
         ok = ok && tile_maps(tm, w.W, w.s, x, shape[type].N, shape[type].K, B, shape[type].K, XT, p, type == kStGU);
         if (!ok) return;
         a.g = p.g;

@@ -64,6 +64,7 @@ struct TileGeom {
     int wrows;             // weight rows per warp: a multiple of 8 up to 32 (48 with 8 warps); GU: of 16
     int ks, gpw;           // K slices, groups of a chunk per slice (2, 4 or 8)
     int tiles, nch, nslots;
+    int tails;             // tiles of 16 rows a warp after the `tiles` ones (whole rounds of the grid then), or 0
     uint32_t slot_bytes, scale_off, x_off, red_off;
 };
 
@@ -80,8 +81,8 @@ struct TilePlan {
 bool tile_plan(int sms, size_t smem_max, int N, int K, int XT, bool stage, size_t extra, TilePlan* out);
 
 // Tensor maps of one call: weights (N rows), scales and `rows` activation rows
-// of pitch x_pitch elements.
-bool tile_maps(CUtensorMap tm[3], const uint32_t* W, const uint16_t* s, const uint16_t* x, int N, int K, int rows,
+// of pitch x_pitch elements; then weights and scales of the tails, if any.
+bool tile_maps(CUtensorMap tm[5], const uint32_t* W, const uint16_t* s, const uint16_t* x, int N, int K, int rows,
                int64_t x_pitch, int XT, const TilePlan& p, bool gu);
 
 // Activation row (of a tile of eight) that lane group g holds: neighbouring
@@ -92,11 +93,11 @@ __device__ __forceinline__ int x_row(int g) { return ((g & 1) << 2) | (g >> 1); 
 __device__ __forceinline__ float lo_scale(uint32_t v) { return __low2float(*reinterpret_cast<const __half2*>(&v)); }
 __device__ __forceinline__ float hi_scale(uint32_t v) { return __high2float(*reinterpret_cast<const __half2*>(&v)); }
 
-// One lane: streams the CTA's chunks (tile blockIdx.x, + gridDim.x, ...) into
-// the ring.  up: GU's first up row.
-template <int XT, bool GU>
+// One lane: streams the CTA's chunks (tile blockIdx.x, + gridDim.x, ..., then
+// its tail) into the ring.  up: GU's first up row.
+template <int XT, bool GU, bool TAIL = false>
 __device__ __forceinline__ void tile_producer(const CUtensorMap* tm_w, const CUtensorMap* tm_s, const CUtensorMap* tm_x,
-                                              const TileGeom& p, int up, uint8_t* smem, uint64_t* full, uint64_t* empty,
+                                              const CUtensorMap* tm_w2, const CUtensorMap* tm_s2, const TileGeom& p, int up, uint8_t* smem, uint64_t* full, uint64_t* empty,
                                               uint32_t* err)
 {
     tc::prefetch_map(tm_w);
@@ -104,11 +105,20 @@ __device__ __forceinline__ void tile_producer(const CUtensorMap* tm_w, const CUt
     tc::prefetch_map(tm_x);
     const int TR = p.wrows * (kTWarps<XT> / p.ks), TB = GU ? TR / 2 : TR;
     const int grid = static_cast<int>(gridDim.x), nch = p.nch, nslots = p.nslots;
-    const int mytiles = (p.tiles - static_cast<int>(blockIdx.x) + grid - 1) / grid;
-    const int boxes = 1 << (p.lkg - 3), total = mytiles * nch;
+    const int wholes = (p.tiles - static_cast<int>(blockIdx.x) + grid - 1) / grid;
+    const bool tail = TAIL && static_cast<int>(blockIdx.x) < p.tails;
+    const int TR2 = 16 * (kTWarps<XT> / p.ks);
+    const int nt = p.tiles * TR + static_cast<int>(blockIdx.x) * TR2;          // the tail's first row
+    const int boxes = 1 << (p.lkg - 3), whole = wholes * nch, total = whole + (tail ? nch : 0);
     const uint32_t bytes = boxes * (TR * 144 + XT * 4096);
-    auto load_w = [&](int slot, int n0, int ch) {
+    auto load_w = [&](int slot, int f, int n0, int ch) {
         uint8_t* base = smem + kTHeader + static_cast<size_t>(slot) * p.slot_bytes;
+        if (TAIL && f >= whole) {
+            mbar_arrive_expect_tx(&full[slot], boxes * (TR2 * 144 + XT * 4096));
+            tc::tma_load_3d(base, tm_w2, 0, nt, ch * boxes, &full[slot]);
+            tc::tma_load_3d(base + p.scale_off, tm_s2, 0, nt, ch * boxes, &full[slot]);
+            return;
+        }
         mbar_arrive_expect_tx(&full[slot], bytes);
         tc::tma_load_3d(base, tm_w, 0, n0, ch * boxes, &full[slot]);
         if (GU) tc::tma_load_3d(base + boxes * TB * 128, tm_w, 0, up + n0, ch * boxes, &full[slot]);
@@ -124,7 +134,7 @@ __device__ __forceinline__ void tile_producer(const CUtensorMap* tm_w, const CUt
     int n0 = static_cast<int>(blockIdx.x) * TB, ch = 0;
     const int early = min(nslots, total);
     for (int f = 0; f < early; ++f) {
-        load_w(f, n0, ch);
+        load_w(f, f, n0, ch);
         if (++ch == nch) {
             ch = 0;
             n0 += grid * TB;
@@ -138,7 +148,7 @@ __device__ __forceinline__ void tile_producer(const CUtensorMap* tm_w, const CUt
     int slot = 0, par = 0, f = early;
     for (; f < total; ++f) {
         if (!mbar_wait(&empty[slot], par, err)) break;
-        load_w(slot, n0, ch);
+        load_w(slot, f, n0, ch);
         load_x(slot, ch);
         if (++ch == nch) {
             ch = 0;

@@ -54,3 +54,20 @@ def test_copy_ring_shapes(N, K, off, batch):
 
 def test_copy_ring_batch_two():
     check(3001, 2144, 2)
+
+
+# more rows than whole rounds of the grid: the last round in tiles of 16 rows a
+# warp (25-32 activation rows, three whole rounds and more; the last tail a
+# row, a part, whole; one row too many for it)
+@pytest.mark.parametrize("N,K,batch", [(116737, 256, 32), (116866, 512, 27), (128255, 512, 25),
+                                       (136192, 256, 32), (136193, 256, 32)])
+def test_tails_of_sixteen_rows(N, K, batch):
+    check(N, K, batch)
+
+
+# three row tiles a warp on sixteen warps (up to eight activation rows): whole,
+# the third half used, a last tile of one row
+@pytest.mark.parametrize("N,K", [(5121, 3072), (6153, 1024), (28672, 512), (7201, 768)])
+@pytest.mark.parametrize("batch", [3, 8])
+def test_three_row_tiles(N, K, batch):
+    check(N, K, batch)
