@@ -575,7 +575,7 @@ __device__ __forceinline__ float warp_allsum(float v)
 // time the queries have.  (Read by the warps themselves once the queries were
 // in, they cost ~5 us of latency a layer: 3B, 4096 tokens, 1212 -> 1082 us a
 // token; the flagged exchange between the ranges 1082 -> 1017, the combine of
-// four heads at a time 1017 -> 981.)  The new token's key and value are polled with the queries.  The
+// four heads at a time 1017 -> 979.)  The new token's key and value are polled with the queries.  The
 // warps take blocks of 16 tokens in ring order, keeping a running maximum, sum
 // and weighted value sum per query head of the group; they are combined in
 // shared memory in warp order (one head at a time).  With one range the unit
@@ -632,31 +632,31 @@ __device__ __forceinline__ void attn_copy(const ChainParamsA& p, int l, const At
     const int P = p.P, p0 = ta / P;
     const int32_t* pt = kv.pt + static_cast<size_t>(a.b) * kv.pt_stride + p0;
     constexpr int kRuns = kAttnMaxChunk / 16 + 1;               // pages of at least 16 tokens
-    int pg[kRuns];
     uint32_t bytes = 0;
-#pragma unroll
-    for (int i = 0; i < kRuns; ++i) pg[i] = (p0 + i) * P < tb ? __ldg(pt + i) : -1;
+    uint32_t good = 0;
 #pragma unroll
     for (int i = 0; i < kRuns; ++i) {
         const int x0 = max(ta, (p0 + i) * P), x1 = min(tb, (p0 + i + 1) * P);
-        if (x0 >= x1) continue;
-        if (pg[i] >= 0 && pg[i] < kv.num_pages) {
-            bytes += static_cast<uint32_t>(x1 - x0) * (4 * kAttnD);
-        } else {
-            atomicOr(p.err, kErrPageId);
-            pg[i] = -1;
-            uint4* kz = reinterpret_cast<uint4*>(dst + (x0 - ta) * (2 * kAttnD));
-            uint4* vz = reinterpret_cast<uint4*>(dst + (ct + x0 - ta) * (2 * kAttnD));
-            for (int e = 0; e < (x1 - x0) * (2 * kAttnD / 16); ++e) kz[e] = vz[e] = make_uint4(0u, 0u, 0u, 0u);
-            asm volatile("fence.proxy.async.shared::cta;" ::: "memory");   // before a later copy into the slot
+        if (x0 < x1) {
+            const int page = __ldg(pt + i);
+            if (page >= 0 && page < kv.num_pages) {
+                bytes += static_cast<uint32_t>(x1 - x0) * (4 * kAttnD);
+                good |= 1u << i;
+            } else {
+                atomicOr(p.err, kErrPageId);
+                uint4* kz = reinterpret_cast<uint4*>(dst + (x0 - ta) * (2 * kAttnD));
+                uint4* vz = reinterpret_cast<uint4*>(dst + (ct + x0 - ta) * (2 * kAttnD));
+                for (int e = 0; e < (x1 - x0) * (2 * kAttnD / 16); ++e) kz[e] = vz[e] = make_uint4(0u, 0u, 0u, 0u);
+                asm volatile("fence.proxy.async.shared::cta;" ::: "memory");   // before a later copy into the slot
+            }
         }
     }
     mbar_arrive_expect_tx(fb, bytes);
-#pragma unroll
+#pragma unroll 1
     for (int i = 0; i < kRuns; ++i) {
+        if (!((good >> i) & 1u)) continue;
         const int x0 = max(ta, (p0 + i) * P), x1 = min(tb, (p0 + i + 1) * P);
-        if (x0 >= x1 || pg[i] < 0) continue;
-        const size_t row = (static_cast<size_t>(pg[i]) * p.Hkv + a.h) * P + (x0 - (p0 + i) * P);
+        const size_t row = (static_cast<size_t>(__ldg(pt + i)) * p.Hkv + a.h) * P + (x0 - (p0 + i) * P);
         const uint32_t n = static_cast<uint32_t>(x1 - x0) * (2 * kAttnD);
         bulk_g2s(dst + (x0 - ta) * (2 * kAttnD), kv.k + row * kAttnD, n, fb, pol);
         bulk_g2s(dst + (ct + x0 - ta) * (2 * kAttnD), kv.v + row * kAttnD, n, fb, pol);
@@ -916,26 +916,36 @@ __device__ __forceinline__ int attention_phase(const ChainParamsA& p, int l, uin
     return chunks;
 }
 
-template <int B, int NW>
+template <int B, int NW, int ATT>
 __device__ __forceinline__ int attention_dispatch(const ChainParamsA& p, int l, uint32_t epoch, float* scratch,
                                                   const int* pos_sh, uint8_t* smem, uint64_t* full,
                                                   uint64_t* empty, uint8_t* slots, int ord0)
 {
-    switch (p.G) {
-        case 1: return attention_phase<B, NW, 1>(p, l, epoch, scratch, pos_sh, smem, full, empty, slots, ord0);
-        case 2: return attention_phase<B, NW, 2>(p, l, epoch, scratch, pos_sh, smem, full, empty, slots, ord0);
-        case 3: return attention_phase<B, NW, 3>(p, l, epoch, scratch, pos_sh, smem, full, empty, slots, ord0);
-        case 4: return attention_phase<B, NW, 4>(p, l, epoch, scratch, pos_sh, smem, full, empty, slots, ord0);
-        case 5: return attention_phase<B, NW, 5>(p, l, epoch, scratch, pos_sh, smem, full, empty, slots, ord0);
-        case 6: return attention_phase<B, NW, 6>(p, l, epoch, scratch, pos_sh, smem, full, empty, slots, ord0);
-        case 7: return attention_phase<B, NW, 7>(p, l, epoch, scratch, pos_sh, smem, full, empty, slots, ord0);
-        default: return attention_phase<B, NW, 8>(p, l, epoch, scratch, pos_sh, smem, full, empty, slots, ord0);
+    if constexpr (ATT == 1) {
+        switch (p.G) {
+            case 1: return attention_phase<B, NW, 1>(p, l, epoch, scratch, pos_sh, smem, full, empty, slots, ord0);
+            case 2: return attention_phase<B, NW, 2>(p, l, epoch, scratch, pos_sh, smem, full, empty, slots, ord0);
+            case 3: return attention_phase<B, NW, 3>(p, l, epoch, scratch, pos_sh, smem, full, empty, slots, ord0);
+            default: return attention_phase<B, NW, 4>(p, l, epoch, scratch, pos_sh, smem, full, empty, slots, ord0);
+        }
+    } else {
+        switch (p.G) {
+            case 5: return attention_phase<B, NW, 5>(p, l, epoch, scratch, pos_sh, smem, full, empty, slots, ord0);
+            case 6: return attention_phase<B, NW, 6>(p, l, epoch, scratch, pos_sh, smem, full, empty, slots, ord0);
+            case 7: return attention_phase<B, NW, 7>(p, l, epoch, scratch, pos_sh, smem, full, empty, slots, ord0);
+            default: return attention_phase<B, NW, 8>(p, l, epoch, scratch, pos_sh, smem, full, empty, slots, ord0);
+        }
     }
 }
 
-template <int B, int NW, bool ATT>
+// ATT: 0 the chain, 1 and 2 the decode step with groups of up to four and of
+// five to eight query heads per kv head.  The larger groups' attention spills
+// registers, also around the stages, where a reload costs a miss (the ring
+// leaves hardly any L1): with every group in one kernel, 3B at batch 1 and 4096
+// tokens took 979 us a token, apart 923; 8B 1613 and 1502.
+template <int B, int NW, int ATT>
 __global__ void __launch_bounds__((NW + 1) * 32, 1)
-    chain_kernel(const __grid_constant__ typename std::conditional<ATT, ChainParamsA, ChainParams>::type p)
+    chain_kernel(const __grid_constant__ typename std::conditional<ATT != 0, ChainParamsA, ChainParams>::type p)
 {
     extern __shared__ __align__(1024) uint8_t smem[];
     uint64_t* full = reinterpret_cast<uint64_t*>(smem);
@@ -970,7 +980,7 @@ __global__ void __launch_bounds__((NW + 1) * 32, 1)
     // row, fp64) and the rows' positions (-1 for an invalid one), after the
     // ring; their addresses are recomputed where used (no registers held)
     constexpr uint32_t kPosOff = B * (kAttnD / 2) * sizeof(double2);
-    if constexpr (ATT) {
+    if constexpr (ATT != 0) {
         rope_table<B>(p, reinterpret_cast<double2*>(smem + p.rope_off));
         int* pos_sh = reinterpret_cast<int*>(smem + p.rope_off + kPosOff);
         if (threadIdx.x < B) {
@@ -1013,7 +1023,7 @@ __global__ void __launch_bounds__((NW + 1) * 32, 1)
                 const StageInfo in = info[g.type];
                 const int w0 = in.w0, w1 = in.w0 + in.nwords, wps = in.wps;
                 const int wpr = g.K >> 3, gpr = g.K >> 5;
-                if constexpr (ATT) {
+                if constexpr (ATT != 0) {
                     // the cached keys and values of this CTA's attention ranges
                     if (g.type == kO) {
                         const int* pos_sh = reinterpret_cast<const int*>(smem + p.rope_off + kPosOff);
@@ -1075,11 +1085,11 @@ __global__ void __launch_bounds__((NW + 1) * 32, 1)
         for (int st = 0; st < nstages; ++st) {
             const Stage g = stage_at(p, st);
             const StageInfo& in = info[g.type];
-            if constexpr (ATT) {
+            if constexpr (ATT != 0) {
                 // every CTA takes its splits of the layer's attention, words or not
                 if (g.type == kO) {
                     int* pos_sh = reinterpret_cast<int*>(smem + p.rope_off + kPosOff);
-                    cord0 += attention_dispatch<B, NW>(p, g.layer, epoch, reinterpret_cast<float*>(xs), pos_sh,
+                    cord0 += attention_dispatch<B, NW, ATT>(p, g.layer, epoch, reinterpret_cast<float*>(xs), pos_sh,
                                                        smem, full, empty, slots, cord0);
                 }
             }
@@ -1100,7 +1110,7 @@ __global__ void __launch_bounds__((NW + 1) * 32, 1)
                 const bool r1 = (blockIdx.x & 1) != 0;   // this CTA's replica
                 if (g.type == kQKV) ll = p.llX + (r1 ? p.rep.X : 0u) + static_cast<size_t>(l) * B * (H / 2);
                 else if (g.type == kO) {
-                    if constexpr (ATT) ll = p.llAt + (r1 ? p.repAt : 0u) + static_cast<size_t>(l) * B * (H / 2);
+                    if constexpr (ATT != 0) ll = p.llAt + (r1 ? p.repAt : 0u) + static_cast<size_t>(l) * B * (H / 2);
                     else ll = p.llA + (r1 ? p.rep.A : 0u) + static_cast<size_t>(l) * B * (H / 2);
                 }
                 else if (g.type == kGU) ll = p.llX1 + (r1 ? p.rep.X1 : 0u) + static_cast<size_t>(l) * B * (H / 2);
@@ -1353,7 +1363,7 @@ __global__ void __launch_bounds__((NW + 1) * 32, 1)
 #pragma unroll
                 for (int bb = 0; bb < B; ++bb) {
                     if (bb != b) continue;
-                    if constexpr (ATT) {
+                    if constexpr (ATT != 0) {
                         if (g.type == kQKV) {
                             const double2* rope = reinterpret_cast<const double2*>(smem + p.rope_off);
                             const int* pos_sh = reinterpret_cast<const int*>(smem + p.rope_off + kPosOff);
@@ -1653,7 +1663,10 @@ bool mat_ok(const wq4_mat& m)
     return m.W && m.s && aligned(m.W, 16) && aligned(m.s, 16);
 }
 
-template <int B, bool ATT>
+// The decode step's kernel (chain_kernel's ATT).
+int attn_kernel(const Dims& d) { return d.nq / d.Hkv <= 4 ? 1 : 2; }
+
+template <int B, int ATT>
 cudaError_t set_chain_attr(int smem)
 {
     return cudaFuncSetAttribute(chain_kernel<B, kChainWarps, ATT>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
@@ -2057,11 +2070,13 @@ int build_plan(const wq4_layer_table* t, const wq4_decode_attn* a, Plan* pl, cud
     // the device maximum so that no plan's launch depends on which plan was
     // built last.
     cudaError_t e = cudaSuccess;
-    switch (d.B * 2 + (a ? 1 : 0)) {
-        case 2: e = set_chain_attr<1, false>(di->smem_optin); break;
-        case 3: e = set_chain_attr<1, true>(di->smem_optin); break;
-        case 4: e = set_chain_attr<2, false>(di->smem_optin); break;
-        default: e = set_chain_attr<2, true>(di->smem_optin); break;
+    switch (d.B * 3 + (a ? attn_kernel(d) : 0)) {
+        case 3: e = set_chain_attr<1, 0>(di->smem_optin); break;
+        case 4: e = set_chain_attr<1, 1>(di->smem_optin); break;
+        case 5: e = set_chain_attr<1, 2>(di->smem_optin); break;
+        case 6: e = set_chain_attr<2, 0>(di->smem_optin); break;
+        case 7: e = set_chain_attr<2, 1>(di->smem_optin); break;
+        default: e = set_chain_attr<2, 2>(di->smem_optin); break;
     }
     if (e != cudaSuccess) return WQ4_ERR_CUDA;
 
@@ -2178,8 +2193,8 @@ int launch_chain(const Plan& pl, const uint16_t* x, uint16_t* logits, cudaStream
         ChainParams p = {};
         if (fill_chain_params(p, pl, x, logits) != WQ4_OK) return WQ4_ERR_CUDA;
         switch (pl.dims.B) {
-            case 1: e = cudaLaunchKernelEx(&cfg, chain_kernel<1, kChainWarps, false>, p); break;
-            default: e = cudaLaunchKernelEx(&cfg, chain_kernel<2, kChainWarps, false>, p); break;
+            case 1: e = cudaLaunchKernelEx(&cfg, chain_kernel<1, kChainWarps, 0>, p); break;
+            default: e = cudaLaunchKernelEx(&cfg, chain_kernel<2, kChainWarps, 0>, p); break;
         }
     } else {
         ChainParamsA p = {};
@@ -2202,9 +2217,11 @@ int launch_chain(const Plan& pl, const uint16_t* x, uint16_t* logits, cudaStream
         p.apart = reinterpret_cast<uint64_t*>(ws + y.apart);
         fill_inv_freq(pl.theta, p.inv_freq);
         for (int l = 0; l < pl.dims.L; ++l) p.kv[l] = kv_layer(pl.kv[l]);
-        switch (pl.dims.B) {
-            case 1: e = cudaLaunchKernelEx(&cfg, chain_kernel<1, kChainWarps, true>, p); break;
-            default: e = cudaLaunchKernelEx(&cfg, chain_kernel<2, kChainWarps, true>, p); break;
+        switch (pl.dims.B * 3 + attn_kernel(pl.dims)) {
+            case 4: e = cudaLaunchKernelEx(&cfg, chain_kernel<1, kChainWarps, 1>, p); break;
+            case 5: e = cudaLaunchKernelEx(&cfg, chain_kernel<1, kChainWarps, 2>, p); break;
+            case 7: e = cudaLaunchKernelEx(&cfg, chain_kernel<2, kChainWarps, 1>, p); break;
+            default: e = cudaLaunchKernelEx(&cfg, chain_kernel<2, kChainWarps, 2>, p); break;
         }
     }
     return e == cudaSuccess ? WQ4_OK : WQ4_ERR_CUDA;
