@@ -34,6 +34,8 @@
 //    words of its input until every epoch matches.  No grid-wide barrier and
 //    no separate flag round trip: one L2 round trip per stage boundary.
 //    Every poll is bounded in time.
+//  * The decode step's cached keys and values move through the same ring,
+//    between a layer's QKV and O weights (see attention_phase).
 //  * Plain fp16 copies of every stage output are written to the workspace for
 //    inspection.
 #include "wq4_device.cuh"
@@ -1400,9 +1402,9 @@ __global__ void __launch_bounds__((NW + 1) * 32, 1)
 // ------------------------------------------------- graph path (batch 3-32) --
 //
 // For batches beyond what the persistent kernel stages in shared memory, the
-// token runs as a CUDA graph (captured once per plan) of tensor-core stage
-// kernels and per-stage epilogues (wq4_tc.cu); they write the same workspace
-// traces as the persistent kernel.
+// token runs as a CUDA graph (captured once per plan) of stage kernels with
+// fused epilogues (wq4_stage.cu); they write the same workspace traces as the
+// persistent kernel.
 
 // Decode step of the graph path: one block per batch row rotates q and k of
 // layer l's QKV output (the same fp64 rotation as the persistent kernel),

@@ -1,8 +1,9 @@
 // wq4_tc.cuh -- tensor-core (tcgen05) and TMA tensor-copy building blocks
 // for sm_103a: tensor-memory allocation, register <-> tensor-memory moves,
 // the kind::f16 MMA with its A operand in tensor memory and B in shared
-// memory (128-byte swizzled, K-major), commits to mbarriers, and 2-D tensor
-// copies.  All inline PTX; used by the batched stage kernels.
+// memory (128-byte swizzled, K-major), commits to mbarriers, and 2-D and
+// 3-D tensor copies.  All inline PTX: the GEMM uses all of it, the batched GEMV,
+// the stages and the attention the tensor copies.
 #pragma once
 
 #include <cstdint>
@@ -12,12 +13,6 @@
 
 namespace wq4 {
 namespace tc {
-
-// Tensor-memory address: lane in bits [16, 32), column in bits [0, 16).
-__device__ __forceinline__ uint32_t tmem_addr(uint32_t base, int lane, int col)
-{
-    return base + (static_cast<uint32_t>(lane) << 16) + static_cast<uint32_t>(col);
-}
 
 // Warp-collective: allocates ncols (power of two, 32..512) columns and writes
 // the base address to *dst (shared memory).
@@ -135,10 +130,6 @@ __device__ __forceinline__ void prefetch_map(const CUtensorMap* map)
 {
     asm volatile("prefetch.tensormap [%0];" ::"l"(map) : "memory");
 }
-
-// Makes this thread's generic-proxy shared-memory writes visible to the async
-// proxy (tensor core, bulk copies).
-__device__ __forceinline__ void fence_proxy_async() { asm volatile("fence.proxy.async.shared::cta;" ::: "memory"); }
 
 __device__ __forceinline__ uint32_t hmul2_u32(uint32_t a, uint32_t b)
 {

@@ -215,7 +215,7 @@ def wq4_chain_plan_destroy(table: wq4_layer_table) -> int:
 
 def wq4_chain_path(table: wq4_layer_table, decode_step: bool = False) -> int:
     """1: the table's cached plan runs the persistent chain kernel; 2: the
-    tensor-core stage graph.  Raises if no plan exists yet."""
+    graph of stage kernels.  Raises if no plan exists yet."""
     rc = load().wq4_chain_path(ctypes.byref(table), 1 if decode_step else 0)
     if rc < 0:
         raise Wq4Error("wq4_chain_path", rc)
