@@ -140,6 +140,21 @@ int wq4_pack_host(const uint8_t* q_host, uint32_t* W_host, int N, int K);
  */
 int wq4_test_gemv_path(int path);
 
+/*
+ * Test hook of the bounded waits for copies into shared memory (no counterpart
+ * in the paper): from now on the named copies are left out of every launch in
+ * this process (WQ4_STALL_NONE, the default: none), so that the waits for them
+ * run out (0.5 s each, all of a block at about the same time).  The kernel
+ * still finishes (its outputs are not valid) and wq4_device_status reports
+ * bit 0.  WQ4_ERR_INVALID for another value.
+ */
+enum wq4_stall {
+    WQ4_STALL_NONE = 0,
+    WQ4_STALL_GEMM_X = 1,     /* wq4_gemm (17 tokens and more): the activations */
+    WQ4_STALL_GEMM_W = 2      /* ... : the weights and scales */
+};
+int wq4_test_copy_stall(int stall);
+
 /* Static, human-readable text of a status code. */
 const char* wq4_status_string(int status);
 

@@ -80,6 +80,7 @@ struct GemmArgs {
     int N, K, M, rtiles, ttiles;
     int split;               // CTAs of a cluster that share a tile's K (1: persistent grid)
     uint32_t* err;
+    int stall;               // test hook: WQ4_STALL_GEMM_X or _W leaves those copies out
 };
 
 __device__ __forceinline__ uint32_t prmt(uint32_t a, uint32_t b, uint32_t sel)
@@ -87,11 +88,6 @@ __device__ __forceinline__ uint32_t prmt(uint32_t a, uint32_t b, uint32_t sel)
     uint32_t d;
     asm("prmt.b32 %0, %1, %2, %3;" : "=r"(d) : "r"(a), "r"(b), "r"(sel));
     return d;
-}
-
-__device__ __forceinline__ bool g_wait(uint64_t* bar, uint32_t parity, uint32_t* err)
-{
-    return mbar_wait(bar, parity, err);
 }
 
 __device__ __forceinline__ void cluster_sync_all()
@@ -157,6 +153,12 @@ __global__ void __launch_bounds__(kGThreads, 1)
     const int u0 = static_cast<int>(blockIdx.x) / split, ustep = static_cast<int>(gridDim.x) / split;
     uint32_t* err = a.err;
 
+    // A wait that gives up (bounded, flagged) leaves invalid outputs, but the
+    // kernel still runs to its end: the dequant, issuer and epilogue warps then
+    // wait no more and go on through every tile with every arrival (a lane or
+    // warp that left its loop alone would leave the others in a warp-wide
+    // instruction, or at a named barrier, for ever), and the producers, who stop,
+    // refill a slot only after its last copy has landed, whoever released it.
     if (threadIdx.x == 0) {
         for (int i = 0; i < XS; ++i) {
             mbar_init(&xfull[i], 1);
@@ -193,10 +195,10 @@ __global__ void __launch_bounds__(kGThreads, 1)
             RingPos<WS> w;
             int n = 0;
             bool ok = true;
-            for (int u = u0; u < tiles && ok; u += ustep) {
+            for (int u = a.stall == WQ4_STALL_GEMM_W ? tiles : u0; u < tiles && ok; u += ustep) {
                 const int n0 = (u / a.ttiles) * 128;
                 for (int k = k0; k < k1; ++k, ++n, w.next()) {
-                    if (n >= WS && !g_wait(&wempty[w.slot], w.par ^ 1u, err)) {
+                    if (n >= WS && (!mbar_wait(&wempty[w.slot], w.par ^ 1u, err) || !mbar_wait(&wfull[w.slot], w.par ^ 1u, err))) {
                         ok = false;
                         break;
                     }
@@ -207,7 +209,7 @@ __global__ void __launch_bounds__(kGThreads, 1)
                 }
             }
             // every copy issued has landed before the CTA's memory goes away
-            for (int i = max(0, n - WS); i < n; ++i) g_wait(&wfull[i % WS], (i / WS) & 1, err);
+            for (int i = max(0, n - WS); i < n; ++i) mbar_wait(&wfull[i % WS], (i / WS) & 1, err);
         }
     } else if (warp == kGXProd) {
         // -------------------------------------------- activation producer
@@ -218,10 +220,10 @@ __global__ void __launch_bounds__(kGThreads, 1)
             int n = 0;
             bool ok = true;
             constexpr int kZ = 2 / C::kXSub;         // boxes of 64 K in a slot
-            for (int u = u0; u < tiles && ok; u += ustep) {
+            for (int u = a.stall == WQ4_STALL_GEMM_X ? tiles : u0; u < tiles && ok; u += ustep) {
                 const int m0 = (u % a.ttiles) * TOK;
                 for (int z = 4 * k0; z < 4 * k1; z += kZ, ++n, x.next()) {
-                    if (n >= XS && !g_wait(&xempty[x.slot], x.par ^ 1u, err)) {
+                    if (n >= XS && (!mbar_wait(&xempty[x.slot], x.par ^ 1u, err) || !mbar_wait(&xfull[x.slot], x.par ^ 1u, err))) {
                         ok = false;
                         break;
                     }
@@ -229,7 +231,7 @@ __global__ void __launch_bounds__(kGThreads, 1)
                     tc::tma_load_3d(xring + static_cast<size_t>(x.slot) * C::kX, &tm_x, 0, m0, z, &xfull[x.slot]);
                 }
             }
-            for (int i = max(0, n - XS); i < n; ++i) g_wait(&xfull[i % XS], (i / XS) & 1, err);
+            for (int i = max(0, n - XS); i < n; ++i) mbar_wait(&xfull[i % XS], (i / XS) & 1, err);
         }
     } else if (warp == kGIssuer) {
         // ---------------------------------------------------- MMA issuer
@@ -243,15 +245,15 @@ __global__ void __launch_bounds__(kGThreads, 1)
         RingPos<XS> x;
         RingPos<NA> ab;
         int dit = 0;
-        bool ok = true;            // after a wait gave up, none is waited for
+        bool ok = true;
         const uint64_t xdesc = tc::sw128_kmajor_desc(smem_addr(xring));
         for (int u = u0; u < tiles; u += ustep, ++dit) {
-            if (dit >= 1 && ok) ok = g_wait(dempty, (dit - 1) & 1, err);
+            if (dit >= 1 && ok) ok = mbar_wait(dempty, (dit - 1) & 1, err);
             for (int it = 2 * k0; it < 2 * k1; ++it) {
-                if (ok) ok = g_wait(&afull[ab.slot], ab.par, err);
+                if (ok) ok = mbar_wait(&afull[ab.slot], ab.par, err);
 #pragma unroll
                 for (int sub = 0; sub < 2; ++sub) {
-                    if (sub < C::kXSub && ok) ok = g_wait(&xfull[x.slot], x.par, err);
+                    if (sub < C::kXSub && ok) ok = mbar_wait(&xfull[x.slot], x.par, err);
                     if (sub == 0) tc::fence_after_sync();
                     const uint64_t xd = xdesc + static_cast<uint64_t>(x.slot) * (C::kX >> 4) +
                                         (C::kXSub == 1 ? sub * (TOK * 128 >> 4) : 0);
@@ -271,7 +273,7 @@ __global__ void __launch_bounds__(kGThreads, 1)
         }
         // all MMAs issued have completed before tensor memory is released
         if (leader) tc::commit(drain);
-        g_wait(drain, 0, err);
+        mbar_wait(drain, 0, err);
     } else if (warp < 4 * kGSets) {
         // ---------------------------------------------------- dequant
         // Item i goes to A buffer i % NA and warp set i % 3, so that several
@@ -283,14 +285,12 @@ __global__ void __launch_bounds__(kGThreads, 1)
         RingPos<NA> ab;
         int i = 0;
         bool ok = true;
-        for (int u = u0; u < tiles && ok; u += ustep) {
-            for (int it = 2 * k0; it < 2 * k1 && ok; ++it, ++i, ab.next()) {
+        for (int u = u0; u < tiles; u += ustep) {
+            for (int it = 2 * k0; it < 2 * k1; ++it, ++i, ab.next()) {
                 if (it > 2 * k0 && (it & 1) == 0) w.next();
                 if (i % kGSets != set) continue;
-                if (!g_wait(&wfull[w.slot], w.par, err) || (i >= NA && !g_wait(&aempty[ab.slot], ab.par ^ 1u, err))) {
-                    ok = false;
-                    break;
-                }
+                if (ok) ok = mbar_wait(&wfull[w.slot], w.par, err) && (i < NA || mbar_wait(&aempty[ab.slot], ab.par ^ 1u, err));
+                __syncwarp();
                 const uint8_t* base = wring + static_cast<size_t>(w.slot) * C::kW;
                 const uint8_t* crow = base + row * 128;
                 const uint2 sv2 = *reinterpret_cast<const uint2*>(base + kGCodes + row * 16 + 8 * (it & 1));
@@ -302,7 +302,8 @@ __global__ void __launch_bounds__(kGThreads, 1)
                     const uint4 cw1 = *reinterpret_cast<const uint4*>(crow + (((j + 1) ^ (row & 7)) << 4));
                     const uint32_t sv = sub ? sv2.y : sv2.x;
                     // (q - 7) s is rounded to fp16 below: a larger scale would overflow
-                    if ((sv & 0x7FFFu) > kMaxFp16ScaleBits || ((sv >> 16) & 0x7FFFu) > kMaxFp16ScaleBits) atomicOr(err, kErrScale);
+                    if ((sv & 0x7FFFu) > kMaxFp16ScaleBits || ((sv >> 16) & 0x7FFFu) > kMaxFp16ScaleBits)
+                        atomicOr(err, ok ? kErrScale : 0u);
                     const uint32_t words[8] = {cw0.x, cw0.y, cw0.z, cw0.w, cw1.x, cw1.y, cw1.z, cw1.w};
                     const uint32_t s0 = prmt(sv, sv, 0x1010u), s1 = prmt(sv, sv, 0x3232u);
                     uint32_t q[32];
@@ -338,9 +339,11 @@ __global__ void __launch_bounds__(kGThreads, 1)
         const int row = 32 * quad + lane;   // 0..127 over the four warps
         const uint32_t lane_base = dcol + (static_cast<uint32_t>(32 * quad) << 16);
         int dit = 0;
+        bool ok = true;
         for (int u = u0; u < tiles; u += ustep, ++dit) {
             const int n0 = (u / a.ttiles) * 128, m0 = (u % a.ttiles) * TOK;
-            if (!g_wait(dfull, dit & 1, err)) break;
+            if (ok) ok = mbar_wait(dfull, dit & 1, err);
+            __syncwarp();
             tc::fence_after_sync();
             if (split > 1) {
                 // fp32 sums of this CTA's K chunks, [token][row], over the idle activation ring
@@ -562,6 +565,7 @@ extern "C" int wq4_gemm(const uint32_t* W_packed, const uint16_t* scales, const 
     a.split = pl.split;
     a.err = status_word();
     if (!a.err) return WQ4_ERR_CUDA;
+    a.stall = test_copy_stall();
     const int64_t tiles = static_cast<int64_t>(a.rtiles) * a.ttiles;
     if (tiles > (static_cast<int64_t>(1) << 30)) return WQ4_ERR_UNSUPPORTED;
     cudaLaunchAttribute attr[2];

@@ -569,6 +569,8 @@ bool plan_mma(const DeviceInfo* di, int N, int K, int B, MmaPlan* pl)
 // 1 the legacy-tensor-path kernels wherever they apply, 2 the CUDA-core one.
 std::atomic<int> g_gemv_path{0};
 
+std::atomic<int> g_copy_stall{WQ4_STALL_NONE};
+
 // Below ~12 M weights a launch is bound by its fixed costs (x staging, the
 // first chunk's round trip, the epilogue), which the smaller CUDA-core
 // kernel pays less of; above it the legacy-tensor-path kernel streams
@@ -725,6 +727,15 @@ extern "C" int wq4_test_gemv_path(int path)
 {
     if (path < 0 || path > 2) return WQ4_ERR_INVALID;
     g_gemv_path.store(path);
+    return WQ4_OK;
+}
+
+int wq4::test_copy_stall() { return g_copy_stall.load(); }
+
+extern "C" int wq4_test_copy_stall(int stall)
+{
+    if (stall < WQ4_STALL_NONE || stall > WQ4_STALL_GEMM_W) return WQ4_ERR_INVALID;
+    g_copy_stall.store(stall);
     return WQ4_OK;
 }
 

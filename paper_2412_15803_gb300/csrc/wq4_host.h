@@ -24,6 +24,9 @@ const DeviceInfo* current_device_info(int* device_out);
 // Device address of the library's status word on the current device.
 uint32_t* status_word();
 
+// The copies that wq4_test_copy_stall leaves out.
+int test_copy_stall();
+
 // wq4_paged_attention that also leaves the sums of squares of every (row,
 // query head)'s outputs in sq [batch][sq_ld] (null: none).
 int launch_paged_attention(const wq4_kv_cache* cache, const uint16_t* q, int q_stride, const int32_t* seq_lens,
