@@ -38,7 +38,6 @@
 
 #include <algorithm>
 #include <atomic>
-#include <mutex>
 
 namespace wq4 {
 namespace {
@@ -429,13 +428,15 @@ __global__ void __launch_bounds__(kGThreads, 1)
 template <int TOK>
 cudaError_t gemm_launch(cudaLaunchConfig_t& cfg, const CUtensorMap* tm, const GemmArgs& a)
 {
-    static std::once_flag once;
-    static cudaError_t rc = cudaErrorUnknown;
-    std::call_once(once, [] {
-        rc = cudaFuncSetAttribute(gemm_kernel<TOK>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                  GCfg<TOK>::kSmem);
-    });
-    if (rc != cudaSuccess) return rc;
+    static std::atomic<bool> ready[64];                // per device; setting the attribute twice is harmless
+    int dev = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e != cudaSuccess) return e;
+    if (dev >= 64 || !ready[dev].load()) {
+        e = cudaFuncSetAttribute(gemm_kernel<TOK>, cudaFuncAttributeMaxDynamicSharedMemorySize, GCfg<TOK>::kSmem);
+        if (e != cudaSuccess) return e;
+        if (dev < 64) ready[dev].store(true);
+    }
     cfg.dynamicSmemBytes = GCfg<TOK>::kSmem;
     return cudaLaunchKernelEx(&cfg, gemm_kernel<TOK>, tm[0], tm[1], tm[2], a);
 }
