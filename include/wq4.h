@@ -84,7 +84,9 @@ enum wq4_status {
  * after the previous kernel in `stream` has completed, but the weight
  * stream may start while it finishes if that kernel lets its dependents
  * launch early (griddepcontrol.launch_dependents), so such a kernel must not
- * write W_packed or scales.
+ * write W_packed or scales.  (A kernel before that one may: every kernel of
+ * this library lets its dependents launch only once its predecessor has
+ * completed.)
  */
 int wq4_gemv(const uint32_t* W_packed, const uint16_t* scales, const uint16_t* x,
              uint16_t* y, int N, int K, int batch, void* stream);
@@ -105,8 +107,9 @@ int wq4_gemv(const uint32_t* W_packed, const uint16_t* scales, const uint16_t* x
  *   M >= 1 (any size), N >= 1 with N % 8 == 0, K % 256 == 0 (other valid
  *   sizes return WQ4_ERR_UNSUPPORTED: use wq4_gemv for them).
  * Deterministic (where K is split over thread blocks, the parts are added in
- * order).  Launched with programmatic dependent launch, as wq4_gemv.  At most
- * 16 tokens run on wq4_gemv's kernels (exact weights).  Returns WQ4_OK, WQ4_ERR_INVALID,
+ * order).  Launched with programmatic dependent launch; everything is read
+ * after the previous kernel in `stream` has completed.  At most 16 tokens run
+ * on wq4_gemv's kernels (exact weights).  Returns WQ4_OK, WQ4_ERR_INVALID,
  * WQ4_ERR_UNSUPPORTED, WQ4_ERR_ALIGN or WQ4_ERR_CUDA.
  */
 int wq4_gemm(const uint32_t* W_packed, const uint16_t* scales, const uint16_t* x,

@@ -217,7 +217,6 @@ __global__ void __launch_bounds__(kThreads, kCtasPerSm) paged_attn_kernel(const 
 
     // tile prefix over the batch (warp 0), barriers (thread 32); every input may
     // come from the previous kernel of the stream (programmatic dependent launch)
-    grid_dependents_launch();
     if (warp != 1) grid_dependency_wait();
     if (warp == 0) {
         int carry = 0, longest = 0;
@@ -286,6 +285,7 @@ __global__ void __launch_bounds__(kThreads, kCtasPerSm) paged_attn_kernel(const 
         mbar_fence_init();
     }
     if (warp == 1) grid_dependency_wait();
+    grid_dependents_launch();             // not before: the next kernel may fetch weights that one before this wrote
     __syncthreads();
 
     const int total = P.Hkv * pre[P.batch];

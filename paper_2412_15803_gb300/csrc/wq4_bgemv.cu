@@ -174,9 +174,10 @@ __global__ void __launch_bounds__(kBThreads, 1) bgemv_kernel(const BGemvParams p
         lstage = (lstage + 1) & (kBStages - 1);
     };
 
-    grid_dependents_launch();
     // weights of the first chunks may be fetched while the previous kernel of
-    // the stream finishes; activations only after it (programmatic dependent launch)
+    // the stream finishes; activations only after it (programmatic dependent
+    // launch).  The next kernel may begin then, and not before: it may fetch
+    // weights that a kernel before this one wrote.
     {
         int c1 = 0, n1 = ln0;
         for (int i = 0; i < kBStages - 1 && i < total; ++i) {
@@ -189,6 +190,7 @@ __global__ void __launch_bounds__(kBThreads, 1) bgemv_kernel(const BGemvParams p
         }
     }
     grid_dependency_wait();
+    grid_dependents_launch();
     for (int i = 0; i < kBStages - 1; ++i) {
         if (i < total) {
             issue_x(lstage, lc);
@@ -339,7 +341,7 @@ struct TGemvParams {
     uint16_t* y;
     int N, batch;
     int y4;                // two outputs may be stored at once
-    int check;             // flag scales beyond +-8188 (wq4_gemm's contract)
+    int check;             // a call of wq4_gemm: flag scales beyond +-8188, copy weights after the previous kernel
     uint32_t* err;
 };
 
@@ -427,13 +429,14 @@ __global__ void __launch_bounds__(32 * (kTWarps<XT> + 1), 1)
         mbar_fence_init();
     }
     __syncthreads();
-    grid_dependents_launch();
     if (warp == NW) {
-        if (lane == 0) tile_producer<XT, false, TAIL>(&tm_w, &tm_s, &tm_x, &tm_w2, &tm_s2, p.g, 0, smem, full, empty, p.err);
+        if (lane == 0)
+            tile_producer<XT, false, TAIL>(&tm_w, &tm_s, &tm_x, &tm_w2, &tm_s2, p.g, 0, smem, full, empty, p.err, XT <= 2 && p.check);
         return;
     }
 
     grid_dependency_wait();               // y is written after the previous kernel
+    grid_dependents_launch();             // ... and the next one may fetch weights that a kernel before this one wrote
     TileWarp<XT, R, false> tw(p.g, smem, warp, lane);
     {
         float acc[R][XT][4];

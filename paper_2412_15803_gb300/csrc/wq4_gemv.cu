@@ -83,7 +83,6 @@ __global__ void __launch_bounds__(kGemvThreads, 1) gemv_tma_kernel(const GemvTma
         mbar_fence_init();
     }
     __syncthreads();
-    grid_dependents_launch();     // the next launch in the stream may start its set-up
 
     if (warp == kGemvConsumerWarps) {
         // ---------------- producer: one elected lane issues the bulk copies
@@ -114,6 +113,8 @@ __global__ void __launch_bounds__(kGemvThreads, 1) gemv_tma_kernel(const GemvTma
     // grid in the stream is complete (programmatic dependent launch: the
     // producer's weight copies may start earlier)
     grid_dependency_wait();
+    // the next launch may start its set-up and fetch its weights, which a kernel before this one may have written
+    grid_dependents_launch();
     {
         const uint4* xg = reinterpret_cast<const uint4*>(p.x);
         const int chunks_per_row = p.K >> 3;
@@ -208,7 +209,6 @@ __global__ void __launch_bounds__(kMmaThreads, 1) gemv_mma_kernel(const GemvMmaP
         mbar_fence_init();
     }
     __syncthreads();
-    grid_dependents_launch();     // the next launch in the stream may start its set-up
 
     if (warp == kMmaWarps) {
         // ---------------- producer: one lane issues the bulk copies
@@ -243,6 +243,8 @@ __global__ void __launch_bounds__(kMmaThreads, 1) gemv_mma_kernel(const GemvMmaP
     // ---------------- consumers: x once, in the MMA's pair-permuted order,
     // after the previous grid in the stream is complete
     grid_dependency_wait();
+    // the next launch may start its set-up and fetch its weights, which a kernel before this one may have written
+    grid_dependents_launch();
     {
         const uint4* xg = reinterpret_cast<const uint4*>(p.x);
         for (int i = threadIdx.x; i < B * cpr; i += kConsumers) xs[i] = pair_permute(xg[i]);

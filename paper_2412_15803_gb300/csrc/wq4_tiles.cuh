@@ -94,11 +94,13 @@ __device__ __forceinline__ float lo_scale(uint32_t v) { return __low2float(*rein
 __device__ __forceinline__ float hi_scale(uint32_t v) { return __high2float(*reinterpret_cast<const __half2*>(&v)); }
 
 // One lane: streams the CTA's chunks (tile blockIdx.x, + gridDim.x, ..., then
-// its tail) into the ring.  up: GU's first up row.
+// its tail) into the ring.  up: GU's first up row.  late: the previous kernel
+// may write the weights (they are fetched into L2 before it has finished; no
+// GU, no tail).
 template <int XT, bool GU, bool TAIL = false>
 __device__ __forceinline__ void tile_producer(const CUtensorMap* tm_w, const CUtensorMap* tm_s, const CUtensorMap* tm_x,
-                                              const CUtensorMap* tm_w2, const CUtensorMap* tm_s2, const TileGeom& p, int up, uint8_t* smem, uint64_t* full, uint64_t* empty,
-                                              uint32_t* err)
+                                              const CUtensorMap* tm_w2, const CUtensorMap* tm_s2, const TileGeom& p, int up,
+                                              uint8_t* smem, uint64_t* full, uint64_t* empty, uint32_t* err, bool late = false)
 {
     tc::prefetch_map(tm_w);
     tc::prefetch_map(tm_s);
@@ -133,6 +135,17 @@ __device__ __forceinline__ void tile_producer(const CUtensorMap* tm_w, const CUt
     // finishes, activations only after it (programmatic dependent launch)
     int n0 = static_cast<int>(blockIdx.x) * TB, ch = 0;
     const int early = min(nslots, total);
+    if (late) {
+        for (int f = 0, c = 0, r = n0; f < early; ++f) {
+            tc::tma_prefetch_3d(tm_w, 0, r, c * boxes);
+            tc::tma_prefetch_3d(tm_s, 0, r, c * boxes);
+            if (++c == nch) {
+                c = 0;
+                r += grid * TB;
+            }
+        }
+        grid_dependency_wait();
+    }
     for (int f = 0; f < early; ++f) {
         load_w(f, f, n0, ch);
         if (++ch == nch) {
