@@ -154,7 +154,8 @@ int wq4_test_gemv_path(int path);
 enum wq4_stall {
     WQ4_STALL_NONE = 0,
     WQ4_STALL_GEMM_X = 1,     /* wq4_gemm (17 tokens and more): the activations */
-    WQ4_STALL_GEMM_W = 2      /* ... : the weights and scales */
+    WQ4_STALL_GEMM_W = 2,     /* ... : the weights and scales */
+    WQ4_STALL_ATTN = 3        /* wq4_paged_attention: the keys and values */
 };
 int wq4_test_copy_stall(int stall);
 

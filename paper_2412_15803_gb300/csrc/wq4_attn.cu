@@ -77,6 +77,7 @@ struct AttnParams {
     int q_stride, out_stride, pt_stride;
     int batch, Hkv, G, page_size, num_pages;
     float sl2;                   // scale * log2(e)
+    int stall;                   // test hook: no tile is copied
     float* sq;                   // per (row, head) sums of squares of the outputs, [batch][sq_ld]; null: none
     int sq_ld;
 };
@@ -205,7 +206,7 @@ __global__ void __launch_bounds__(kThreads, kCtasPerSm) paged_attn_kernel(const 
     uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
     uint64_t* full = reinterpret_cast<uint64_t*>(smem + kOffBars);
     uint64_t* empty = full + kSlots;
-    volatile int* misc = reinterpret_cast<volatile int*>(smem + kOffMisc);   // [0] abort, [1] last arriver, [2] one piece per CTA
+    volatile int* misc = reinterpret_cast<volatile int*>(smem + kOffMisc);   // [0] last arriver, [1] one piece per CTA
     float* mrow = reinterpret_cast<float*>(smem + kOffMrow);
     float* lrow = reinterpret_cast<float*>(smem + kOffLrow);
     float* scr = reinterpret_cast<float*>(smem + kOffScr);
@@ -274,14 +275,13 @@ __global__ void __launch_bounds__(kThreads, kCtasPerSm) paged_attn_kernel(const 
             fits = P.Hkv * sum <= grid;
         }
         __syncwarp();
-        if (lane == 0) misc[2] = fits ? 1 : 0;
+        if (lane == 0) misc[1] = fits ? 1 : 0;
     } else if (tid == 32) {
         for (int i = 0; i < kSlots; ++i) {
             mbar_init(&full[i], 1);
             mbar_init(&empty[i], 1);
         }
         misc[0] = 0;
-        misc[1] = 0;
         mbar_fence_init();
     }
     if (warp == 1) grid_dependency_wait();
@@ -290,7 +290,7 @@ __global__ void __launch_bounds__(kThreads, kCtasPerSm) paged_attn_kernel(const 
 
     const int total = P.Hkv * pre[P.batch];
     const int cta = blockIdx.x;
-    const bool whole = misc[2] != 0;
+    const bool whole = misc[1] != 0;
     const int R = max((total + static_cast<int>(gridDim.x) - 1) / static_cast<int>(gridDim.x), kShareMin);
     const int g_begin = whole ? 0 : min(total, cta * R);
     const int g_end = whole ? (cta < P.Hkv * parts[P.batch] ? 1 : 0) : min(total, g_begin + R);
@@ -307,7 +307,7 @@ __global__ void __launch_bounds__(kThreads, kCtasPerSm) paged_attn_kernel(const 
             asm volatile("prefetch.tensormap [%0];" ::"l"(&P.mv) : "memory");
         }
         int i = 0;   // CTA-wide tile counter
-        bool ok = true;
+        bool ok = P.stall == 0;
         for (int g = g_begin; g < g_end && ok;) {
             const Piece pc = piece(g);
             const int32_t* pt = P.page_table + static_cast<size_t>(pc.b) * P.pt_stride;
@@ -327,7 +327,6 @@ __global__ void __launch_bounds__(kThreads, kCtasPerSm) paged_attn_kernel(const 
                     if (lane == 0) {
                         const int slot = i % kSlots;
                         if (i >= kSlots && !mbar_wait(&empty[slot], ((i / kSlots) - 1) & 1, P.err)) {
-                            misc[0] = 1;
                             ok = false;
                         } else {
                             int y;
@@ -378,6 +377,12 @@ __global__ void __launch_bounds__(kThreads, kCtasPerSm) paged_attn_kernel(const 
     const int qc = 2 * (lane & 3);     // column pair within 8
     const uint32_t ring = smem_addr(smem + kOffRing);
     int ibase = 0;                     // CTA-wide index of the piece's first tile
+    // After a wait gave up (bounded, flagged) a lane waits no more but goes on
+    // through every tile: the shuffles, copies of fragments and barriers below
+    // are for whole warps and all of them.  It releases no slot then (its copy may
+    // still be in flight), so the producer gives up as well, and the outputs are
+    // not valid.
+    bool ok = true;
     for (int g = g_begin; g < g_end;) {
         const Piece pc = piece(g);
         const int ntile = pc.t1 - pc.t0;
@@ -407,13 +412,9 @@ __global__ void __launch_bounds__(kThreads, kCtasPerSm) paged_attn_kernel(const 
         // tiles k of the piece with (ibase + k) % W == warp
         int k0 = (warp - ibase % kConsumers + kConsumers) % kConsumers;
         for (int k = k0; k < ntile; k += kConsumers) {
-            if (misc[0]) break;
             const int i = ibase + k;
             const int slot = i % kSlots;
-            if (!mbar_wait(&full[slot], (i / kSlots) & 1, P.err)) {
-                misc[0] = 1;
-                break;
-            }
+            if (ok) ok = mbar_wait(&full[slot], (i / kSlots) & 1, P.err);
             const int tok0 = (pc.t0 + k) * kTile;
             const int valid = min(kTile, T - tok0);
             const uint32_t kb = ring + slot * kSlotBytes;
@@ -479,7 +480,7 @@ __global__ void __launch_bounds__(kThreads, kCtasPerSm) paged_attn_kernel(const 
                 }
             }
             __syncwarp();
-            if (lane == 0) mbar_arrive(&empty[slot]);
+            if (lane == 0 && ok) mbar_arrive(&empty[slot]);
         }
 
         // ---- merge the warps' states of this piece (fixed warp order)
@@ -552,11 +553,11 @@ __global__ void __launch_bounds__(kThreads, kCtasPerSm) paged_attn_kernel(const 
             named_barrier_sync(1, kConsumers * 32);
             if (tid == 0) {
                 const uint32_t old = atomicAdd(P.cnt + pc.seg, 1u);
-                misc[1] = (old == static_cast<uint32_t>(pc.npieces - 1)) ? 1 : 0;
+                misc[0] = (old == static_cast<uint32_t>(pc.npieces - 1)) ? 1 : 0;
             }
             named_barrier_sync(1, kConsumers * 32);
-            if (misc[1]) __threadfence();
-            for (int gg = warp; misc[1] && gg < G; gg += kConsumers) {
+            if (misc[0]) __threadfence();
+            for (int gg = warp; misc[0] && gg < G; gg += kConsumers) {
                 // Merge parts p = 0..np-1 of this segment, a warp per head.  The
                 // lanes read the parts' (M_p, L_p) and, at the same time, the
                 // first parts' outputs; the running maximum and normaliser are
@@ -611,7 +612,7 @@ __global__ void __launch_bounds__(kThreads, kCtasPerSm) paged_attn_kernel(const 
                 for (int p = kPre; p < np; ++p) add(__ldcg(reinterpret_cast<const float4*>(po + p * pstride)), p);
                 store(gg, a0, a1, a2, a3, l);
             }
-            if (tid == 0 && misc[1]) P.cnt[pc.seg] = 0u;
+            if (tid == 0 && misc[0]) P.cnt[pc.seg] = 0u;
         }
         named_barrier_sync(1, kConsumers * 32);   // scratch and flags free for the next piece
         ibase += ntile;
@@ -760,6 +761,7 @@ int launch_paged_attention(const wq4_kv_cache* cache, const uint16_t* q, int q_s
     p.sl2 = static_cast<float>(static_cast<double>(scale) * 1.4426950408889634);
     p.sq = sq;
     p.sq_ld = sq_ld;
+    p.stall = test_copy_stall() == WQ4_STALL_ATTN ? 1 : 0;
     if (!p.err) return WQ4_ERR_CUDA;
     cudaLaunchAttribute attr[1];
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;

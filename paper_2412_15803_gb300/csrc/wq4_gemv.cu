@@ -736,7 +736,7 @@ int wq4::test_copy_stall() { return g_copy_stall.load(); }
 
 extern "C" int wq4_test_copy_stall(int stall)
 {
-    if (stall < WQ4_STALL_NONE || stall > WQ4_STALL_GEMM_W) return WQ4_ERR_INVALID;
+    if (stall < WQ4_STALL_NONE || stall > WQ4_STALL_ATTN) return WQ4_ERR_INVALID;
     g_copy_stall.store(stall);
     return WQ4_OK;
 }

@@ -11,11 +11,13 @@ import pytest
 import torch
 
 from paper_2412_15803_gb300 import wq4
+from paper_2412_15803_gb300.attention import PagedAttentionLayer
+from paper_2412_15803_gb300.model import ModelShape
 
 pytestmark = pytest.mark.gpu
 
 PIPE_TIMEOUT = 1
-GEMM_X, GEMM_W = 1, 2
+GEMM_X, GEMM_W, ATTN = 1, 2, 3
 
 
 def _stalled(stall, call):
@@ -56,3 +58,19 @@ def test_gemm_without_its_copies_ends(N, K, M, stall):
     torch.cuda.synchronize()
     assert wq4.wq4_device_status() == 0
     assert torch.equal(y, ref)
+
+
+# one piece a block (merged over blocks), several pieces a block with more tiles
+# than ring slots, an empty sequence among them
+@pytest.mark.parametrize("lens", [[4096], [9000, 0, 3000, 1] * 8])
+def test_attention_without_its_tiles_ends(lens):
+    layer = PagedAttentionLayer(ModelShape("stall", 1, 4096, 512, 32, 8, 128, 1000), lens, seed=3)
+    layer.run()
+    torch.cuda.synchronize()
+    ref = layer.out.clone()
+    _stalled(ATTN, layer.run)
+    layer.out.zero_()
+    layer.run()
+    torch.cuda.synchronize()
+    assert wq4.wq4_device_status() == 0
+    assert torch.equal(layer.out, ref)
