@@ -17,6 +17,7 @@ pytestmark = pytest.mark.gpu
 @pytest.mark.parametrize("lens", [
     [16], [129], [128 * 9 + 1], [4000],                    # one sequence: whole tiles, a tile over, many parts
     [1] * 40, [17] * 40, [300, 0, 1, 2000, 0],               # as many segments as blocks and more, empty ones
+    [40, 0] * 38, [40, 0, 7] * 38, [40, 0] * 76, [40] * 77,  # as many as blocks and one sequence more (8 and 4 heads)
     [64 * k + 1 for k in range(1, 20)],                      # a fair share that no cut at the ends fits
     [2500 + 7 * k for k in range(12)],                        # large shares
 ])
