@@ -547,7 +547,7 @@ def gemv_copies(mats) -> int:
 
 
 def gemv_kernel_names(mats, B: int) -> str:
-    """The kernels wq4_gemv's size rules pick for the set (K % 256 == 0)."""
+    """The kernels wq4_gemv's size rules pick for the set (K % 256 == 0, more than 8 rows an SM)."""
     names = []
     for _, N, K in mats:
         if B > 2 or (B == 2 and N * K >= 8 << 20):

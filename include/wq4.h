@@ -72,8 +72,9 @@ enum wq4_status {
  *              K % 256 == 0 select the TMA-staged fast paths: batch 1 from
  *              12 Mi weights, batch 2 from 8 Mi and every larger batch run on
  *              the legacy tensor path, exact in fp16 products with fp32 sums,
- *              else the CUDA cores; other rows at batch 3 and up run on the
- *              legacy tensor path too).
+ *              else, and with few long rows at batch 2-4, the CUDA cores;
+ *              other rows at batch 3 and up run on the legacy tensor path
+ *              too).
  *   x        : fp16 bits [batch][K], 16-byte aligned.
  *   y        : fp16 bits [batch][N], 2-byte aligned; must not overlap x, W or
  *              scales.
@@ -134,11 +135,11 @@ int wq4_unpack_debug(const uint32_t* W_packed, const uint16_t* scales,
 int wq4_pack_host(const uint8_t* q_host, uint32_t* W_host, int N, int K);
 
 /*
- * Test hook: which kernel wq4_gemv takes at batch 1-2 with K % 256 == 0 and
+ * Test hook: which kernel wq4_gemv takes at batch 1-4 with K % 256 == 0 and
  * 16-byte aligned scales, for every later call in this process.  0 (the
- * default) picks by size (the legacy-tensor-path kernels from 12 Mi weights
- * up, 8 Mi at batch 2, the CUDA-core kernel below), 1 always a legacy-tensor-path kernel,
- * 2 always the CUDA-core kernel.  Results agree within the tolerance; no
+ * default) picks by size (wq4_gemv above), 1 always a legacy-tensor-path
+ * kernel, 2 always the CUDA-core kernel (where its activations fit in shared
+ * memory).  Results agree within the tolerance; no
  * counterpart in the paper.  WQ4_ERR_INVALID for another value.
  */
 int wq4_test_gemv_path(int path);

@@ -3,8 +3,8 @@
 //
 // y[b][n] = fp16( sum_k (q(n,k) - 7) * s[n][k/32] * x[b][k] ), the projection
 // every decoded token applies to every 4-bit weight matrix (Section 3,
-// Table 1).  The kernels of batch 1-2 (batch 2 from 8 Mi weights and every
-// larger batch run in wq4_bgemv.cu):
+// Table 1).  The kernels of batch 1 and of few rows at batch 2-4 (the others run
+// in wq4_bgemv.cu):
 //
 //  * gemv_mma_kernel (batch 1, K % 256 == 0, 16-byte aligned scales): the
 //    persistent decode chain's weight stream for one projection.  A
@@ -14,7 +14,7 @@
 //    and run them on the legacy tensor path (wq4_items.cuh: exact fp16
 //    q - 7, eight groups of x as the MMA's columns, scales in fp32 on the
 //    diagonal); K parts are added in part order in shared memory.
-//  * gemv_tma_kernel<B> (batch B <= 2, K % 256 == 0): one persistent CTA per
+//  * gemv_tma_kernel<B> (batch B <= 4, K % 256 == 0): one persistent CTA per
 //    SM.  A producer warp streams the CTA's contiguous block of rows through a
 //    ring of shared-memory slots with 1-D bulk copies (TMA) and mbarriers;
 //    consumer warps take rows round-robin, unpack in registers and accumulate
@@ -484,7 +484,9 @@ const DeviceInfo* current_device_info(int* device_out)
         if (cudaDeviceGetAttribute(&d.smem_optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev) != cudaSuccess)
             return nullptr;
         if (cudaDeviceGetAttribute(&d.coop_launch, cudaDevAttrCooperativeLaunch, dev) != cudaSuccess) return nullptr;
-        if (!set_tma_attr<1>(d.smem_optin) || !set_tma_attr<2>(d.smem_optin) || !set_mma_attr(d.smem_optin)) return nullptr;
+        if (!set_tma_attr<1>(d.smem_optin) || !set_tma_attr<2>(d.smem_optin) || !set_tma_attr<3>(d.smem_optin) ||
+            !set_tma_attr<4>(d.smem_optin) || !set_mma_attr(d.smem_optin))
+            return nullptr;
         void* ptr = nullptr;
         if (cudaGetSymbolAddress(&ptr, g_status_word) != cudaSuccess) return nullptr;
         g_status_ptr[dev] = static_cast<uint32_t*>(ptr);
@@ -567,7 +569,7 @@ bool plan_mma(const DeviceInfo* di, int N, int K, int B, MmaPlan* pl)
     return true;
 }
 
-// Which batch 1-2 kernel a call takes (wq4_test_gemv_path): 0 the size rules,
+// Which batch 1-4 kernel a call takes (wq4_test_gemv_path): 0 the size rules,
 // 1 the legacy-tensor-path kernels wherever they apply, 2 the CUDA-core one.
 std::atomic<int> g_gemv_path{0};
 
@@ -582,13 +584,34 @@ std::atomic<int> g_copy_stall{WQ4_STALL_NONE};
 // 16384 x 3072 8.69 / 12.20, 128256 x 3072 45.1 / 75.1.
 constexpr int64_t kMmaMinWeights = int64_t(12) << 20;
 
-// From here on batch 2 takes the batched kernel (wq4_bgemv.cu): batch 2, us
-// (batched / the CUDA-core kernel here, or above 12 Mi weights the two-row
-// form that gemv_mma_kernel had): 2048 x 2048 2.99 / 3.00, 512 x 14336 6.86 /
-// 4.36, 3072 x 3072 3.68 / 4.70, 16384 x 3072 9.15 / 10.61, 128256 x 3072
-// 43.8 / 57.4.  At batch 1 the kernels here stay ahead (128256 x 3072 42.4 /
-// 43.8).
+// Batch 2-4 on the CUDA cores, or (false) the batched kernel (wq4_bgemv.cu).
+// The batched kernel takes at least eight rows a block, so with few rows most
+// of the SMs idle while a block walks all of K; here a row has a warp of its
+// own up to 8 rows an SM.  us a launch, batched / CUDA cores:
+//   batch 2: 600 x 14336 7.2 / 4.4, 1216 x 14336 8.1 / 6.3, 1216 x 8192 5.9 /
+//     4.3; below 8 Mi weights 512 x 4096 3.2 / 2.6, 2048 x 2048 2.9 / 3.0; from
+//     there on more rows take the batched kernel: 1536 x 6144 4.6 / 4.8, 16384 x
+//     3072 9.2 / 10.6, 128256 x 3072 43.8 / 57.4 (at batch 1 the kernels here stay
+//     ahead, 43.8 / 42.4).
+//   batch 3: 152 x 4608 3.3 / 3.4, 152 x 5120 3.4 / 3.4, 152 x 14336 6.8 / 4.9,
+//     608 x 4096 3.2 / 3.1, 768 x 3072 3.1 / 3.0, 1216 x 3072 3.5 / 3.1, 1280 x
+//     3072 3.0 / 3.7.
+//   batch 4: 304 x 5120 3.4 / 3.7, 304 x 6144 3.8 / 3.7, 608 x 14336 7.2 / 6.1,
+//     768 x 11008 6.3 / 6.9.
+//   Rows for two thirds of the SMs or fewer leave the next launch room to begin:
+//     batch 3 100 x 3072 2.7 / 2.5, 64 x 2048 2.2 / 2.1, batch 4 100 x 4096 3.0 /
+//     2.9.
 constexpr int64_t kBatch2MinWeights = int64_t(8) << 20;
+
+bool cuda_cores(int batch, int N, int K, int sms)
+{
+    const int64_t weights = static_cast<int64_t>(N) * K;
+    if (batch == 2) return weights < kBatch2MinWeights || N <= 8 * sms;
+    if (batch == 3)
+        return (N <= 8 * sms && (K >= 5120 || 10 * weights >= (int64_t(22) << 20))) || (3 * N <= 2 * sms && K >= 3072) ||
+               (2 * N <= sms && K >= 2048);
+    return batch == 4 && ((N <= 4 * sms && K >= 5632) || (3 * N <= 2 * sms && K >= 4096) || (2 * N <= sms && K >= 2048));
+}
 
 // Rows that the bulk copies cannot take (K % 256 != 0 or unaligned scales):
 // the batched kernel's copy ring from here on at batch 1 and 2, the warp-per-row
@@ -606,7 +629,12 @@ int launch_gemv(const uint32_t* W, const uint16_t* s, const uint16_t* x, uint16_
     const int path = g_gemv_path.load();
     const int64_t weights = static_cast<int64_t>(N) * K;
     const bool bulk = (K % 256) == 0 && aligned(s, 16);
-    if (batch > 2 || (batch == 2 && bulk && path != 2 && (weights >= kBatch2MinWeights || path == 1)))
+    const size_t row_bytes = static_cast<size_t>(K) / 2 + static_cast<size_t>(K) / 16;
+    const size_t x_bytes = align_up(static_cast<size_t>(batch) * K * 2, 128);
+    const bool fast = batch <= 4 && bulk &&
+                      kHeaderBytes + x_bytes + 2 * align_up(row_bytes, 128) <= static_cast<size_t>(di->smem_optin);
+    if ((batch > 2 && !fast) ||
+        (batch >= 2 && bulk && path != 2 && (path == 1 || !cuda_cores(batch, N, K, di->sm_count))))
         return launch_bgemv(di, W, s, x, y, N, K, batch, stream);
     MmaPlan mp;
     if (path != 2 && (weights >= kMmaMinWeights || path == 1) && batch == 1 && bulk && plan_mma(di, N, K, batch, &mp)) {
@@ -637,9 +665,6 @@ int launch_gemv(const uint32_t* W, const uint16_t* s, const uint16_t* x, uint16_
         const cudaError_t e = cudaLaunchKernelEx(&cfg, gemv_mma_kernel, p);
         return e == cudaSuccess ? WQ4_OK : WQ4_ERR_CUDA;
     }
-    const size_t row_bytes = static_cast<size_t>(K) / 2 + static_cast<size_t>(K) / 16;
-    const size_t x_bytes = align_up(static_cast<size_t>(batch) * K * 2, 128);
-    const bool fast = bulk && kHeaderBytes + x_bytes + 2 * align_up(row_bytes, 128) <= static_cast<size_t>(di->smem_optin);
     if (fast) {
         const int grid = N < di->sm_count ? N : di->sm_count;
         const int rows_per_cta = (N + grid - 1) / grid;
@@ -679,8 +704,13 @@ int launch_gemv(const uint32_t* W, const uint16_t* s, const uint16_t* x, uint16_
         cfg.stream = stream;
         cfg.attrs = attr;
         cfg.numAttrs = 1;
-        const cudaError_t e = batch == 1 ? cudaLaunchKernelEx(&cfg, gemv_tma_kernel<1>, p)
-                                         : cudaLaunchKernelEx(&cfg, gemv_tma_kernel<2>, p);
+        cudaError_t e;
+        switch (batch) {
+            case 1: e = cudaLaunchKernelEx(&cfg, gemv_tma_kernel<1>, p); break;
+            case 2: e = cudaLaunchKernelEx(&cfg, gemv_tma_kernel<2>, p); break;
+            case 3: e = cudaLaunchKernelEx(&cfg, gemv_tma_kernel<3>, p); break;
+            default: e = cudaLaunchKernelEx(&cfg, gemv_tma_kernel<4>, p); break;
+        }
         if (e != cudaSuccess) return WQ4_ERR_CUDA;
     } else if (weights >= kRingMinWeights[batch]) {
         return launch_bgemv(di, W, s, x, y, N, K, batch, stream);

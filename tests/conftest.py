@@ -27,3 +27,17 @@ def pytest_collection_modifyitems(config, items):
     for item in items:
         if "gpu" in item.keywords:
             item.add_marker(skip)
+
+
+@pytest.fixture(scope="session")
+def fake_cudart(tmp_path_factory):
+    """Path of the stand-in for the CUDA runtime (fake_cudart.c), to preload in a child process."""
+    import subprocess
+
+    from paper_2412_15803_gb300 import build
+    cuda = os.path.dirname(os.path.dirname(os.path.realpath(build.nvcc())))
+    so = str(tmp_path_factory.mktemp("fake") / "libfake_cudart.so")
+    subprocess.check_call(["gcc", "-O1", "-Wall", "-Werror", "-shared", "-fPIC", "-I", os.path.join(cuda, "include"),
+                           "-o", so, os.path.join(ROOT, "tests", "fake_cudart.c")])
+    build.build()
+    return so

@@ -1,0 +1,46 @@
+"""Which kernel wq4_gemv launches at batch 2-4: the CUDA-core kernel where the
+rows are few and long (measured faster there), the batched one elsewhere.
+
+The lines are those of the dispatch rule, a size on each side; run without a
+GPU over a stand-in for the CUDA runtime (fake_cudart.c), which tells the
+kernel of the last launch.
+"""
+import os
+import subprocess
+import sys
+
+HERE = os.path.dirname(os.path.abspath(__file__))
+
+CHILD = r"""
+import ctypes, sys
+fake = ctypes.CDLL(sys.argv[1])
+from paper_2412_15803_gb300 import wq4
+L = wq4.load(build_if_missing=False)
+A = 1 << 40          # 16-byte aligned "device" addresses, never read
+
+def kernel(path, batch, N, K, off=0):
+    assert L.wq4_test_gemv_path(path) == 0
+    assert L.wq4_gemv(A, 2 * A + off, 4 * A, 8 * A, N, K, batch, None) == 0
+    return fake.fake_last_kernel()
+
+CORES = [(2, 600, 14336), (2, 1216, 14336), (2, 1216, 8192), (2, 2048, 2048), (2, 64, 256),
+         (3, 64, 2048), (3, 76, 2048), (3, 101, 3072), (3, 152, 5120), (3, 608, 4096), (3, 768, 3072), (3, 1216, 14336),
+         (4, 64, 2048), (4, 101, 4096), (4, 152, 5632), (4, 608, 14336)]
+BATCHED = [(2, 1217, 14336), (2, 4096, 2048), (2, 128256, 4096),
+           (3, 64, 1792), (3, 77, 2048), (3, 102, 3072), (3, 152, 4864), (3, 608, 3584), (3, 1217, 14336), (3, 64, 256),
+           (4, 64, 1792), (4, 101, 3840), (4, 152, 5376), (4, 609, 14336), (4, 4096, 4096)]
+for c in CORES:
+    assert kernel(0, *c) == kernel(2, *c) != kernel(1, *c), c
+for c in BATCHED:
+    assert kernel(0, *c) == kernel(1, *c) != kernel(2, *c), c
+# activations beyond shared memory, batch 5 and scales off 16 bytes: the batched kernels, whatever the hook says
+for c in ((3, 64, 36864), (4, 64, 28672), (5, 64, 14336)):
+    assert kernel(0, *c) == kernel(1, *c) == kernel(2, *c), c
+assert kernel(0, 3, 64, 14336, 2) == kernel(2, 3, 64, 14336, 2) != kernel(2, 3, 64, 14336)
+"""
+
+
+def test_routes(fake_cudart):
+    env = dict(os.environ, LD_PRELOAD=fake_cudart, PYTHONPATH=os.path.dirname(HERE))
+    r = subprocess.run([sys.executable, "-c", CHILD, fake_cudart], env=env, capture_output=True, text=True)
+    assert r.returncode == 0, r.stderr[-2000:]

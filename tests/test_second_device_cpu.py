@@ -11,8 +11,6 @@ import sys
 
 import pytest
 
-from paper_2412_15803_gb300 import build
-
 HERE = os.path.dirname(os.path.abspath(__file__))
 
 CHILD = r"""
@@ -36,16 +34,6 @@ for device in (0, 1, 0, 2):
 """
 
 
-@pytest.fixture(scope="module")
-def fake(tmp_path_factory):
-    cuda = os.path.dirname(os.path.dirname(os.path.realpath(build.nvcc())))
-    so = str(tmp_path_factory.mktemp("fake") / "libfake_cudart.so")
-    subprocess.check_call(["gcc", "-O1", "-Wall", "-Werror", "-shared", "-fPIC", "-I", os.path.join(cuda, "include"),
-                           "-o", so, os.path.join(HERE, "fake_cudart.c")])
-    build.build()
-    return so
-
-
 # one size of every kernel: GEMM token tiles 64, 128, 192 and 256 and a split K;
 # batch 1 small and large, 2, the batched tile loop with and without a tail
 # round, rows of the copy ring; attention
@@ -55,8 +43,8 @@ def fake(tmp_path_factory):
     ("wq4_gemv", 1, 2048, 2048), ("wq4_gemv", 1, 16384, 3072), ("wq4_gemv", 2, 2048, 2048), ("wq4_gemv", 2, 16384, 3072),
     ("wq4_gemv", 4, 600, 14336), ("wq4_gemv", 8, 3072, 8192), ("wq4_gemv", 24, 8192, 4096), ("wq4_gemv", 32, 128256, 4096),
     ("wq4_gemv", 5, 1003, 2080), ("wq4_gemv", 1, 1003, 2080), ("attention", 4, 0, 0)])
-def test_launches_on_every_device(fake, name, rows, N, K):
-    env = dict(os.environ, LD_PRELOAD=fake, PYTHONPATH=os.path.dirname(HERE))
-    r = subprocess.run([sys.executable, "-c", CHILD, fake, name, str(rows), str(N), str(K)], env=env,
+def test_launches_on_every_device(fake_cudart, name, rows, N, K):
+    env = dict(os.environ, LD_PRELOAD=fake_cudart, PYTHONPATH=os.path.dirname(HERE))
+    r = subprocess.run([sys.executable, "-c", CHILD, fake_cudart, name, str(rows), str(N), str(K)], env=env,
                        capture_output=True, text=True)
     assert r.returncode == 0, r.stderr[-2000:]
