@@ -391,9 +391,23 @@ __global__ void __launch_bounds__(256) gemv_generic_kernel(const uint32_t* __res
         float acc[B];
 #pragma unroll
         for (int b = 0; b < B; ++b) acc[b] = 0.f;
+        // The next group's codes and scale are loaded ahead.  (Unrolled by the
+        // compiler instead, four groups a turn, batch 1 took 6.3 us for 64 x 8160
+        // against 5.0, 8192 x 4128 15.7 against 13.4, 20000 x 3104 24.2 against 21.1.)
+        uint4 ncw = make_uint4(0u, 0u, 0u, 0u);
+        uint16_t nsc = 0;
+        if (lane < gpr) {
+            ncw = __ldg(crow + lane);
+            nsc = __ldg(srow + lane);
+        }
+#pragma unroll 1
         for (int g = lane; g < gpr; g += 32) {
-            const uint4 cw = __ldg(crow + g);
-            const float sc = half_bits_to_float(__ldg(srow + g));
+            const uint4 cw = ncw;
+            const float sc = half_bits_to_float(nsc);
+            if (g + 32 < gpr) {
+                ncw = __ldg(crow + g + 32);
+                nsc = __ldg(srow + g + 32);
+            }
             uint32_t pq[16];
             unpack_word(cw.x, pq + 0);
             unpack_word(cw.y, pq + 4);
@@ -613,12 +627,20 @@ bool cuda_cores(int batch, int N, int K, int sms)
     return batch == 4 && ((N <= 4 * sms && K >= 5632) || (3 * N <= 2 * sms && K >= 4096) || (2 * N <= sms && K >= 2048));
 }
 
-// Rows that the bulk copies cannot take (K % 256 != 0 or unaligned scales):
-// the batched kernel's copy ring from here on at batch 1 and 2, the warp-per-row
-// kernel below.  us (ring / warp per row): batch 1 1003 x 2080 4.83 / 2.99,
-// 20000 x 3104 27.5 / 21.6, 100000 x 3104 78.6 / 95.4; batch 2 1003 x 2080
-// 4.62 / 4.27, 4000 x 2080 6.53 / 7.33, 100000 x 3104 78.5 / 155.8.
-constexpr int64_t kRingMinWeights[3] = {0, int64_t(128) << 20, int64_t(6) << 20};
+// Rows that the bulk copies cannot take (K % 256 != 0 or unaligned scales) at
+// batch 1-2: the batched kernel's copy ring, or (false) a warp per row, which
+// reads every activation once more per row but takes every row's codes at once
+// up to 8 rows an SM.  The lines lie where the two cross, us, ring / warp per row:
+//   batch 1: 1003 x 2080 4.7 / 2.7, 40000 x 3104 45.7 / 39.2, 50000 x 3104 42.2 /
+//     46.5, 100000 x 3104 77.8 / 92.6, 20000 x 8160 56.5 / 47.7, 24000 x 8160 57.3 /
+//     56.3, 30000 x 8160 68.9 / 70.1;
+//   batch 2: 1003 x 2080 4.4 / 3.4, 3000 x 2080 6.1 / 5.6, 4000 x 2080 6.7 / 6.9,
+//     1000 x 8160 9.6 / 7.1, 1500 x 8160 10.5 / 11.0, 100000 x 3104 77.7 / 150.
+bool copy_ring(int batch, int N, int K, int sms)
+{
+    const int64_t weights = static_cast<int64_t>(N) * K;
+    return batch == 1 ? weights >= (int64_t(128) << 20) && K <= 4096 : weights >= (int64_t(6) << 20) && N > 8 * sms;
+}
 
 int launch_gemv(const uint32_t* W, const uint16_t* s, const uint16_t* x, uint16_t* y, int N, int K, int batch,
                 cudaStream_t stream)
@@ -712,7 +734,7 @@ int launch_gemv(const uint32_t* W, const uint16_t* s, const uint16_t* x, uint16_
             default: e = cudaLaunchKernelEx(&cfg, gemv_tma_kernel<4>, p); break;
         }
         if (e != cudaSuccess) return WQ4_ERR_CUDA;
-    } else if (weights >= kRingMinWeights[batch]) {
+    } else if (copy_ring(batch, N, K, di->sm_count)) {
         return launch_bgemv(di, W, s, x, y, N, K, batch, stream);
     } else {
         const int warps_per_block = 8;

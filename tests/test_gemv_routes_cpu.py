@@ -1,5 +1,6 @@
-"""Which kernel wq4_gemv launches at batch 2-4: the CUDA-core kernel where the
-rows are few and long (measured faster there), the batched one elsewhere.
+"""Which kernel wq4_gemv launches where a rule on sizes decides: at batch 2-4
+the CUDA-core kernel for few long rows and the batched one elsewhere, at batch
+1-2 the copy ring or a warp per row for rows that bulk copies cannot take.
 
 The lines are those of the dispatch rule, a size on each side; run without a
 GPU over a stand-in for the CUDA runtime (fake_cudart.c), which tells the
@@ -37,6 +38,15 @@ for c in BATCHED:
 for c in ((3, 64, 36864), (4, 64, 28672), (5, 64, 14336)):
     assert kernel(0, *c) == kernel(1, *c) == kernel(2, *c), c
 assert kernel(0, 3, 64, 14336, 2) == kernel(2, 3, 64, 14336, 2) != kernel(2, 3, 64, 14336)
+# rows of odd groups at batch 1-2: the copy ring of the batched kernels (as at batch 3), or a warp per row
+RING = [(1, 50000, 3104), (1, 100000, 3104), (2, 4000, 2080), (2, 1500, 8160), (2, 1217, 8160)]
+WARPS = [(1, 1003, 2080), (1, 40000, 3104), (1, 20000, 8160), (1, 30000, 8160), (2, 1003, 2080), (2, 3000, 2080), (2, 1000, 8160),
+         (2, 1216, 8160)]
+warps = {b: kernel(0, b, 3, 32) for b in (1, 2)}
+for c in RING:
+    assert kernel(0, *c) != warps[c[0]], c
+for c in WARPS:
+    assert kernel(0, *c) == warps[c[0]], c
 """
 
 
