@@ -408,11 +408,16 @@ __device__ __noinline__ bool tail_tile(const TGemvParams& p, uint8_t* smem, int 
     return tl.bad;
 }
 
+// The call's tensor maps: weights, scales, activations, and the tails' weights and
+// scales where there are any.
+template <bool TAIL>
+struct TMaps {
+    CUtensorMap m[TAIL ? 5 : 3];
+};
+
 template <int XT, int R, bool TAIL>
 __global__ void __launch_bounds__(32 * (kTWarps<XT> + 1), 1)
-    bgemv_tma_kernel(const __grid_constant__ CUtensorMap tm_w, const __grid_constant__ CUtensorMap tm_s,
-                     const __grid_constant__ CUtensorMap tm_x, const __grid_constant__ CUtensorMap tm_w2,
-                     const __grid_constant__ CUtensorMap tm_s2, const __grid_constant__ TGemvParams p)
+    bgemv_tma_kernel(const __grid_constant__ TMaps<TAIL> t, const __grid_constant__ TGemvParams p)
 {
     extern __shared__ __align__(1024) uint8_t smem[];
     constexpr int NW = kTWarps<XT>, kConsumers = 32 * NW;
@@ -431,7 +436,7 @@ __global__ void __launch_bounds__(32 * (kTWarps<XT> + 1), 1)
     __syncthreads();
     if (warp == NW) {
         if (lane == 0)
-            tile_producer<XT, false, TAIL>(&tm_w, &tm_s, &tm_x, &tm_w2, &tm_s2, p.g, 0, smem, full, empty, p.err, XT <= 2 && p.check);
+            tile_producer<XT, false, TAIL>(&t.m[0], &t.m[1], &t.m[2], &t.m[TAIL ? 3 : 0], &t.m[TAIL ? 4 : 1], p.g, 0, smem, full, empty, p.err, XT <= 2 && p.check);
         return;
     }
 
@@ -512,67 +517,89 @@ bool plan_bgemv(int sms, size_t smem_max, int N, int K, int XT, bool s2, BPlan* 
 }
 
 template <int XT, int R, bool S2>
-cudaError_t launch_one(const cudaLaunchConfig_t& cfg, const BGemvParams& p, int smem_max)
+cudaError_t launch_one(const cudaLaunchConfig_t& cfg, const BGemvParams& p, const DeviceInfo* di)
 {
-    static std::atomic<bool> ready[64];                // per device; setting the attribute twice is harmless
-    int dev = 0;
-    cudaError_t e = cudaGetDevice(&dev);
-    if (e != cudaSuccess) return e;
-    if (dev >= 64 || !ready[dev].load()) {
-        e = cudaFuncSetAttribute(bgemv_kernel<XT, R, S2>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_max);
+    static std::atomic<bool> ready[kMaxDevices];       // setting the attribute twice is harmless
+    if (!ready[di->dev].load()) {
+        const cudaError_t e =
+            cudaFuncSetAttribute(bgemv_kernel<XT, R, S2>, cudaFuncAttributeMaxDynamicSharedMemorySize, di->smem_optin);
         if (e != cudaSuccess) return e;
-        if (dev < 64) ready[dev].store(true);
+        ready[di->dev].store(true);
     }
     return cudaLaunchKernelEx(&cfg, bgemv_kernel<XT, R, S2>, p);
 }
 
 template <int XT>
-cudaError_t launch_xt(int R, bool s2, const cudaLaunchConfig_t& cfg, const BGemvParams& p, int smem_max)
+cudaError_t launch_xt(int R, bool s2, const cudaLaunchConfig_t& cfg, const BGemvParams& p, const DeviceInfo* di)
 {
-    if (s2) return R == 1 ? launch_one<XT, 1, true>(cfg, p, smem_max) : launch_one<XT, 2, true>(cfg, p, smem_max);
+    if (s2) return R == 1 ? launch_one<XT, 1, true>(cfg, p, di) : launch_one<XT, 2, true>(cfg, p, di);
     switch (R) {
-        case 1: return launch_one<XT, 1, false>(cfg, p, smem_max);
-        case 2: return launch_one<XT, 2, false>(cfg, p, smem_max);
-        case 3: return launch_one<XT, 3, false>(cfg, p, smem_max);
-        default: return launch_one<XT, 4, false>(cfg, p, smem_max);
+        case 1: return launch_one<XT, 1, false>(cfg, p, di);
+        case 2: return launch_one<XT, 2, false>(cfg, p, di);
+        case 3: return launch_one<XT, 3, false>(cfg, p, di);
+        default: return launch_one<XT, 4, false>(cfg, p, di);
     }
 }
 
 template <int XT, int R, bool TAIL>
-cudaError_t launch_tma(const cudaLaunchConfig_t& cfg, const CUtensorMap* tm, const TGemvParams& p, int smem_max)
+cudaError_t launch_tma(const cudaLaunchConfig_t& cfg, const CUtensorMap* tm, const TGemvParams& p, const DeviceInfo* di)
 {
-    static std::atomic<bool> ready[64];                // per device; setting the attribute twice is harmless
-    int dev = 0;
-    cudaError_t e = cudaGetDevice(&dev);
-    if (e != cudaSuccess) return e;
-    if (dev >= 64 || !ready[dev].load()) {
-        e = cudaFuncSetAttribute(bgemv_tma_kernel<XT, R, TAIL>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_max);
+    static std::atomic<bool> ready[kMaxDevices];       // setting the attribute twice is harmless
+    if (!ready[di->dev].load()) {
+        const cudaError_t e =
+            cudaFuncSetAttribute(bgemv_tma_kernel<XT, R, TAIL>, cudaFuncAttributeMaxDynamicSharedMemorySize, di->smem_optin);
         if (e != cudaSuccess) return e;
-        if (dev < 64) ready[dev].store(true);
+        ready[di->dev].store(true);
     }
-    return cudaLaunchKernelEx(&cfg, bgemv_tma_kernel<XT, R, TAIL>, tm[0], tm[1], tm[2], tm[3], tm[4], p);
+    TMaps<TAIL> t;
+    std::copy(tm, tm + (TAIL ? 5 : 3), t.m);
+    return cudaLaunchKernelEx(&cfg, bgemv_tma_kernel<XT, R, TAIL>, t, p);
 }
 
 template <int XT>
-cudaError_t launch_tma_xt(int R, const cudaLaunchConfig_t& cfg, const CUtensorMap* tm, const TGemvParams& p, int smem_max)
+cudaError_t launch_tma_xt(int R, const cudaLaunchConfig_t& cfg, const CUtensorMap* tm, const TGemvParams& p, const DeviceInfo* di)
 {
     if constexpr (XT == 4)
-        if (p.g.tails != 0) return launch_tma<XT, 2, true>(cfg, tm, p, smem_max);    // one slice: 32 rows a warp at most
-    if (R == 1) return launch_tma<XT, 1, false>(cfg, tm, p, smem_max);
+        if (p.g.tails != 0) return launch_tma<XT, 2, true>(cfg, tm, p, di);    // one slice: 32 rows a warp at most
+    if (R == 1) return launch_tma<XT, 1, false>(cfg, tm, p, di);
     if constexpr (XT != 2)
-        if (R == 3) return launch_tma<XT, 3, false>(cfg, tm, p, smem_max);
-    return launch_tma<XT, 2, false>(cfg, tm, p, smem_max);
+        if (R == 3) return launch_tma<XT, 3, false>(cfg, tm, p, di);
+    return launch_tma<XT, 2, false>(cfg, tm, p, di);
+}
+
+// The launch shape of a GEMV's sizes, kept by this thread for its next call of
+// the same ones: the search takes 0.7 us.  (Host time of a small batch 3-4 call:
+// 3.6 us on the CUDA-core kernel, 4.7 here with a search a call, 3.9 now; the
+// rest is three tensor maps, which hold the call's pointers.)
+const TilePlan* gemv_plan(const DeviceInfo* di, int N, int K, int XT)
+{
+    struct Kept {
+        int N = 0, K = 0, XT = 0, sms = 0, smem = 0;
+        TilePlan plan;
+    };
+    thread_local Kept kept[64];
+    const uint32_t h = (static_cast<uint32_t>(N) * 2654435761u) ^ (static_cast<uint32_t>(K / 256 * 4 + XT) * 2246822519u);
+    Kept& k = kept[h >> 26];
+    if (k.N != N || k.K != K || k.XT != XT || k.sms != di->sm_count || k.smem != di->smem_optin) {
+        k = Kept{};
+        if (!tile_plan(di->sm_count, static_cast<size_t>(di->smem_optin), N, K, XT, false, 0, &k.plan)) return nullptr;
+        k.N = N;
+        k.K = K;
+        k.XT = XT;
+        k.sms = di->sm_count;
+        k.smem = di->smem_optin;
+    }
+    return &k.plan;
 }
 
 int launch_bgemv_tma(const DeviceInfo* di, const uint32_t* W, const uint16_t* s, const uint16_t* x, uint16_t* y, int N,
                      int K, int batch, bool check_scales, cudaStream_t stream)
 {
     const int XT = (batch + 7) / 8;
-    TilePlan b;
+    const TilePlan* plan = gemv_plan(di, N, K, XT);
     CUtensorMap tm[5];
-    if (!tile_plan(di->sm_count, static_cast<size_t>(di->smem_optin), N, K, XT, false, 0, &b) ||
-        !tile_maps(tm, W, s, x, N, K, batch, K, XT, b, false))
-        return WQ4_ERR_CUDA;
+    if (!plan || !tile_maps(tm, W, s, x, N, K, batch, K, XT, *plan, false)) return WQ4_ERR_CUDA;
+    const TilePlan& b = *plan;
     TGemvParams p;
     p.g = b.g;
     p.y = y;
@@ -580,7 +607,7 @@ int launch_bgemv_tma(const DeviceInfo* di, const uint32_t* W, const uint16_t* s,
     p.batch = batch;
     p.y4 = (N % 2) == 0 && aligned(y, 4);
     p.check = check_scales ? 1 : 0;
-    p.err = status_word();
+    p.err = di->status;
     cudaLaunchAttribute attr[1];
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr[0].val.programmaticStreamSerializationAllowed = 1;
@@ -593,10 +620,10 @@ int launch_bgemv_tma(const DeviceInfo* di, const uint32_t* W, const uint16_t* s,
     cfg.numAttrs = 1;
     cudaError_t e;
     switch (XT) {
-        case 1: e = launch_tma_xt<1>(b.R, cfg, tm, p, di->smem_optin); break;
-        case 2: e = launch_tma_xt<2>(b.R, cfg, tm, p, di->smem_optin); break;
-        case 3: e = launch_tma_xt<3>(b.R, cfg, tm, p, di->smem_optin); break;
-        default: e = launch_tma_xt<4>(b.R, cfg, tm, p, di->smem_optin); break;
+        case 1: e = launch_tma_xt<1>(b.R, cfg, tm, p, di); break;
+        case 2: e = launch_tma_xt<2>(b.R, cfg, tm, p, di); break;
+        case 3: e = launch_tma_xt<3>(b.R, cfg, tm, p, di); break;
+        default: e = launch_tma_xt<4>(b.R, cfg, tm, p, di); break;
     }
     return e == cudaSuccess ? WQ4_OK : WQ4_ERR_CUDA;
 }
@@ -736,10 +763,10 @@ int launch_bgemv(const DeviceInfo* di, const uint32_t* W, const uint16_t* s, con
     cfg.numAttrs = 1;
     cudaError_t e;
     switch (XT) {
-        case 1: e = launch_xt<1>(b.R, s2, cfg, p, di->smem_optin); break;
-        case 2: e = launch_xt<2>(b.R, s2, cfg, p, di->smem_optin); break;
-        case 3: e = launch_xt<3>(b.R, s2, cfg, p, di->smem_optin); break;
-        default: e = launch_xt<4>(b.R, s2, cfg, p, di->smem_optin); break;
+        case 1: e = launch_xt<1>(b.R, s2, cfg, p, di); break;
+        case 2: e = launch_xt<2>(b.R, s2, cfg, p, di); break;
+        case 3: e = launch_xt<3>(b.R, s2, cfg, p, di); break;
+        default: e = launch_xt<4>(b.R, s2, cfg, p, di); break;
     }
     return e == cudaSuccess ? WQ4_OK : WQ4_ERR_CUDA;
 }

@@ -465,10 +465,8 @@ __global__ void unpack_debug_kernel(const uint32_t* __restrict__ W, const uint16
 
 namespace {
 
-constexpr int kMaxDevices = 64;
 DeviceInfo g_info[kMaxDevices];
 bool g_info_ready[kMaxDevices];
-uint32_t* g_status_ptr[kMaxDevices];
 std::mutex g_mu;
 
 template <int B>
@@ -503,7 +501,8 @@ const DeviceInfo* current_device_info(int* device_out)
             return nullptr;
         void* ptr = nullptr;
         if (cudaGetSymbolAddress(&ptr, g_status_word) != cudaSuccess) return nullptr;
-        g_status_ptr[dev] = static_cast<uint32_t*>(ptr);
+        d.dev = dev;
+        d.status = static_cast<uint32_t*>(ptr);
         g_info[dev] = d;
         g_info_ready[dev] = true;
     }
@@ -512,9 +511,8 @@ const DeviceInfo* current_device_info(int* device_out)
 
 uint32_t* status_word()
 {
-    int dev = 0;
-    if (!current_device_info(&dev)) return nullptr;
-    return g_status_ptr[dev];
+    const DeviceInfo* di = current_device_info(nullptr);
+    return di ? di->status : nullptr;
 }
 
 namespace {
@@ -673,7 +671,7 @@ int launch_gemv(const uint32_t* W, const uint16_t* s, const uint16_t* x, uint16_
         p.x_bytes = mp.x_bytes;
         p.spw = mp.spw;
         p.q = mp.q;
-        p.err = status_word();
+        p.err = di->status;
         cudaLaunchAttribute attr[1];
         attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
         attr[0].val.programmaticStreamSerializationAllowed = 1;
@@ -714,7 +712,7 @@ int launch_gemv(const uint32_t* W, const uint16_t* s, const uint16_t* x, uint16_
         p.slot_bytes = static_cast<uint32_t>(slot_bytes);
         p.scales_offset = static_cast<uint32_t>(static_cast<size_t>(rps) * (K / 2));
         p.x_bytes = static_cast<uint32_t>(x_bytes);
-        p.err = status_word();
+        p.err = di->status;
         const size_t smem = kHeaderBytes + x_bytes + static_cast<size_t>(nslots) * slot_bytes;
         cudaLaunchAttribute attr[1];
         attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;

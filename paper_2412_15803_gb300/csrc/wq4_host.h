@@ -12,10 +12,14 @@
 
 namespace wq4 {
 
+constexpr int kMaxDevices = 64;
+
 struct DeviceInfo {
     int sm_count = 0;
     int smem_optin = 0;      // max dynamic shared memory per block (opt-in)
     int coop_launch = 0;     // cooperative launch supported
+    int dev = 0;             // its number
+    uint32_t* status = nullptr;   // device address of the library's status word there
 };
 
 // Properties of the current device, queried once per device.

@@ -13,6 +13,7 @@ static int g_limit[kKernels][kDevices];
 static unsigned g_word[kDevices];
 static int g_launches;
 static int g_last = -1;
+static size_t g_last_shape;
 
 static int kernel_index(const void* f)
 {
@@ -29,12 +30,14 @@ static cudaError_t launch(const void* f, dim3 grid, size_t smem)
     if (smem > 48 * 1024 && smem > (size_t)g_limit[i][g_device]) return cudaErrorInvalidValue;
     ++g_launches;
     g_last = i;
+    g_last_shape = (size_t)grid.x << 32 | smem;
     return cudaSuccess;
 }
 
 void fake_set_device(int d) { g_device = d; }
 int fake_launches(void) { return g_launches; }
 int fake_last_kernel(void) { return g_last; }
+size_t fake_last_shape(void) { return g_last_shape; }   /* grid << 32 | shared memory */
 
 cudaError_t cudaGetDevice(int* d) { *d = g_device; return cudaSuccess; }
 cudaError_t cudaGetLastError(void) { return cudaSuccess; }

@@ -10,6 +10,8 @@ import os
 import subprocess
 import sys
 
+import pytest
+
 HERE = os.path.dirname(os.path.abspath(__file__))
 
 CHILD = r"""
@@ -49,8 +51,39 @@ for c in WARPS:
     assert kernel(0, *c) == warps[c[0]], c
 """
 
+# launch shapes kept from call to call: the same in any order of sizes, and in a thread that kept none
+SHAPES = r"""
+import ctypes, random, sys, threading
+fake = ctypes.CDLL(sys.argv[1])
+fake.fake_last_shape.restype = ctypes.c_size_t
+from paper_2412_15803_gb300 import wq4
+L = wq4.load(build_if_missing=False)
+A = 1 << 40
+rng = random.Random(1)
+sizes = [(rng.randrange(1, 40000), 256 * rng.randrange(1, 57), rng.randrange(5, 33)) for _ in range(300)]
 
-def test_routes(fake_cudart):
+def shapes(order):
+    out = {}
+    for N, K, batch in order:
+        assert L.wq4_gemv(A, 2 * A, 4 * A, 8 * A, N, K, batch, None) == 0
+        out[N, K, batch] = (fake.fake_last_kernel(), fake.fake_last_shape())
+    return out
+
+first = shapes(sizes)
+assert len(set(first.values())) > 50
+for _ in range(3):
+    rng.shuffle(sizes)
+    assert shapes(sizes) == first and shapes([c for c in sizes[:100] for _ in range(2)]).items() <= first.items()
+other = []
+t = threading.Thread(target=lambda: other.append(shapes(sizes)))
+t.start()
+t.join()
+assert other == [first]
+"""
+
+
+@pytest.mark.parametrize("child", [CHILD, SHAPES], ids=["routes", "shapes"])
+def test_launches(fake_cudart, child):
     env = dict(os.environ, LD_PRELOAD=fake_cudart, PYTHONPATH=os.path.dirname(HERE))
-    r = subprocess.run([sys.executable, "-c", CHILD, fake_cudart], env=env, capture_output=True, text=True)
+    r = subprocess.run([sys.executable, "-c", child, fake_cudart], env=env, capture_output=True, text=True)
     assert r.returncode == 0, r.stderr[-2000:]
