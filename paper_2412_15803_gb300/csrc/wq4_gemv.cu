@@ -393,7 +393,7 @@ __global__ void __launch_bounds__(256) gemv_generic_kernel(const uint32_t* __res
         for (int b = 0; b < B; ++b) acc[b] = 0.f;
         // The next group's codes and scale are loaded ahead.  (Unrolled by the
         // compiler instead, four groups a turn, batch 1 took 6.3 us for 64 x 8160
-        // against 5.0, 8192 x 4128 15.7 against 13.4, 20000 x 3104 24.2 against 21.1.)
+        // against 5.0, 8192 x 4128 15.7 against 13.4, 20000 x 3104 24.2 against 21.2.)
         uint4 ncw = make_uint4(0u, 0u, 0u, 0u);
         uint16_t nsc = 0;
         if (lane < gpr) {
@@ -599,45 +599,44 @@ constexpr int64_t kMmaMinWeights = int64_t(12) << 20;
 // Batch 2-4 on the CUDA cores, or (false) the batched kernel (wq4_bgemv.cu).
 // The batched kernel takes at least eight rows a block, so with few rows most
 // of the SMs idle while a block walks all of K; here a row has a warp of its
-// own up to 8 rows an SM.  us a launch, batched / CUDA cores:
-//   batch 2: 600 x 14336 7.2 / 4.4, 1216 x 14336 8.1 / 6.3, 1216 x 8192 5.9 /
-//     4.3; below 8 Mi weights 512 x 4096 3.2 / 2.6, 2048 x 2048 2.9 / 3.0; from
-//     there on more rows take the batched kernel: 1536 x 6144 4.6 / 4.8, 16384 x
+// own up to 8 rows an SM, and a lane takes K / 1024 groups, rounded up.  us a
+// launch over copies of 520 MB, batched / CUDA cores:
+//   batch 2, few rows from 8 Mi weights on: 608 x 14336 7.1 / 4.4, 1216 x 14336
+//     8.0 / 6.2, 1216 x 8192 5.8 / 4.2, 1536 x 8192 5.3 / 5.4; below, 1024 x 4096
+//     3.8 / 2.9, 2048 x 2048 3.1 / 3.1.  More rows: 2048 x 6144 4.9 / 5.4, 16384 x
 //     3072 9.2 / 10.6, 128256 x 3072 43.8 / 57.4 (at batch 1 the kernels here stay
 //     ahead, 43.8 / 42.4).
-//   batch 3: 152 x 4608 3.3 / 3.4, 152 x 5120 3.4 / 3.4, 152 x 14336 6.8 / 4.9,
-//     608 x 4096 3.2 / 3.1, 768 x 3072 3.1 / 3.0, 1216 x 3072 3.5 / 3.1, 1280 x
-//     3072 3.0 / 3.7.
-//   batch 4: 304 x 5120 3.4 / 3.7, 304 x 6144 3.8 / 3.7, 608 x 14336 7.2 / 6.1,
-//     768 x 11008 6.3 / 6.9.
-//   Rows for two thirds of the SMs or fewer leave the next launch room to begin:
-//     batch 3 100 x 3072 2.7 / 2.5, 64 x 2048 2.2 / 2.1, batch 4 100 x 4096 3.0 /
-//     2.9.
+//   batch 3: 304 x 2560 2.7 / 2.8, 304 x 2816 2.8 / 2.8, 304 x 4096 3.2 / 3.0, 152 x
+//     14336 6.8 / 4.8, 1216 x 2048 3.1 / 2.9, 1024 x 2048 2.9 / 2.9, 1536 x 14336 7.6 /
+//     10.0; 76 x 1792 2.0 / 2.1, 76 x 2048 2.1 / 2.0.
+//   batch 4: 304 x 3840 3.1 / 3.5, 304 x 4096 3.2 / 3.1, 304 x 5120 3.5 / 3.6, 304 x
+//     8192 4.6 / 4.0, 608 x 14336 7.0 / 6.0, 768 x 14336 7.4 / 8.0, 1024 x 4096 3.7 /
+//     3.5, 1024 x 4352 4.0 / 4.2; 76 x 2048 2.1 / 1.9.
 constexpr int64_t kBatch2MinWeights = int64_t(8) << 20;
 
 bool cuda_cores(int batch, int N, int K, int sms)
 {
     const int64_t weights = static_cast<int64_t>(N) * K;
     if (batch == 2) return weights < kBatch2MinWeights || N <= 8 * sms;
-    if (batch == 3)
-        return (N <= 8 * sms && (K >= 5120 || 10 * weights >= (int64_t(22) << 20))) || (3 * N <= 2 * sms && K >= 3072) ||
-               (2 * N <= sms && K >= 2048);
-    return batch == 4 && ((N <= 4 * sms && K >= 5632) || (3 * N <= 2 * sms && K >= 4096) || (2 * N <= sms && K >= 2048));
+    if (2 * N <= sms && K >= 2048) return batch <= 4;
+    if (batch == 3) return N <= 8 * sms && (K >= 2816 || 10 * weights >= (int64_t(22) << 20));
+    return batch == 4 && K >= 4096 && N <= (K == 4096 ? 8 : 4) * sms;
 }
 
 // Rows that the bulk copies cannot take (K % 256 != 0 or unaligned scales) at
 // batch 1-2: the batched kernel's copy ring, or (false) a warp per row, which
 // reads every activation once more per row but takes every row's codes at once
-// up to 8 rows an SM.  The lines lie where the two cross, us, ring / warp per row:
-//   batch 1: 1003 x 2080 4.7 / 2.7, 40000 x 3104 45.7 / 39.2, 50000 x 3104 42.2 /
-//     46.5, 100000 x 3104 77.8 / 92.6, 20000 x 8160 56.5 / 47.7, 24000 x 8160 57.3 /
-//     56.3, 30000 x 8160 68.9 / 70.1;
-//   batch 2: 1003 x 2080 4.4 / 3.4, 3000 x 2080 6.1 / 5.6, 4000 x 2080 6.7 / 6.9,
-//     1000 x 8160 9.6 / 7.1, 1500 x 8160 10.5 / 11.0, 100000 x 3104 77.7 / 150.
-bool copy_ring(int batch, int N, int K, int sms)
+// up to 8 rows an SM.  The lines lie where the two cross, us over copies of
+// 520 MB, ring / warp per row:
+//   batch 1: 1003 x 2080 5.1 / 3.6, 40000 x 3104 45.9 / 38.7, 50000 x 3104 42.2 /
+//     47.2, 100000 x 3104 77.9 / 93.1, 20000 x 8160 56.3 / 47.7, 24000 x 8160 57.2 /
+//     56.3, 30000 x 8160 69.0 / 70.0;
+//   batch 2: 1003 x 2080 5.0 / 4.5, 3000 x 2080 6.7 / 6.3, 4000 x 2080 7.2 / 7.5,
+//     512 x 14304 12.7 / 16.2, 1000 x 8160 9.8 / 10.6, 100000 x 3104 77.9 / 150.
+bool copy_ring(int batch, int N, int K)
 {
     const int64_t weights = static_cast<int64_t>(N) * K;
-    return batch == 1 ? weights >= (int64_t(128) << 20) && K <= 4096 : weights >= (int64_t(6) << 20) && N > 8 * sms;
+    return batch == 1 ? weights >= (int64_t(128) << 20) && K <= 4096 : weights >= (int64_t(6) << 20);
 }
 
 int launch_gemv(const uint32_t* W, const uint16_t* s, const uint16_t* x, uint16_t* y, int N, int K, int batch,
@@ -732,7 +731,7 @@ int launch_gemv(const uint32_t* W, const uint16_t* s, const uint16_t* x, uint16_
             default: e = cudaLaunchKernelEx(&cfg, gemv_tma_kernel<4>, p); break;
         }
         if (e != cudaSuccess) return WQ4_ERR_CUDA;
-    } else if (copy_ring(batch, N, K, di->sm_count)) {
+    } else if (copy_ring(batch, N, K)) {
         return launch_bgemv(di, W, s, x, y, N, K, batch, stream);
     } else {
         const int warps_per_block = 8;

@@ -75,7 +75,7 @@ def test_three_row_tiles(N, K, batch):
 
 # few long rows at batch 2-4 on the CUDA cores: a row, an odd count, a warp's
 # second row, the largest of the rule; K of one set of groups more than 4096
-@pytest.mark.parametrize("batch,N,K", [(3, 1, 2048), (3, 75, 2304), (4, 76, 2048), (3, 153, 5376), (2, 1216, 7168), (3, 1215, 4352),
-                                       (4, 607, 5632), (3, 64, 28672), (4, 33, 20480)])
+@pytest.mark.parametrize("batch,N,K", [(3, 1, 2048), (3, 75, 2304), (4, 76, 2048), (3, 153, 2816), (2, 1216, 7168), (3, 1215, 4352),
+                                       (4, 607, 5632), (4, 1215, 4096), (3, 64, 28672), (4, 33, 20480)])
 def test_few_long_rows(batch, N, K):
     check(N, K, batch)

@@ -27,11 +27,11 @@ def kernel(path, batch, N, K, off=0):
     return fake.fake_last_kernel()
 
 CORES = [(2, 600, 14336), (2, 1216, 14336), (2, 1216, 8192), (2, 2048, 2048), (2, 64, 256),
-         (3, 64, 2048), (3, 76, 2048), (3, 101, 3072), (3, 152, 5120), (3, 608, 4096), (3, 768, 3072), (3, 1216, 14336),
-         (4, 64, 2048), (4, 101, 4096), (4, 152, 5632), (4, 608, 14336)]
+         (3, 64, 2048), (3, 76, 2048), (3, 77, 2816), (3, 608, 4096), (3, 1216, 2048), (3, 1216, 14336),
+         (4, 64, 2048), (4, 76, 3840), (4, 77, 4096), (4, 608, 4352), (4, 608, 14336), (4, 1216, 4096)]
 BATCHED = [(2, 1217, 14336), (2, 4096, 2048), (2, 128256, 4096),
-           (3, 64, 1792), (3, 77, 2048), (3, 102, 3072), (3, 152, 4864), (3, 608, 3584), (3, 1217, 14336), (3, 64, 256),
-           (4, 64, 1792), (4, 101, 3840), (4, 152, 5376), (4, 609, 14336), (4, 4096, 4096)]
+           (3, 76, 1792), (3, 77, 2560), (3, 1024, 2048), (3, 1217, 14336), (3, 64, 256),
+           (4, 76, 1792), (4, 77, 3840), (4, 609, 4352), (4, 609, 14336), (4, 1217, 4096), (4, 4096, 4096)]
 for c in CORES:
     assert kernel(0, *c) == kernel(2, *c) != kernel(1, *c), c
 for c in BATCHED:
@@ -41,9 +41,8 @@ for c in ((3, 64, 36864), (4, 64, 28672), (5, 64, 14336)):
     assert kernel(0, *c) == kernel(1, *c) == kernel(2, *c), c
 assert kernel(0, 3, 64, 14336, 2) == kernel(2, 3, 64, 14336, 2) != kernel(2, 3, 64, 14336)
 # rows of odd groups at batch 1-2: the copy ring of the batched kernels (as at batch 3), or a warp per row
-RING = [(1, 50000, 3104), (1, 100000, 3104), (2, 4000, 2080), (2, 1500, 8160), (2, 1217, 8160)]
-WARPS = [(1, 1003, 2080), (1, 40000, 3104), (1, 20000, 8160), (1, 30000, 8160), (2, 1003, 2080), (2, 3000, 2080), (2, 1000, 8160),
-         (2, 1216, 8160)]
+RING = [(1, 50000, 3104), (1, 100000, 3104), (2, 4000, 2080), (2, 1000, 8160), (2, 512, 14304)]
+WARPS = [(1, 1003, 2080), (1, 40000, 3104), (1, 20000, 8160), (1, 30000, 8160), (2, 1003, 2080), (2, 3000, 2080), (2, 700, 8160)]
 warps = {b: kernel(0, b, 3, 32) for b in (1, 2)}
 for c in RING:
     assert kernel(0, *c) != warps[c[0]], c
