@@ -590,6 +590,7 @@ __device__ __forceinline__ float warp_allsum(float v)
 constexpr int kAttnHeads = 4;                // heads combined at a time
 constexpr int kAttnSplitTokens = 128;
 constexpr int kAttnMaxChunk = 64;            // tokens of a ring slot, at most
+constexpr int kAttnBlk = 16;                 // tokens of a warp's block: one per lane pair
 static_assert(kHdrRes + 8 * (kAttnMaxSplits * kAttnMaxGroup + kAttnMaxGroup * kAttnD / 2 + kAttnMaxSplits) <= kChainHeader,
               "attention scratch overlaps the staged input");
 
@@ -619,10 +620,12 @@ __device__ __forceinline__ bool attn_unit(const ChainParamsA& p, int l, const in
     return true;
 }
 
-// Tokens of one ring slot (keys, then values, 256 bytes a token each).
-__device__ __forceinline__ int attn_chunk_tokens(uint32_t slot_bytes)
+// Tokens of one ring slot (keys, then values, 256 bytes a token each): whole
+// blocks of kAttnBlk.
+__host__ __device__ __forceinline__ int attn_chunk_tokens(uint32_t slot_bytes)
 {
-    return min(kAttnMaxChunk, static_cast<int>(slot_bytes / (4 * kAttnD))) & ~15;
+    const int n = static_cast<int>(slot_bytes / (4 * kAttnD));
+    return (n < kAttnMaxChunk ? n : kAttnMaxChunk) / kAttnBlk * kAttnBlk;
 }
 
 // Producer lane: the bulk copies of tokens [ta, tb) of a unit into one slot.
@@ -672,7 +675,7 @@ __device__ __forceinline__ int attention_phase(const ChainParamsA& p, int l, uin
                                              uint8_t* slots, int ord0)
 {
     constexpr int kConsumers = NW * 32;
-    constexpr int kBlk = 16;                   // tokens of a warp's block: one per lane pair
+    constexpr int kBlk = kAttnBlk;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int H = p.H, Hkv = p.Hkv, S = p.S, KD = Hkv * kAttnD;
     const float scale = p.scale * 1.4426950408889634f;   // base-2 scores
@@ -1784,9 +1787,14 @@ bool choose_parts(const Dims& d, int grid, int nw, const int spw[5], int nslots,
 
 // True when no consumer wait on the ring can alias: for every stage,
 // nslots + ceil(NW / items per slot) <= the number of full barriers (items
-// per slot = superpairs per slot x K parts).
-bool ring_ok(const Dims& d, int nslots, uint32_t slot_bytes, int nw, const int spw[5], const int q[5])
+// per slot = superpairs per slot x K parts; with attention also the blocks of
+// cached tokens in a slot, which must hold one).
+bool ring_ok(const Dims& d, int nslots, uint32_t slot_bytes, int nw, const int spw[5], const int q[5], bool att)
 {
+    if (att) {
+        const int blocks = attn_chunk_tokens(slot_bytes) / kAttnBlk;
+        if (blocks < 1 || nslots + (nw + blocks - 1) / blocks > full_bars(nslots)) return false;
+    }
     size_t wb[5];
     word_bytes(d, wb);
     for (int t = 0; t < 5; ++t) {
@@ -2060,7 +2068,7 @@ int build_plan(const wq4_layer_table* t, const wq4_decode_attn* a, Plan* pl, cud
     if (!choose_parts(d, di->sm_count, kChainWarps, spw, nslots, slot_bytes, q)) return WQ4_ERR_UNSUPPORTED;
     // fewer slots give more full barriers per slot: take the deepest ring
     // whose barriers cannot alias
-    while (nslots >= 2 && !ring_ok(d, nslots, slot_bytes, kChainWarps, spw, q)) --nslots;
+    while (nslots >= 2 && !ring_ok(d, nslots, slot_bytes, kChainWarps, spw, q, a != nullptr)) --nslots;
     if (nslots < 2) return WQ4_ERR_UNSUPPORTED;
     const size_t smem = header + x_bytes + static_cast<size_t>(nslots) * slot_bytes + rope_bytes;
     pl->rope_off = static_cast<uint32_t>(header + x_bytes + static_cast<size_t>(nslots) * slot_bytes);

@@ -121,7 +121,9 @@ def simulate(stages, nslots, nbars, nw, rng):
 
 def plan_nbars(nslots, stages, nw, max_bars=48):
     """The planner's choice: the largest multiple of nslots up to 48 barriers,
-    accepted only if nslots + ceil(nw / ips) <= nbars for every stage."""
+    accepted only if nslots + ceil(nw / ips) <= nbars for every stage (the decode
+    step's cached tokens are a stage of 16-token blocks, slot bytes / 8192 a chunk
+    and at most four)."""
     nbars = (max_bars // nslots) * nslots
     ok = all(nslots + math.ceil(nw / ips) <= nbars for _, ips in stages)
     return nbars, ok
@@ -133,8 +135,16 @@ LAYER_8B = [(21, 4), (14, 4), (48, 2), (14, 1)]
 NARROW = [(3, 1), (2, 1), (5, 1), (1, 1)]
 
 
-@pytest.mark.parametrize("layer", [LAYER_3B, LAYER_8B, NARROW])
-@pytest.mark.parametrize("nslots", [3, 6, 9, 12, 16])
+# the decode step: blocks of cached tokens between QKV and O, few to many a CTA
+# (a range of one block, of more than the ring holds), none in a CTA without one
+STEP_SHORT = [(17, 5), (1, 2), (10, 5), (27, 2), (10, 2)]
+STEP_LONG = [(17, 5), (130, 4), (10, 5), (27, 2), (10, 2)]
+STEP_NARROW = [(3, 1), (37, 1), (2, 1), (5, 1), (1, 1)]
+STEP_NONE = [(3, 1), (0, 2), (2, 1), (5, 1), (1, 1)]
+
+
+@pytest.mark.parametrize("layer", [LAYER_3B, LAYER_8B, NARROW, STEP_SHORT, STEP_LONG, STEP_NARROW, STEP_NONE])
+@pytest.mark.parametrize("nslots", [3, 6, 9, 12, 13, 16])
 def test_no_aliased_wait_under_the_planner_rule(layer, nslots):
     stages = layer * 4 + [(211, 4)]
     nbars, ok = plan_nbars(nslots, stages, 15)
@@ -152,6 +162,17 @@ def test_waits_alias_when_barriers_equal_slots():
     rng = random.Random(7)
     total = sum(simulate(stages, 4, 4, 15, rng) for _ in range(40))
     assert total > 0
+
+
+def test_waits_alias_without_the_rule_for_cached_tokens():
+    """The rule kept for the weights alone (five items a chunk, 8 barriers) does
+    not hold for one block of cached tokens a chunk."""
+    layer = [(17, 5), (61, 1), (10, 5)]
+    nslots, nbars = 4, 8
+    assert all(nslots + math.ceil(15 / ips) <= nbars for _, ips in (layer[0], layer[2]))
+    assert nslots + math.ceil(15 / layer[1][1]) > nbars
+    rng = random.Random(11)
+    assert sum(simulate(layer * 4, nslots, nbars, 15, rng) for _ in range(40)) > 0
 
 
 def test_model_has_no_false_alarms_in_lockstep():
