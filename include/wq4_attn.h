@@ -122,7 +122,9 @@ int wq4_kv_append(const wq4_kv_cache* cache, const uint16_t* new_k, const uint16
  *                all with the table's n_kv_heads, head_dim 128 and one common
  *                page_size (a multiple of 16); page tables [batch][stride].
  *                Sequences of a batch must not map their new positions to
- *                the same cache row.
+ *                the same cache row.  (One may map another's new position as
+ *                a token that it has cached, as two consecutive tokens of one
+ *                sequence do: it attends to the new key and value.)
  *   positions  : device int32 [batch]: the new token's place in its sequence
  *                (the number of tokens already cached).
  *   rope_theta : rotary base (> 1; Llama-3.x 500000, Phi-3.5 10000).

@@ -594,6 +594,17 @@ constexpr int kAttnBlk = 16;                 // tokens of a warp's block: one pe
 static_assert(kHdrRes + 8 * (kAttnMaxSplits * kAttnMaxGroup + kAttnMaxGroup * kAttnD / 2 + kAttnMaxSplits) <= kChainHeader,
               "attention scratch overlaps the staged input");
 
+// After the ring: the rotation table, the rows' positions and, at batch 2, the
+// shared tokens of every slot (see AttnShared).
+template <int B>
+__host__ __device__ constexpr uint32_t attn_pos_off() { return B * (kAttnD / 2) * sizeof(double2); }
+template <int B>
+__host__ __device__ constexpr uint32_t attn_shared_off() { return attn_pos_off<B>() + 16; }
+constexpr size_t attn_tail_bytes(int B)
+{
+    return static_cast<size_t>(B) * (kAttnD / 2) * sizeof(double2) + 16 + (B == 2 ? 8 * kChainMaxSlots : 0);
+}
+
 struct AttnUnit {
     int b, h, c, Sb, pos;
     int t0, t1;          // the range's tokens
@@ -628,13 +639,72 @@ __host__ __device__ __forceinline__ int attn_chunk_tokens(uint32_t slot_bytes)
     return (n < kAttnMaxChunk ? n : kAttnMaxChunk) / kAttnBlk * kAttnBlk;
 }
 
-// Producer lane: the bulk copies of tokens [ta, tb) of a unit into one slot.
-// Rows of a page id outside the pool become zeros (and are flagged).
-__device__ __forceinline__ void attn_copy(const ChainParamsA& p, int l, const AttnUnit& a, int ta, int tb, int ct,
-                                          uint8_t* dst, uint64_t* fb, uint64_t pol)
+// Batch 2: one row's new token may be a cached token of the other (two tokens
+// of one sequence in a step, a page in both).  The copies into the ring run
+// ahead of it, so the producer notes such tokens of a slot, 16 bits a block, and
+// the warp that takes the block puts the other row's new key and value in their
+// place.
+struct AttnShared {
+    int page = -1, off = 0;       // the other row's new token: its page (-1: none), its row there
+    uint64_t* tokens = nullptr;   // of this slot
+};
+
+template <int B>
+__device__ __forceinline__ AttnShared attn_shared(const ChainParamsA& p, int l, const AttnUnit& a, const int* pos_sh)
+{
+    AttnShared s;
+    if constexpr (B == 2) {
+        const KvLayer& kv = p.kv[l];
+        const int pos = pos_sh[1 - a.b];
+        if (pos >= 0 && pos / p.P < kv.pt_stride) {
+            s.page = __ldg(kv.pt + static_cast<size_t>(1 - a.b) * kv.pt_stride + pos / p.P);
+            s.off = pos % p.P;
+        }
+    }
+    return s;
+}
+
+// The tokens of [ta, tb) of row b, from page p0 on, that are the other row's new
+// one, as bits from ta (out of the producer's loop: it runs into nearly none).
+__device__ __noinline__ uint64_t attn_shared_tokens(const KvLayer& kv, int P, int b, int p0, int ta, int tb, int page, int off)
+{
+    uint64_t bits = 0;
+    for (int pi = p0; pi * P < tb; ++pi) {
+        const int t = pi * P + off;
+        if (t >= ta && t < tb && __ldg(kv.pt + static_cast<size_t>(b) * kv.pt_stride + pi) == page) bits |= 1ull << (t - ta);
+    }
+    return bits;
+}
+
+// The other row's new key and value over rows `tokens` of a block (keys at ka,
+// values at va in shared memory), by one warp.
+__device__ __noinline__ void attn_place_shared(const ChainParamsA& p, int l, int other, int h, uint32_t ka, uint32_t va,
+                                               uint32_t tokens, uint32_t epoch)
+{
+    const int lane = threadIdx.x & 31;
+    const size_t at = (static_cast<size_t>(l) * 2 + other) * (p.Hkv * (kAttnD / 2)) + h * (kAttnD / 2) + 2 * lane;
+    uint32_t w[4];
+#pragma unroll
+    for (int i = 0; i < 4; ++i)
+        w[i] = ll_load((i < 2 ? p.llK : p.llVn) + at + (i & 1), epoch, epoch, p.err, p.abort, p.wait_ns);
+    for (; tokens; tokens &= tokens - 1) {
+        const uint32_t row = (__ffs(tokens) - 1) * (2 * kAttnD) + 8 * lane;
+        asm volatile("st.shared.v2.b32 [%0], {%1, %2};" ::"r"(ka + row), "r"(w[0]), "r"(w[1]) : "memory");
+        asm volatile("st.shared.v2.b32 [%0], {%1, %2};" ::"r"(va + row), "r"(w[2]), "r"(w[3]) : "memory");
+    }
+    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");   // before a later copy into the slot
+    __syncwarp();
+}
+
+// Producer lane: the bulk copies of tokens [ta, tb) of a unit, from its page p0
+// on, into one slot.  Rows of a page id outside the pool become zeros (and are flagged).
+template <int B>
+__device__ __forceinline__ void attn_copy(const ChainParamsA& p, int l, const AttnUnit& a, int p0, int ta, int tb, int ct,
+                                          uint8_t* dst, uint64_t* fb, uint64_t pol, const AttnShared& sh)
 {
     const KvLayer& kv = p.kv[l];
-    const int P = p.P, p0 = ta / P;
+    const int P = p.P;
+    [[maybe_unused]] bool hit = false;
     const int32_t* pt = kv.pt + static_cast<size_t>(a.b) * kv.pt_stride + p0;
     constexpr int kRuns = kAttnMaxChunk / 16 + 1;               // pages of at least 16 tokens
     uint32_t bytes = 0;
@@ -647,6 +717,7 @@ __device__ __forceinline__ void attn_copy(const ChainParamsA& p, int l, const At
             if (page >= 0 && page < kv.num_pages) {
                 bytes += static_cast<uint32_t>(x1 - x0) * (4 * kAttnD);
                 good |= 1u << i;
+                if constexpr (B == 2) hit = hit || page == sh.page;
             } else {
                 atomicOr(p.err, kErrPageId);
                 uint4* kz = reinterpret_cast<uint4*>(dst + (x0 - ta) * (2 * kAttnD));
@@ -656,6 +727,7 @@ __device__ __forceinline__ void attn_copy(const ChainParamsA& p, int l, const At
             }
         }
     }
+    if constexpr (B == 2) *sh.tokens = hit ? attn_shared_tokens(kv, P, a.b, p0, ta, tb, sh.page, sh.off) : 0;
     mbar_arrive_expect_tx(fb, bytes);
 #pragma unroll 1
     for (int i = 0; i < kRuns; ++i) {
@@ -735,6 +807,10 @@ __device__ __forceinline__ int attention_phase(const ChainParamsA& p, int l, uin
             const uint32_t va = ka + ct * (2 * kAttnD);
             const int nb = min(kBlk, au.te - (au.t0 + it * kBlk));
             const bool valid = ti < nb;
+            if constexpr (B == 2) {
+                const uint32_t shared = reinterpret_cast<const uint16_t*>(smem + p.rope_off + attn_shared_off<B>())[4 * slot + it - i0];
+                if (shared) attn_place_shared(p, l, 1 - b, h, ka, va, shared, epoch);
+            }
             float sp[G][2];
 #pragma unroll
             for (int j = 0; j < G; ++j) sp[j][0] = sp[j][1] = 0.f;
@@ -984,7 +1060,7 @@ __global__ void __launch_bounds__((NW + 1) * 32, 1)
     // decode step: the rotation table (cos, sin of pos * theta^(-2i/128) per
     // row, fp64) and the rows' positions (-1 for an invalid one), after the
     // ring; their addresses are recomputed where used (no registers held)
-    constexpr uint32_t kPosOff = B * (kAttnD / 2) * sizeof(double2);
+    constexpr uint32_t kPosOff = attn_pos_off<B>();
     if constexpr (ATT != 0) {
         rope_table<B>(p, reinterpret_cast<double2*>(smem + p.rope_off));
         int* pos_sh = reinterpret_cast<int*>(smem + p.rope_off + kPosOff);
@@ -1023,6 +1099,15 @@ __global__ void __launch_bounds__((NW + 1) * 32, 1)
             int ord = 0;                // ring ordinal of the next chunk
             int slot = 0, round = 0;    // its slot and the slot's use count
             int fbi = 0;                // its full barrier
+            // Cached tokens of a chunk, its whole pages and the rest.  (This lane's
+            // instructions bound long contexts: a chunk's first page is carried on, a
+            // division a chunk cost more than the look for shared tokens.)
+            [[maybe_unused]] int ct = 0, ctp = 0, ctr = 0;
+            if constexpr (ATT != 0) {
+                ct = attn_chunk_tokens(p.slot_bytes);
+                ctp = ct / p.P;
+                ctr = ct - ctp * p.P;
+            }
             for (int st = 0; st < nstages; ++st) {
                 const Stage g = stage_at(p, st);
                 const StageInfo in = info[g.type];
@@ -1032,14 +1117,22 @@ __global__ void __launch_bounds__((NW + 1) * 32, 1)
                     // the cached keys and values of this CTA's attention ranges
                     if (g.type == kO) {
                         const int* pos_sh = reinterpret_cast<const int*>(smem + p.rope_off + kPosOff);
-                        const int ct = attn_chunk_tokens(p.slot_bytes);
                         for (int u = blockIdx.x; u < B * p.Hkv * p.S; u += gridDim.x) {
                             AttnUnit au;
                             if (!attn_unit<B>(p, g.layer, pos_sh, u, &au)) continue;
+                            AttnShared sh = attn_shared<B>(p, g.layer, au, pos_sh);
+                            int p0 = au.t0 / p.P, row = au.t0 - p0 * p.P;
                             for (int ta = au.t0; ta < au.te; ta += ct, ++ord) {
                                 if (round > 0) mbar_wait(&empty[slot], (round - 1) & 1, p.err);
-                                attn_copy(p, g.layer, au, ta, min(au.te, ta + ct), ct,
-                                          slots + static_cast<size_t>(slot) * p.slot_bytes, &full[fbi], pol);
+                                if constexpr (B == 2)
+                                    sh.tokens = reinterpret_cast<uint64_t*>(smem + p.rope_off + attn_shared_off<B>()) + slot;
+                                attn_copy<B>(p, g.layer, au, p0, ta, min(au.te, ta + ct), ct,
+                                             slots + static_cast<size_t>(slot) * p.slot_bytes, &full[fbi], pol, sh);
+                                p0 += ctp;
+                                if ((row += ctr) >= p.P) {
+                                    row -= p.P;
+                                    ++p0;
+                                }
                                 if (++slot == p.nslots) {
                                     slot = 0;
                                     ++round;
@@ -2052,8 +2145,7 @@ int build_plan(const wq4_layer_table* t, const wq4_decode_attn* a, Plan* pl, cud
         xb = std::max(xb, align_up(4 * static_cast<size_t>(G * kAttnD + std::min(G, kAttnHeads) * kChainWarps * kAttnPart), 128));
     }
     const uint32_t x_bytes = static_cast<uint32_t>(xb);
-    // the rotation table (double2 [B][64]), the positions and a flag sit after the ring
-    const size_t rope_bytes = a ? align_up(static_cast<size_t>(d.B) * (kAttnD / 2) * 16 + 16, 128) : 0;
+    const size_t rope_bytes = a ? align_up(attn_tail_bytes(d.B), 128) : 0;
     // the residual words of a CTA's words must fit in shared memory
     if (static_cast<long>((d.H / 2 + di->sm_count - 1) / di->sm_count) * d.B > kMaxResWords) return WQ4_ERR_UNSUPPORTED;
     int spw[5];
