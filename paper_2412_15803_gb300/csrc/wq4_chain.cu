@@ -156,6 +156,14 @@ static_assert(sizeof(ChainParams) <= 32764, "kernel parameter space");
 constexpr int kAttnD = 128;          // head dimension
 constexpr int kAttnMaxGroup = 8;     // query heads per kv head
 constexpr int kAttnMaxSplits = 32;   // token ranges per (row, kv head)
+// ... and as many as give each of these many SMs one (the 152 of the chip and a
+// few): the workspace's size holds without a device.
+constexpr int kAttnSms = 160;
+inline int attn_splits(int B, int Hkv)
+{
+    const int s = kAttnSms / (B * Hkv);
+    return s < 1 ? 1 : (s > kAttnMaxSplits ? kAttnMaxSplits : s);
+}
 constexpr int kAttnPart = kAttnD + 4;   // floats of one split partial: o[128], m, l, pad
 
 struct KvLayer {
@@ -1669,7 +1677,7 @@ Layout make_layout(const Dims& d, bool att = false, size_t attn_ws_bytes = 0)
         y.llK = take(8 * L * B * (KD / 2));
         y.llVn = take(8 * L * B * (KD / 2));
         y.llAt = take(8 * 2 * L * B * (H / 2));          // two replicas
-        if (d.B <= kMaxChainBatch) y.apart = take(8 * L * B * d.Hkv * kAttnMaxSplits * G * kAttnPart);
+        if (d.B <= kMaxChainBatch) y.apart = take(8 * L * B * d.Hkv * attn_splits(d.B, d.Hkv) * G * kAttnPart);
         y.att_ll_end = o;
         y.pQr = take(2 * L * B * H);
         y.pKr = take(2 * L * B * KD);
@@ -2165,8 +2173,8 @@ int build_plan(const wq4_layer_table* t, const wq4_decode_attn* a, Plan* pl, cud
     const size_t smem = header + x_bytes + static_cast<size_t>(nslots) * slot_bytes + rope_bytes;
     pl->rope_off = static_cast<uint32_t>(header + x_bytes + static_cast<size_t>(nslots) * slot_bytes);
     if (a) {
-        int S = di->sm_count / (d.B * d.Hkv);
-        pl->S = S < 1 ? 1 : (S > kAttnMaxSplits ? kAttnMaxSplits : S);
+        const int S = di->sm_count / (d.B * d.Hkv);
+        pl->S = S < 1 ? 1 : std::min(S, attn_splits(d.B, d.Hkv));
     }
     // The limit is a property of the kernel, shared by every plan: set it to
     // the device maximum so that no plan's launch depends on which plan was

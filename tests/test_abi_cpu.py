@@ -224,3 +224,23 @@ def test_gemv_path_hook_rejects_bad_values():
     assert lib.wq4_test_gemv_path(-1) == wq4.WQ4_ERR_INVALID
     assert lib.wq4_test_gemv_path(3) == wq4.WQ4_ERR_INVALID
     assert lib.wq4_test_gemv_path(0) == wq4.WQ4_OK
+
+
+# (hidden, ffn, q heads, kv heads, layers): the 3B and the 8B shape, many kv heads, one
+@pytest.mark.parametrize("shape", [(3072, 8192, 24, 8, 28), (4096, 14336, 32, 8, 32), (4096, 14336, 32, 32, 4), (1024, 512, 8, 1, 4)])
+@pytest.mark.parametrize("batch", [1, 2])
+def test_step_workspace_holds_the_ranges_a_step_can_have(shape, batch):
+    """Beside the chain's workspace: flagged keys, values and outputs, their plain
+    copies, and per layer, row and head a flagged partial of every range (one an
+    SM, at most 32)."""
+    H, F, nq, nkv, L = shape
+    layers = (wq4.wq4_layer * L)()
+    t, _ = _table(hidden=H, ffn=F, n_q_heads=nq, n_kv_heads=nkv, num_layers=L, batch=batch)
+    t.layers = layers
+    lib = wq4.load()
+    KD = nkv * 128
+    words = L * batch * (2 * (KD // 2) * 8 + 2 * (H // 2) * 8 + 2 * (2 * H + KD))
+    ranges = min(32, max(1, 160 // (batch * nkv)))
+    partials = 8 * L * batch * nq * ranges * 132
+    extra = lib.wq4_decode_step_workspace_bytes(ctypes.byref(t)) - lib.wq4_chain_workspace_bytes(ctypes.byref(t))
+    assert words + partials <= extra <= words + partials + 16 * 256
