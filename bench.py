@@ -88,18 +88,37 @@ def measured_peak():
         return FALLBACK_HBM_GBS, "fallback"
 
 
+CSRC = os.path.join(ROOT, "paper_2412_15803_gb300", "csrc")
+
+# The files that decide a kernel's traffic: its own and the one with its launch
+# shapes (tile_plan and tile_maps of wq4_bgemv.cu); what they include counts too.
 KERNEL_SOURCES = {
-    "chain_kernel": ("wq4_chain.cu", "wq4_items.cuh", "wq4_device.cuh"),
-    "stage_kernel": ("wq4_stage.cu", "wq4_tiles.cuh", "wq4_items.cuh", "wq4_device.cuh"),
+    "chain_kernel": ("wq4_chain.cu",),
+    "stage_kernel": ("wq4_stage.cu", "wq4_bgemv.cu"),
+    "gemv_kernels": ("wq4_gemv.cu", "wq4_bgemv.cu"),
+    "paged_attn_kernel": ("wq4_attn.cu",),
+    "gemm_kernel": ("wq4_gemm.cu",),
 }
 
 
-def chain_source_sha(kernel: str) -> str:
+def kernel_files(kernel: str) -> list[str]:
+    """The kernel's source files and every header of the library that they include."""
+    files, todo = [], list(KERNEL_SOURCES[kernel])
+    while todo:
+        f = todo.pop(0)
+        if f not in files:
+            files.append(f)
+            text = open(os.path.join(CSRC, f)).read()
+            todo += [h for h in re.findall(r'#include "([^"]+)"', text) if os.path.exists(os.path.join(CSRC, h))]
+    return files
+
+
+def source_sha(kernel: str) -> str:
     """Hash of the sources of one kernel (the committed ncu summary of that
     kernel carries the same hash)."""
     h = hashlib.sha256()
-    for f in KERNEL_SOURCES[kernel]:
-        h.update(open(os.path.join(ROOT, "paper_2412_15803_gb300", "csrc", f), "rb").read())
+    for f in kernel_files(kernel):
+        h.update(open(os.path.join(CSRC, f), "rb").read())
     return h.hexdigest()[:16]
 
 
@@ -113,7 +132,7 @@ def profiled_traffic(name: str, workload: str, batch: int, context: int = 0):
     text = open(path).read()
     m = re.search(r"traffic_bytes_per_launch:\s*(\d+)", text)
     s = re.search(r"source_sha:\s*([0-9a-f]+)", text)
-    if not m or not s or s.group(1) != chain_source_sha(name):
+    if not m or not s or s.group(1) != source_sha(name):
         return None
     return int(m.group(1))
 
@@ -563,13 +582,6 @@ def gemv_io_bytes(mats, B: int) -> int:
     return sum(2 * B * (N + K) for _, N, K in mats)
 
 
-def gemv_source_sha() -> str:
-    h = hashlib.sha256()
-    for f in ("wq4_gemv.cu", "wq4_bgemv.cu", "wq4_items.cuh", "wq4_device.cuh"):
-        h.update(open(os.path.join(ROOT, "paper_2412_15803_gb300", "csrc", f), "rb").read())
-    return h.hexdigest()[:16]
-
-
 def gemv_profiled_traffic(workload: str):
     path = os.path.join(ROOT, "profiles", f"gemv_kernels_{workload}.md")
     if not os.path.exists(path):
@@ -577,7 +589,7 @@ def gemv_profiled_traffic(workload: str):
     text = open(path).read()
     m = re.search(r"traffic_bytes_per_set:\s*(\d+)", text)
     h = re.search(r"source_sha:\s*([0-9a-f]+)", text)
-    if not m or not h or h.group(1) != gemv_source_sha():
+    if not m or not h or h.group(1) != source_sha("gemv_kernels"):
         return None
     return int(m.group(1))
 
@@ -812,13 +824,6 @@ def run_gemv(args, rank, world, local):
 ATTN_METRIC = "paged decode attention sequences/s (one decode step per sequence) and achieved HBM GB/s"
 
 
-def attn_source_sha() -> str:
-    h = hashlib.sha256()
-    for f in ("wq4_attn.cu", "wq4_device.cuh"):
-        h.update(open(os.path.join(ROOT, "paper_2412_15803_gb300", "csrc", f), "rb").read())
-    return h.hexdigest()[:16]
-
-
 def attn_profiled_traffic(workload: str):
     path = os.path.join(ROOT, "profiles", f"paged_attn_kernel_{workload}.md")
     if not os.path.exists(path):
@@ -826,7 +831,7 @@ def attn_profiled_traffic(workload: str):
     text = open(path).read()
     m = re.search(r"traffic_bytes_per_launch:\s*(\d+)", text)
     s = re.search(r"source_sha:\s*([0-9a-f]+)", text)
-    if not m or not s or s.group(1) != attn_source_sha():
+    if not m or not s or s.group(1) != source_sha("paged_attn_kernel"):
         return None
     return int(m.group(1))
 
