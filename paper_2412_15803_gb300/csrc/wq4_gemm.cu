@@ -23,11 +23,12 @@
 // What bounds it: over long prompts the power limit (28672 x 4096 over 2048
 // tokens: 363 -> 311 us, 1.55 PFLOP/s; in a loop the SMs settle at 1.42 GHz,
 // where 256-token tiles run at 87 % of the MMA rate), over short ones the MMA
-// issuer's own latency (~340 cycles a 64-wide chunk) and the launch.  Before,
-// each 64-wide chunk cost the issuer ~870 cycles whatever the tile: one lane's
-// branch with two waits and two commits for four MMAs.  5120 x 3072 over 77
-// tokens 22.7 -> 9.5 us, 3072 x 8192 over 1000 tokens 57 -> 39, 512 x 14336
-// over 200 tokens 91 -> 11.3.
+// issuer's own latency (~340 cycles a 64-wide chunk), the launch and the first
+// weights, which are copied after the previous kernel.  Before, each 64-wide
+// chunk cost the issuer ~870 cycles whatever the tile: one lane's branch with
+// two waits and two commits for four MMAs.  5120 x 3072 over 77 tokens 22.7 ->
+// 9.9 us, 3072 x 8192 over 1000 tokens 57 -> 36.7, 512 x 14336 over 200 tokens
+// 91 -> 12.2.
 #include "wq4.h"
 #include "wq4_device.cuh"
 #include "wq4_host.h"
@@ -64,7 +65,7 @@ struct GCfg {
     static constexpr int kX = TOK * 2 * (128 / kXSub);            // activation slot: boxes of TOK tokens x 64 K fp16
     static constexpr int kW = kGCodes + kGScales;
     static constexpr int kXSlots = TOK == 256 ? 4 : (TOK == 192 ? 5 : (TOK == 128 ? 4 : 6));
-    static constexpr int kWSlots = TOK == 256 ? 3 : 3;
+    static constexpr int kWSlots = 3;
     static constexpr int kT = kGHeader;                           // two transpose blocks: kGBlk tokens x 128 outputs fp16
     static constexpr int kXRing = kT + 2 * kGBlk * 128 * 2;
     static constexpr int kWRing = kXRing + kXSlots * kX;
@@ -195,8 +196,8 @@ __global__ void __launch_bounds__(kGThreads, 1)
             tc::prefetch_map(&tm_scales);
             // The previous kernel may write the weights too: they are fetched into
             // L2 while it finishes and copied after it.  (Copied before, they would be
-            // dequantized by the time it ends: 5120 x 3072 over 77 tokens 11.8 -> 10.9
-            // us between calls, 128 x 256 over 17 3.2 -> 2.6.)
+            // dequantized by the time it ends: 1024 x 1024 over 64 tokens 5.4 -> 4.2 us
+            // in a row of calls, 128 x 256 over 17 3.2 -> 2.6.)
             if (u0 < tiles)
                 for (int k = k0; k < min(k1, k0 + WS); ++k) {
                     tc::tma_prefetch_2d(&tm_codes, k * 128, (u0 / a.ttiles) * 128);
@@ -486,18 +487,21 @@ struct GemmPlan {
 };
 
 // Token tile and K split: the least estimated time.  Per 64-wide K chunk a
-// tile takes (us, one CTA alone .. every SM busy) 0.165 .. 0.18 with 64
-// tokens, 0.177 .. 0.22 with 128, 0.214 .. 0.304 with 192 and 0.287 .. 0.394
-// with 256, beside a launch's fixed 1.8, 2.3, 3.3 and 4; a split (the
+// tile takes (us, one CTA alone .. every SM busy) 0.188 .. 0.205 with 64
+// tokens, 0.203 .. 0.235 with 128, 0.22 .. 0.285 with 192 and 0.287 .. 0.394
+// with 256, beside a launch's fixed 2.3, 2.65, 3.4 and 4.2; a split (the
 // cluster's CTAs take K blocks in order, one tile a cluster, all resident)
-// adds 1.7 and 0.025 a CTA.  Measured: 5120 x 3072 over 77 tokens 10.8 us
-// whole, 9.5 split in 3; 512 x 14336 over 200 tokens 42 whole, 11.3 split in 8;
-// 1024 x 1024 over 77 tokens 4.9 whole, 5.8 split in 2.
+// adds 1.3, 1.5 or 1.7 and 0.016, 0.023 or 0.03 a CTA.  Fitted to every choice
+// over 34 sizes, each over copies of 520 MB: the picks are 0.1 % from the best on
+// average, 3 % at most.  Measured: 5120 x 3072 over 77 tokens 11.6 us whole, 9.9
+// split in 3; 512 x 14336 over 200 tokens 42 whole, 12.2 split in 8; 1024 x 1024
+// over 300 tokens 5.6 whole, 6.4 split in 2.
 GemmPlan pick_gemm(int N, int K, int M, int sms, int dev)
 {
     static constexpr int kTok[4] = {64, 128, 192, 256};
-    static constexpr double kB0[4] = {0.165, 0.177, 0.214, 0.287}, kB1[4] = {0.18, 0.22, 0.304, 0.394};
-    static constexpr double kFix[4] = {1.8, 2.3, 3.3, 4.0};
+    static constexpr double kB0[4] = {0.188, 0.203, 0.22, 0.287}, kB1[4] = {0.205, 0.235, 0.285, 0.394};
+    static constexpr double kFix[4] = {2.3, 2.65, 3.4, 4.2};
+    static constexpr double kSplit[4] = {1.3, 1.5, 1.7, 1.7}, kCta[4] = {0.0155, 0.023, 0.03, 0.03};
     GemmPlan best;
     double best_t = 1e300;
     const int nblk = K >> 8;
@@ -512,7 +516,7 @@ GemmPlan pick_gemm(int N, int K, int M, int sms, int dev)
                 t += nch * (full * kB1[i] + (rest ? rate(static_cast<double>(rest)) : 0.0)) + 0.6 * full;
             } else {
                 if (tiles * s > sms) break;
-                t += nch * rate(static_cast<double>(tiles * s)) + 1.7 + 0.025 * (tiles * s) * (i >= 2 ? 1.2 : 1.0);
+                t += nch * rate(static_cast<double>(tiles * s)) + kSplit[i] + kCta[i] * (tiles * s);
             }
             if (t >= best_t - 1e-9) continue;
             if (s > 1) {
@@ -531,8 +535,8 @@ GemmPlan pick_gemm(int N, int K, int M, int sms, int dev)
 }
 
 // Up to this many tokens the batched GEMV kernel takes the call (exact
-// weights; 5120 x 3072 over 8 tokens 4.7 us against 8.3 here, 128256 x 4096
-// over 16 tokens 75 against 81).
+// weights; 5120 x 3072 over 8 tokens 5.3 us against 9.4 here, 128256 x 4096
+// over 16 tokens 82.8 against 85.2).
 constexpr int kGemvTokens = 16;
 
 }  // namespace
