@@ -158,7 +158,7 @@ constexpr int kMmaThreads = (kMmaWarps + 1) * 32;     // + the producer warp
 constexpr int kMmaMaxSlots = 16;
 constexpr int kMmaFullBars = 48;                      // full barriers: nbars = (48 / nslots) * nslots
 constexpr uint32_t kMmaRelease = 1024;                // arrivals that release a slot (see below)
-constexpr int kMmaMaxPart = 384;                      // float4 partial sums [superpair][part][batch]
+constexpr int kMmaMaxPart = 384;                      // float4 partial sums [superpair][part]
 constexpr int kMmaHdrPart = 8 * (kMmaFullBars + kMmaMaxSlots);
 constexpr int kMmaHeader = kMmaHdrPart + 16 * kMmaMaxPart;
 static_assert(kMmaHdrPart % 16 == 0 && kMmaHeader % 128 == 0, "header alignment");
@@ -184,7 +184,6 @@ struct GemvMmaParams {
 // can alias, as in the chain kernel.
 __global__ void __launch_bounds__(kMmaThreads, 1) gemv_mma_kernel(const GemvMmaParams p)
 {
-    constexpr int B = 1;                          // activation rows
     extern __shared__ __align__(1024) uint8_t smem[];
     uint64_t* full = reinterpret_cast<uint64_t*>(smem);
     uint64_t* empty = full + kMmaFullBars;
@@ -247,7 +246,7 @@ __global__ void __launch_bounds__(kMmaThreads, 1) gemv_mma_kernel(const GemvMmaP
     grid_dependents_launch();
     {
         const uint4* xg = reinterpret_cast<const uint4*>(p.x);
-        for (int i = threadIdx.x; i < B * cpr; i += kConsumers) xs[i] = pair_permute(xg[i]);
+        for (int i = threadIdx.x; i < cpr; i += kConsumers) xs[i] = pair_permute(xg[i]);
         named_barrier_sync(1, kConsumers);
     }
     const int J = K >> 8, upp = J / q;
@@ -302,46 +301,32 @@ __global__ void __launch_bounds__(kMmaThreads, 1) gemv_mma_kernel(const GemvMmaP
                     sa[pr] = sbase + ra * (K / 16);
                     sb2[pr] = sbase + rb * (K / 16);
                 }
-                float acc[2][B];
-#pragma unroll
-                for (int pr = 0; pr < 2; ++pr)
-#pragma unroll
-                    for (int b = 0; b < B; ++b) acc[pr][b] = 0.f;
+                float acc[2][1] = {{0.f}, {0.f}};
                 if (spw == 2) {
-                    item_units<B, 2>(ca, cb2, sa, sb2, xsa, cpr, jb, je, acc);
+                    item_units<1, 2>(ca, cb2, sa, sb2, xsa, cpr, jb, je, acc);
                 } else {
                     const uint32_t ca1[1] = {ca[0]}, cb1[1] = {cb2[0]}, sa1[1] = {sa[0]}, sb1[1] = {sb2[0]};
-                    float (&acc1)[1][B] = *reinterpret_cast<float (*)[1][B]>(&acc[0]);
-                    item_units<B, 1>(ca1, cb1, sa1, sb1, xsa, cpr, jb, je, acc1);
+                    float (&acc1)[1][1] = *reinterpret_cast<float (*)[1][1]>(&acc[0]);
+                    item_units<1, 1>(ca1, cb1, sa1, sb1, xsa, cpr, jb, je, acc1);
                 }
-#pragma unroll
-                for (int pr = 0; pr < 2; ++pr)
-#pragma unroll
-                    for (int b = 0; b < B; ++b) acc[pr][b] = pair_reduce(acc[pr][b]);
+                const float r0 = pair_reduce(acc[0][0]), r1 = pair_reduce(acc[1][0]);
                 if (q == 1) {
                     // whole superpairs: lane 0 writes rows 2w (and 2w + 2), lane 16
                     // rows 2w + 1 (and 2w + 3)
                     const int n0 = 2 * (w0 + sw0) + (lane == 16 ? 1 : 0);
                     if (lane == 0 || lane == 16) {
-#pragma unroll
-                        for (int b = 0; b < B; ++b) {
-                            uint16_t* out = p.y + static_cast<size_t>(b) * N;
-                            if (n0 < N) out[n0] = float_to_half_bits(acc[0][b]);
-                            if (spw == 2 && sw0 + 1 < nwd && n0 + 2 < N) out[n0 + 2] = float_to_half_bits(acc[1][b]);
-                        }
+                        if (n0 < N) p.y[n0] = float_to_half_bits(r0);
+                        if (spw == 2 && sw0 + 1 < nwd && n0 + 2 < N) p.y[n0 + 2] = float_to_half_bits(r1);
                     }
                 } else {
-                    float* pf = reinterpret_cast<float*>(part + (sl * q + pt) * B);
-#pragma unroll
-                    for (int b = 0; b < B; ++b) {
-                        if (lane == 0) {
-                            pf[4 * b + 0] = acc[0][b];
-                            pf[4 * b + 2] = acc[1][b];
-                        }
-                        if (lane == 16) {
-                            pf[4 * b + 1] = acc[0][b];
-                            pf[4 * b + 3] = acc[1][b];
-                        }
+                    float* pf = reinterpret_cast<float*>(part + sl * q + pt);
+                    if (lane == 0) {
+                        pf[0] = r0;
+                        pf[2] = r1;
+                    }
+                    if (lane == 16) {
+                        pf[1] = r0;
+                        pf[3] = r1;
                     }
                 }
             }
@@ -350,26 +335,24 @@ __global__ void __launch_bounds__(kMmaThreads, 1) gemv_mma_kernel(const GemvMmaP
         }
     }
     if (q > 1) {
-        // every part is in: add them in part order, one thread per (superpair, row)
+        // every part is in: add them in part order, one thread per superpair
         named_barrier_sync(1, kConsumers);
-        for (int e = threadIdx.x; e < nsp * B; e += kConsumers) {
-            const int sl = e / B, b = e - sl * B;
-            const float4* pp = part + sl * q * B + b;
+        for (int sl = threadIdx.x; sl < nsp; sl += kConsumers) {
+            const float4* pp = part + sl * q;
             float4 sum = pp[0];
             for (int r = 1; r < q; ++r) {
-                const float4 t = pp[r * B];
+                const float4 t = pp[r];
                 sum.x += t.x;
                 sum.y += t.y;
                 sum.z += t.z;
                 sum.w += t.w;
             }
             const int n = 2 * (w0 + (sl << sps));
-            uint16_t* out = p.y + static_cast<size_t>(b) * N;
-            out[n] = float_to_half_bits(sum.x);
-            if (n + 1 < N) out[n + 1] = float_to_half_bits(sum.y);
+            p.y[n] = float_to_half_bits(sum.x);
+            if (n + 1 < N) p.y[n + 1] = float_to_half_bits(sum.y);
             if (spw == 2 && (sl << sps) + 1 < nwd) {
-                out[n + 2] = float_to_half_bits(sum.z);
-                if (n + 3 < N) out[n + 3] = float_to_half_bits(sum.w);
+                p.y[n + 2] = float_to_half_bits(sum.z);
+                if (n + 3 < N) p.y[n + 3] = float_to_half_bits(sum.w);
             }
         }
     }
@@ -529,7 +512,7 @@ struct MmaPlan {
     size_t smem;
 };
 
-bool plan_mma(const DeviceInfo* di, int N, int K, int B, MmaPlan* pl)
+bool plan_mma(const DeviceInfo* di, int N, int K, MmaPlan* pl)
 {
     const int nw = (N + 1) / 2;
     const int grid = nw < di->sm_count ? nw : di->sm_count;
@@ -537,7 +520,7 @@ bool plan_mma(const DeviceInfo* di, int N, int K, int B, MmaPlan* pl)
     const size_t word_bytes = 2 * (static_cast<size_t>(K) / 2 + static_cast<size_t>(K) / 16);
     const int spw = (2 * word_bytes <= 20 * 1024 && nwc >= 2) ? 2 : 1;
     const size_t sp_bytes = spw * word_bytes;
-    const size_t x_bytes = align_up(static_cast<size_t>(B) * K * 2, 128);
+    const size_t x_bytes = align_up(static_cast<size_t>(K) * 2, 128);
     if (static_cast<size_t>(di->smem_optin) < kMmaHeader + x_bytes) return false;
     const size_t avail = static_cast<size_t>(di->smem_optin) - kMmaHeader - x_bytes;
     size_t per = sp_bytes < 20 * 1024 ? (20 * 1024) / sp_bytes : 1;
@@ -553,12 +536,12 @@ bool plan_mma(const DeviceInfo* di, int N, int K, int B, MmaPlan* pl)
     const int J = K / 256;
     const int nsp = (nwc + spw - 1) / spw;
     const int sp_per_chunk = static_cast<int>((slot_bytes / word_bytes) / spw);
-    const double unit = (spw == 2 ? 300.0 : 200.0) * (1.0 + 0.5 * (B - 1));
+    const double unit = spw == 2 ? 300.0 : 200.0;
     int best_q = 0;
     double best = 0.0;
     for (int qq = 1; qq <= J; ++qq) {
         if (J % qq) continue;
-        if (qq > 1 && nsp * qq * B > kMmaMaxPart) continue;
+        if (qq > 1 && nsp * qq > kMmaMaxPart) continue;
         const int ips = sp_per_chunk * qq;
         const int first_chunks = (kMmaWarps + ips - 1) / ips;
         if (first_chunks > nslots - 2 || nslots + first_chunks > nbars) continue;
@@ -656,7 +639,7 @@ int launch_gemv(const uint32_t* W, const uint16_t* s, const uint16_t* x, uint16_
         (batch >= 2 && bulk && path != 2 && (path == 1 || !cuda_cores(batch, N, K, di->sm_count))))
         return launch_bgemv(di, W, s, x, y, N, K, batch, stream);
     MmaPlan mp;
-    if (path != 2 && (weights >= kMmaMinWeights || path == 1) && batch == 1 && bulk && plan_mma(di, N, K, batch, &mp)) {
+    if (path != 2 && (weights >= kMmaMinWeights || path == 1) && batch == 1 && bulk && plan_mma(di, N, K, &mp)) {
         GemvMmaParams p;
         p.W = W;
         p.s = s;
