@@ -1,31 +1,34 @@
-// wq4_bgemv.cu -- the fused dequantize x GEMV for several activation rows
-// (batch 3-32, and batch 1-2 where the TMA-staged kernels do not apply): one
+// wq4_bgemv.cu -- the fused dequantize x GEMV for several activation rows: one
 // decode step of a serving batch through one projection (Section 3, Table 1).
+// It takes batch 5-32, batch 2-4 but for few long rows (and batch 2 below 8 Mi
+// weights), rows that bulk copies cannot take from the sizes on where its ring
+// wins (cuda_cores and copy_ring, wq4_gemv.cu), and wq4_gemm's calls of up to 16
+// tokens.
 //
 // y[b][n] = fp16( sum_k (q(n,k) - 7) * s[n][k/32] * x[b][k] )
 //
-// The contraction runs on mma.sync m16n8k16 with the activations as the 16
-// rows and eight weight rows as the columns: per 32-code group and tile of
-// eight rows two MMAs add the group's exact fp16 products (q - 7) x in fp32,
-// and the group's scales multiply the fp32 result into the running sums, so
-// no weight is ever rounded and every fp16 scale is valid.  (tcgen05 would
-// need the scale inside the fp16 operand, or one accumulator per group.)
+// The contraction runs on mma.sync m16n8k16: per 32-code group two MMAs add the
+// group's exact fp16 products (q - 7) x in fp32, and the group's scales multiply
+// the fp32 result into the running sums, so no weight is ever rounded and every
+// fp16 scale is valid.  (tcgen05 would need the scale inside the fp16 operand,
+// or one accumulator per group.)  A CTA owns tiles of weight rows; its warps
+// are row groups times slices of every K chunk, and the slices' sums are added
+// in slice order in shared memory at the tile's end: the same inputs give the
+// same bits.  The next tile's chunks are in flight while a tile is finished.
 //
-// A CTA owns tiles of 8 R RG weight rows; its 16 warps are RG row groups of R
-// tiles times KS slices of every K chunk, and the slices' sums are added in
-// slice order in shared memory at the tile's end: the same inputs give the
-// same bits.  Chunks of KG groups (codes, scales, activations) move through a
-// four-stage cp.async ring; rows are padded so that ldmatrix of the codes and
-// the 16-byte loads of the activations are free of bank conflicts.  The next
-// tile's chunks are in flight while a tile is finished.
+// Two kernels:
+//  * bgemv_tma_kernel (K % 256 == 0, 16-byte aligned scales): the tile loop of
+//    wq4_tiles.cuh, weights as the MMA's 16 rows, chunks by tensor copies.
+//  * bgemv_kernel (other rows): activations as the 16 rows and eight weight rows
+//    as the columns, 16 warps, chunks of KG groups through a four-stage cp.async
+//    ring, rows padded so that ldmatrix of the codes and the 16-byte loads of
+//    the activations are free of bank conflicts.
 //
-// Two forms: rows that tensor copies can take (K % 256 == 0, 16-byte aligned
-// scales) run in bgemv_tma_kernel below, others in bgemv_kernel.  Measured
-// (us a launch in a graph over rotated copies, before: CUDA-core kernels that
-// read the activations through L1): 3072 x 8192 batch 8 76.5 -> 6.9,
-// 16384 x 3072 batch 8 100 -> 8.8 and batch 32 387 -> 17.3, 128256 x 4096
-// batch 8 927 -> 54.6 (5.4 TB/s) and batch 32 3739 -> 118; 1003 x 2080 (copy
-// ring) batch 5 7.3 -> 4.1.  Up to batch 8 the wide shapes are bound by
+// Measured (us a launch in a graph over copies of 520 MB, before: CUDA-core
+// kernels that read the activations through L1): 3072 x 8192 batch 8 76.5 ->
+// 6.9, 16384 x 3072 batch 8 100 -> 8.8 and batch 32 387 -> 17.4, 128256 x 4096
+// batch 8 927 -> 54.7 (5.4 TB/s) and batch 32 3739 -> 119; 1003 x 2080 (copy
+// ring) batch 5 7.3 -> 4.5.  Up to batch 8 the wide shapes are bound by
 // instruction issue and HBM together, at batch 32 by the MMAs (two per tile,
 // group and eight activation rows) and their issue; the narrow ones by the
 // launch and a chunk's latency.

@@ -585,10 +585,10 @@ __device__ __forceinline__ float warp_allsum(float v)
 // time the queries have.  (Read by the warps themselves once the queries were
 // in, they cost ~5 us of latency a layer: 3B, 4096 tokens, 1212 -> 1082 us a
 // token; the flagged exchange between the ranges 1082 -> 1017, the combine of
-// four heads at a time 1017 -> 979.)  The new token's key and value are polled with the queries.  The
-// warps take blocks of 16 tokens in ring order, keeping a running maximum, sum
-// and weighted value sum per query head of the group; they are combined in
-// shared memory in warp order (one head at a time).  With one range the unit
+// four heads at a time 1017 -> 979.)  The new token's key and value are polled
+// with the queries.  The warps take blocks of 16 tokens in ring order, keeping a
+// running maximum, sum and weighted value sum per query head of the group; they
+// are combined in shared memory in warp order (four heads at a time).  With one range the unit
 // publishes a = o / l itself; otherwise it publishes its (o, m, l), and each of
 // the S_b ranges merges its share of the output over all of them.
 // Shared memory: xs area = qs[G][128] | wp[min(G, kAttnHeads)][NW][kAttnPart];
@@ -1510,12 +1510,11 @@ __global__ void __launch_bounds__((NW + 1) * 32, 1)
 // fused epilogues (wq4_stage.cu); they write the same workspace traces as the
 // persistent kernel.
 
-// Decode step of the graph path: one block per batch row rotates q and k of
-// layer l's QKV output (the same fp64 rotation as the persistent kernel),
-// writes the traces, appends k and v to the cache and sets the row's
-// sequence length (positions + 1; 0 for an invalid position).  Launched
-// after the QKV stage with programmatic dependent launch: it reads the QKV
-// output only after that grid has completed.
+// Decode step of the graph path: a word a thread, some blocks a batch row, rotate
+// q and k of layer l's QKV output (by the token's table, the same fp64 rotation
+// as the persistent kernel), write the traces and append k and v to the cache.
+// Launched after the QKV stage with programmatic dependent launch: it reads the
+// QKV output only after that grid has completed.
 struct RopeAppendArgs {
     const uint16_t* qkv;        // [B][Nqkv]
     uint16_t* qr;               // [B][H] rotated queries

@@ -49,10 +49,10 @@ bool encode_tensor_map_3d(CUtensorMap* m, CUtensorMapDataType dt, const void* ba
                           const std::array<uint64_t, 2>& strides, const std::array<uint32_t, 3>& box,
                           CUtensorMapSwizzle swz);
 
-// wq4_gemv for the batches and sizes that the TMA-staged kernels do not take
-// (wq4_bgemv.cu): any N, K % 32 == 0, batch 1-32, scales at any 2-byte address.
-// check_scales (16-byte aligned scales, K % 256 == 0 only): flag scales beyond
-// +-8188 in the status word, as wq4_gemm promises.
+// The batched GEMV (wq4_bgemv.cu): any N, K % 32 == 0, batch 1-32, scales at any
+// 2-byte address.  check_scales (a call of wq4_gemm; 16-byte aligned scales, K %
+// 256 == 0, batch <= 16 only): flag scales beyond +-8188 in the status word and
+// copy weights only after the previous kernel, as wq4_gemm promises.
 int launch_bgemv(const DeviceInfo* di, const uint32_t* W, const uint16_t* s, const uint16_t* x, uint16_t* y, int N,
                  int K, int batch, cudaStream_t stream, bool check_scales = false);
 

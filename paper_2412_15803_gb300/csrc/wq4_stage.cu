@@ -9,10 +9,11 @@
 // every stage output, and per tile the sums of squares from which the next
 // stage's RMS factors follow.  A warp beside the producer computes this
 // stage's factors while the tiles run.  Weights may be fetched before the
-// previous stage has finished; its outputs are read after.
+// previous stage has finished, its outputs are read after: on the SMs that it
+// leaves free, that is, since two blocks of ~200 KB do not share one.
 //
-// Measured (us a token, 3B shape, batch 4 / 8 / 16 / 32): 773 / 809 / 1115 /
-// 1878, against 1176 / 1228 / 1349 / 2171 with tcgen05 stages, whose
+// Measured (us a token, 3B shape, batch 4 / 8 / 16 / 32): 783 / 822 / 1093 /
+// 1866, against 1176 / 1228 / 1349 / 2171 with tcgen05 stages, whose
 // MMA-issuing lanes and K parts' exchange through global memory took most of
 // a narrow stage.  Bound by each stage's launch, first chunk and epilogue
 // (~3 us of ~7 at batch 8), then as the tile loop.

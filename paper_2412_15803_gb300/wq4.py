@@ -247,7 +247,7 @@ def wq4_decode_step_host(table: wq4_layer_table, attn: wq4_decode_attn, x_host, 
 
 
 def wq4_test_gemv_path(path: int) -> None:
-    """Test hook: 0 size rule, 1 legacy-tensor-path kernel, 2 CUDA-core kernel (batch 1-2)."""
+    """Test hook: 0 size rule, 1 legacy-tensor-path kernel, 2 CUDA-core kernel (batch 1-4)."""
     _check("wq4_test_gemv_path", load().wq4_test_gemv_path(path))
 
 

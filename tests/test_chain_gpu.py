@@ -108,9 +108,9 @@ def check_logits(model, logits, rows=None):
 
 @pytest.mark.parametrize("batch", [1, 2, 3, 4, 5, 6, 7, 8, 9, 13, 17, 32])
 def test_tiny_chain_every_stage_every_element(batch):
-    """Batch 1-2: the persistent kernel; 3-32: the graph of tensor-core stage
-    kernels (batch padded to 16 up to 16, else to 32; 13 and 17 leave a
-    partly padded group of four batch rows)."""
+    """Batch 1-2: the persistent kernel; 3-32: the graph of stage kernels (batch
+    padded to tiles of eight activation rows: whole ones, partly padded ones,
+    one to four of them)."""
     model = DecodeModel(TINY, batch=batch, seed=batch)
     x = synth.activations(100 + batch, batch, TINY.hidden)
     logits = run(model, x)
@@ -132,7 +132,7 @@ def test_tiny_chain_every_stage_every_element(batch):
 def test_chain_full_range_codes_every_element(shape, batch):
     """Codes uniform on 0..15 (every code value, code 15 = weight 8 s, on
     every path: the persistent kernel's exact tensor-path dequantization at
-    batch 1-2, the fp16 dequantized weights of the stage graph at 3-32);
+    batch 1-2, the exact weights of the stage kernels at 3-32);
     every stage, every element, and the logits."""
     model = DecodeModel(shape, batch=batch, seed=40 + batch, symmetric=False)
     x = synth.activations(140 + batch, batch, shape.hidden)
@@ -193,7 +193,7 @@ def test_plan_rebuilds_when_table_changes():
 @pytest.mark.parametrize("batch", [1, 3, 8])
 def test_3b_chain_full_size_sampled(batch):
     """The 28-layer 3B-shaped chain at batch 1 (the persistent kernel, as the
-    benchmark runs it) and at batch 3 and 8 (the tensor-core stage graph):
+    benchmark runs it) and at batch 3 and 8 (the graph of stage kernels):
     sampled rows of every projection of three layers, and of the LM head."""
     model = DecodeModel(SHAPE_3B, batch=batch, seed=0)
     x = synth.activations(0, batch, SHAPE_3B.hidden)
@@ -217,8 +217,8 @@ def test_3b_chain_full_size_sampled(batch):
 @pytest.mark.parametrize("shape,batch", [(SHAPE_3B, 1), (SHAPE_3B, 8), (SHAPE_8B, 1)], ids=["3b-b1", "3b-b8", "8b-b1"])
 def test_full_size_every_layer_every_element(shape, batch):
     """Full-size chains checked whole: the 28-layer 3B shape at batch 1 (the
-    benchmarked configuration, persistent kernel) and 8 (tensor-core stage
-    graph), the 32-layer 8B shape at batch 1: every output element of every
+    benchmarked configuration, persistent kernel) and 8 (graph of stage
+    kernels), the 32-layer 8B shape at batch 1: every output element of every
     projection of every layer (stage by stage, each on the GPU's own input to
     that stage; residual adds bit-exact) and every logit, against the oracle.
     The host side (weights regenerated from the seeded generator, the fp64
@@ -255,10 +255,10 @@ def test_full_size_every_layer_every_element(shape, batch):
 def test_8b_chain_full_size_sampled(batch):
     """The 32-layer 8B-shaped chain over the batch sweep: batch 1-2 on the
     persistent kernel (the longest rows, K = 14336 in the down projection,
-    one row pair per item), 4-32 on the tensor-core stage graph (batch 5: a
-    partly padded group of four batch rows; batch 17-32: 32-column tiles and
-    8-part K splits at K = 14336).  Sampled rows of three layers and of the
-    LM head, and twenty tokens with identical bits."""
+    one row pair per item), 4-32 on the graph of stage kernels (batch 5: a
+    partly padded tile of eight activation rows; 8 and 16: whole ones, 16
+    consumer warps; 32: four tiles, eight warps).  Sampled rows of three
+    layers and of the LM head, and twenty tokens with identical bits."""
     sh = SHAPE_8B
     model = DecodeModel(sh, batch=batch, seed=3)
     x = synth.activations(5, batch, sh.hidden)
@@ -280,8 +280,8 @@ def test_8b_chain_full_size_sampled(batch):
 @pytest.mark.parametrize("batch", [1, 8])
 def test_phi_chain_full_size_sampled(batch):
     """The Phi-3.5-mini-shaped chain (32 layers, 32 + 32 heads of 96, QKV
-    9216 x 3072, vocabulary 32064: the LM head's last 128-row tile is
-    partial) on the persistent kernel (batch 1) and the tensor-core graph
+    9216 x 3072, vocabulary 32064: no multiple of the LM head's row tiles)
+    on the persistent kernel (batch 1) and the graph of stage kernels
     (batch 8): sampled rows of three layers and of the LM head."""
     sh = SHAPE_PHI
     model = DecodeModel(sh, batch=batch, seed=7)

@@ -153,7 +153,7 @@ def test_tiny_step_every_stage(positions):
 @pytest.mark.parametrize("positions", [[0, 17, 300], [31, 32, 33, 64, 5, 1, 250, 999]])
 def test_tiny_step_graph_path(positions):
     """Batch 3 and 8: the graph path's rotation/append kernel and
-    wq4_paged_attention between the tensor-core stages."""
+    wq4_paged_attention between the stage kernels."""
     model, caches, x, logits = step_and_check(TINY, positions, seed=20 + len(positions))
     check_logits(model, logits)
 

@@ -1,5 +1,5 @@
-"""GPU parity of the batched GEMV kernels (batch 2-32) at the edges of their
-tiles, against the fp64 oracle: every element within
+"""GPU parity of wq4_gemv at batch 2-32 at the edges of its kernels' tiles,
+against the fp64 oracle: every element within
 |y_gpu - y_ref| <= 1e-3 * sum_k |w x| + ulp16(|y_ref|).
 """
 import numpy as np
