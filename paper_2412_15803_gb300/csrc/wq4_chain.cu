@@ -1107,12 +1107,13 @@ __global__ void __launch_bounds__((NW + 1) * 32, 1)
             int ord = 0;                // ring ordinal of the next chunk
             int slot = 0, round = 0;    // its slot and the slot's use count
             int fbi = 0;                // its full barrier
-            // Cached tokens of a chunk, its whole pages and the rest.  (This lane's
-            // instructions bound long contexts: a chunk's first page is carried on, a
-            // division a chunk cost more than the look for shared tokens.)
-            [[maybe_unused]] int ct = 0, ctp = 0, ctr = 0;
-            if constexpr (ATT != 0) {
-                ct = attn_chunk_tokens(p.slot_bytes);
+            // Batch 2: whole pages of a chunk of cached tokens and the rest.  (This lane's
+            // instructions bound long contexts there: a chunk's first page is carried on,
+            // a division a chunk cost more than the look for shared tokens.  At batch 1,
+            // without that look, the division is as fast up to 4096 tokens.)
+            [[maybe_unused]] int ctp = 0, ctr = 0;
+            if constexpr (ATT != 0 && B == 2) {
+                const int ct = attn_chunk_tokens(p.slot_bytes);
                 ctp = ct / p.P;
                 ctr = ct - ctp * p.P;
             }
@@ -1125,21 +1126,28 @@ __global__ void __launch_bounds__((NW + 1) * 32, 1)
                     // the cached keys and values of this CTA's attention ranges
                     if (g.type == kO) {
                         const int* pos_sh = reinterpret_cast<const int*>(smem + p.rope_off + kPosOff);
+                        const int ct = attn_chunk_tokens(p.slot_bytes);
                         for (int u = blockIdx.x; u < B * p.Hkv * p.S; u += gridDim.x) {
                             AttnUnit au;
                             if (!attn_unit<B>(p, g.layer, pos_sh, u, &au)) continue;
                             AttnShared sh = attn_shared<B>(p, g.layer, au, pos_sh);
-                            int p0 = au.t0 / p.P, row = au.t0 - p0 * p.P;
+                            [[maybe_unused]] int p0 = 0, row = 0;
+                            if constexpr (B == 2) {
+                                p0 = au.t0 / p.P;
+                                row = au.t0 - p0 * p.P;
+                            }
                             for (int ta = au.t0; ta < au.te; ta += ct, ++ord) {
                                 if (round > 0) mbar_wait(&empty[slot], (round - 1) & 1, p.err);
                                 if constexpr (B == 2)
                                     sh.tokens = reinterpret_cast<uint64_t*>(smem + p.rope_off + attn_shared_off<B>()) + slot;
-                                attn_copy<B>(p, g.layer, au, p0, ta, min(au.te, ta + ct), ct,
+                                attn_copy<B>(p, g.layer, au, B == 2 ? p0 : ta / p.P, ta, min(au.te, ta + ct), ct,
                                              slots + static_cast<size_t>(slot) * p.slot_bytes, &full[fbi], pol, sh);
-                                p0 += ctp;
-                                if ((row += ctr) >= p.P) {
-                                    row -= p.P;
-                                    ++p0;
+                                if constexpr (B == 2) {
+                                    p0 += ctp;
+                                    if ((row += ctr) >= p.P) {
+                                        row -= p.P;
+                                        ++p0;
+                                    }
                                 }
                                 if (++slot == p.nslots) {
                                     slot = 0;
