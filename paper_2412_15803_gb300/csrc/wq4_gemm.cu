@@ -488,8 +488,8 @@ struct GemmPlan {
 
 // Token tile and K split: the least estimated time.  Per 64-wide K chunk a
 // tile takes (us, one CTA alone .. every SM busy) 0.188 .. 0.205 with 64
-// tokens, 0.203 .. 0.235 with 128, 0.22 .. 0.285 with 192 and 0.287 .. 0.394
-// with 256, beside a launch's fixed 2.3, 2.65, 3.4 and 4.2; a split (the
+// tokens, 0.203 .. 0.235 with 128, 0.214 .. 0.304 with 192 and 0.287 .. 0.394
+// with 256, beside a launch's fixed 2.3, 2.65, 3.3 and 4; a split (the
 // cluster's CTAs take K blocks in order, one tile a cluster, all resident)
 // adds 1.3, 1.5 or 1.7 and 0.016, 0.023 or 0.03 a CTA.  Fitted to every choice
 // over 34 sizes, each over copies of 520 MB: the picks are 0.1 % from the best on
@@ -499,8 +499,8 @@ struct GemmPlan {
 GemmPlan pick_gemm(int N, int K, int M, int sms, int dev)
 {
     static constexpr int kTok[4] = {64, 128, 192, 256};
-    static constexpr double kB0[4] = {0.188, 0.203, 0.22, 0.287}, kB1[4] = {0.205, 0.235, 0.285, 0.394};
-    static constexpr double kFix[4] = {2.3, 2.65, 3.4, 4.2};
+    static constexpr double kB0[4] = {0.188, 0.203, 0.214, 0.287}, kB1[4] = {0.205, 0.235, 0.304, 0.394};
+    static constexpr double kFix[4] = {2.3, 2.65, 3.3, 4.0};
     static constexpr double kSplit[4] = {1.3, 1.5, 1.7, 1.7}, kCta[4] = {0.0155, 0.023, 0.03, 0.03};
     GemmPlan best;
     double best_t = 1e300;
